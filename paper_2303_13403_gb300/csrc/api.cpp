@@ -401,14 +401,21 @@ pqmc_status build_ctx(int n, const pqmc_chain_spec* specs, const pqmc_opts* opts
   }
   ctx->off_last = take((size_t)n * kRecord * 8);
   // default CTA size (measured on GB300): the FP64 path packs 4 chains of 64
-  // threads per SM; the reduced paths 2 chains of 256 threads, whose G and
+  // threads per SM, or 2 of 128 or 1 of 256 when the batch leaves the SMs room
+  // (304 chains of 72 sites, 2Theta = 4: 90.4 ms per sweep with 64 threads,
+  // 74.6 with 128; one chain of 72 sites finishes in half the time with 256);
+  // the reduced paths 2 chains of 256 threads, whose G and
   // scratch then fit in shared memory at 72 sites, and one chain of 512
   // threads per SM once a chain has 128 sites or more (its G lives in global
   // memory and more warps hide the latency: 1.4-1.6x at 162-648 sites)
   int nmax_sites = 0;
   for (const HostChain& h : ctx->chains) nmax_sites = std::max(nmax_sites, h.N);
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int fp64_tpb = n <= sms ? 256 : n <= 2 * sms ? 128 : 64;
   const int reduced_tpb = (nmax_sites >= 128 && !o.dense_chains) ? 512 : 256;
-  ctx->tpb = o.cta_threads != 0 ? o.cta_threads : (ctx->prec == PQMC_FP64 ? (o.spread ? 256 : 64) : reduced_tpb);
+  ctx->tpb = o.cta_threads != 0 ? o.cta_threads : (ctx->prec == PQMC_FP64 ? (o.spread ? 256 : fp64_tpb) : reduced_tpb);
   {
     ctx->boost = (ctx->prec != PQMC_FP64 && o.dense_chains) ? 1 : 0;
     const size_t cap = smem_resident_cap(ctx->prec, ctx->tpb, ctx->boost);

@@ -123,8 +123,9 @@ PQMC_HDI constexpr size_t al16(size_t v) { return (v + 15) & ~(size_t)15; }
 // ratios of one decision sub-block, Delta and Delta/R of each accepted flip of
 // a delayed block, accepted sites); the layout is FlipBuf<T> in
 // sweep_kernels.cuh.
+constexpr int kSvLd = kBlock + 4;   // row length of the vector tables in FlipBuf
 PQMC_HDI constexpr size_t flipbuf_bytes(int tsize) {
-  return al16(2 * (size_t)kBlock * (kBlock + 1) * tsize + 2 * (size_t)kBlock * tsize +
+  return al16(2 * (size_t)kBlock * kSvLd * tsize + 2 * (size_t)kBlock * tsize +
               4 * (size_t)kMaxDelay * tsize + 2 * (size_t)kMaxDelay * 4);
 }
 

@@ -223,13 +223,13 @@ __device__ __forceinline__ T* sp_gcur(const ChainDesc& c, int alt, int tsize = (
 template <typename T>
 __global__ void __launch_bounds__(256) sp_decide_kernel(const ChainDesc* chains, uint64_t seed,
                                                         const uint32_t* sweep_ctr, int tau, int i0, int alt, int* err) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
   if (chains[blockIdx.x].st->err) return;
-  Cta<T> x = make_cta<T>(chains[blockIdx.x], smem_raw, 0, seed);
+  setup_cta<T>(chains[blockIdx.x], 0, seed);
+  auto x = this_cta<T, false>();
   load_state(x);
   const ChainDesc& c = x.c;
   x.Gp = sp_gcur<T>(c, alt);
-  decide_sub_block(x, tau, *sweep_ctr, i0, min(kBlock, c.N - i0), 0);
+  decide<true>(x, tau, *sweep_ctr, i0, min(kBlock, c.N - i0), 0);
   __syncthreads();
   x.mark(kPhFlip);
   const int a = x.sh.na;
@@ -470,9 +470,9 @@ enum : int { kSpMeasure = 1, kSpRecord = 2, kSpInit = 4 };
 template <typename T>
 __global__ void __launch_bounds__(256) sp_tail_kernel(const ChainDesc* chains, uint64_t seed, int b, int left,
                                                       int flags, int* err) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
   if (chains[blockIdx.x].st->err) return;
-  Cta<T> x = make_cta<T>(chains[blockIdx.x], smem_raw, 0, seed);
+  setup_cta<T>(chains[blockIdx.x], 0, seed);
+  auto x = this_cta<T, false>();
   load_state(x);
   const ChainDesc& c = x.c;
   Smem<T>& sh = x.sh;

@@ -313,7 +313,10 @@ __device__ void cta_gemm_bf16x3(int M, int Nn, int K, const float* A, int sai, i
 // Buffers of one flip block (lives in shared memory, see make_cta).
 template <typename T>
 struct FlipBuf {
-  T Tu[2][kBlock][kBlock + 1];      // t-V: 1 + (1 - G_SS) Gamma, inverted in place, then M
+  union {
+    T Tu[2][kBlock][kBlock + 1];    // t-V: 1 + (1 - G_SS) Gamma, inverted in place, then M
+    alignas(16) T sv[2][kBlock][kSvLd];   // Hubbard: the update vectors at the accepted sites (sm_vectors)
+  };
   T rs[2][kBlock];                  // ratio R_sigma of each proposal of the decision sub-block
   T cl[2][kMaxDelay];               // Delta of each accepted flip of the delayed block (diagonal of Gamma)
   T fr[2][kMaxDelay];               // Delta / R_sigma of each accepted flip
@@ -348,25 +351,36 @@ struct Smem {
   double dGmax;
   long long n_prop, n_acc, acc_pos;
   int err;
+  int res;                          // G and the scratch live in shared memory
+  uint64_t seed;
+  ScratchLayout L;                  // offsets of the phase buffers in the scratch
+  uint32_t scr_off;                 // RES: the scratch's offset from the shared-memory base
+  uint32_t tcs_off;                 // tensor-core staging area (BF16X3, chains in global memory), or 0
+  uint32_t tmem;                    // its TMEM accumulator
+  double gj_logabs[2], gj_sign[2];  // log|det O| and sign of the last Gauss-Jordan inverse
 };
 
 // One chain CTA: its descriptor, shared memory, and where G and the phase
-// scratch live (shared memory when they fit, else the chain's global buffers).
-template <typename T>
+// scratch live (RES: shared memory, when they fit; else the chain's global
+// buffers).  Each phase of the sweep is a function of its own (not inlined:
+// ptxas gives every phase the whole register budget, where one inlined kernel
+// spilled) that builds its Cta from the shared-memory base, so that with RES
+// every access is a shared-memory instruction on a 32-bit address.
+template <typename T, bool RES>
 struct Cta {
+  static constexpr bool resident = RES;
   const ChainDesc& c;
   Smem<T>& sh;
-  uint64_t seed;
   T* Gp;
   unsigned char* scr;
-  ScratchLayout L;
-  bool resident;
+  const ScratchLayout& L;
   FlipBuf<T>* fb;
-  unsigned char* tcs = nullptr;     // tensor-core staging area (BF16X3, chains in global memory), or null
-  uint32_t tmem = 0;                // its TMEM accumulator
   __device__ T* G(int s) const { return Gp + (long)s * c.N * c.ld; }
   __device__ T* Gt() const { return reinterpret_cast<T*>(scr + L.gt); }
   __device__ T* Ub() const { return reinterpret_cast<T*>(scr + L.u); }
+  // update vectors of spin s: U (column m at m N), V (row m at m ld)
+  __device__ T* Uv(int s) const { return reinterpret_cast<T*>(scr + (s == 0 ? L.u : L.u2)); }
+  __device__ T* Vv(int s) const { return reinterpret_cast<T*>(scr + (s == 0 ? L.w : L.mw)); }
   __device__ T* Wb() const { return reinterpret_cast<T*>(scr + L.w); }
   __device__ double* M64() const { return reinterpret_cast<double*>(scr + L.m64); }
   __device__ double* Q64() const { return reinterpret_cast<double*>(scr + L.mtq); }
@@ -384,6 +398,11 @@ struct Cta {
   __device__ T* QRt() const { return reinterpret_cast<T*>(scr + L.qrt); }
   __device__ T* QLt() const { return reinterpret_cast<T*>(scr + L.qlt); }
   __device__ T* Ot() const { return reinterpret_cast<T*>(scr + L.ot); }
+  // staging area of the tensor-core products (when sh.tcs_off != 0)
+  __device__ unsigned char* tcs() const {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    return smem_raw + sh.tcs_off;
+  }
   __device__ double* pval(int s) const { return reinterpret_cast<double*>(scr + L.laux) + s * 3 * c.nmax; }
   __device__ double* pinv(int s) const { return pval(s) + c.nmax; }
   __device__ double* lmul(int s) const { return pval(s) + 2 * c.nmax; }
@@ -424,30 +443,47 @@ struct Cta {
   }
 };
 
-// Path GEMM of the wrap (deep = true, K = N) and of the delayed update
-// (deep = false, K = accepted flips of a block).  On the BF16X3 path the
-// wrap runs as split-precision tensor-core products: tcgen05 MMAs into tensor
-// memory when the CTA holds a staging area for them (a chain kept in global
-// memory on a 512-thread CTA), mma.sync otherwise.  The delayed update is a
-// rank-a correction (a <= 64) whose cost is reading and writing G: it runs
-// in FP32 on the CUDA cores on the BF16X3 path too (measured faster than
-// either tensor-core form at 162-648 sites, and exact to FP32).  FP32 and
-// FP64 paths: CUDA-core FMA.
-template <typename T, typename Epi>
-__device__ void path_gemm(Cta<T>& x, bool deep, int M, int Nn, int K, const T* A, int sai, int sak, const T* B,
-                          int sbk, int sbj, T* C, int sci, int scj, Epi epi) {
+// The Cta of this block, from the shared-memory base (setup_cta has run).
+template <typename T, bool RES>
+__device__ __forceinline__ Cta<T, RES> this_cta() {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  Smem<T>& sh = *reinterpret_cast<Smem<T>*>(smem_raw);
+  unsigned char* dyn = smem_raw + al16(sizeof(Smem<T>));
+  if constexpr (RES) {
+    unsigned char* scr = smem_raw + sh.scr_off;
+    return Cta<T, RES>{sh.desc, sh, reinterpret_cast<T*>(dyn), scr, sh.L, reinterpret_cast<FlipBuf<T>*>(scr + sh.L.fb)};
+  } else {
+    return Cta<T, RES>{sh.desc, sh, reinterpret_cast<T*>(sh.desc.G), reinterpret_cast<unsigned char*>(sh.desc.scratch),
+                       sh.L, reinterpret_cast<FlipBuf<T>*>(dyn)};
+  }
+}
+
+// Product of the wrap in the path's arithmetic.  On the BF16X3 path it runs
+// as split-precision tensor-core products: tcgen05 MMAs into tensor memory
+// when the CTA holds a staging area for them (kTc: 512-thread CTAs, a chain
+// kept in global memory; a kernel that holds tcgen05 code runs one CTA per
+// SM, so the smaller CTAs are built without it), mma.sync otherwise.  The
+// delayed update is a rank-a correction (a <= 64) whose cost is reading and
+// writing G: it runs in FP32 on the CUDA cores on the BF16X3 path too
+// (measured faster than either tensor-core form at 162-648 sites, and exact
+// to FP32).  FP32 and FP64 paths: CUDA-core FMA.
+template <bool kTc, typename T, bool RES, typename Epi>
+__device__ __forceinline__ void wrap_gemm(Cta<T, RES>& x, int n, const T* A, int sai, int sak, const T* B, T* C, int ld,
+                                          Epi epi) {
   if constexpr (std::is_same<T, float>::value) {
-    if (x.c.tc && deep) {
-      if (x.tcs) {
-        cta_gemm_tc(M, Nn, K, A, sai, sak, B, sbk, sbj, C, sci, scj, epi, x.tcs, x.tmem, &x.sh.err, kErrTimeout);
-        __syncthreads();
-      } else {
-        cta_gemm_bf16x3(M, Nn, K, A, sai, sak, B, sbk, sbj, C, sci, scj, epi);
+    if (x.c.tc) {
+      if constexpr (kTc && !RES) {
+        if (x.sh.tcs_off) {
+          cta_gemm_tc(n, n, n, A, sai, sak, B, ld, 1, C, ld, 1, epi, x.tcs(), x.sh.tmem, &x.sh.err, kErrTimeout);
+          __syncthreads();
+          return;
+        }
       }
+      cta_gemm_bf16x3(n, n, n, A, sai, sak, B, ld, 1, C, ld, 1, epi);
       return;
     }
   }
-  cta_gemm<T>(M, Nn, K, A, sai, sak, B, sbk, sbj, C, sci, scj, epi);
+  cta_gemm<T>(n, n, n, A, sai, sak, B, ld, 1, C, ld, 1, epi);
 }
 
 // --------------------------------------------------------------------------
@@ -482,8 +518,8 @@ __device__ __forceinline__ T uniform_of(uint64_t m53) {
 // M = Gamma (1 + (1 - G_SS) Gamma)^{-1} of the a accepted flips of a block
 // into fb.Tu[s] for every species s (collective; G is the G of the block
 // start).
-template <typename T>
-__device__ void block_inverse(Cta<T>& x, int a, bool pivot) {
+template <typename T, bool RES>
+__device__ __forceinline__ void block_inverse(Cta<T, RES>& x, int a, bool pivot) {
   FlipBuf<T>& fb = *x.fb;
   const int ld = x.c.ld, ns = x.nspec();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -548,8 +584,8 @@ __device__ void block_inverse(Cta<T>& x, int a, bool pivot) {
   __syncthreads();
 }
 
-template <typename T>
-__device__ void flush_block(Cta<T>& x, int a, bool pivot) {
+template <typename T, bool RES>
+__device__ __forceinline__ void flush_block(Cta<T, RES>& x, int a, bool pivot) {
   const ChainDesc& c = x.c;
   FlipBuf<T>& fb = *x.fb;
   const int N = c.N, ld = c.ld, ns = x.nspec();
@@ -569,7 +605,7 @@ __device__ void flush_block(Cta<T>& x, int a, bool pivot) {
     __syncthreads();
     cta_gemm<T>(a, N, a, &fb.Tu[s][0][0], kBlock + 1, 1, Wbuf, ld, 1, MW, ld, 1, EpiStore());
     __syncthreads();
-    path_gemm<T>(x, false, N, N, a, Ubuf, 1, N, MW, ld, 1, Gs, ld, 1, EpiSub());
+    cta_gemm<T>(N, N, a, Ubuf, 1, N, MW, ld, 1, Gs, ld, 1, EpiSub());
     __syncthreads();
   }
   x.mark(kPhFlush);
@@ -581,57 +617,211 @@ __device__ void flush_block(Cta<T>& x, int a, bool pivot) {
 //     G <- G - (e_i - G_{:,i}) (Delta_i / R_i) G_{i,:}.
 // Written as G <- G - U V over the block: column m of U and row m of V are
 // the vectors of flip m, obtained from the block-start G and the earlier
-// vectors (c = G_{:,s_m} - U V_{:,s_m}, r = G_{s_m,:} - U_{s_m,:} V), one
-// step per flip for the two spins at once (half of the CTA each)
+// vectors (c = G_{:,s_m} - U V_{:,s_m}, r = G_{s_m,:} - U_{s_m,:} V)
 // (sm_vectors, for flips m0..m1-1 once their decisions are taken), then one
 // rank-a product per spin (apply_vectors).  Same result as the block form of
 // flush_block, without the a x a inverse.
+//
+// Step m of any row o or column j needs of the other flips only their
+// vectors' elements at the accepted sites, V_m[s_p] and U_m[s_p] (p > m).  So
+// the chain first runs on the accepted sites alone (sm_core) and leaves those
+// elements in a table; then every row and column of G is an independent
+// thread that keeps its own vector in registers and reads the table as
+// 16-byte broadcasts (sm_vectors): one CTA barrier per block instead of one
+// per flip.  Every element sees the same FMAs in the same order as flip by
+// flip.
+//
+// The loops over the flips stay rolled and move the register window down
+// instead (the element of flip m is always in register 0): unrolled over the
+// 32 flips, one warp runs through 20-40 KB of code once per block and waits
+// for instruction fetches.
+
+// The table of a spin (FlipBuf::sv): V_m[s_p] at row m, column p; U_m[s_p] at
+// row 31 - m, column 31 - p (p > m: above and below the diagonal).
 template <typename T>
-__device__ void sm_vectors(Cta<T>& x, int m0, int m1) {
+__device__ __forceinline__ T& sm_v(T (*tab)[kSvLd], int m, int p) { return tab[m][p]; }
+template <typename T>
+__device__ __forceinline__ T& sm_u(T (*tab)[kSvLd], int m, int p) { return tab[kBlock - 1 - m][kBlock - 1 - p]; }
+
+// The chain on the accepted sites, one warp per spin and role: rows (lane q:
+// row s_q, register p: column s_p; gives the U_m) or columns (transposed; the
+// V_m).  The two roles form the same elements and need no word of each other.
+template <typename T, bool RES>
+__device__ __forceinline__ void sm_core(Cta<T, RES>& x, int m0, int cnt) {
+  const ChainDesc& c = x.c;
+  FlipBuf<T>& fb = *x.fb;
+  const int N = c.N, ld = c.ld;
+  const int lane = threadIdx.x & 31;
+  for (int w = threadIdx.x >> 5; w < 4; w += blockDim.x >> 5) {
+    const int s = w >> 1;
+    const bool row = (w & 1) == 0;
+    const T* Gs = x.G(s);
+    const T* U = x.Uv(s);
+    const T* V = x.Vv(s);
+    T (*tab)[kSvLd] = fb.sv[s];
+    const int sq = fb.gsite[m0 + min(lane, cnt - 1)];
+    T a[kBlock];
+#pragma unroll
+    for (int p = 0; p < kBlock; ++p) {
+      const int sp = fb.gsite[m0 + min(p, cnt - 1)];
+      a[p] = row ? Gs[(long)sq * ld + sp] : Gs[(long)sp * ld + sq];
+    }
+    for (int l = 0; l < m0; ++l) {
+      // flips of the delayed block's earlier sub-blocks
+      const T own = row ? U[(long)l * N + sq] : V[(long)l * ld + sq];
+#pragma unroll
+      for (int p = 0; p < kBlock; ++p) {
+        const int sp = fb.gsite[m0 + min(p, cnt - 1)];
+        a[p] = fma(-own, row ? V[(long)l * ld + sp] : U[(long)l * N + sp], a[p]);
+      }
+    }
+#pragma unroll 1
+    for (int m = 0; m < cnt; ++m) {
+      const T f = fb.fr[s][m0 + m];
+      const int rem = cnt - 1 - m;       // flips after this one
+      if (row) {
+        const T u = (T(0) - a[0]) * f;
+        if (lane > m && lane < cnt) sm_u(tab, m, lane) = u;
+#pragma unroll
+        for (int p0 = 1; p0 < kBlock; p0 += 8)
+          if (p0 <= rem) {
+#pragma unroll
+            for (int p = p0; p < (p0 + 8 < kBlock ? p0 + 8 : kBlock); ++p)
+              a[p - 1] = fma(-u, __shfl_sync(0xffffffffu, a[p], m), a[p]);
+          }
+      } else {
+        const T v = a[0];
+        if (lane > m && lane < cnt) sm_v(tab, m, lane) = v;
+#pragma unroll
+        for (int p0 = 1; p0 < kBlock; p0 += 8)
+          if (p0 <= rem) {
+#pragma unroll
+            for (int p = p0; p < (p0 + 8 < kBlock ? p0 + 8 : kBlock); ++p) {
+              const T u = (T(0) - __shfl_sync(0xffffffffu, a[p], m)) * f;
+              a[p - 1] = fma(-u, v, a[p]);
+            }
+          }
+      }
+    }
+  }
+}
+
+// Four flips k .. k + 3 on a thread's window w of kW elements (register i:
+// flip k + i): the flips' vector elements go out, the later elements take
+// their updates.  No branch inside: the table rows are read ahead of the
+// FMAs (flips beyond cnt work on leftovers that nothing reads).
+template <bool kRow, int kW, typename T>
+__device__ __forceinline__ void sm_four(T (&w)[kBlock], const T (*tab)[kSvLd], int k, int cnt, int j, const int* site,
+                                        const T* fr, T* out, long os) {
+  const T* tr = kRow ? &tab[k][k] : &tab[kBlock - 1 - k][kBlock - 4 - k];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    T cv = w[i];
+    if (kRow) cv = (T(j == site[k + i] ? 1 : 0) - cv) * fr[k + i];
+    if (k + i < cnt) out[(k + i) * os] = cv;
+#pragma unroll
+    for (int q = 0; q < kW; q += 4)
+      if (q + 3 > i) {
+        T t[4];
+        Vec4<T>::load(kRow ? tr + i * kSvLd + q : tr - i * kSvLd - q, t);
+#pragma unroll
+        for (int h = 0; h < 4; ++h)
+          if (q + h > i) w[q + h] = fma(-cv, kRow ? t[h] : t[3 - h], w[q + h]);
+      }
+  }
+#pragma unroll
+  for (int p = 0; p + 4 < kW; ++p) w[p] = w[p + 4];
+}
+
+template <bool kRow, typename T, bool RES>
+__device__ __forceinline__ void sm_line(Cta<T, RES>& x, int s, int j, int m0, int cnt) {
+  const ChainDesc& c = x.c;
+  FlipBuf<T>& fb = *x.fb;
+  const int ld = c.ld;
+  // element p of this line: G[j][s_p] (row) or G[s_p][j] (column)
+  const T* g = kRow ? x.G(s) + (long)j * ld : x.G(s) + j;
+  T* out = kRow ? x.Uv(s) + j : x.Vv(s) + j;
+  const long os = kRow ? c.N : ld;
+  const int* site = fb.gsite + m0;
+  T w[kBlock];
+#pragma unroll
+  for (int p = 0; p < kBlock; ++p) {
+    const int sp = site[min(p, cnt - 1)];
+    w[p] = g[kRow ? sp : sp * ld];
+  }
+  const T* other = kRow ? x.Vv(s) : x.Uv(s);
+  const long ot = kRow ? ld : c.N;
+  for (int l = 0; l < m0; ++l) {         // flips of the delayed block's earlier sub-blocks
+    const T a = out[l * os];
+#pragma unroll
+    for (int p = 0; p < kBlock; ++p) w[p] = fma(-a, other[l * ot + site[min(p, cnt - 1)]], w[p]);
+  }
+  out += m0 * os;
+  int k = 0;
+#pragma unroll 1
+  for (; cnt - k > 16; k += 4) sm_four<kRow, 32>(w, fb.sv[s], k, cnt, j, site, fb.fr[s] + m0, out, os);
+#pragma unroll 1
+  for (; k < cnt; k += 4) sm_four<kRow, 16>(w, fb.sv[s], k, cnt, j, site, fb.fr[s] + m0, out, os);
+}
+
+// every row of U and every column of V, both spins: a warp takes 32 rows or
+// 32 columns of one spin at a time
+template <typename T, bool RES>
+__device__ __forceinline__ void sm_vectors(Cta<T, RES>& x, int m0, int cnt) {
+  const int N = x.c.N, lane = threadIdx.x & 31;
+  const int groups = (N + 31) >> 5;
+  for (int t = threadIdx.x >> 5; t < 4 * groups; t += blockDim.x >> 5) {
+    const int s = t & 1, j = 32 * (t >> 2) + lane;
+    if (j >= N) continue;
+    if (t & 2) sm_line<true>(x, s, j, m0, cnt);
+    else sm_line<false>(x, s, j, m0, cnt);
+  }
+}
+
+// FP64: flip by flip, one step per flip for the two spins at once (half of
+// the CTA each).  Here the FP64 pipe sets the time (16 cycles per warp
+// instruction and SM): the form above, which repeats the accepted sites'
+// part and works on padding, takes 1.9 times as long.
+template <typename T, bool RES>
+__device__ __forceinline__ void sm_vectors_by_flip(Cta<T, RES>& x, int m0, int m1) {
   const ChainDesc& c = x.c;
   FlipBuf<T>& fb = *x.fb;
   const int N = c.N, ld = c.ld;
   const int half = (int)blockDim.x >> 1;
   const int s = (int)threadIdx.x >= half ? 1 : 0;
   const int t = (int)threadIdx.x - s * half;
-  T* Us[2] = {reinterpret_cast<T*>(x.scr + x.L.u), reinterpret_cast<T*>(x.scr + x.L.u2)};
-  T* Vs[2] = {reinterpret_cast<T*>(x.scr + x.L.w), reinterpret_cast<T*>(x.scr + x.L.mw)};
-  {
-    const T* Gs = x.G(s);
-    T* U = Us[s];
-    T* V = Vs[s];
-    for (int m = m0; m < m1; ++m) {
-      const int sm = fb.gsite[m];
-      const T f = fb.fr[s][m];
-      for (int o = t; o < 2 * N; o += half) {
-        if (o < N) {
-          T cv = Gs[(long)o * ld + sm];
-          for (int l = 0; l < m; ++l) cv = fma(-U[(long)l * N + o], V[(long)l * ld + sm], cv);
-          U[(long)m * N + o] = ((o == sm ? T(1) : T(0)) - cv) * f;
-        } else {
-          const int j = o - N;
-          T rv = Gs[(long)sm * ld + j];
-          for (int l = 0; l < m; ++l) rv = fma(-U[(long)l * N + sm], V[(long)l * ld + j], rv);
-          V[(long)m * ld + j] = rv;
-        }
+  const T* Gs = x.G(s);
+  T* U = x.Uv(s);
+  T* V = x.Vv(s);
+  for (int m = m0; m < m1; ++m) {
+    const int sm = fb.gsite[m];
+    const T f = fb.fr[s][m];
+    for (int o = t; o < 2 * N; o += half) {
+      if (o < N) {
+        T cv = Gs[(long)o * ld + sm];
+        for (int l = 0; l < m; ++l) cv = fma(-U[(long)l * N + o], V[(long)l * ld + sm], cv);
+        U[(long)m * N + o] = ((o == sm ? T(1) : T(0)) - cv) * f;
+      } else {
+        const int j = o - N;
+        T rv = Gs[(long)sm * ld + j];
+        for (int l = 0; l < m; ++l) rv = fma(-U[(long)l * N + sm], V[(long)l * ld + j], rv);
+        V[(long)m * ld + j] = rv;
       }
-      // the two halves step independently: one named barrier per spin
-      if (s == 0) asm volatile("bar.sync 2, %0;" ::"r"(half) : "memory");
-      else asm volatile("bar.sync 3, %0;" ::"r"(half) : "memory");
     }
+    // the two halves step independently: one named barrier per spin
+    if (s == 0) asm volatile("bar.sync 2, %0;" ::"r"(half) : "memory");
+    else asm volatile("bar.sync 3, %0;" ::"r"(half) : "memory");
   }
-  __syncthreads();
-  x.mark(kPhFlushVec);
 }
 
-template <typename T>
-__device__ void apply_vectors(Cta<T>& x, int a) {
+template <typename T, bool RES>
+__device__ __forceinline__ void apply_vectors(Cta<T, RES>& x, int a) {
   const ChainDesc& c = x.c;
   const int N = c.N, ld = c.ld;
   T* Us[2] = {reinterpret_cast<T*>(x.scr + x.L.u), reinterpret_cast<T*>(x.scr + x.L.u2)};
   T* Vs[2] = {reinterpret_cast<T*>(x.scr + x.L.w), reinterpret_cast<T*>(x.scr + x.L.mw)};
   for (int sp = 0; sp < 2; ++sp)
-    path_gemm<T>(x, false, N, N, a, Us[sp], 1, N, Vs[sp], ld, 1, x.G(sp), ld, 1, EpiSub());
+    cta_gemm<T>(N, N, a, Us[sp], 1, N, Vs[sp], ld, 1, x.G(sp), ld, 1, EpiSub());
   __syncthreads();
   x.mark(kPhFlush);
 }
@@ -646,8 +836,8 @@ __device__ void apply_vectors(Cta<T>& x, int a) {
 // (their update vectors in the scratch correct the diagonal block read from
 // G): warps 0 and 1 decide; sh.na receives the accepted count of the delayed
 // block, fb the accepted sites and their Delta, Delta / R.
-template <typename T>
-__device__ void decide_sub_block(Cta<T>& x, int tau, uint32_t sweep, int i0, int nbk, int a_done) {
+template <typename T, bool RES>
+__device__ __forceinline__ void decide_sub_block(Cta<T, RES>& x, int tau, uint32_t sweep, int i0, int nbk, int a_done) {
   const ChainDesc& c = x.c;
   Smem<T>& sh = x.sh;
   FlipBuf<T>& fb = *x.fb;
@@ -680,8 +870,8 @@ __device__ void decide_sub_block(Cta<T>& x, int tau, uint32_t sweep, int i0, int
     T uj = T(2);
     int flj = 1;
     if (colq) {
-      const U4 w = philox4x32_10((uint32_t)(i0 + lane), (uint32_t)tau, sweep, c.chain_index, (uint32_t)x.seed,
-                                 (uint32_t)(x.seed >> 32));
+      const U4 w = philox4x32_10((uint32_t)(i0 + lane), (uint32_t)tau, sweep, c.chain_index, (uint32_t)x.sh.seed,
+                                 (uint32_t)(x.sh.seed >> 32));
       uj = uniform_of<T>(((uint64_t)w.x0 << 21) | (uint64_t)(w.x1 >> 11));
       flj = (int)f[i0 + lane];
     }
@@ -732,27 +922,202 @@ __device__ void decide_sub_block(Cta<T>& x, int tau, uint32_t sweep, int i0, int
   }
 }
 
-template <typename T>
-__device__ void update_slice(Cta<T>& x, int tau, uint32_t sweep) {
+// The same in FP32 by one warp: half-warp s holds spin s's diagonal block,
+// lane q of it the columns q and q + 16 in registers.  A proposal's chain is
+// then two shuffles (the diagonal element, the other spin's ratio), the
+// ratios' arithmetic and a compare, with no barrier; an accepted flip costs
+// one shuffle per future row for both spins together.  Every value is formed
+// by the operations of the two-warp form above, so the decisions and the
+// factors are the same bits.  What a decision leaves behind (fields, logs,
+// sites, Delta) is written after the loop, by all lanes at once.
+template <bool RES>
+__device__ __forceinline__ void decide_sub_block_pair(Cta<float, RES>& x, int tau, uint32_t sweep, int i0, int nbk,
+                                                             int a_done) {
+  if (threadIdx.x >= 32) return;
   const ChainDesc& c = x.c;
-  Smem<T>& sh = x.sh;
-  const int N = c.N;
-  const int kd = c.kb;
+  Smem<float>& sh = x.sh;
+  FlipBuf<float>& fb = *x.fb;
+  const unsigned full = 0xffffffffu;
+  const int N = c.N, ld = c.ld;
+  const int lane = threadIdx.x, s = lane >> 4, q = lane & 15, half = lane & 16;
+  const int kap = x.gutz(tau) ? 1 : 0;
+  int8_t* f = c.fields + (long)tau * c.nfld;
+  const float d0 = (float)c.delta[kap][s][0], d1 = (float)c.delta[kap][s][1];
+  const bool on0 = q < nbk, on1 = q + 16 < nbk;
+  float ga[kBlock], gb[kBlock];
+  {
+    const float* G = x.G(s) + (long)i0 * ld + i0 + q;
+#pragma unroll
+    for (int r = 0; r < kBlock; ++r) {
+      ga[r] = (on0 && r < nbk) ? G[(long)r * ld] : 0.f;
+      gb[r] = (on1 && r < nbk) ? G[(long)r * ld + 16] : 0.f;
+    }
+  }
+  if (a_done > 0) {
+    // G_SS - U_S V_S over the vectors of the block's earlier flips
+    const float* U = reinterpret_cast<const float*>(x.scr + (s == 0 ? x.L.u : x.L.u2)) + i0;
+    const float* V = reinterpret_cast<const float*>(x.scr + (s == 0 ? x.L.w : x.L.mw)) + i0 + q;
+    for (int l = 0; l < a_done; ++l) {
+      const float va = on0 ? V[(long)l * ld] : 0.f, vb = on1 ? V[(long)l * ld + 16] : 0.f;
+#pragma unroll
+      for (int r = 0; r < kBlock; ++r)
+        if (r < nbk) {
+          const float u = U[(long)l * N + r];
+          if (on0) ga[r] = fma(-u, va, ga[r]);
+          if (on1) gb[r] = fma(-u, vb, gb[r]);
+        }
+    }
+  }
+  // lane j: uniform (in the decision precision) and field of site i0 + j
+  float uj = 2.f;
+  int flj = 1;
+  if (lane < nbk) {
+    const U4 w = philox4x32_10((uint32_t)(i0 + lane), (uint32_t)tau, sweep, c.chain_index, (uint32_t)x.sh.seed,
+                               (uint32_t)(x.sh.seed >> 32));
+    uj = uniform_of<float>(((uint64_t)w.x0 << 21) | (uint64_t)(w.x1 >> 11));
+    flj = (int)f[i0 + lane];
+  }
+  const unsigned up = __ballot_sync(full, flj > 0);
+  unsigned accepted = 0;
+  int a = a_done, bad = 0, nneg = 0;
+  float* frs = &fb.fr[s][0];
+  // sites 0..15 (their columns in ga), then 16..31 (in gb).  The loops stay
+  // rolled: the register window moves down one row per proposal, so row j is
+  // always register 0 (see sm_core on code size).
+  const int n_lo = min(nbk, 16);
+#pragma unroll 1
+  for (int j = 0; j < n_lo; ++j) {
+    const float u = __shfl_sync(full, uj, j);
+    const float ds = ((up >> j) & 1u) ? d0 : d1;
+    const float rs = 1.f + ds * (1.f - __shfl_sync(full, ga[0], half | j));
+    const float R = rs * __shfl_xor_sync(full, rs, 16);
+    const float fac = ds / rs;
+    bad |= isfinite(R) ? 0 : 1;
+    const bool acc = u < fabsf(R);     // the same value in every lane
+    // G_rq += c G_rj G_jq for future rows r > j and columns q > j
+    const float ya = acc && q > j ? fac * ga[0] : 0.f, yb = acc ? fac * gb[0] : 0.f;
+    if (acc) {
+      accepted |= 1u << j;
+      nneg += R < 0.f ? 1 : 0;
+      if (q == 0) frs[a] = fac;
+      ++a;
+#pragma unroll
+      for (int r0 = 1; r0 < kBlock; r0 += 8)
+        if (r0 < nbk - j) {
+#pragma unroll
+          for (int r = r0; r < (r0 + 8 < kBlock ? r0 + 8 : kBlock); ++r) {
+            const float xr = __shfl_sync(full, ga[r], half | j);
+            ga[r - 1] = fma(xr, ya, ga[r]);
+            gb[r - 1] = fma(xr, yb, gb[r]);
+          }
+        }
+    } else {
+#pragma unroll
+      for (int r = 1; r < kBlock; ++r) {
+        ga[r - 1] = ga[r];
+        gb[r - 1] = gb[r];
+      }
+    }
+  }
+#pragma unroll 1
+  for (int j = 16; j < nbk; ++j) {
+    const float u = __shfl_sync(full, uj, j);
+    const float ds = ((up >> j) & 1u) ? d0 : d1;
+    const float rs = 1.f + ds * (1.f - __shfl_sync(full, gb[0], half | (j - 16)));
+    const float R = rs * __shfl_xor_sync(full, rs, 16);
+    const float fac = ds / rs;
+    bad |= isfinite(R) ? 0 : 1;
+    const bool acc = u < fabsf(R);
+    const float yb = acc && q + 16 > j ? fac * gb[0] : 0.f;
+    if (acc) {
+      accepted |= 1u << j;
+      nneg += R < 0.f ? 1 : 0;
+      if (q == 0) frs[a] = fac;
+      ++a;
+#pragma unroll
+      for (int r0 = 1; r0 < 16; r0 += 8)
+        if (r0 < nbk - j) {
+#pragma unroll
+          for (int r = r0; r < (r0 + 8 < 16 ? r0 + 8 : 16); ++r)
+            gb[r - 1] = fma(__shfl_sync(full, gb[r], half | (j - 16)), yb, gb[r]);
+        }
+    } else {
+#pragma unroll
+      for (int r = 1; r < 16; ++r) gb[r - 1] = gb[r];
+    }
+  }
+  const bool mine = (accepted >> lane) & 1u;
+  if (mine) {
+    const int at = a_done + __popc(accepted & ((1u << lane) - 1u));
+    const int si = flj > 0 ? 0 : 1;
+    fb.gsite[at] = i0 + lane;
+    fb.cl[0][at] = (float)c.delta[kap][0][si];
+    fb.cl[1][at] = (float)c.delta[kap][1][si];
+    f[i0 + lane] = (int8_t)-flj;
+  }
+  const long long pos0 = sh.acc_pos;
+  if (lane < nbk && pos0 + lane < c.acc_cap) c.acc_log[pos0 + lane] = mine ? 1 : 0;
+  __syncwarp();
+  if (lane == 0) {
+    sh.na = a;
+    sh.acc_pos = pos0 + nbk;
+    sh.n_prop += nbk;
+    sh.n_acc += a - a_done;
+    if (nneg & 1) sh.sign_running = -sh.sign_running;
+    if (bad) sh.err |= kErrNaN;
+  }
+}
+
+// kPair: the one-warp form (FP32 kernels with room for its 64 block registers)
+template <bool kPair, typename T, bool RES>
+__device__ __forceinline__ void decide(Cta<T, RES>& x, int tau, uint32_t sweep, int i0, int nbk, int a_done) {
+  if constexpr (kPair && std::is_same<T, float>::value) decide_sub_block_pair(x, tau, sweep, i0, nbk, a_done);
+  else decide_sub_block(x, tau, sweep, i0, nbk, a_done);
+}
+
+template <typename T, bool RES, bool kPair>
+__device__ __noinline__ void phase_decide(int tau, uint32_t sweep, int i0, int nbk, int a_done) {
+  auto x = this_cta<T, RES>();
+  decide<kPair>(x, tau, sweep, i0, nbk, a_done);
+  __syncthreads();
+  x.mark(kPhFlip);
+}
+template <typename T, bool RES>
+__device__ __noinline__ void phase_vectors(int m0, int m1) {
+  auto x = this_cta<T, RES>();
+  if constexpr (std::is_same<T, double>::value) {
+    sm_vectors_by_flip(x, m0, m1);
+  } else {
+    sm_core(x, m0, m1 - m0);
+    __syncthreads();
+    sm_vectors(x, m0, m1 - m0);
+  }
+  __syncthreads();
+  x.mark(kPhFlushVec);
+}
+template <typename T, bool RES>
+__device__ __noinline__ void phase_apply(int a) {
+  auto x = this_cta<T, RES>();
+  apply_vectors(x, a);
+}
+
+template <typename T, bool RES, bool kPair>
+__device__ __forceinline__ void update_slice(int tau, uint32_t sweep) {
+  auto x = this_cta<T, RES>();
+  const int N = x.c.N;
+  const int kd = x.c.kb;
   const int sub = kd < kBlock ? kd : kBlock;
 
   for (int d0 = 0; d0 < N; d0 += kd) {
     const int d1 = min(d0 + kd, N);
     int a_done = 0;                                  // flips of the delayed block already accepted
     for (int i0 = d0; i0 < d1; i0 += sub) {
-      const int nbk = min(sub, d1 - i0);
-      decide_sub_block(x, tau, sweep, i0, nbk, a_done);
-      __syncthreads();
-      x.mark(kPhFlip);
-      const int a = sh.na;
-      if (a > a_done) sm_vectors(x, a_done, a);
+      phase_decide<T, RES, kPair>(tau, sweep, i0, min(sub, d1 - i0), a_done);
+      const int a = x.sh.na;
+      if (a > a_done) phase_vectors<T, RES>(a_done, a);
       a_done = a;
     }
-    if (a_done > 0) apply_vectors(x, a_done);
+    if (a_done > 0) phase_apply<T, RES>(a_done);
   }
 }
 
@@ -766,8 +1131,8 @@ __device__ void update_slice(Cta<T>& x, int tau, uint32_t sweep) {
 // columns of the later pairs by the rank-2 form
 //     G_rq <- G_rq + sum_{s in S} G_rs (M G_{S,q})_s,  M = Gamma (1 + (1 - G_SS) Gamma)^{-1}.
 // The accepted ends then go to flush_block as one set.
-template <typename T>
-__device__ void update_slice_tv(Cta<T>& x, int tau, uint32_t sweep) {
+template <typename T, bool RES>
+__device__ __forceinline__ void update_slice_tv(Cta<T, RES>& x, int tau, uint32_t sweep) {
   const ChainDesc& c = x.c;
   Smem<T>& sh = x.sh;
   FlipBuf<T>& fb = *x.fb;
@@ -796,8 +1161,8 @@ __device__ void update_slice_tv(Cta<T>& x, int tau, uint32_t sweep) {
         int fp = 1;
         if (lane < np) {
           const int b = 3 * (c0 + lane) + k;
-          const U4 w = philox4x32_10((uint32_t)b, (uint32_t)tau, sweep, c.chain_index, (uint32_t)x.seed,
-                                     (uint32_t)(x.seed >> 32));
+          const U4 w = philox4x32_10((uint32_t)b, (uint32_t)tau, sweep, c.chain_index, (uint32_t)x.sh.seed,
+                                     (uint32_t)(x.sh.seed >> 32));
           up = uniform_of<T>(((uint64_t)w.x0 << 21) | (uint64_t)(w.x1 >> 11));
           fp = (int)f[b];
         }
@@ -875,15 +1240,15 @@ __device__ void update_slice_tv(Cta<T>& x, int tau, uint32_t sweep) {
 // Slice wrapping.  dir = +1: G(tau) = B_tau G(tau-1) B_tau^{-1};
 // dir = -1: G(tau-1) = B_tau^{-1} G(tau) B_tau.
 
-template <typename T>
-__device__ void wrap(Cta<T>& x, int tau, int dir) {
+template <bool kTc, typename T, bool RES>
+__device__ __forceinline__ void wrap(Cta<T, RES>& x, int tau, int dir) {
   const ChainDesc& c = x.c;
   const int N = c.N, ld = c.ld;
   const bool gz = x.gutz(tau);
   T* Gt = x.Gt();
   const T* Em = x.Em();
   const T* Ep = x.Ep();
-  if (!gz && x.resident && x.L.em) {
+  if (!gz && RES && x.L.em) {
     // a chain resident in shared memory reads e^{-+dtau K} there: the two
     // tables are copied in from the L2-resident copy shared by all chains
     // (the wrap phase leaves room for them in the scratch)
@@ -910,17 +1275,17 @@ __device__ void wrap(Cta<T>& x, int tau, int dir) {
     if (gz) return;
     // Gt = e^{-dtau K} G, G = Gt e^{+dtau K}
     for (int s = 0; s < x.nspec(); ++s) {
-      path_gemm<T>(x, true, N, N, N, Em, 1, ld, x.G(s), ld, 1, Gt, ld, 1, EpiStore());
+      wrap_gemm<kTc>(x, N, Em, 1, ld, x.G(s), Gt, ld, EpiStore());
       __syncthreads();
-      path_gemm<T>(x, true, N, N, N, Gt, ld, 1, Ep, ld, 1, x.G(s), ld, 1, EpiStore());
+      wrap_gemm<kTc>(x, N, Gt, ld, 1, Ep, x.G(s), ld, EpiStore());
       __syncthreads();
     }
   } else {
     if (!gz) {
       for (int s = 0; s < x.nspec(); ++s) {
-        path_gemm<T>(x, true, N, N, N, Ep, 1, ld, x.G(s), ld, 1, Gt, ld, 1, EpiStore());
+        wrap_gemm<kTc>(x, N, Ep, 1, ld, x.G(s), Gt, ld, EpiStore());
         __syncthreads();
-        path_gemm<T>(x, true, N, N, N, Gt, ld, 1, Em, ld, 1, x.G(s), ld, 1, EpiStore());
+        wrap_gemm<kTc>(x, N, Gt, ld, 1, Em, x.G(s), ld, EpiStore());
         __syncthreads();
       }
     }
@@ -937,8 +1302,8 @@ __device__ void wrap(Cta<T>& x, int tau, int dir) {
 
 // log|prod_j d_j| and sign(prod_j d_j) of n values in shared memory, summed by
 // warp 0 and broadcast through shared memory (collective).
-template <typename T>
-__device__ void log_det_of(Cta<T>& x, const double* d, int n, int extra_sign_flips, double& logabs, double& sgn) {
+template <typename T, bool RES>
+__device__ __forceinline__ void log_det_of(Cta<T, RES>& x, const double* d, int n, int extra_sign_flips, double& logabs, double& sgn) {
   Smem<T>& sh = x.sh;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   __syncthreads();
@@ -969,8 +1334,8 @@ __device__ void log_det_of(Cta<T>& x, const double* d, int n, int extra_sign_fli
 // columns in three CTA-wide phases (partial column dots over row chunks, one
 // thread per column adds the chunks, a parallel rank-1 update), so no FP64
 // work sits in warp-shuffle reductions.
-template <typename T>
-__device__ void householder_apply(Cta<T>& x, int N, int lda, const double* v, double beta, double* A, int c0, int c1,
+template <typename T, bool RES>
+__device__ __forceinline__ void householder_apply(Cta<T, RES>& x, int N, int lda, const double* v, double beta, double* A, int c0, int c1,
                                   int j) {
   double* part = x.qpart();
   double* w = x.qw();
@@ -1014,8 +1379,8 @@ __device__ void householder_apply(Cta<T>& x, int N, int lda, const double* v, do
 }
 
 // reflector of column j (warp 0): v = x - alpha e_j stored over the column
-template <typename T>
-__device__ void householder_reflector(Cta<T>& x, int N, int ldm, double* M, int j) {
+template <typename T, bool RES>
+__device__ __forceinline__ void householder_reflector(Cta<T, RES>& x, int N, int ldm, double* M, int j) {
   const int lane = threadIdx.x & 31;
   if ((threadIdx.x >> 5) == 0) {
     double* v = M + (long)j * ldm;
@@ -1036,8 +1401,8 @@ __device__ void householder_reflector(Cta<T>& x, int N, int ldm, double* M, int 
   __syncthreads();
 }
 
-template <typename T>
-__device__ void qr_householder(Cta<T>& x, int N, int ldm, int n, double* M, double* Q, double& logabs, double& sgn) {
+template <typename T, bool RES>
+__device__ __forceinline__ void qr_householder(Cta<T, RES>& x, int N, int ldm, int n, double* M, double* Q, double& logabs, double& sgn) {
   for (int j = 0; j < n; ++j) {
     householder_reflector(x, N, ldm, M, j);
     householder_apply(x, N, ldm, M + (long)j * ldm, x.qbeta()[j], M, j + 1, n, j);
@@ -1096,8 +1461,8 @@ static __device__ void gram_upper_f64(int n, int N, int ldm, const double* M, do
 // pivot falls below 1e-12 of its original diagonal entry (cond(M) above about
 // 1e6); the caller then takes the Householder QR.  R has a positive diagonal,
 // so only log|det R| = (1/2) sum_k log(pivot_k) is returned.
-template <typename T>
-__device__ bool qr_cholesky(Cta<T>& x, int N, int ldm, int n, double* M, double* Q, double& logabs) {
+template <typename T, bool RES>
+__device__ __forceinline__ bool qr_cholesky(Cta<T, RES>& x, int N, int ldm, int n, double* M, double* Q, double& logabs) {
   Smem<T>& sh = x.sh;
   double* C = x.chol();                 // n x n row-major (upper part): Gram, then Schur complements
   double* U = C + (long)n * n;          // n x n row-major (upper part): U_kj = R_kj / R_kk
@@ -1215,8 +1580,8 @@ __device__ bool qr_cholesky(Cta<T>& x, int N, int ldm, int n, double* M, double*
 // and saves the pivot column; the CTA then eliminates that column from every
 // other row; the row interchanges are undone on the columns at the end.
 // Returns log|det O_s| and sign(det O_s) to every thread.
-template <typename T>
-__device__ void gj_invert2(Cta<T>& x, const int n[2], double* O[2], double logabs[2], double sgn[2]) {
+template <typename T, bool RES>
+__device__ __forceinline__ void gj_invert2(Cta<T, RES>& x, const int n[2], double* O[2], double logabs[2], double sgn[2]) {
   Smem<T>& sh = x.sh;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nmax = n[0] > n[1] ? n[0] : n[1];
@@ -1347,34 +1712,36 @@ static __device__ void copy_block(const double* src, double* dst, int n) {
   __syncthreads();
 }
 
-template <typename T>
-__device__ double* stack_block(const Cta<T>& x, double* base, int b, int s) {
+template <typename T, bool RES>
+__device__ __forceinline__ double* stack_block(const Cta<T, RES>& x, double* base, int b, int s) {
   return base + ((long)b * 2 + s) * x.c.N * x.c.nmax;
 }
 
 // Right stack block b: QR of B_{b n} ... B_{(b-1)n+1} Q_R[b-1] (b >= 1) or of B_0 P (b = 0).
-// The slice products run in the path precision on a row-major copy.
-template <typename T>
-__device__ void push_R(Cta<T>& x, int b) {
+// Left stack block b holds (B_L(b n))^T = Q T^T: QR of
+// B_{bn+1}^T ... B_{(b+1)n}^T Q_L[b+1] (b < nb) or of e^{V(s_{Ltau+1})} P (b = nb).
+// phase_stack forms the block to factorise, of spin s, in M64: the slice
+// products run in the path precision on a row-major copy.
+template <typename T, bool RES>
+__device__ __noinline__ void phase_stack(int b, int left, int s) {
+  auto x = this_cta<T, RES>();
   const ChainDesc& c = x.c;
   const int N = c.N, n_stab = c.n_stab;
   const int ldm = m64_ld(N);
   double* M = x.M64();
-  for (int s = 0; s < x.nspec(); ++s) {
-    const int n = x.nsig(s);
+  const int n = x.nsig(s);
+  T* Mt = x.Mt();
+  T* Mt2 = x.Mt2();
+  if (left ? b == c.nb : b == 0) {
     const double* P = c.P + (long)s * N * c.nmax;
-    T* Mt = x.Mt();
-    T* Mt2 = x.Mt2();
-    double prev_l = 0.0, prev_s = 1.0;
-    if (b == 0) {
-      x.stage(0);
-      PQMC_FOR_2D(k, 0, n, i, 0, N) M[(long)k * ldm + i] = x.vexp(0, s, i) * P[(long)k * N + i];
-      __syncthreads();
-    } else {
-      const double* prev = stack_block(x, c.Rst, b - 1, s);
-      PQMC_FOR_2D(k, 0, n, i, 0, N) Mt[(long)i * n + k] = (T)prev[(long)k * N + i];
-      prev_l = c.Rlog[((b - 1) * 2 + s) * 2 + 0];
-      prev_s = c.Rlog[((b - 1) * 2 + s) * 2 + 1];
+    const int tau = left ? c.Ltau + 1 : 0;
+    x.stage(tau);
+    PQMC_FOR_2D(k, 0, n, i, 0, N) M[(long)k * ldm + i] = x.vexp(tau, s, i) * P[(long)k * N + i];
+    __syncthreads();
+  } else {
+    const double* prev = left ? stack_block(x, c.Lst, b + 1, s) : stack_block(x, c.Rst, b - 1, s);
+    PQMC_FOR_2D(k, 0, n, i, 0, N) Mt[(long)i * n + k] = (T)prev[(long)k * N + i];
+    if (!left) {
       for (int tau = (b - 1) * n_stab + 1; tau <= b * n_stab; ++tau) {
         x.stage(tau);
         PQMC_FOR_2D(i, 0, N, k, 0, n) Mt[(long)i * n + k] *= x.vexpT(tau, s, i);
@@ -1383,46 +1750,7 @@ __device__ void push_R(Cta<T>& x, int b) {
         __syncthreads();
         T* t = Mt; Mt = Mt2; Mt2 = t;
       }
-      PQMC_FOR_2D(k, 0, n, i, 0, N) M[(long)k * ldm + i] = (double)Mt[(long)i * n + k];
-      __syncthreads();
-    }
-    double la, sg = 1.0;
-    x.mark(kPhStack);
-    if (std::is_same<T, double>::value || !qr_cholesky(x, N, ldm, n, M, x.Q64(), la))
-      qr_householder(x, N, ldm, n, M, x.Q64(), la, sg);
-    copy_block(x.Q64(), stack_block(x, c.Rst, b, s), N * n);
-    x.mark(kPhQR);
-    if (threadIdx.x == 0) {
-      c.Rlog[(b * 2 + s) * 2 + 0] = prev_l + la;
-      c.Rlog[(b * 2 + s) * 2 + 1] = prev_s * sg;
-    }
-    __syncthreads();
-  }
-}
-
-// Left stack block b holds (B_L(b n))^T = Q T^T: QR of
-// B_{bn+1}^T ... B_{(b+1)n}^T Q_L[b+1] (b < nb) or of e^{V(s_{Ltau+1})} P (b = nb).
-template <typename T>
-__device__ void push_L(Cta<T>& x, int b) {
-  const ChainDesc& c = x.c;
-  const int N = c.N, n_stab = c.n_stab;
-  const int ldm = m64_ld(N);
-  double* M = x.M64();
-  for (int s = 0; s < x.nspec(); ++s) {
-    const int n = x.nsig(s);
-    const double* P = c.P + (long)s * N * c.nmax;
-    T* Mt = x.Mt();
-    T* Mt2 = x.Mt2();
-    double prev_l = 0.0, prev_s = 1.0;
-    if (b == c.nb) {
-      x.stage(c.Ltau + 1);
-      PQMC_FOR_2D(k, 0, n, i, 0, N) M[(long)k * ldm + i] = x.vexp(c.Ltau + 1, s, i) * P[(long)k * N + i];
-      __syncthreads();
     } else {
-      const double* prev = stack_block(x, c.Lst, b + 1, s);
-      PQMC_FOR_2D(k, 0, n, i, 0, N) Mt[(long)i * n + k] = (T)prev[(long)k * N + i];
-      prev_l = c.Llog[((b + 1) * 2 + s) * 2 + 0];
-      prev_s = c.Llog[((b + 1) * 2 + s) * 2 + 1];
       __syncthreads();
       for (int tau = (b + 1) * n_stab; tau > b * n_stab; --tau) {
         cta_gemm<T>(N, n, N, x.Em(), 1, c.ld, Mt, n, 1, Mt2, n, 1, EpiStore());
@@ -1430,18 +1758,44 @@ __device__ void push_L(Cta<T>& x, int b) {
         PQMC_FOR_2D(i, 0, N, k, 0, n) Mt[(long)i * n + k] = x.vexpT(tau, s, i) * Mt2[(long)i * n + k];
         __syncthreads();
       }
-      PQMC_FOR_2D(k, 0, n, i, 0, N) M[(long)k * ldm + i] = (double)Mt[(long)i * n + k];
-      __syncthreads();
     }
+    PQMC_FOR_2D(k, 0, n, i, 0, N) M[(long)k * ldm + i] = (double)Mt[(long)i * n + k];
+    __syncthreads();
+  }
+  x.mark(kPhStack);
+}
+
+template <typename T, bool RES>
+__device__ __noinline__ bool phase_chol(int n, double* logabs) {
+  auto x = this_cta<T, RES>();
+  return qr_cholesky(x, x.c.N, m64_ld(x.c.N), n, x.M64(), x.Q64(), *logabs);
+}
+template <typename T, bool RES>
+__device__ __noinline__ void phase_householder(int n, double* logabs, double* sgn) {
+  auto x = this_cta<T, RES>();
+  qr_householder(x, x.c.N, m64_ld(x.c.N), n, x.M64(), x.Q64(), *logabs, *sgn);
+}
+
+// the new stack block b of both species
+template <typename T, bool RES>
+__device__ __forceinline__ void push_block(int b, int left) {
+  auto x = this_cta<T, RES>();
+  const ChainDesc& c = x.c;
+  for (int s = 0; s < x.nspec(); ++s) {
+    const int n = x.nsig(s);
+    phase_stack<T, RES>(b, left, s);
     double la, sg = 1.0;
-    x.mark(kPhStack);
-    if (std::is_same<T, double>::value || !qr_cholesky(x, N, ldm, n, M, x.Q64(), la))
-      qr_householder(x, N, ldm, n, M, x.Q64(), la, sg);
-    copy_block(x.Q64(), stack_block(x, c.Lst, b, s), N * n);
+    bool done = false;
+    if constexpr (!std::is_same<T, double>::value) done = phase_chol<T, RES>(n, &la);
+    if (!done) phase_householder<T, RES>(n, &la, &sg);
+    copy_block(x.Q64(), stack_block(x, left ? c.Lst : c.Rst, b, s), c.N * n);
     x.mark(kPhQR);
     if (threadIdx.x == 0) {
-      c.Llog[(b * 2 + s) * 2 + 0] = prev_l + la;
-      c.Llog[(b * 2 + s) * 2 + 1] = prev_s * sg;
+      double* lg = left ? c.Llog : c.Rlog;
+      const bool first = left ? b == c.nb : b == 0;
+      const int bp = left ? b + 1 : b - 1;
+      lg[(b * 2 + s) * 2 + 0] = (first ? 0.0 : lg[(bp * 2 + s) * 2 + 0]) + la;
+      lg[(b * 2 + s) * 2 + 1] = (first ? 1.0 : lg[(bp * 2 + s) * 2 + 1]) * sg;
     }
     __syncthreads();
   }
@@ -1482,8 +1836,8 @@ struct EpiDiff64 {
 // G_fresh = 1 - Q_R X Q_L^T for spin s with X = (Q_L^T Q_R)^{-1} (FP64, n x n
 // row-major at Xinv), in the path precision; the FP64 diagnostics of
 // opts.dg_fp64 around it.
-template <typename T>
-__device__ void assemble_spin(Cta<T>& x, int s, const double* QR, const double* QL, const double* Xinv, int ns,
+template <typename T, bool RES>
+__device__ __forceinline__ void assemble_spin(Cta<T, RES>& x, int s, const double* QR, const double* QL, const double* Xinv, int ns,
                               bool record, T& dmax, double& dmax64) {
   const ChainDesc& c = x.c;
   Smem<T>& sh = x.sh;
@@ -1555,29 +1909,44 @@ __device__ void assemble_spin(Cta<T>& x, int s, const double* QR, const double* 
 // propagated G against the same formula assembled in FP64 from the FP64
 // factors; the G that replaces the propagated one is still the
 // path-precision assembly, so the chain itself is unchanged.
-template <typename T>
-__device__ void refresh(Cta<T>& x, int b, bool record) {
+template <typename T, bool RES>
+__device__ __noinline__ void phase_overlap(int b) {
+  // O_s = Q_L^T Q_R in FP64, both spins
+  auto x = this_cta<T, RES>();
+  const ChainDesc& c = x.c;
+  for (int s = 0; s < 2; ++s) {
+    const int n = x.nsig(s);
+    gemm_tn_f64(n, n, c.N, stack_block(x, c.Lst, b, s), stack_block(x, c.Rst, b, s), x.Ob(s), n);
+  }
+  __syncthreads();
+  x.mark(kPhOverlap);
+}
+template <typename T, bool RES>
+__device__ __noinline__ void phase_inverse() {
+  auto x = this_cta<T, RES>();
+  int n[2] = {x.nsig(0), x.nsig(1)};
+  double* O[2] = {x.Ob(0), x.Ob(1)};
+  double la[2], sg[2];
+  gj_invert2(x, n, O, la, sg);
+  if (threadIdx.x < 2) {
+    x.sh.gj_logabs[threadIdx.x] = threadIdx.x ? la[1] : la[0];
+    x.sh.gj_sign[threadIdx.x] = threadIdx.x ? sg[1] : sg[0];
+  }
+  __syncthreads();
+  x.mark(kPhLU);
+}
+template <typename T, bool RES>
+__device__ __noinline__ void phase_assemble(int b, bool record) {
+  auto x = this_cta<T, RES>();
   const ChainDesc& c = x.c;
   Smem<T>& sh = x.sh;
-  const int N = c.N;
   T dmax = T(0);
   double dmax64 = 0.0;
   double sign_total = 1.0;
-  int n[2] = {x.nsig(0), x.nsig(1)};
-  double* O[2] = {x.Ob(0), x.Ob(1)};
-  const double* QR[2] = {stack_block(x, c.Rst, b, 0), stack_block(x, c.Rst, b, 1)};
-  const double* QL[2] = {stack_block(x, c.Lst, b, 0), stack_block(x, c.Lst, b, 1)};
-  // O_s = Q_L^T Q_R and its inverse in FP64, both spins together
-  for (int s = 0; s < 2; ++s) gemm_tn_f64(n[s], n[s], N, QL[s], QR[s], O[s], n[s]);
-  __syncthreads();
-  x.mark(kPhOverlap);
-  double la[2], sg[2];
-  gj_invert2(x, n, O, la, sg);
-  x.mark(kPhLU);
   for (int s = 0; s < x.nspec(); ++s) {
-    assemble_spin(x, s, QR[s], QL[s], O[s], n[s], record, dmax, dmax64);
-    const double l_tot = c.Rlog[(b * 2 + s) * 2 + 0] + la[s] + c.Llog[(b * 2 + s) * 2 + 0];
-    const double s_tot = c.Rlog[(b * 2 + s) * 2 + 1] * sg[s] * c.Llog[(b * 2 + s) * 2 + 1];
+    assemble_spin(x, s, stack_block(x, c.Rst, b, s), stack_block(x, c.Lst, b, s), x.Ob(s), x.nsig(s), record, dmax, dmax64);
+    const double l_tot = c.Rlog[(b * 2 + s) * 2 + 0] + sh.gj_logabs[s] + c.Llog[(b * 2 + s) * 2 + 0];
+    const double s_tot = c.Rlog[(b * 2 + s) * 2 + 1] * sh.gj_sign[s] * c.Llog[(b * 2 + s) * 2 + 1];
     if (threadIdx.x == 0) {
       sh.logw_spin[s] = l_tot;
       sh.sign_spin[s] = s_tot;
@@ -1592,16 +1961,22 @@ __device__ void refresh(Cta<T>& x, int b, bool record) {
       sh.logw_spin[s] = 0.0;
       sh.sign_spin[s] = 1.0;
     }
-    const double dmax = dm;
-    if (!isfinite(dmax)) sh.err |= kErrNaN;
+    if (!isfinite(dm)) sh.err |= kErrNaN;
     if (record) {
-      sh.dGmax = fmax(sh.dGmax, dmax);
-      c.dG[c.st->n_dG % kDGHistory] = dmax;
+      sh.dGmax = fmax(sh.dGmax, dm);
+      c.dG[c.st->n_dG % kDGHistory] = dm;
       c.st->n_dG++;
     }
     c.st->sign_stack = sign_total;
   }
   __syncthreads();
+}
+
+template <typename T, bool RES>
+__device__ __forceinline__ void refresh(int b, bool record) {
+  phase_overlap<T, RES>(b);
+  phase_inverse<T, RES>();
+  phase_assemble<T, RES>(b, record);
 }
 
 // Wick estimates on the fresh G at the middle slice: E/site for Eq. (2),
@@ -1614,8 +1989,8 @@ __device__ void refresh(Cta<T>& x, int b, bool record) {
 // V sum_<ij> [(n_i - 1/2)(n_j - 1/2) - G_ji G_ij] / N, kinetic/site, the weight
 // sign, the running sign, and S_CDW = [(sum_i eps_i (n_i - 1/2))^2 +
 // sum_ij eps_i eps_j (delta_ij - G_ji) G_ij] / N^2.
-template <typename T>
-__device__ void measure_tv(Cta<T>& x) {
+template <typename T, bool RES>
+__device__ __forceinline__ void measure_tv(Cta<T, RES>& x) {
   const ChainDesc& c = x.c;
   Smem<T>& sh = x.sh;
   const int N = c.N, ld = c.ld;
@@ -1649,8 +2024,8 @@ __device__ void measure_tv(Cta<T>& x) {
   __syncthreads();
 }
 
-template <typename T>
-__device__ void measure(Cta<T>& x) {
+template <typename T, bool RES>
+__device__ __forceinline__ void measure(Cta<T, RES>& x) {
   const ChainDesc& c = x.c;
   if (c.tv) {
     measure_tv(x);
@@ -1693,47 +2068,54 @@ __device__ void measure(Cta<T>& x) {
 // --------------------------------------------------------------------------
 // sweeps
 
-template <typename T>
-__device__ void sweep_up(Cta<T>& x, uint32_t sweep, bool do_measure) {
-  const ChainDesc& c = x.c;
-  for (int tau = 0; tau <= c.Ltau + 1; ++tau) {
-    if (c.tv) update_slice_tv(x, tau, sweep);
-    else update_slice(x, tau, sweep);
-    wrap(x, tau, +1);
-    x.mark(kPhWrap);
-    if (tau <= c.Ltau && tau % c.n_stab == 0) {
-      const int b = tau / c.n_stab;
-      push_R(x, b);
-      refresh(x, b, true);
-      x.mark(kPhRefresh);
-      if (do_measure && tau == c.Ltau / 2) measure(x);
-      x.mark(kPhMeasure);
-    }
+template <typename T, bool RES>
+__device__ __noinline__ void phase_slice_tv(int tau, uint32_t sweep) {
+  auto x = this_cta<T, RES>();
+  update_slice_tv(x, tau, sweep);
+}
+template <typename T, bool RES, bool kTc>
+__device__ __noinline__ void phase_wrap(int tau, int dir) {
+  auto x = this_cta<T, RES>();
+  wrap<kTc>(x, tau, dir);
+  x.mark(kPhWrap);
+}
+template <typename T, bool RES>
+__device__ __noinline__ void phase_measure() {
+  auto x = this_cta<T, RES>();
+  measure(x);
+}
+
+// The stabilisation at slice t (a multiple of n_stab): the new stack block,
+// G from the stacks, the measurement at the middle slice.
+template <typename T, bool RES>
+__device__ __forceinline__ void stabilise(int t, int left, bool do_measure) {
+  auto x = this_cta<T, RES>();
+  const int b = t / x.c.n_stab;
+  push_block<T, RES>(b, left);
+  refresh<T, RES>(b, true);
+  x.mark(kPhRefresh);
+  if (do_measure && t == x.c.Ltau / 2) phase_measure<T, RES>();
+  x.mark(kPhMeasure);
+}
+
+template <typename T, bool RES, bool kPair, bool kTc>
+__device__ __forceinline__ void sweep_once(uint32_t sweep, bool do_measure) {
+  auto x = this_cta<T, RES>();
+  const int Lt = x.c.Ltau, n_stab = x.c.n_stab;
+  const bool down = (sweep & 1u) != 0;
+  for (int k = 0; k <= Lt + 1; ++k) {
+    const int tau = down ? Lt + 1 - k : k;
+    if (down) phase_wrap<T, RES, kTc>(tau, -1);
+    if (x.c.tv) phase_slice_tv<T, RES>(tau, sweep);
+    else update_slice<T, RES, kPair>(tau, sweep);
+    if (!down) phase_wrap<T, RES, kTc>(tau, +1);
+    const int t = down ? tau - 1 : tau;              // G is G(t) now
+    if (t >= 0 && t <= Lt && t % n_stab == 0) stabilise<T, RES>(t, down ? 1 : 0, do_measure);
   }
 }
 
-template <typename T>
-__device__ void sweep_down(Cta<T>& x, uint32_t sweep, bool do_measure) {
-  const ChainDesc& c = x.c;
-  for (int tau = c.Ltau + 1; tau >= 0; --tau) {
-    wrap(x, tau, -1);
-    x.mark(kPhWrap);
-    if (c.tv) update_slice_tv(x, tau, sweep);
-    else update_slice(x, tau, sweep);
-    const int t1 = tau - 1;
-    if (t1 >= 0 && t1 % c.n_stab == 0) {
-      const int b = t1 / c.n_stab;
-      push_L(x, b);
-      refresh(x, b, true);
-      x.mark(kPhRefresh);
-      if (do_measure && t1 == c.Ltau / 2) measure(x);
-      x.mark(kPhMeasure);
-    }
-  }
-}
-
-template <typename T>
-__device__ void load_state(Cta<T>& x) {
+template <typename T, bool RES>
+__device__ __forceinline__ void load_state(Cta<T, RES>& x) {
   if (threadIdx.x == 0) {
     const ChainState& st = *x.c.st;
     x.sh.sign_running = st.sign_running;
@@ -1765,8 +2147,8 @@ __device__ void load_state(Cta<T>& x) {
   __syncthreads();
 }
 
-template <typename T>
-__device__ void store_state(Cta<T>& x, int* err) {
+template <typename T, bool RES>
+__device__ __forceinline__ void store_state(Cta<T, RES>& x, int* err) {
   __syncthreads();
   if (threadIdx.x == 0) {
     ChainState& st = *x.c.st;
@@ -1787,8 +2169,10 @@ __device__ void store_state(Cta<T>& x, int* err) {
 
 // Place G and the scratch: in shared memory after the fixed part when the
 // chain's footprint fits in res_bytes (G is copied in), else in global memory.
+// Every phase finds them again through this_cta.
 template <typename T>
-__device__ Cta<T> make_cta(const ChainDesc& cg, unsigned char* smem_raw, size_t res_bytes, uint64_t seed) {
+__device__ __forceinline__ Smem<T>& setup_cta(const ChainDesc& cg, size_t res_bytes, uint64_t seed) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
   Smem<T>& sh = *reinterpret_cast<Smem<T>*>(smem_raw);
   // the descriptor is read all through the sweep: keep a shared-memory copy
   {
@@ -1800,28 +2184,51 @@ __device__ Cta<T> make_cta(const ChainDesc& cg, unsigned char* smem_raw, size_t 
   }
   const ChainDesc& c = sh.desc;
   const int ts = (int)sizeof(T);
-  const ScratchLayout L = scratch_layout(c.N, c.ld, c.nmax, ts, c.kb);
   const bool res = resident_bytes(c.N, c.ld, c.nmax, ts, c.kb) <= res_bytes;
-  unsigned char* dyn = smem_raw + al16(sizeof(Smem<T>));
-  T* Gp = res ? reinterpret_cast<T*>(dyn) : reinterpret_cast<T*>(c.G);
-  unsigned char* scr = res ? dyn + al16(2 * (size_t)c.N * c.ld * ts) : reinterpret_cast<unsigned char*>(c.scratch);
-  FlipBuf<T>* fb = reinterpret_cast<FlipBuf<T>*>(res ? scr + L.fb : dyn);
-  Cta<T> x{c, sh, seed, Gp, scr, L, res, fb};
+  if (threadIdx.x == 0) {
+    sh.L = scratch_layout(c.N, c.ld, c.nmax, ts, c.kb);
+    sh.res = res ? 1 : 0;
+    sh.seed = seed;
+    sh.scr_off = (uint32_t)(al16(sizeof(Smem<T>)) + al16(2 * (size_t)c.N * c.ld * ts));
+    sh.tcs_off = 0;
+    sh.tmem = 0;
+  }
   if (res) {
+    T* Gp = reinterpret_cast<T*>(smem_raw + al16(sizeof(Smem<T>)));
     const T* g = reinterpret_cast<const T*>(c.G);
     for (long e = threadIdx.x; e < 2L * c.N * c.ld; e += blockDim.x) Gp[e] = g[e];
   }
-  return x;
+  __syncthreads();
+  return sh;
 }
 
-template <typename T>
-__device__ void write_back(Cta<T>& x) {
+template <typename T, bool RES>
+__device__ __forceinline__ void write_back() {
+  auto x = this_cta<T, RES>();
   __syncthreads();
-  if (x.resident) {
+  if (RES) {
     T* g = reinterpret_cast<T*>(x.c.G);
     for (long e = threadIdx.x; e < 2L * x.c.N * x.c.ld; e += blockDim.x) g[e] = x.Gp[e];
   }
   __syncthreads();
+}
+
+template <typename T, bool RES>
+__device__ __forceinline__ void run_init(int* err, int b_at) {
+  auto x = this_cta<T, RES>();
+  Smem<T>& sh = x.sh;
+  load_state(x);
+  const int bt = b_at < 0 ? 0 : b_at;
+  for (int b = x.c.nb; b >= bt; --b) push_block<T, RES>(b, 1);
+  for (int b = 0; b <= bt; ++b) push_block<T, RES>(b, 0);
+  refresh<T, RES>(bt, false);
+  if (b_at < 0) {
+    if (threadIdx.x == 0) sh.sign_running = sh.sign_spin[0] * sh.sign_spin[1];
+    __syncthreads();
+    phase_wrap<T, RES, false>(0, -1);
+  }
+  write_back<T, RES>();
+  store_state(x, err);
 }
 
 // b_at < 0: initialisation from the chain's fields (left stack, right block
@@ -1832,59 +2239,67 @@ __device__ void write_back(Cta<T>& x) {
 template <typename T, int TPB, int MINB>
 __global__ void __launch_bounds__(TPB, MINB) init_kernel(const ChainDesc* chains, int chain0, uint64_t seed,
                                                           size_t res_bytes, int* err, int b_at) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  Cta<T> x = make_cta<T>(chains[chain0 + blockIdx.x], smem_raw, res_bytes, seed);
+  Smem<T>& sh = setup_cta<T>(chains[chain0 + blockIdx.x], res_bytes, seed);
+  if (sh.res) run_init<T, true>(err, b_at);
+  else run_init<T, false>(err, b_at);
+}
+
+template <typename T, bool RES, bool kPair, bool kTc>
+__device__ __forceinline__ void run_sweeps(uint32_t sweep0, int n_sweeps, int do_measure, int* err) {
+  auto x = this_cta<T, RES>();
   Smem<T>& sh = x.sh;
-  load_state(x);
-  const ChainDesc& c = x.c;
-  const int bt = b_at < 0 ? 0 : b_at;
-  for (int b = c.nb; b >= bt; --b) push_L(x, b);
-  for (int b = 0; b <= bt; ++b) push_R(x, b);
-  refresh(x, bt, false);
-  if (b_at < 0) {
-    if (threadIdx.x == 0) sh.sign_running = sh.sign_spin[0] * sh.sign_spin[1];
+  const long long t_start = clock64();
+  for (int k = 0; k < n_sweeps; ++k) {
+    sweep_once<T, RES, kPair, kTc>(sweep0 + (uint32_t)k, do_measure != 0);
     __syncthreads();
-    wrap(x, 0, -1);
+    if (sh.err) break;
   }
-  write_back(x);
-  store_state(x, err);
+  if (threadIdx.x == 0) sh.cyc[kPhTotal] += clock64() - t_start;
+  (void)err;
 }
 
 template <typename T, int TPB, int MINB>
 __global__ void __launch_bounds__(TPB, MINB) sweep_kernel(const ChainDesc* chains, uint64_t seed,
                                                        const uint32_t* sweep_ctr, int n_sweeps, int do_measure,
                                                        size_t res_bytes, int* err, int tc_on) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
   if (chains[blockIdx.x].st->err) return;
+  constexpr bool kPair = TPB * MINB <= 512;   // 128 registers per thread: room for the one-warp decisions
   const uint32_t sweep0 = *sweep_ctr;
-  Cta<T> x = make_cta<T>(chains[blockIdx.x], smem_raw, res_bytes, seed);
-  Smem<T>& sh = x.sh;
-  load_state(x);
-  if constexpr (std::is_same<T, float>::value && TPB == 512) {
-    // BF16X3 chains kept in global memory run their products on the tensor
-    // cores: a staging area after the dynamic shared memory the launch
-    // reserves for it, and TMEM columns held until the CTA ends
-    if (tc_on && x.c.tc && !x.resident) {
-      const size_t fbb = flipbuf_bytes((int)sizeof(T));
-      const uintptr_t at = reinterpret_cast<uintptr_t>(smem_raw) + al16(sizeof(Smem<T>)) + (res_bytes > fbb ? res_bytes : fbb);
-      x.tcs = reinterpret_cast<unsigned char*>((at + 127) & ~(uintptr_t)127);
-      x.tmem = tc_alloc(x.tcs);
+  Smem<T>& sh = setup_cta<T>(chains[blockIdx.x], res_bytes, seed);
+  if (sh.res) {
+    auto x = this_cta<T, true>();
+    load_state(x);
+    run_sweeps<T, true, kPair, (TPB == 512)>(sweep0, n_sweeps, do_measure, err);
+    write_back<T, true>();
+    store_state(x, err);
+  } else {
+    auto x = this_cta<T, false>();
+    load_state(x);
+    if constexpr (std::is_same<T, float>::value && TPB == 512) {
+      // BF16X3 chains kept in global memory run their products on the tensor
+      // cores: a staging area after the dynamic shared memory the launch
+      // reserves for it, and TMEM columns held until the CTA ends
+      if (tc_on && x.c.tc) {
+        extern __shared__ __align__(16) unsigned char smem_raw[];
+        const size_t fbb = flipbuf_bytes((int)sizeof(T));
+        const uint32_t base = smem_addr(smem_raw);
+        const uint32_t at = base + (uint32_t)(al16(sizeof(Smem<T>)) + (res_bytes > fbb ? res_bytes : fbb));
+        const uint32_t off = ((at + 127) & ~127u) - base;
+        const uint32_t tmem = tc_alloc(smem_raw + off);
+        if (threadIdx.x == 0) {
+          sh.tcs_off = off;
+          sh.tmem = tmem;
+        }
+        __syncthreads();
+      }
     }
+    run_sweeps<T, false, kPair, (TPB == 512)>(sweep0, n_sweeps, do_measure, err);
+    if constexpr (std::is_same<T, float>::value && TPB == 512) {
+      if (sh.tcs_off) tc_free(sh.tmem);
+    }
+    write_back<T, false>();
+    store_state(x, err);
   }
-  const long long t_start = clock64();
-  for (int k = 0; k < n_sweeps; ++k) {
-    const uint32_t sw = sweep0 + (uint32_t)k;
-    if ((sw & 1u) == 0) sweep_up(x, sw, do_measure != 0);
-    else sweep_down(x, sw, do_measure != 0);
-    __syncthreads();
-    if (sh.err) break;
-  }
-  if (threadIdx.x == 0) sh.cyc[kPhTotal] += clock64() - t_start;
-  if constexpr (std::is_same<T, float>::value && TPB == 512) {
-    if (x.tcs) tc_free(x.tmem);
-  }
-  write_back(x);
-  store_state(x, err);
 }
 
 // --------------------------------------------------------------------------
