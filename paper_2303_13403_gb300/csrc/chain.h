@@ -106,15 +106,18 @@ namespace pqmc {
 //             (kw x ld, T) of each spin (u, w for spin 0; u2, mw for
 //             spin 1), kw = max(delayed block, kBlock); for t-V blocks A_S
 //             (u), W and M W (w, mw); and the per-block flip buffers
-//   stack   : M64 (N x n, FP64, column-major, ld m64_ld(N)), then a region holding the two
+//   stack   : M64 (N x n, FP64, column-major, ld m64_ld(N); Cholesky QR: the packed digits of
+//             the block, ld digit_ld(N)), then a region holding the two
 //             path-precision product buffers Mt, Mt2 (N x n, T, row-major)
-//             and later the FP64 Q of the QR; Householder betas / R_jj;
-//             the Gram matrix and pivots of the Cholesky QR
-//   refresh : O (n x n, FP64, both spins, inverted in place), Y (n x ld, T), Q_R and Q_L in the
+//             and later the FP64 Q of the Householder QR or the packed digits of R^{-1};
+//             Householder betas / R_jj;
+//             the Gram matrix, its inverse factor and pivots of the Cholesky QR
+//   refresh : O (n x n, FP64, both spins, inverted in place), the packed digits of Q_L and Q_R of
+//             one spin (dq), then in their place Y (n x ld, T), Q_R and Q_L in the
 //             path precision (N x n, T); GJ pivots / multipliers; O^{-1} in
 //             the path precision (n x n, T)
 struct ScratchLayout {
-  size_t gt, em, ep, u, u2, w, mw, fb, m64, mtq, mt2, qaux, chol, o, y, qrt, qlt, laux, ot, total;
+  size_t gt, em, ep, u, u2, w, mw, fb, m64, mtq, mt2, qaux, chol, o, dq, y, qrt, qlt, laux, ot, total;
 };
 
 PQMC_HDI constexpr size_t al16(size_t v) { return (v + 15) & ~(size_t)15; }
@@ -123,9 +126,8 @@ PQMC_HDI constexpr size_t al16(size_t v) { return (v + 15) & ~(size_t)15; }
 // ratios of one decision sub-block, Delta and Delta/R of each accepted flip of
 // a delayed block, accepted sites); the layout is FlipBuf<T> in
 // sweep_kernels.cuh.
-constexpr int kSvLd = kBlock + 4;   // row length of the vector tables in FlipBuf
 PQMC_HDI constexpr size_t flipbuf_bytes(int tsize) {
-  return al16(2 * (size_t)kBlock * kSvLd * tsize + 2 * (size_t)kBlock * tsize +
+  return al16(2 * (size_t)kBlock * (kBlock + 1) * tsize + 2 * (size_t)kBlock * tsize +
               4 * (size_t)kMaxDelay * tsize + 2 * (size_t)kMaxDelay * 4);
 }
 
@@ -135,6 +137,10 @@ PQMC_HDI constexpr size_t flipbuf_bytes(int tsize) {
 // that the Gram matrix's threads, each on its own columns, read different
 // shared-memory banks
 PQMC_HDI constexpr int m64_ld(int N) { return N | 1; }
+// leading dimension of packed digits (digit_gemm.cuh) for K contiguous elements:
+// = 2 mod 8, so that the fragments' 16-byte loads along K and 8-byte loads
+// across it meet few bank conflicts (and K pairs stay 16-byte aligned)
+PQMC_HDI constexpr int digit_ld(int K) { return ((K + 5) & ~7) + 2; }
 
 PQMC_HDI ScratchLayout scratch_layout(int N, int ld, int n, int tsize, int kd) {
   ScratchLayout L;
@@ -148,21 +154,27 @@ PQMC_HDI ScratchLayout scratch_layout(int N, int ld, int n, int tsize, int kd) {
   L.mw = L.w + al16(kw * ld * tsize);
   L.fb = L.mw + al16(kw * ld * tsize);
   size_t flush = L.fb + flipbuf_bytes(tsize);
+  const bool chol = tsize == 4;              // the reduced paths' stack blocks take the Cholesky QR
+  const size_t dig = al16((size_t)digit_ld(N) * n * 8);
   L.m64 = 0;
   L.mtq = al16((size_t)m64_ld(N) * n * 8);
+  if (chol && dig > L.mtq) L.mtq = dig;
   L.mt2 = L.mtq + al16(Nn * tsize);
-  const size_t two_mt = 2 * al16(Nn * tsize);
-  const size_t mtq_sz = two_mt > al16(Nn * 8) ? two_mt : al16(Nn * 8);
+  size_t mtq_sz = 2 * al16(Nn * tsize);
+  if (al16(Nn * 8) > mtq_sz) mtq_sz = al16(Nn * 8);
+  if (chol && al16((size_t)digit_ld(n) * n * 8) > mtq_sz) mtq_sz = al16((size_t)digit_ld(n) * n * 8);
   L.qaux = L.mtq + mtq_sz;
   L.chol = L.qaux + al16((3 * (size_t)n + (size_t)kQRParts * n) * 8);
-  size_t stack = L.chol + al16((2 * (size_t)n * n + 3 * (size_t)n) * 8);
+  size_t stack = L.chol + (chol ? al16(((size_t)n * n + 6 * (size_t)n) * 8) : 0);
   L.o = 0;                                   // O for spin 0, then spin 1 (inverted in place)
-  L.y = 2 * al16((size_t)n * n * 8);
+  L.dq = 2 * al16((size_t)n * n * 8);
+  L.y = L.dq;
   L.qrt = L.y + al16((size_t)n * ld * tsize);
   L.qlt = L.qrt + al16(Nn * tsize);
   L.laux = L.qlt + al16(Nn * tsize);
-  L.ot = L.laux + al16(2 * 3 * (size_t)n * 8);
-  size_t refresh = L.ot + al16((size_t)n * n * tsize);
+  L.ot = L.laux + al16(2 * 6 * (size_t)n * 8);
+  size_t refresh = L.ot + (chol ? al16((size_t)n * n * tsize) : 0);   // (no copy of O^{-1} on the FP64 path)
+  if (L.dq + 2 * dig > refresh) refresh = L.dq + 2 * dig;
   size_t t = wrap;
   if (flush > t) t = flush;
   if (stack > t) t = stack;

@@ -43,6 +43,7 @@
 #include "model.h"
 #include "philox.cuh"
 #include "tc_gemm.cuh"
+#include "digit_gemm.cuh"
 
 namespace pqmc {
 
@@ -315,7 +316,7 @@ template <typename T>
 struct FlipBuf {
   union {
     T Tu[2][kBlock][kBlock + 1];    // t-V: 1 + (1 - G_SS) Gamma, inverted in place, then M
-    alignas(16) T sv[2][kBlock][kSvLd];   // Hubbard: the update vectors at the accepted sites (sm_vectors)
+    alignas(16) T sv[2][kBlock][kBlock];  // Hubbard: the update vectors at the accepted sites (sm_vectors)
   };
   T rs[2][kBlock];                  // ratio R_sigma of each proposal of the decision sub-block
   T cl[2][kMaxDelay];               // Delta of each accepted flip of the delayed block (diagonal of Gamma)
@@ -357,6 +358,8 @@ struct Smem {
   uint32_t scr_off;                 // RES: the scratch's offset from the shared-memory base
   uint32_t tcs_off;                 // tensor-core staging area (BF16X3, chains in global memory), or 0
   uint32_t tmem;                    // its TMEM accumulator
+  int src;                          // where phase_stack left the block: Mt (0), Mt2 (1), e^V P (2)
+  double gj_ip[2];                  // reciprocal of the Gauss-Jordan pivot
   double gj_logabs[2], gj_sign[2];  // log|det O| and sign of the last Gauss-Jordan inverse
 };
 
@@ -403,9 +406,11 @@ struct Cta {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     return smem_raw + sh.tcs_off;
   }
-  __device__ double* pval(int s) const { return reinterpret_cast<double*>(scr + L.laux) + s * 3 * c.nmax; }
-  __device__ double* pinv(int s) const { return pval(s) + c.nmax; }
-  __device__ double* lmul(int s) const { return pval(s) + 2 * c.nmax; }
+  // Gauss-Jordan of spin s: pivots, column in hand (two), pivot row, row of each step (and two work arrays)
+  __device__ double* pval(int s) const { return reinterpret_cast<double*>(scr + L.laux) + s * 6 * c.nmax; }
+  __device__ double* gj_col(int s) const { return pval(s) + c.nmax; }
+  __device__ double* gj_row(int s) const { return pval(s) + 3 * c.nmax; }
+  __device__ int* gj_rows(int s) const { return reinterpret_cast<int*>(pval(s) + 4 * c.nmax); }
   __device__ const T* Em() const { return reinterpret_cast<const T*>(c.expKm); }
   __device__ const T* Ep() const { return reinterpret_cast<const T*>(c.expKp); }
   __device__ int nsig(int s) const { return s == 0 ? c.nup : c.ndn; }
@@ -639,9 +644,9 @@ __device__ __forceinline__ void flush_block(Cta<T, RES>& x, int a, bool pivot) {
 // The table of a spin (FlipBuf::sv): V_m[s_p] at row m, column p; U_m[s_p] at
 // row 31 - m, column 31 - p (p > m: above and below the diagonal).
 template <typename T>
-__device__ __forceinline__ T& sm_v(T (*tab)[kSvLd], int m, int p) { return tab[m][p]; }
+__device__ __forceinline__ T& sm_v(T (*tab)[kBlock], int m, int p) { return tab[m][p]; }
 template <typename T>
-__device__ __forceinline__ T& sm_u(T (*tab)[kSvLd], int m, int p) { return tab[kBlock - 1 - m][kBlock - 1 - p]; }
+__device__ __forceinline__ T& sm_u(T (*tab)[kBlock], int m, int p) { return tab[kBlock - 1 - m][kBlock - 1 - p]; }
 
 // The chain on the accepted sites, one warp per spin and role: rows (lane q:
 // row s_q, register p: column s_p; gives the U_m) or columns (transposed; the
@@ -658,7 +663,7 @@ __device__ __forceinline__ void sm_core(Cta<T, RES>& x, int m0, int cnt) {
     const T* Gs = x.G(s);
     const T* U = x.Uv(s);
     const T* V = x.Vv(s);
-    T (*tab)[kSvLd] = fb.sv[s];
+    T (*tab)[kBlock] = fb.sv[s];
     const int sq = fb.gsite[m0 + min(lane, cnt - 1)];
     T a[kBlock];
 #pragma unroll
@@ -711,7 +716,7 @@ __device__ __forceinline__ void sm_core(Cta<T, RES>& x, int m0, int cnt) {
 // their updates.  No branch inside: the table rows are read ahead of the
 // FMAs (flips beyond cnt work on leftovers that nothing reads).
 template <bool kRow, int kW, typename T>
-__device__ __forceinline__ void sm_four(T (&w)[kBlock], const T (*tab)[kSvLd], int k, int cnt, int j, const int* site,
+__device__ __forceinline__ void sm_four(T (&w)[kBlock], const T (*tab)[kBlock], int k, int cnt, int j, const int* site,
                                         const T* fr, T* out, long os) {
   const T* tr = kRow ? &tab[k][k] : &tab[kBlock - 1 - k][kBlock - 4 - k];
 #pragma unroll
@@ -723,7 +728,7 @@ __device__ __forceinline__ void sm_four(T (&w)[kBlock], const T (*tab)[kSvLd], i
     for (int q = 0; q < kW; q += 4)
       if (q + 3 > i) {
         T t[4];
-        Vec4<T>::load(kRow ? tr + i * kSvLd + q : tr - i * kSvLd - q, t);
+        Vec4<T>::load(kRow ? tr + i * kBlock + q : tr - i * kBlock - q, t);
 #pragma unroll
         for (int h = 0; h < 4; ++h)
           if (q + h > i) w[q + h] = fma(-cv, kRow ? t[h] : t[3 - h], w[q + h]);
@@ -1415,295 +1420,306 @@ __device__ __forceinline__ void qr_householder(Cta<T, RES>& x, int N, int ldm, i
   x.mark(kPhQRForm);
 }
 
-// Upper triangle (2 x 2 tiles on or above the diagonal) of C = M^T M for the
-// column-major N x n matrix M (ld ldm, odd so that the threads' columns fall
-// in different shared-memory banks); C row-major n x n.
-static __device__ void gram_upper_f64(int n, int N, int ldm, const double* M, double* C) {
-  // 2 x 2 output tiles (ti, tj), ti <= tj, enumerated over a flat index so
-  // that every warp carries only tiles of the upper triangle (the FP64 pipe
-  // takes the same time for a partial warp as for a full one)
-  const int tn = (n + 1) >> 1;
-  for (int t = threadIdx.x; t < tn * (tn + 1) / 2; t += blockDim.x) {
-    int ti = 0, tj = t;
-    while (tj >= tn - ti) { tj -= tn - ti; ++ti; }
-    tj += ti;
-    const int i0 = ti << 1, j0 = tj << 1;
-    const double* a0 = M + (long)i0 * ldm;
-    const double* a1 = M + (long)min(i0 + 1, n - 1) * ldm;
-    const double* b0 = M + (long)j0 * ldm;
-    const double* b1 = M + (long)min(j0 + 1, n - 1) * ldm;
-    double c00 = 0, c01 = 0, c10 = 0, c11 = 0;
-#pragma unroll 4
-    for (int k = 0; k < N; ++k) {
-      const double x0 = a0[k], x1 = a1[k], y0 = b0[k], y1 = b1[k];
-      c00 = fma(x0, y0, c00);
-      c01 = fma(x0, y1, c01);
-      c10 = fma(x1, y0, c10);
-      c11 = fma(x1, y1, c11);
-    }
-    C[(long)i0 * n + j0] = c00;
-    if (j0 + 1 < n) C[(long)i0 * n + j0 + 1] = c01;
-    if (i0 + 1 < n) {
-      C[(long)(i0 + 1) * n + j0] = c10;
-      if (j0 + 1 < n) C[(long)(i0 + 1) * n + j0 + 1] = c11;
-    }
-  }
+// 1 / x: the hardware's approximation (about 20 bits) and two Newton steps
+// y <- y + y (1 - x y), four dependent FMAs (65 cycles each) where the division
+// takes 646; outside the approximation's range the division.
+static __device__ __forceinline__ double recip64(double x) {
+  const double ax = fabs(x);
+  if (!(ax > 1e-290 && ax < 1e290)) return 1.0 / x;
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  y = fma(y, fma(-x, y, 1.0), y);
+  return fma(y, fma(-x, y, 1.0), y);
 }
 
-// Cholesky QR of the column-major N x n matrix M (ld N), used for the stack
-// blocks of the reduced-precision paths: C = M^T M = R^T R, Q = M R^{-1}
+// Cholesky QR of a stack block M (N x n) of the reduced-precision paths:
+// C = M^T M = R^T R, Q = M R^{-1}
 // (Stathopoulos & Wu, SIAM J. Sci. Comput. 23 (2002); the loss of
 // orthogonality grows like eps cond(M)^2, Yamamoto et al., ETNA 44 (2015)).
-// With two slices per stabilisation cond(M) stays near 1e2, and it needs n
-// CTA barriers per factor and per solve instead of the Householder QR's
-// sequence of reflector, dot and update phases.  Every FP64 step runs over a
-// flat or 2D index of the whole CTA.  Returns false, with M unchanged, when a
+// With two slices per stabilisation cond(M) stays near 1e2.  The two products,
+// M^T M and M R^{-1}, run on the tensor cores from the digits of M
+// (digit_gemm.cuh); the factor and its inverse come from one elimination of
+// [C | I] on the FP64 pipe.  M(i, k): element of the block.
+// Q goes column-major (ld N) to the stack block.  Returns false, with nothing
+// written, when a
 // pivot falls below 1e-12 of its original diagonal entry (cond(M) above about
 // 1e6); the caller then takes the Householder QR.  R has a positive diagonal,
 // so only log|det R| = (1/2) sum_k log(pivot_k) is returned.
-template <typename T, bool RES>
-__device__ __forceinline__ bool qr_cholesky(Cta<T, RES>& x, int N, int ldm, int n, double* M, double* Q, double& logabs) {
+//
+// 72 sites, n = 36, one chain alone on its SM, per block and spin: the FP64
+// Gram matrix, factor (two barriers, a division and a row scaling per column)
+// and column-by-column Q took 122 + 57 kcycles.
+template <typename T, bool RES, typename Elem>
+__device__ __forceinline__ bool qr_cholesky(Cta<T, RES>& x, int N, int n, double* Q, double& logabs, Elem M) {
   Smem<T>& sh = x.sh;
-  double* C = x.chol();                 // n x n row-major (upper part): Gram, then Schur complements
-  double* U = C + (long)n * n;          // n x n row-major (upper part): U_kj = R_kj / R_kk
-  double* d0 = U + (long)n * n;         // original diagonal
-  double* ip = d0 + n;                  // 1 / pivot
-  double* isq = ip + n;                 // 1 / sqrt(pivot)
-  gram_upper_f64(n, N, ldm, M, C);
+  unsigned long long* D = reinterpret_cast<unsigned long long*>(x.scr + x.L.m64);
+  unsigned long long* X = reinterpret_cast<unsigned long long*>(x.scr + x.L.mtq);   // the block's source is free by then
+  double* C = x.chol();                 // n x n row-major: see below
+  double* u[2] = {C + (long)n * n, C + (long)n * n + n};
+  double* dlim = u[1] + n;              // smallest pivot accepted
+  double* pv = dlim + n;                // pivots
+  double* isq = pv + n;                 // 1 / sqrt(pivot)
+  int* ex = reinterpret_cast<int*>(isq + n);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (int)blockDim.x >> 5;
+  const int ldd = digit_ld(N), ldx = digit_ld(n);
+  int E = kDigitNone;
+  PQMC_FOR_2D(i, 0, N, k, 0, n) E = max(E, digit_exp(M(i, k)));
+  E = digit_cta_max(E, reinterpret_cast<int*>(sh.red));
+  PQMC_FOR_2D(i, 0, N, k, 0, n) D[(long)k * ldd + i] = digit_pack(M(i, k), E);
   if (threadIdx.x == 0) sh.chol_bad = 0;
   __syncthreads();
-  for (int k = threadIdx.x; k < n; k += blockDim.x) d0[k] = C[(long)k * n + k];
-  if (threadIdx.x == 0) ip[0] = 1.0 / C[0];
+  auto eM = [E](int) { return E; };
+  digit_gemm<true>(n, n, N, D, ldd, 1, D, ldd, eM, eM, true, false,
+                   [C, n](int i, int j, double v) { C[(long)i * n + j] = v; });
   __syncthreads();
-  // right-looking factorisation: step k scales row k into U (U_kj = C_kj / p_k)
-  // and then updates the trailing block, C_ij -= C_ki U_kj (i, j > k; the
-  // part below the diagonal is updated too, so the flat loop keeps the warps
-  // full, and never read)
-  const int step = (int)blockDim.x;
-  for (int k = 0; k < n; ++k) {
-    const double p = C[(long)k * n + k];
-    if (!(p > 1e-12 * d0[k])) {          // same value in every thread: uniform exit
-      if (threadIdx.x == 0) sh.chol_bad = 1;
-      break;
+  for (int k = threadIdx.x; k < n; k += blockDim.x) dlim[k] = 1e-12 * C[(long)k * n + k];
+  __syncthreads();
+  x.mark(kPhOverlap);
+  // Elimination of [C | I], the part of I that has filled in kept below the
+  // diagonal: step k takes row k, u_j = row_kj / p_k, from the rows below,
+  //     row_ij -= C_ki u_j   (C_ki = C_ik; column k, still zero: -C_ki / p_k).
+  // Row k then holds the Schur complements C_kj right of the diagonal and row
+  // k of L^{-1} (L unit lower, C = L diag(p) L^T) left of it.  Warp 0 runs
+  // ahead: it takes row k + 1 first, its pivot, reciprocal and u, while the
+  // others do the rest of step k: one barrier per column, the reciprocal's
+  // latency beside the other rows' FMAs (a flat index with constant row
+  // length: full FP64 warp instructions, no division).
+  auto pivot_row = [&](int r, double* un) {
+    const double p = C[(long)r * n + r];
+    const bool ok = p > dlim[r];
+    const double ip = ok ? recip64(p) : 0.0;
+    if (lane == 0) {
+      pv[r] = p;
+      if (!ok) sh.chol_bad = 1;
     }
-    const double ipk = ip[k];
-    for (int j = k + 1 + (int)threadIdx.x; j < n; j += step) U[(long)k * n + j] = C[(long)k * n + j] * ipk;
-    __syncthreads();
-    const int m = n - k - 1;
-    if (m > 0) {
-      const int sq = step / m, sr = step - sq * m;
-      int i = (int)threadIdx.x / m, j = (int)threadIdx.x - i * m;
-      const double* Ck = C + (long)k * n + k + 1;
-      const double* Uk = U + (long)k * n + k + 1;
-      double* Cb = C + (long)(k + 1) * n + k + 1;
-      while (i < m) {
-        Cb[(long)i * n + j] = fma(-Ck[i], Uk[j], Cb[(long)i * n + j]);
-        if (i == 0 && j == 0) ip[k + 1] = 1.0 / Cb[0];
-        j += sr;
-        i += sq;
-        if (j >= m) { j -= m; ++i; }
+    for (int j = lane; j < n; j += 32) un[j] = j == r ? ip : C[(long)r * n + j] * ip;
+  };
+  if (warp == 0) pivot_row(0, u[0]);
+  __syncthreads();
+  {
+    const int rest = (int)blockDim.x - 32, tr = (int)threadIdx.x - 32;
+    const int sq = rest / n, sr = rest - sq * n;
+    const int i0 = tr / n, j0 = tr - i0 * n;
+    for (int k = 0; k + 1 < n && !sh.chol_bad; ++k) {
+      const double* uk = u[k & 1];
+      const double* Ck = C + (long)k * n;
+      if (warp == 0) {
+        const int r = k + 1;
+        double* Cr = C + (long)r * n;
+        const double m = Ck[r];
+        for (int j = lane; j < n; j += 32) Cr[j] = fma(-m, uk[j], j == k ? 0.0 : Cr[j]);
+        __syncwarp();
+        pivot_row(r, u[r & 1]);
+      } else {
+        int i = k + 2 + i0, j = j0;
+        while (i < n) {
+          double* c = C + (long)i * n + j;
+          *c = fma(-Ck[i], uk[j], j == k ? 0.0 : *c);
+          j += sr;
+          i += sq;
+          if (j >= n) { j -= n; ++i; }
+        }
       }
+      __syncthreads();
     }
-    __syncthreads();
   }
   __syncthreads();
   if (sh.chol_bad) return false;
-  for (int k = threadIdx.x; k < n; k += blockDim.x) isq[k] = rsqrt(C[(long)k * n + k]);
+  for (int k = threadIdx.x; k < n; k += blockDim.x) isq[k] = rsqrt(pv[k]);
   __syncthreads();
   x.mark(kPhQR);
-  {
-    // Q = M R^{-1}, right-looking over the columns of M: q_k = m_k / R_kk,
-    // m_j -= m_k U_kj for j > k, in blocks of four columns: each row first
-    // takes its block's own triangle in registers, then one flat pass
-    // applies the block's four updates to the later columns (a barrier pair
-    // per block instead of per column; every element sees the same FMAs in
-    // the same order as column by column)
-    for (int K = 0; K < n; K += 4) {
-      const int kb = min(4, n - K);
-      for (int i = threadIdx.x; i < N; i += blockDim.x) {
-        double mv[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) mv[u] = u < kb ? M[(long)(K + u) * ldm + i] : 0.0;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          if (u < kb) {
-            Q[(long)(K + u) * N + i] = mv[u] * isq[K + u];
-#pragma unroll
-            for (int v = u + 1; v < 4; ++v)
-              if (v < kb) mv[v] = fma(-mv[u], U[(long)(K + u) * n + K + v], mv[v]);
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (u < kb) M[(long)(K + u) * ldm + i] = mv[u];
-      }
-      __syncthreads();
-      const int j0 = K + kb;
-      if (j0 < n) {
-        const int sq = step / N, sr = step - sq * N;
-        const int t0 = (int)threadIdx.x / N, r0 = (int)threadIdx.x - t0 * N;
-        int jj = j0 + t0, i = r0;
-        while (jj < n) {
-          double acc = M[(long)jj * ldm + i];
-#pragma unroll
-          for (int u = 0; u < 4; ++u)
-            if (u < kb) acc = fma(-M[(long)(K + u) * ldm + i], U[(long)(K + u) * n + jj], acc);
-          M[(long)jj * ldm + i] = acc;
-          i += sr;
-          jj += sq;
-          if (i >= N) { i -= N; ++jj; }
-        }
-      }
-      __syncthreads();
-    }
+  // digits of R^{-1}: column j is row j of L^{-1} / sqrt(p_j), 1 / sqrt(p_j) on the diagonal
+  for (int j = warp; j < n; j += nw) {
+    const double f = isq[j];
+    int e = lane == 0 ? digit_exp(f) : kDigitNone;
+    for (int c = lane; c < j; c += 32) e = max(e, digit_exp(C[(long)j * n + c] * f));
+    e = __reduce_max_sync(0xffffffffu, e);
+    for (int c = lane; c < ldx; c += 32)
+      X[(long)j * ldx + c] = c < j ? digit_pack(C[(long)j * n + c] * f, e) : c == j ? digit_pack(f, e) : kDigitZero;
+    if (lane == 0) ex[j] = e;
   }
+  __syncthreads();
+  digit_gemm<false>(N, n, n, D, 1, ldd, X, ldx, eM, [ex](int j) { return ex[j]; }, false, true,
+                    [Q, N](int i, int j, double v) { Q[(long)j * N + i] = v; });
   // log|det R|
-  {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (warp == 0) {
-      double la = 0.0;
-      for (int k = lane; k < n; k += 32) la += log(C[(long)k * n + k]);
-      la = warp_sum(la);
-      if (lane == 0) sh.red[0] = 0.5 * la;
-    }
-    __syncthreads();
-    logabs = sh.red[0];
-    __syncthreads();
+  if (warp == 0) {
+    double la = 0.0;
+    for (int k = lane; k < n; k += 32) la += log(pv[k]);
+    la = warp_sum(la);
+    if (lane == 0) sh.red[0] = 0.5 * la;
   }
+  __syncthreads();
+  logabs = sh.red[0];
+  __syncthreads();
   x.mark(kPhQRForm);
   return true;
 }
 
 // Invert O_s (n_s x n_s, row-major) in place for both spins at once by
 // Gauss-Jordan elimination with partial pivoting (Golub & Van Loan, section
-// 3.2): warp s finds the pivot of spin s, swaps the rows, scales the pivot row
-// and saves the pivot column; the CTA then eliminates that column from every
-// other row; the row interchanges are undone on the columns at the end.
-// Returns log|det O_s| and sign(det O_s) to every thread.
+// 3.2), one half of the CTA per spin.  Rows are not interchanged: step j
+// takes the largest |A_ij| over the rows not used yet (row r_j), and at the end
+// (O^{-1})_{j, r_c} = A_{r_j, c} (gj_rows; the caller reads the inverse through
+// it).  A step is one barrier for the scaled pivot row and one for the
+// elimination, one FP64 FMA per element over a flat index; meanwhile the
+// half's first warp eliminates column j + 1 first and finds its pivot and
+// reciprocal, so that their latency (shuffles, five dependent FP64 steps)
+// passes beside the others' FMAs, which the FP64 pipe bounds: 2 n^2 / 32 warp
+// instructions of 16 cycles (1300 cycles at n = 36; a step took 5.7 kcycles
+// with the search, the interchange and a division between two barriers).
+// Leaves log|det O_s| and sign(det O_s) in sh.gj_logabs, sh.gj_sign.
 template <typename T, bool RES>
-__device__ __forceinline__ void gj_invert2(Cta<T, RES>& x, const int n[2], double* O[2], double logabs[2], double sgn[2]) {
+__device__ __forceinline__ void gj_invert2(Cta<T, RES>& x) {
   Smem<T>& sh = x.sh;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int nmax = n[0] > n[1] ? n[0] : n[1];
-  if (threadIdx.x < 2) sh.nswap[threadIdx.x] = 0;
+  const int half = (int)blockDim.x >> 1;
+  const int s = (int)threadIdx.x >= half ? 1 : 0;
+  const int tid = (int)threadIdx.x - s * half, lane = threadIdx.x & 31;
+  const bool first = tid < 32;
+  const int n = x.nsig(s), nmax = max(x.nsig(0), x.nsig(1));
+  double* A = x.Ob(s);
+  double* f = x.gj_col(s);              // column j before step j, two steps in flight: f[(j & 1) n ..]
+  double* R = x.gj_row(s);              // scaled pivot row of the step
+  int* rows = x.gj_rows(s);
+  unsigned used = 0;                    // bit b: row lane + 32 b has been a pivot row
+  // column j at hand in f: pivot row and reciprocal (first warp of the half)
+  auto pick = [&](int j) {
+    const double* fj = f + (j & 1) * n;
+    unsigned long long best = 0;
+    int bi = -1;
+    for (int i = lane, b = 0; i < n; i += 32, ++b) {
+      // |x| is compared through the bit pattern with the sign cleared, which
+      // orders non-negative doubles like their values
+      const unsigned long long v = (unsigned long long)__double_as_longlong(fj[i]) & 0x7fffffffffffffffull;
+      if (!((used >> b) & 1u) && (bi < 0 || v > best)) { best = v; bi = i; }
+    }
+    const unsigned hi = (unsigned)(best >> 32), top = __reduce_max_sync(0xffffffffu, bi < 0 ? 0u : hi);
+    const unsigned lo = __reduce_max_sync(0xffffffffu, (bi >= 0 && hi == top) ? (unsigned)best : 0u);
+    const bool mine = bi >= 0 && hi == top && (unsigned)best == lo;
+    const int r = (int)__reduce_min_sync(0xffffffffu, mine ? (unsigned)bi : 0xffffffffu);   // ties to the lower row
+    if ((r & 31) == lane) used |= 1u << (r >> 5);
+    const double p = fj[r];
+    if (lane == 0) {
+      x.pval(s)[j] = p;
+      rows[j] = r;
+      sh.gj_ip[s] = p != 0.0 ? recip64(p) : 0.0;
+      if (p == 0.0) atomicOr(&sh.err, kErrStab);
+    }
+  };
+  if (first && n > 0) {
+    for (int i = lane; i < n; i += 32) f[i] = A[(long)i * n];
+    __syncwarp();
+    pick(0);
+  }
+  const int rest = half > 32 ? half - 32 : half, tr = half > 32 ? tid - 32 : tid;
+  const int sq = n > 0 ? rest / n : 0, sr = n > 0 ? rest - sq * n : 0;
+  const int i0 = n > 0 && tr >= 0 ? tr / n : 0, j0 = tr - i0 * n;
   __syncthreads();
   for (int j = 0; j < nmax; ++j) {
-    if (warp < 2 && j < n[warp]) {
-      const int s = warp, ns = n[s];
-      double* A = O[s];
-      double* f = x.lmul(s);
-      // pivot: largest |A_ij|, i >= j, ties to the lower row; |x| is compared
-      // through the bit pattern with the sign cleared, which orders
-      // non-negative doubles like their values
-      unsigned long long best = 0;
-      int bi = j;
-      for (int i = j + lane; i < ns; i += 32) {
-        const unsigned long long v = (unsigned long long)__double_as_longlong(A[(long)i * ns + j]) & 0x7fffffffffffffffull;
-        if (v > best || bi == j && i == j) { best = v; bi = i; }
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long ob = __shfl_xor_sync(0xffffffffu, best, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-      }
-      if (bi != j) {
-        for (int col = lane; col < ns; col += 32) {
-          const double t = A[(long)j * ns + col];
-          A[(long)j * ns + col] = A[(long)bi * ns + col];
-          A[(long)bi * ns + col] = t;
-        }
-        if (lane == 0) sh.nswap[s]++;
-      }
-      if (lane == 0) x.pinv(s)[j] = (double)bi;         // row interchange of step j
-      __syncwarp();
-      const double pv = A[(long)j * ns + j];
-      const double ip = pv != 0.0 ? 1.0 / pv : 0.0;
-      if (lane == 0) {
-        x.pval(s)[j] = pv;
-        if (pv == 0.0) sh.err |= kErrStab;
-      }
-      for (int i = lane; i < ns; i += 32) f[i] = A[(long)i * ns + j];
-      __syncwarp();
-      for (int col = lane; col < ns; col += 32) A[(long)j * ns + col] = (col == j) ? ip : A[(long)j * ns + col] * ip;
+    const double* fj = f + (j & 1) * n;
+    double* fn = f + ((j + 1) & 1) * n;
+    const int r = j < n ? rows[j] : 0;
+    if (j < n) {
+      const double ip = sh.gj_ip[s];
+      for (int c = tid; c < n; c += half) R[c] = c == j ? ip : A[(long)r * n + c] * ip;
     }
     __syncthreads();
     x.mark(kPhGJPivot);
-    // eliminate column j from every other row of both spins: one FMA per
-    // element over a flat index (full warps on the FP64 pipe); the pivot
-    // column takes -f_i / pivot through the same FMA with a zero addend
-    for (int s = 0; s < 2; ++s) {
-      const int ns = n[s];
-      if (j >= ns) continue;
-      double* A = O[s];
-      const double* fl = x.lmul(s);
-      // flat (row, column) index stepped incrementally
-      const int step = (int)blockDim.x, sq = step / ns, sr = step - sq * ns;
-      int i = (int)threadIdx.x / ns, col = (int)threadIdx.x - i * ns;
-      while (i < ns) {
-        const double add = col == j ? 0.0 : A[(long)i * ns + col];
-        const double r = fma(-fl[i], A[(long)j * ns + col], add);
-        if (i != j) A[(long)i * ns + col] = r;
-        col += sr;
-        i += sq;
-        if (col >= ns) { col -= ns; ++i; }
+    if (j < n) {
+      if (first && j + 1 < n) {
+        const double rn = R[j + 1];
+        for (int i = lane; i < n; i += 32) {
+          const double v = i == r ? rn : fma(-fj[i], rn, A[(long)i * n + j + 1]);
+          A[(long)i * n + j + 1] = v;
+          fn[i] = v;
+        }
+        __syncwarp();
+        pick(j + 1);
+      }
+      if (!first || half <= 32) {
+        int i = i0, c = j0;
+        while (i < n) {
+          if (c != j + 1) {
+            double* a = A + (long)i * n + c;
+            const double v = fma(-fj[i], R[c], c == j ? 0.0 : *a);
+            *a = i == r ? R[c] : v;
+          }
+          c += sr;
+          i += sq;
+          if (c >= n) { c -= n; ++i; }
+        }
       }
     }
     __syncthreads();
     x.mark(kPhGJElim);
   }
-  // undo the row interchanges on the columns, last step first
-  if (warp < 2) {
-    const int s = warp, ns = n[s];
-    double* A = O[s];
-    for (int j = ns - 1; j >= 0; --j) {
-      const int p = (int)x.pinv(s)[j];
+  // parity of the permutation j -> r_j: its inversions
+  if (threadIdx.x < 2) sh.nswap[threadIdx.x] = 0;
+  __syncthreads();
+  {
+    int inv = 0;
+    for (int a = tid; a < n; a += half)
+      for (int b = a + 1; b < n; ++b) inv += rows[a] > rows[b] ? 1 : 0;
+    if (inv) atomicAdd(&sh.nswap[s], inv);
+  }
+  __syncthreads();
+  for (int sp = 0; sp < 2; ++sp) {
+    double la, sg;
+    log_det_of(x, x.pval(sp), x.nsig(sp), sh.nswap[sp], la, sg);
+    if (threadIdx.x == 0) {
+      sh.gj_logabs[sp] = la;
+      sh.gj_sign[sp] = sg;
+    }
+  }
+  __syncthreads();
+  x.mark(kPhGJTail);
+}
+
+// The inverse of spin s as a plain matrix, in place: row j from row r_j, then
+// column r_c from column c, as interchanges by one warp (the FP64 path and the
+// FP64 diagnostics; the reduced paths read through gj_rows instead).
+template <typename T, bool RES>
+__device__ __forceinline__ void gj_unpermute(Cta<T, RES>& x, int s) {
+  const int n = x.nsig(s);
+  double* A = x.Ob(s);
+  const int* rows = x.gj_rows(s);
+  int* at = x.gj_rows(s) + n;           // original row at each place
+  int* swp = at + n;                    // place interchanged with j
+  if (threadIdx.x < 32) {
+    const int lane = threadIdx.x;
+    for (int i = lane; i < n; i += 32) at[i] = i;
+    __syncwarp();
+    for (int j = 0; j < n; ++j) {
+      // place j takes original row r_j: find where it is now (at or after j)
+      unsigned p = 0xffffffffu;
+      for (int i = j + lane; i < n; i += 32)
+        if (at[i] == rows[j]) p = (unsigned)i;
+      p = __reduce_min_sync(0xffffffffu, p);
+      if ((int)p != j)
+        for (int c = lane; c < n; c += 32) {
+          const double t = A[(long)j * n + c];
+          A[(long)j * n + c] = A[(long)p * n + c];
+          A[(long)p * n + c] = t;
+        }
+      if (lane == 0) {
+        at[p] = at[j];
+        at[j] = rows[j];
+        swp[j] = (int)p;
+      }
+      __syncwarp();
+    }
+    // columns: the same interchanges, last first (column r_c from column c)
+    for (int j = n - 1; j >= 0; --j) {
+      const int p = swp[j];
       if (p != j)
-        for (int i = lane; i < ns; i += 32) {
-          const double t = A[(long)i * ns + j];
-          A[(long)i * ns + j] = A[(long)i * ns + p];
-          A[(long)i * ns + p] = t;
+        for (int i = lane; i < n; i += 32) {
+          const double t = A[(long)i * n + j];
+          A[(long)i * n + j] = A[(long)i * n + p];
+          A[(long)i * n + p] = t;
         }
       __syncwarp();
     }
   }
   __syncthreads();
-  for (int s = 0; s < 2; ++s) log_det_of(x, x.pval(s), n[s], sh.nswap[s], logabs[s], sgn[s]);
-  x.mark(kPhGJTail);
-}
-
-// C = A^T B for column-major A, B (K x m and K x m', ld K): FP64, 2 x 3
-// outputs per thread (a 36 x 36 product is 216 tiles: one pass of a
-// 256-thread CTA).
-static __device__ void gemm_tn_f64(int m, int mp, int K, const double* A, const double* B, double* C, int ldc) {
-  const int tm = (m + 1) >> 1, tn = (mp + 2) / 3;
-  for (int t = threadIdx.x; t < tm * tn; t += blockDim.x) {
-    const int i0 = (t / tn) << 1, j0 = (t % tn) * 3;
-    const double* a0 = A + (long)i0 * K;
-    const double* a1 = A + (long)min(i0 + 1, m - 1) * K;
-    const double* b0 = B + (long)j0 * K;
-    const double* b1 = B + (long)min(j0 + 1, mp - 1) * K;
-    const double* b2 = B + (long)min(j0 + 2, mp - 1) * K;
-    double c00 = 0, c01 = 0, c02 = 0, c10 = 0, c11 = 0, c12 = 0;
-#pragma unroll 4
-    for (int k = 0; k < K; ++k) {
-      const double x0 = a0[k], x1 = a1[k], y0 = b0[k], y1 = b1[k], y2 = b2[k];
-      c00 = fma(x0, y0, c00);
-      c01 = fma(x0, y1, c01);
-      c02 = fma(x0, y2, c02);
-      c10 = fma(x1, y0, c10);
-      c11 = fma(x1, y1, c11);
-      c12 = fma(x1, y2, c12);
-    }
-    C[(long)i0 * ldc + j0] = c00;
-    if (j0 + 1 < mp) C[(long)i0 * ldc + j0 + 1] = c01;
-    if (j0 + 2 < mp) C[(long)i0 * ldc + j0 + 2] = c02;
-    if (i0 + 1 < m) {
-      C[(long)(i0 + 1) * ldc + j0] = c10;
-      if (j0 + 1 < mp) C[(long)(i0 + 1) * ldc + j0 + 1] = c11;
-      if (j0 + 2 < mp) C[(long)(i0 + 1) * ldc + j0 + 2] = c12;
-    }
-  }
 }
 
 static __device__ void copy_block(const double* src, double* dst, int n) {
@@ -1717,27 +1733,51 @@ __device__ __forceinline__ double* stack_block(const Cta<T, RES>& x, double* bas
   return base + ((long)b * 2 + s) * x.c.N * x.c.nmax;
 }
 
+// Calls f(element(i, k)) with the accessor of the block phase_stack left for
+// spin s: a product in the path precision, or e^{V(s_tau0)} P in FP64 for the
+// blocks at the ends of the projection.
+template <typename T, bool RES, typename F>
+__device__ __forceinline__ void with_block(Cta<T, RES>& x, int left, int s, F f) {
+  const int n = x.nsig(s), N = x.c.N;
+  if (x.sh.src == 2) {
+    const double* P = x.c.P + (long)s * N * x.c.nmax;
+    const int tau = left ? x.c.Ltau + 1 : 0;
+    f([&x, P, tau, s, N](int i, int k) { return x.vexp(tau, s, i) * P[(long)k * N + i]; });
+  } else {
+    const T* Mt = x.sh.src ? x.Mt2() : x.Mt();
+    f([Mt, n](int i, int k) { return Mt[(long)i * n + k]; });
+  }
+}
+// M64 = that block, column-major
+template <typename T, bool RES>
+__device__ __forceinline__ void block_to_m64(Cta<T, RES>& x, int b, int left, int s) {
+  const int ldm = m64_ld(x.c.N);
+  double* M = x.M64();
+  with_block(x, left, s, [&](auto e) {
+    PQMC_FOR_2D(k, 0, x.nsig(s), i, 0, x.c.N) M[(long)k * ldm + i] = (double)e(i, k);
+  });
+  __syncthreads();
+}
+
 // Right stack block b: QR of B_{b n} ... B_{(b-1)n+1} Q_R[b-1] (b >= 1) or of B_0 P (b = 0).
 // Left stack block b holds (B_L(b n))^T = Q T^T: QR of
 // B_{bn+1}^T ... B_{(b+1)n}^T Q_L[b+1] (b < nb) or of e^{V(s_{Ltau+1})} P (b = nb).
-// phase_stack forms the block to factorise, of spin s, in M64: the slice
-// products run in the path precision on a row-major copy.
+// phase_stack forms the block to factorise, of spin s (sh.src says where): the
+// slice products run in the path precision on a row-major copy.
 template <typename T, bool RES>
 __device__ __noinline__ void phase_stack(int b, int left, int s) {
   auto x = this_cta<T, RES>();
   const ChainDesc& c = x.c;
   const int N = c.N, n_stab = c.n_stab;
-  const int ldm = m64_ld(N);
-  double* M = x.M64();
   const int n = x.nsig(s);
   T* Mt = x.Mt();
   T* Mt2 = x.Mt2();
+  constexpr bool f64 = std::is_same<T, double>::value;
+  int src = 0;
   if (left ? b == c.nb : b == 0) {
-    const double* P = c.P + (long)s * N * c.nmax;
     const int tau = left ? c.Ltau + 1 : 0;
     x.stage(tau);
-    PQMC_FOR_2D(k, 0, n, i, 0, N) M[(long)k * ldm + i] = x.vexp(tau, s, i) * P[(long)k * N + i];
-    __syncthreads();
+    src = 2;
   } else {
     const double* prev = left ? stack_block(x, c.Lst, b + 1, s) : stack_block(x, c.Rst, b - 1, s);
     PQMC_FOR_2D(k, 0, n, i, 0, N) Mt[(long)i * n + k] = (T)prev[(long)k * N + i];
@@ -1749,6 +1789,7 @@ __device__ __noinline__ void phase_stack(int b, int left, int s) {
         cta_gemm<T>(N, n, N, x.Em(), 1, c.ld, Mt, n, 1, Mt2, n, 1, EpiStore());
         __syncthreads();
         T* t = Mt; Mt = Mt2; Mt2 = t;
+        src ^= 1;
       }
     } else {
       __syncthreads();
@@ -1759,21 +1800,30 @@ __device__ __noinline__ void phase_stack(int b, int left, int s) {
         __syncthreads();
       }
     }
-    PQMC_FOR_2D(k, 0, n, i, 0, N) M[(long)k * ldm + i] = (double)Mt[(long)i * n + k];
-    __syncthreads();
   }
+  if (threadIdx.x == 0) x.sh.src = src;
+  __syncthreads();
+  if (f64) block_to_m64(x, b, left, s);
   x.mark(kPhStack);
 }
 
 template <typename T, bool RES>
-__device__ __noinline__ bool phase_chol(int n, double* logabs) {
+__device__ __noinline__ bool phase_chol(int b, int left, int s, double* logabs) {
   auto x = this_cta<T, RES>();
-  return qr_cholesky(x, x.c.N, m64_ld(x.c.N), n, x.M64(), x.Q64(), *logabs);
+  const int N = x.c.N, n = x.nsig(s);
+  double* Q = stack_block(x, left ? x.c.Lst : x.c.Rst, b, s);
+  bool ok = false;
+  with_block(x, left, s, [&](auto e) { ok = qr_cholesky(x, N, n, Q, *logabs, e); });
+  return ok;
 }
 template <typename T, bool RES>
-__device__ __noinline__ void phase_householder(int n, double* logabs, double* sgn) {
+__device__ __noinline__ void phase_householder(int b, int left, int s, double* logabs, double* sgn) {
   auto x = this_cta<T, RES>();
-  qr_householder(x, x.c.N, m64_ld(x.c.N), n, x.M64(), x.Q64(), *logabs, *sgn);
+  const int N = x.c.N, n = x.nsig(s);
+  if (!std::is_same<T, double>::value) block_to_m64(x, b, left, s);
+  qr_householder(x, N, m64_ld(N), n, x.M64(), x.Q64(), *logabs, *sgn);
+  copy_block(x.Q64(), stack_block(x, left ? x.c.Lst : x.c.Rst, b, s), N * n);
+  x.mark(kPhQR);
 }
 
 // the new stack block b of both species
@@ -1782,14 +1832,11 @@ __device__ __forceinline__ void push_block(int b, int left) {
   auto x = this_cta<T, RES>();
   const ChainDesc& c = x.c;
   for (int s = 0; s < x.nspec(); ++s) {
-    const int n = x.nsig(s);
     phase_stack<T, RES>(b, left, s);
     double la, sg = 1.0;
     bool done = false;
-    if constexpr (!std::is_same<T, double>::value) done = phase_chol<T, RES>(n, &la);
-    if (!done) phase_householder<T, RES>(n, &la, &sg);
-    copy_block(x.Q64(), stack_block(x, left ? c.Lst : c.Rst, b, s), c.N * n);
-    x.mark(kPhQR);
+    if constexpr (!std::is_same<T, double>::value) done = phase_chol<T, RES>(b, left, s, &la);
+    if (!done) phase_householder<T, RES>(b, left, s, &la, &sg);
     if (threadIdx.x == 0) {
       double* lg = left ? c.Llog : c.Rlog;
       const bool first = left ? b == c.nb : b == 0;
@@ -1878,9 +1925,15 @@ __device__ __forceinline__ void assemble_spin(Cta<T, RES>& x, int s, const doubl
   if constexpr (std::is_same<T, double>::value) {
     cta_gemm<T>(ns, N, ns, Xinv, ns, 1, ql, N, 1, Y, ld, 1, EpiStore());
   } else {
-    // O^{-1} to the path precision once, then a path-precision product
+    // O^{-1} to the path precision once (in the order of its rows and columns),
+    // then a path-precision product
     T* ot = x.Ot();
-    for (int e = threadIdx.x; e < ns * ns; e += blockDim.x) ot[e] = (T)Xinv[e];
+    if (c.dg64) {
+      for (int e = threadIdx.x; e < ns * ns; e += blockDim.x) ot[e] = (T)Xinv[e];
+    } else {
+      const int* rows = x.gj_rows(s);
+      PQMC_FOR_2D(j, 0, ns, k, 0, ns) ot[(long)j * ns + rows[k]] = (T)Xinv[(long)rows[j] * ns + k];
+    }
     __syncthreads();
     cta_gemm<T>(ns, N, ns, ot, ns, 1, ql, N, 1, Y, ld, 1, EpiStore());
   }
@@ -1909,30 +1962,48 @@ __device__ __forceinline__ void assemble_spin(Cta<T, RES>& x, int s, const doubl
 // propagated G against the same formula assembled in FP64 from the FP64
 // factors; the G that replaces the propagated one is still the
 // path-precision assembly, so the chain itself is unchanged.
+// O_s = Q_L^T Q_R of both spins, from the digits of the two blocks (columns of
+// orthonormal matrices: exponent 1; should an element reach 2, the blocks are
+// packed again against the largest).
 template <typename T, bool RES>
 __device__ __noinline__ void phase_overlap(int b) {
-  // O_s = Q_L^T Q_R in FP64, both spins
   auto x = this_cta<T, RES>();
   const ChainDesc& c = x.c;
-  for (int s = 0; s < 2; ++s) {
+  const int N = c.N, ldd = digit_ld(N);
+  unsigned long long* DL = reinterpret_cast<unsigned long long*>(x.scr + x.L.dq);
+  for (int s = 0; s < x.nspec(); ++s) {
     const int n = x.nsig(s);
-    gemm_tn_f64(n, n, c.N, stack_block(x, c.Lst, b, s), stack_block(x, c.Rst, b, s), x.Ob(s), n);
+    unsigned long long* DR = DL + (long)ldd * n;
+    const double* QL = stack_block(x, c.Lst, b, s);
+    const double* QR = stack_block(x, c.Rst, b, s);
+    int E = 1;
+    for (int pass = 0; pass < 2; ++pass) {
+      int e = kDigitNone;
+      PQMC_FOR_2D(k, 0, n, i, 0, N) {
+        const double l = QL[(long)k * N + i], r = QR[(long)k * N + i];
+        e = max(e, max(digit_exp(l), digit_exp(r)));
+        DL[(long)k * ldd + i] = digit_pack(l, E);
+        DR[(long)k * ldd + i] = digit_pack(r, E);
+      }
+      const bool again = __syncthreads_or(e > E) != 0;
+      if (!again) break;
+      E = digit_cta_max(e, reinterpret_cast<int*>(x.sh.red));
+      __syncthreads();
+    }
+    double* O = x.Ob(s);
+    auto eQ = [E](int) { return E; };
+    digit_gemm<true>(n, n, N, DL, ldd, 1, DR, ldd, eQ, eQ, false, false,
+                     [O, n](int i, int j, double v) { O[(long)i * n + j] = v; });
+    __syncthreads();
   }
-  __syncthreads();
   x.mark(kPhOverlap);
 }
 template <typename T, bool RES>
 __device__ __noinline__ void phase_inverse() {
   auto x = this_cta<T, RES>();
-  int n[2] = {x.nsig(0), x.nsig(1)};
-  double* O[2] = {x.Ob(0), x.Ob(1)};
-  double la[2], sg[2];
-  gj_invert2(x, n, O, la, sg);
-  if (threadIdx.x < 2) {
-    x.sh.gj_logabs[threadIdx.x] = threadIdx.x ? la[1] : la[0];
-    x.sh.gj_sign[threadIdx.x] = threadIdx.x ? sg[1] : sg[0];
-  }
-  __syncthreads();
+  gj_invert2(x);
+  if (std::is_same<T, double>::value || x.c.dg64)
+    for (int s = 0; s < x.nspec(); ++s) gj_unpermute(x, s);
   x.mark(kPhLU);
 }
 template <typename T, bool RES>
