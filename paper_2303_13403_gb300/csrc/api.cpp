@@ -56,7 +56,7 @@ struct HostChain {
   pqmc_chain_spec spec;
   int N, ld, nup, ndn, nmax, Ltau, nb, nfld;
   size_t off_fields, off_G, off_Rst, off_Lst, off_Rlog, off_Llog, off_meas, off_dG,
-      off_acc, off_state, off_P, off_scratch, off_expKm, off_expKp, off_expKm64, off_K64, off_eps, off_bonds,
+      off_acc, off_state, off_P, off_scratch, off_expKm, off_expKp, off_digits, off_expKm64, off_K64, off_eps, off_bonds,
       off_sbonds, off_spread;
 };
 
@@ -112,6 +112,7 @@ bool is_tv(const pqmc_chain_spec& s) { return s.lattice.kind == PQMC_HONEYCOMB_T
 // model tables shared by chains with the same lattice and dtau
 struct ModelTables {
   std::vector<double> K, eps, w, V, expKm, expKp;
+  int eEm = 0, eEp = 0;                     // exponents of the two exponentials (digit_gemm.cuh)
   std::vector<int> bond_ends, site_bonds;   // t-V only
 };
 
@@ -207,6 +208,26 @@ void put(Staged& a, size_t off, const std::vector<double>& src, int rows, int co
   T* p = reinterpret_cast<T*>(a.at(off, (size_t)rows * ld * sizeof(T)));
   for (int i = 0; i < rows; ++i)
     for (int j = 0; j < cols; ++j) p[(size_t)i * ld + j] = (T)src[(size_t)i * cols + j];
+}
+
+// smallest E with |x| < 2^E for every x of v
+int max_exponent(const std::vector<double>& v) {
+  int e = -1000;
+  for (double x : v) {
+    int k = 0;
+    std::frexp(x, &k);
+    if (x != 0.0) e = std::max(e, k);
+  }
+  return e;
+}
+
+// Digits of an N x N matrix for digit_gemm.cuh: element (b, a) at
+// a digit_ld(N) + b, x = X 2^{E - 62} packed as X + 0x80...80.
+void pack_digits(uint64_t* dig, const std::vector<double>& m, int N, int E) {
+  const int ldd = digit_ld(N);
+  for (int a = 0; a < N; ++a)
+    for (int b = 0; b < N; ++b)
+      dig[(size_t)a * ldd + b] = (uint64_t)std::llround(std::ldexp(m[(size_t)b * N + a], 62 - E)) + 0x8080808080808080ull;
 }
 
 void put_raw(Staged& a, size_t off, const void* src, size_t n) { memcpy(a.at(off, n), src, n); }
@@ -346,10 +367,13 @@ pqmc_status build_ctx(int n, const pqmc_chain_spec* specs, const pqmc_opts* opts
       if (!sym_eig(h.N, mt.K, mt.w, mt.V)) { delete ctx; return fail(nullptr, PQMC_EINVAL, "eigensolver failed on K"); }
       expm_from_eig(h.N, mt.w, mt.V, -s.dtau, mt.expKm);
       expm_from_eig(h.N, mt.w, mt.V, +s.dtau, mt.expKp);
+      mt.eEm = max_exponent(mt.expKm);
+      mt.eEp = max_exponent(mt.expKp);
       models[key] = std::move(mt);
       const size_t Tm = (size_t)h.N * h.ld * ctx->tsize;
       const size_t o1 = take(Tm);
       take(Tm);
+      if (ctx->prec == PQMC_FP64) take(2 * (size_t)h.N * digit_ld(h.N) * 8);   // digits of e^{-+dtau K}
       take((size_t)h.N * h.N * 8);
       take((size_t)h.N * h.N * 8);
       take((size_t)h.N * 8);
@@ -378,7 +402,8 @@ pqmc_status build_ctx(int n, const pqmc_chain_spec* specs, const pqmc_opts* opts
     }
     h.off_expKm = model_off[key];
     h.off_expKp = h.off_expKm + align_up((size_t)h.N * h.ld * ctx->tsize, 256);
-    h.off_expKm64 = h.off_expKp + align_up((size_t)h.N * h.ld * ctx->tsize, 256);
+    h.off_digits = h.off_expKp + align_up((size_t)h.N * h.ld * ctx->tsize, 256);
+    h.off_expKm64 = h.off_digits + (ctx->prec == PQMC_FP64 ? align_up(2 * (size_t)h.N * digit_ld(h.N) * 8, 256) : 0);
     h.off_K64 = h.off_expKm64 + align_up((size_t)h.N * h.N * 8, 256);
     h.off_eps = h.off_K64 + align_up((size_t)h.N * h.N * 8, 256);
     h.off_bonds = h.off_eps + align_up((size_t)h.N * 8, 256);
@@ -439,6 +464,10 @@ pqmc_status build_ctx(int n, const pqmc_chain_spec* specs, const pqmc_opts* opts
       if (ctx->prec == PQMC_FP64) {
         put<double>(A, h.off_expKm, mt.expKm, h.N, h.N, h.ld);
         put<double>(A, h.off_expKp, mt.expKp, h.N, h.N, h.ld);
+        const size_t tab = (size_t)h.N * digit_ld(h.N);
+        uint64_t* dig = reinterpret_cast<uint64_t*>(A.at(h.off_digits, 2 * tab * 8));
+        pack_digits(dig, mt.expKm, h.N, mt.eEm);
+        pack_digits(dig + tab, mt.expKp, h.N, mt.eEp);
       } else {
         put<float>(A, h.off_expKm, mt.expKm, h.N, h.N, h.ld);
         put<float>(A, h.off_expKp, mt.expKp, h.N, h.N, h.ld);
@@ -517,6 +546,13 @@ pqmc_status build_ctx(int n, const pqmc_chain_spec* specs, const pqmc_opts* opts
     d.G = b + h.off_G;
     d.expKm = b + h.off_expKm;
     d.expKp = b + h.off_expKp;
+    if (ctx->prec == PQMC_FP64) {
+      const ModelTables& mt = models[lattice_key(s)];
+      d.dEm = reinterpret_cast<const unsigned long long*>(b + h.off_digits);
+      d.dEp = d.dEm + (size_t)h.N * digit_ld(h.N);
+      d.eEm = mt.eEm;
+      d.eEp = mt.eEp;
+    }
     d.expKm64 = reinterpret_cast<const double*>(b + h.off_expKm64);
     d.K64 = reinterpret_cast<const double*>(b + h.off_K64);
     d.eps = reinterpret_cast<const double*>(b + h.off_eps);

@@ -64,6 +64,9 @@ struct ChainDesc {
   const void* expKm;       // N x ld (T): e^{-dtau K}
   const void* expKp;       // N x ld (T): e^{+dtau K}
   const double* expKm64;   // N x N FP64
+  const unsigned long long* dEm;  // FP64 path: packed digits of e^{-dtau K}, element (b, a) at a digit_ld(N) + b, or null
+  const unsigned long long* dEp;  // the same of e^{+dtau K}
+  int eEm, eEp;            // their exponents
   const double* K64;       // N x N FP64
   const double* eps;       // N: staggered sublattice sign (+1 A, -1 B)
   const int* bond_ends;    // tv: 3N/2 x 2 (A end, B end) of each bond
@@ -99,7 +102,7 @@ namespace pqmc {
 
 // Byte offsets of the phase buffers inside one chain's scratch region.  The
 // phases never overlap in time, so their buffers share the region:
-//   wrap    : Gt (N x ld, T) for one spin at a time; for a chain resident in
+//   wrap    : Gt (N x ld, T; FP64 path: packed digits of G) for one spin at a time; for a chain resident in
 //             shared memory also copies of e^{-dtau K} and e^{+dtau K}
 //             (em, ep; 0 when they would make the scratch larger)
 //   flips   : the update vectors of a delayed block, U (N x kw, T) and V
@@ -159,6 +162,7 @@ PQMC_HDI ScratchLayout scratch_layout(int N, int ld, int n, int tsize, int kd) {
   L.m64 = 0;
   L.mtq = al16((size_t)m64_ld(N) * n * 8);
   if (chol && dig > L.mtq) L.mtq = dig;
+  if (!chol) L.mtq = al16((size_t)(N + 1) * n * 8);     // digits of a product's right factor, ld even
   L.mt2 = L.mtq + al16(Nn * tsize);
   size_t mtq_sz = 2 * al16(Nn * tsize);
   if (al16(Nn * 8) > mtq_sz) mtq_sz = al16(Nn * 8);

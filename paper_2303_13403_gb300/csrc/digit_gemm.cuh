@@ -130,14 +130,14 @@ static __device__ __forceinline__ void digit_mma(float c[4], uint32_t a0, uint32
 }
 
 // C = A B by one CTA (every thread calls; no barrier inside): A(i, k) =
-// A[i sai + k sak], B(k, j) = B[j sbj + k] packed digits, k contiguous in B
-// and, with kAk, in A (sak = 1); rows 16-byte aligned then.  ea(i), eb(j):
+// A[i sai + k sak], B(k, j) = B[j sbj + k sbk] packed digits; kAk (kBk): k
+// contiguous in A (B), sak = 1 (sbk = 1) and rows 16-byte aligned.  ea(i), eb(j):
 // exponents.  epi(i, j, value) for every element; with upper, only the 16 x 8
 // tiles that reach j >= i; with btri, B(k, j) = 0 for k > j is left out.  One warp per tile, its 36 digit-pair sums in 32
 // accumulator registers.
-template <bool kAk, typename EA, typename EB, typename Epi>
+template <bool kAk, bool kBk, typename EA, typename EB, typename Epi>
 __device__ __forceinline__ void digit_gemm(int M, int Nn, int K, const unsigned long long* A, int sai, int sak,
-                                           const unsigned long long* B, int sbj, EA ea, EB eb, bool upper, bool btri, Epi epi) {
+                                           const unsigned long long* B, int sbj, int sbk, EA ea, EB eb, bool upper, bool btri, Epi epi) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int tm = (M + 15) >> 4, tn = (Nn + 7) >> 3;
   int m0 = 0, n0 = 8 * (int)(threadIdx.x >> 5);
@@ -175,8 +175,16 @@ __device__ __forceinline__ void digit_gemm(int M, int Nn, int K, const unsigned 
               ya[6 + e] = pa1[(long)(k + 8 + e) * sak];
             }
           }
-          const ulonglong2 w0 = *reinterpret_cast<const ulonglong2*>(pb + k), w1 = *reinterpret_cast<const ulonglong2*>(pb + k + 8);
-          yb[0] = w0.x; yb[1] = w0.y; yb[2] = w1.x; yb[3] = w1.y;
+          if (kBk) {
+            const ulonglong2 w0 = *reinterpret_cast<const ulonglong2*>(pb + k), w1 = *reinterpret_cast<const ulonglong2*>(pb + k + 8);
+            yb[0] = w0.x; yb[1] = w0.y; yb[2] = w1.x; yb[3] = w1.y;
+          } else {
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+              yb[e] = pb[(long)(k + e) * sbk];
+              yb[2 + e] = pb[(long)(k + 8 + e) * sbk];
+            }
+          }
         } else {
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
@@ -184,7 +192,7 @@ __device__ __forceinline__ void digit_gemm(int M, int Nn, int K, const unsigned 
             const bool in = kk < K;
             ya[4 * (e >> 1) + (e & 1)] = in ? pa0[(long)kk * sak] : kDigitZero;
             ya[4 * (e >> 1) + 2 + (e & 1)] = in ? pa1[(long)kk * sak] : kDigitZero;
-            yb[e] = in ? pb[kk] : kDigitZero;
+            yb[e] = in ? pb[(long)kk * sbk] : kDigitZero;
           }
         }
         uint32_t b0[8], b1[8], a0[8], a1[8], a2[8], a3[8];

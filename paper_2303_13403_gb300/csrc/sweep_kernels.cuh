@@ -819,14 +819,37 @@ __device__ __forceinline__ void sm_vectors_by_flip(Cta<T, RES>& x, int m0, int m
   }
 }
 
+// FP64: the product on the tensor cores, U and V turned into digits in place.
 template <typename T, bool RES>
 __device__ __forceinline__ void apply_vectors(Cta<T, RES>& x, int a) {
   const ChainDesc& c = x.c;
   const int N = c.N, ld = c.ld;
-  T* Us[2] = {reinterpret_cast<T*>(x.scr + x.L.u), reinterpret_cast<T*>(x.scr + x.L.u2)};
-  T* Vs[2] = {reinterpret_cast<T*>(x.scr + x.L.w), reinterpret_cast<T*>(x.scr + x.L.mw)};
-  for (int sp = 0; sp < 2; ++sp)
-    cta_gemm<T>(N, N, a, Us[sp], 1, N, Vs[sp], ld, 1, x.G(sp), ld, 1, EpiSub());
+  if constexpr (std::is_same<T, double>::value) {
+    int* red = reinterpret_cast<int*>(x.sh.red);
+    for (int sp = 0; sp < 2; ++sp) {
+      double* U = x.Uv(sp);
+      double* V = x.Vv(sp);
+      double* G = x.G(sp);
+      int eu = kDigitNone, ev = kDigitNone;
+      PQMC_FOR_2D(m, 0, a, i, 0, N) {
+        eu = max(eu, digit_exp(U[(long)m * N + i]));
+        ev = max(ev, digit_exp(V[(long)m * ld + i]));
+      }
+      const int EU = digit_cta_max(eu, red), EV = digit_cta_max(ev, red);
+      unsigned long long* DU = reinterpret_cast<unsigned long long*>(U);
+      unsigned long long* DV = reinterpret_cast<unsigned long long*>(V);
+      PQMC_FOR_2D(m, 0, a, i, 0, N) {
+        DU[(long)m * N + i] = digit_pack(U[(long)m * N + i], EU);
+        DV[(long)m * ld + i] = digit_pack(V[(long)m * ld + i], EV);
+      }
+      __syncthreads();
+      digit_gemm<false, false>(N, N, a, DU, 1, N, DV, 1, ld, [EU](int) { return EU; }, [EV](int) { return EV; }, false,
+                               false, [G, ld](int i, int j, double v) { G[(long)i * ld + j] -= v; });
+    }
+  } else {
+    for (int sp = 0; sp < 2; ++sp)
+      cta_gemm<T>(N, N, a, x.Uv(sp), 1, N, x.Vv(sp), ld, 1, x.G(sp), ld, 1, EpiSub());
+  }
   __syncthreads();
   x.mark(kPhFlush);
 }
@@ -1245,12 +1268,60 @@ __device__ __forceinline__ void update_slice_tv(Cta<T, RES>& x, int tau, uint32_
 // Slice wrapping.  dir = +1: G(tau) = B_tau G(tau-1) B_tau^{-1};
 // dir = -1: G(tau-1) = B_tau^{-1} G(tau) B_tau.
 
+// The two products of an FP64 wrap on the tensor cores (digit_gemm.cuh): G_s
+// <- E1 (f G_s) E2 with f the diagonal factors of pre (or 1), E1 and E2 the
+// digit tables of the model; G_s is packed, receives the first product, is
+// packed again and receives the second.  E1 is read transposed, as the other
+// paths read it.
+template <typename T, bool RES, typename F>
+__device__ __forceinline__ void wrap_digits(Cta<T, RES>& x, int s, const unsigned long long* E1, int e1,
+                                            const unsigned long long* E2, int e2, F pre) {
+  const int N = x.c.N, ld = x.c.ld, ldd = digit_ld(N);
+  T* G = x.G(s);
+  unsigned long long* D = reinterpret_cast<unsigned long long*>(x.Gt());
+  int* red = reinterpret_cast<int*>(x.sh.red);
+  int e = kDigitNone;
+  PQMC_FOR_2D(i, 0, N, j, 0, N) e = max(e, digit_exp(G[(long)i * ld + j] * pre(i, j)));
+  const int EG = digit_cta_max(e, red);
+  PQMC_FOR_2D(i, 0, N, j, 0, N) D[(long)j * ld + i] = digit_pack(G[(long)i * ld + j] * pre(i, j), EG);
+  __syncthreads();
+  e = kDigitNone;
+  digit_gemm<true, true>(N, N, N, E1, ldd, 1, D, ld, 1, [e1](int) { return e1; }, [EG](int) { return EG; }, false, false,
+                         [&e, G, ld](int i, int j, double v) {
+                           G[(long)i * ld + j] = v;
+                           e = max(e, digit_exp(v));
+                         });
+  const int ET = digit_cta_max(e, red);
+  PQMC_FOR_2D(i, 0, N, j, 0, N) D[(long)i * ld + j] = digit_pack(G[(long)i * ld + j], ET);
+  __syncthreads();
+  digit_gemm<true, true>(N, N, N, D, ld, 1, E2, ldd, 1, [ET](int) { return ET; }, [e2](int) { return e2; }, false, false,
+                         [G, ld](int i, int j, double v) { G[(long)i * ld + j] = v; });
+  __syncthreads();
+}
+
 template <bool kTc, typename T, bool RES>
 __device__ __forceinline__ void wrap(Cta<T, RES>& x, int tau, int dir) {
   const ChainDesc& c = x.c;
   const int N = c.N, ld = c.ld;
   const bool gz = x.gutz(tau);
   T* Gt = x.Gt();
+  if constexpr (std::is_same<T, double>::value) {
+    if (!gz && c.dEm) {
+      x.stage(tau);
+      for (int s = 0; s < x.nspec(); ++s) {
+        if (dir > 0) {
+          wrap_digits(x, s, c.dEm, c.eEm, c.dEp, c.eEp,
+                      [&](int i, int j) { return x.vexpT(tau, s, i) * x.vinvT(tau, s, j); });
+        } else {
+          wrap_digits(x, s, c.dEp, c.eEp, c.dEm, c.eEm, [](int, int) { return 1.0; });
+          T* Gs = x.G(s);
+          PQMC_FOR_2D(i, 0, N, j, 0, N) Gs[(long)i * ld + j] *= x.vexpT(tau, s, j) * x.vinvT(tau, s, i);
+        }
+      }
+      __syncthreads();
+      return;
+    }
+  }
   const T* Em = x.Em();
   const T* Ep = x.Ep();
   if (!gz && RES && x.L.em) {
@@ -1469,7 +1540,7 @@ __device__ __forceinline__ bool qr_cholesky(Cta<T, RES>& x, int N, int n, double
   if (threadIdx.x == 0) sh.chol_bad = 0;
   __syncthreads();
   auto eM = [E](int) { return E; };
-  digit_gemm<true>(n, n, N, D, ldd, 1, D, ldd, eM, eM, true, false,
+  digit_gemm<true, true>(n, n, N, D, ldd, 1, D, ldd, 1, eM, eM, true, false,
                    [C, n](int i, int j, double v) { C[(long)i * n + j] = v; });
   __syncthreads();
   for (int k = threadIdx.x; k < n; k += blockDim.x) dlim[k] = 1e-12 * C[(long)k * n + k];
@@ -1539,7 +1610,7 @@ __device__ __forceinline__ bool qr_cholesky(Cta<T, RES>& x, int N, int n, double
     if (lane == 0) ex[j] = e;
   }
   __syncthreads();
-  digit_gemm<false>(N, n, n, D, 1, ldd, X, ldx, eM, [ex](int j) { return ex[j]; }, false, true,
+  digit_gemm<false, true>(N, n, n, D, 1, ldd, X, ldx, 1, eM, [ex](int j) { return ex[j]; }, false, true,
                     [Q, N](int i, int j, double v) { Q[(long)j * N + i] = v; });
   // log|det R|
   if (warp == 0) {
@@ -1773,6 +1844,24 @@ __device__ __noinline__ void phase_stack(int b, int left, int s) {
   T* Mt = x.Mt();
   T* Mt2 = x.Mt2();
   constexpr bool f64 = std::is_same<T, double>::value;
+  // Mt2 = e^{-dtau K} Mt: on the tensor cores in FP64 (digits of Mt in M64's place)
+  auto product = [&](const T* from, T* to) {
+    if constexpr (f64) {
+      if (c.dEm) {
+        const int ldd = digit_ld(N), ldk = N + (N & 1);
+        unsigned long long* D = reinterpret_cast<unsigned long long*>(x.M64());
+        int e = kDigitNone;
+        PQMC_FOR_2D(i, 0, N, k, 0, n) e = max(e, digit_exp(from[(long)i * n + k]));
+        const int E = digit_cta_max(e, reinterpret_cast<int*>(x.sh.red)), e1 = c.eEm;
+        PQMC_FOR_2D(i, 0, N, k, 0, n) D[(long)k * ldk + i] = digit_pack(from[(long)i * n + k], E);
+        __syncthreads();
+        digit_gemm<true, true>(N, n, N, c.dEm, ldd, 1, D, ldk, 1, [e1](int) { return e1; }, [E](int) { return E; }, false,
+                               false, [to, n](int i, int j, double v) { to[(long)i * n + j] = v; });
+        return;
+      }
+    }
+    cta_gemm<T>(N, n, N, x.Em(), 1, c.ld, from, n, 1, to, n, 1, EpiStore());
+  };
   int src = 0;
   if (left ? b == c.nb : b == 0) {
     const int tau = left ? c.Ltau + 1 : 0;
@@ -1786,7 +1875,7 @@ __device__ __noinline__ void phase_stack(int b, int left, int s) {
         x.stage(tau);
         PQMC_FOR_2D(i, 0, N, k, 0, n) Mt[(long)i * n + k] *= x.vexpT(tau, s, i);
         __syncthreads();
-        cta_gemm<T>(N, n, N, x.Em(), 1, c.ld, Mt, n, 1, Mt2, n, 1, EpiStore());
+        product(Mt, Mt2);
         __syncthreads();
         T* t = Mt; Mt = Mt2; Mt2 = t;
         src ^= 1;
@@ -1794,7 +1883,7 @@ __device__ __noinline__ void phase_stack(int b, int left, int s) {
     } else {
       __syncthreads();
       for (int tau = (b + 1) * n_stab; tau > b * n_stab; --tau) {
-        cta_gemm<T>(N, n, N, x.Em(), 1, c.ld, Mt, n, 1, Mt2, n, 1, EpiStore());
+        product(Mt, Mt2);
         x.stage(tau);
         PQMC_FOR_2D(i, 0, N, k, 0, n) Mt[(long)i * n + k] = x.vexpT(tau, s, i) * Mt2[(long)i * n + k];
         __syncthreads();
@@ -1992,7 +2081,7 @@ __device__ __noinline__ void phase_overlap(int b) {
     }
     double* O = x.Ob(s);
     auto eQ = [E](int) { return E; };
-    digit_gemm<true>(n, n, N, DL, ldd, 1, DR, ldd, eQ, eQ, false, false,
+    digit_gemm<true, true>(n, n, N, DL, ldd, 1, DR, ldd, 1, eQ, eQ, false, false,
                      [O, n](int i, int j, double v) { O[(long)i * n + j] = v; });
     __syncthreads();
   }
