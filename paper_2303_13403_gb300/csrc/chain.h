@@ -105,22 +105,24 @@ namespace pqmc {
 //   wrap    : Gt (N x ld, T; FP64 path: packed digits of G) for one spin at a time; for a chain resident in
 //             shared memory also copies of e^{-dtau K} and e^{+dtau K}
 //             (em, ep; 0 when they would make the scratch larger)
-//   flips   : the update vectors of a delayed block, U (N x kw, T) and V
+//   flips   : the update vectors of a delayed block, U (kw columns, N apart, reduced paths ld, T) and V
 //             (kw x ld, T) of each spin (u, w for spin 0; u2, mw for
 //             spin 1), kw = max(delayed block, kBlock); for t-V blocks A_S
 //             (u), W and M W (w, mw); and the per-block flip buffers
-//   stack   : M64 (N x n, FP64, column-major, ld m64_ld(N); Cholesky QR: the packed digits of
-//             the block, ld digit_ld(N)), then a region holding the two
-//             path-precision product buffers Mt, Mt2 (N x n, T, row-major)
-//             and later the FP64 Q of the Householder QR or the packed digits of R^{-1};
-//             Householder betas / R_jj;
-//             the Gram matrix, its inverse factor and pivots of the Cholesky QR
+//   stack   : FP64 path: M64 (N x n, FP64, column-major, ld m64_ld(N)), the two product
+//             buffers Mt, Mt2 (N x n, row-major) and later the FP64 Q, Householder betas / R_jj.
+//             Reduced paths, both spins: m64 holds a product buffer (mt2), then the packed
+//             digits of one spin's block (ld digit_ld(N)); mtq the two spins' blocks (N x n, T,
+//             row-major, mts bytes apart); chol per spin (chs bytes) the Gram matrix,
+//             its inverse factor and in its place that factor's digits (ld digit_ld(n)), and pivots.
+//             A block that takes the Householder QR after all: M64 at m64, Q and its vectors
+//             at q64 (= chol) and qaux, before spin 1's block
 //   refresh : O (n x n, FP64, both spins, inverted in place), the packed digits of Q_L and Q_R of
 //             one spin (dq), then in their place Y (n x ld, T), Q_R and Q_L in the
 //             path precision (N x n, T); GJ pivots / multipliers; O^{-1} in
 //             the path precision (n x n, T)
 struct ScratchLayout {
-  size_t gt, em, ep, u, u2, w, mw, fb, m64, mtq, mt2, qaux, chol, o, dq, y, qrt, qlt, laux, ot, total;
+  size_t gt, em, ep, u, u2, w, mw, fb, m64, mtq, mt2, mts, q64, qaux, chol, chs, o, dq, y, qrt, qlt, laux, ot, total;
 };
 
 PQMC_HDI constexpr size_t al16(size_t v) { return (v + 15) & ~(size_t)15; }
@@ -143,6 +145,8 @@ PQMC_HDI constexpr int m64_ld(int N) { return N | 1; }
 // leading dimension of packed digits (digit_gemm.cuh) for K contiguous elements:
 // = 2 mod 8, so that the fragments' 16-byte loads along K and 8-byte loads
 // across it meet few bank conflicts (and K pairs stay 16-byte aligned)
+// n rounded up to whole 16-byte vectors of FP32
+PQMC_HDI constexpr int pad4(int n) { return (n + 3) & ~3; }
 PQMC_HDI constexpr int digit_ld(int K) { return ((K + 5) & ~7) + 2; }
 
 PQMC_HDI ScratchLayout scratch_layout(int N, int ld, int n, int tsize, int kd) {
@@ -152,32 +156,47 @@ PQMC_HDI ScratchLayout scratch_layout(int N, int ld, int n, int tsize, int kd) {
   L.gt = 0;
   size_t wrap = al16((size_t)N * ld * tsize);
   L.u = 0;
-  L.u2 = al16((size_t)N * kw * tsize);
-  L.w = L.u2 + al16((size_t)N * kw * tsize);
+  L.u2 = al16((size_t)(tsize == 4 ? ld : N) * kw * tsize);
+  L.w = L.u2 + al16((size_t)(tsize == 4 ? ld : N) * kw * tsize);
   L.mw = L.w + al16(kw * ld * tsize);
   L.fb = L.mw + al16(kw * ld * tsize);
   size_t flush = L.fb + flipbuf_bytes(tsize);
   const bool chol = tsize == 4;              // the reduced paths' stack blocks take the Cholesky QR
   const size_t dig = al16((size_t)digit_ld(N) * n * 8);
   L.m64 = 0;
-  L.mtq = al16((size_t)m64_ld(N) * n * 8);
-  if (chol && dig > L.mtq) L.mtq = dig;
-  if (!chol) L.mtq = al16((size_t)(N + 1) * n * 8);     // digits of a product's right factor, ld even
-  L.mt2 = L.mtq + al16(Nn * tsize);
-  size_t mtq_sz = 2 * al16(Nn * tsize);
-  if (al16(Nn * 8) > mtq_sz) mtq_sz = al16(Nn * 8);
-  if (chol && al16((size_t)digit_ld(n) * n * 8) > mtq_sz) mtq_sz = al16((size_t)digit_ld(n) * n * 8);
-  L.qaux = L.mtq + mtq_sz;
-  L.chol = L.qaux + al16((3 * (size_t)n + (size_t)kQRParts * n) * 8);
-  size_t stack = L.chol + (chol ? al16(((size_t)n * n + 6 * (size_t)n) * 8) : 0);
+  const size_t qaux_sz = al16((3 * (size_t)n + (size_t)kQRParts * n) * 8);
+  size_t stack;
+  if (chol) {
+    size_t d = dig;
+    if (al16((size_t)m64_ld(N) * n * 8) > d) d = al16((size_t)m64_ld(N) * n * 8);
+    if (al16((size_t)N * pad4(n) * tsize) > d) d = al16((size_t)N * pad4(n) * tsize);
+    L.mt2 = L.m64;
+    L.chol = L.m64 + d;
+    L.chs = al16(((size_t)digit_ld(n) * n + 6 * (size_t)n) * 8);
+    const size_t mt = al16((size_t)N * pad4(n) * tsize);
+    L.mtq = L.chol + 2 * L.chs;
+    L.q64 = L.chol;
+    L.qaux = L.chol + al16(Nn * 8);
+    L.mts = mt;                                // spin 1's block lies behind a Householder QR's Q and vectors
+    if (L.qaux + qaux_sz > L.mtq + mt) L.mts = L.qaux + qaux_sz - L.mtq;
+    stack = L.mtq + L.mts + mt;
+  } else {
+    L.mtq = al16((size_t)(N + 1) * n * 8);     // (room for the digits of a product's right factor, ld even)
+    L.mt2 = L.mtq + al16(Nn * tsize);
+    L.mts = 0;
+    L.q64 = L.mtq;
+    L.qaux = L.mtq + 2 * al16(Nn * tsize);
+    L.chol = L.chs = 0;
+    stack = L.qaux + qaux_sz;
+  }
   L.o = 0;                                   // O for spin 0, then spin 1 (inverted in place)
   L.dq = 2 * al16((size_t)n * n * 8);
   L.y = L.dq;
   L.qrt = L.y + al16((size_t)n * ld * tsize);
-  L.qlt = L.qrt + al16(Nn * tsize);
-  L.laux = L.qlt + al16(Nn * tsize);
+  L.qlt = L.qrt + (chol ? al16((size_t)ld * n * tsize) : al16(Nn * tsize));
+  L.laux = L.qlt + (chol ? al16((size_t)ld * n * tsize) : al16(Nn * tsize));
   L.ot = L.laux + al16(2 * 6 * (size_t)n * 8);
-  size_t refresh = L.ot + (chol ? al16((size_t)n * n * tsize) : 0);   // (no copy of O^{-1} on the FP64 path)
+  size_t refresh = L.ot + (chol ? al16((size_t)n * pad4(n) * tsize) : 0);   // (no copy of O^{-1} on the FP64 path)
   if (L.dq + 2 * dig > refresh) refresh = L.dq + 2 * dig;
   size_t t = wrap;
   if (flush > t) t = flush;

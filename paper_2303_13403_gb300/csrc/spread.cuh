@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(256) sp_decide_kernel(const ChainDesc* chains,
   load_state(x);
   const ChainDesc& c = x.c;
   x.Gp = sp_gcur<T>(c, alt);
-  decide<true>(x, tau, *sweep_ctr, i0, min(kBlock, c.N - i0), 0);
+  decide<true, false>(x, tau, *sweep_ctr, i0, min(kBlock, c.N - i0), 0);
   __syncthreads();
   x.mark(kPhFlip);
   const int a = x.sh.na;

@@ -94,7 +94,11 @@ static __device__ double cta_max(double v, double* red) {
 // on load; the epilogue receives (i, j, value).  Every thread owns 4x4
 // outputs.  When A is contiguous in i and B in j (sai = sbj = 1, strides and
 // pointers 16-byte aligned, same type as T) the operands are read with
-// 16-byte vector loads.
+// 16-byte vector loads.  pad: the caller's rows of A and B can be read up to
+// the next multiple of four elements, whatever they hold there, so that sizes
+// that are no multiple of four take the vector loads too (162 sites: rank-21
+// update, stack products and assembly 29 + 22 + 24 Mcycles per 42 slices with
+// scalar loads and a bounds check per element).
 
 struct EpiStore {
   static constexpr bool kRow4 = true;   // supports 4 contiguous outputs of a row at once
@@ -139,18 +143,18 @@ __device__ __forceinline__ bool vec_ok(const T* p, long stride) {
 
 template <typename T, typename TA, typename TB, typename TC, typename Epi>
 __device__ void cta_gemm(int M, int Nn, int K, const TA* A, int sai, int sak, const TB* B, int sbk, int sbj,
-                         TC* C, int sci, int scj, Epi epi) {
+                         TC* C, int sci, int scj, Epi epi, bool pad = false) {
   const int tm = (M + 3) >> 2, tn = (Nn + 3) >> 2;
   bool vec = false, vec_row = false, st_row = false;
   if constexpr (std::is_same<T, TA>::value && std::is_same<T, TB>::value) {
     vec = sai == 1 && sbj == 1 && vec_ok<T>((const T*)A, sak) && vec_ok<T>((const T*)B, sbk) &&
-          (M % 4 == 0) && (Nn % 4 == 0);
+          (pad || ((M % 4 == 0) && (Nn % 4 == 0)));
     // A contiguous along k (row-major): 4 x 4 blocks of A per four k-steps
     vec_row = !vec && sak == 1 && sbj == 1 && vec_ok<T>((const T*)A, sai) && vec_ok<T>((const T*)B, sbk) &&
-              (M % 4 == 0) && (Nn % 4 == 0) && (K % 4 == 0);
+              (pad || (Nn % 4 == 0));
   }
   if constexpr (std::is_same<T, TC>::value && HasRow4<Epi>::value) {
-    st_row = scj == 1 && vec_ok<T>((const T*)C, sci) && (Nn % 4 == 0);
+    st_row = scj == 1 && vec_ok<T>((const T*)C, sci);
   }
   for (int t = threadIdx.x; t < tm * tn; t += blockDim.x) {
     const int i0 = (t / tn) << 2, j0 = (t % tn) << 2;
@@ -177,12 +181,15 @@ __device__ void cta_gemm(int M, int Nn, int K, const TA* A, int sai, int sak, co
     }
     if constexpr (std::is_same<T, TA>::value && std::is_same<T, TB>::value) {
       if (vec_row) {
-        const T* pa = (const T*)A + (long)i0 * sai;
+        const T* pa[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) pa[r] = (const T*)A + (long)min(i0 + r, M - 1) * sai;
         const T* pb = (const T*)B + j0;
-        for (int k = 0; k < K; k += 4) {
+        int k = 0;
+        for (; k + 4 <= K; k += 4) {
           T a[4][4], b[4][4];
 #pragma unroll
-          for (int r = 0; r < 4; ++r) Vec4<T>::load(pa + (long)r * sai + k, a[r]);
+          for (int r = 0; r < 4; ++r) Vec4<T>::load(pa[r] + k, a[r]);
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk) Vec4<T>::load(pb + (long)(k + kk) * sbk, b[kk]);
 #pragma unroll
@@ -191,6 +198,16 @@ __device__ void cta_gemm(int M, int Nn, int K, const TA* A, int sai, int sak, co
             for (int r = 0; r < 4; ++r)
 #pragma unroll
               for (int q = 0; q < 4; ++q) acc[r][q] = fma(a[r][kk], b[kk][q], acc[r][q]);
+        }
+        for (; k < K; ++k) {
+          T b[4];
+          Vec4<T>::load(pb + (long)k * sbk, b);
+#pragma unroll
+          for (int r = 0; r < 4; ++r) {
+            const T ar = pa[r][k];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[r][q] = fma(ar, b[q], acc[r][q]);
+          }
         }
       }
     }
@@ -208,7 +225,7 @@ __device__ void cta_gemm(int M, int Nn, int K, const TA* A, int sai, int sak, co
       }
     }
     if constexpr (std::is_same<T, TC>::value && HasRow4<Epi>::value) {
-      if (st_row) {
+      if (st_row && j0 + 4 <= Nn) {
 #pragma unroll
         for (int r = 0; r < 4; ++r)
           if (i0 + r < M) epi.row4((T*)C + (long)(i0 + r) * sci + j0, acc[r]);
@@ -343,7 +360,7 @@ struct Smem {
   int na;                           // accepted flips in the block
   int piv;
   int nswap[2];
-  int chol_bad;
+  int chol_bad[2];                  // the spin's Cholesky factor broke down
   int fperm[kBlock];                // row interchanges of the flush inverse (t-V)
   int staged;                       // slice held in fr, or -1
   double sign_running;
@@ -358,7 +375,7 @@ struct Smem {
   uint32_t scr_off;                 // RES: the scratch's offset from the shared-memory base
   uint32_t tcs_off;                 // tensor-core staging area (BF16X3, chains in global memory), or 0
   uint32_t tmem;                    // its TMEM accumulator
-  int src;                          // where phase_stack left the block: Mt (0), Mt2 (1), e^V P (2)
+  int src;                          // where phase_stack left the block: Mt (0; FP64 path also Mt2, 1), e^V P (2)
   double gj_ip[2];                  // reciprocal of the Gauss-Jordan pivot
   double gj_logabs[2], gj_sign[2];  // log|det O| and sign of the last Gauss-Jordan inverse
 };
@@ -381,19 +398,22 @@ struct Cta {
   __device__ T* G(int s) const { return Gp + (long)s * c.N * c.ld; }
   __device__ T* Gt() const { return reinterpret_cast<T*>(scr + L.gt); }
   __device__ T* Ub() const { return reinterpret_cast<T*>(scr + L.u); }
-  // update vectors of spin s: U (column m at m N), V (row m at m ld)
+  // update vectors of spin s: U (column m at m ldu()), V (row m at m ld)
+  __device__ int ldu() const { return std::is_same<T, double>::value ? c.N : c.ld; }
   __device__ T* Uv(int s) const { return reinterpret_cast<T*>(scr + (s == 0 ? L.u : L.u2)); }
   __device__ T* Vv(int s) const { return reinterpret_cast<T*>(scr + (s == 0 ? L.w : L.mw)); }
   __device__ T* Wb() const { return reinterpret_cast<T*>(scr + L.w); }
   __device__ double* M64() const { return reinterpret_cast<double*>(scr + L.m64); }
-  __device__ double* Q64() const { return reinterpret_cast<double*>(scr + L.mtq); }
-  __device__ T* Mt() const { return reinterpret_cast<T*>(scr + L.mtq); }
+  __device__ double* Q64() const { return reinterpret_cast<double*>(scr + L.q64); }
+  // row length of the stack products' buffers (FP32: whole vectors)
+  __device__ int ldn(int s) const { return std::is_same<T, double>::value ? nsig(s) : pad4(nsig(s)); }
+  __device__ T* Mt(int s) const { return reinterpret_cast<T*>(scr + L.mtq + s * L.mts); }
   __device__ T* Mt2() const { return reinterpret_cast<T*>(scr + L.mt2); }
   __device__ double* qbeta() const { return reinterpret_cast<double*>(scr + L.qaux); }
   __device__ double* qalpha() const { return qbeta() + c.nmax; }
   __device__ double* qw() const { return qbeta() + 2 * c.nmax; }
   __device__ double* qpart() const { return qbeta() + 3 * c.nmax; }
-  __device__ double* chol() const { return reinterpret_cast<double*>(scr + L.chol); }
+  __device__ double* chol(int s) const { return reinterpret_cast<double*>(scr + L.chol + s * L.chs); }
   __device__ double* Ob(int s) const {
     return reinterpret_cast<double*>(scr + L.o + s * al16((size_t)c.nmax * c.nmax * 8));
   }
@@ -488,7 +508,7 @@ __device__ __forceinline__ void wrap_gemm(Cta<T, RES>& x, int n, const T* A, int
       return;
     }
   }
-  cta_gemm<T>(n, n, n, A, sai, sak, B, ld, 1, C, ld, 1, epi);
+  cta_gemm<T>(n, n, n, A, sai, sak, B, ld, 1, C, ld, 1, epi, !std::is_same<T, double>::value);
 }
 
 // --------------------------------------------------------------------------
@@ -517,28 +537,35 @@ __device__ __forceinline__ T uniform_of(uint64_t m53) {
 // gsite, Delta per species cl), to the whole G of every species:
 //     G <- G - (E_S - G_{:,S}) Gamma (1 + (1 - G_SS) Gamma)^{-1} G_{S,:}
 // with G the G of the block start.  X = 1 + (1 - G_SS) Gamma is inverted in
-// place by one warp per species; Hubbard blocks need no pivoting (its pivots
+// place; Hubbard blocks need no pivoting (its pivots
 // are the accepted ratios), the bond blocks of the t-V model pivot on rows
 // (a single end of an accepted bond may have a vanishing ratio).
 // M = Gamma (1 + (1 - G_SS) Gamma)^{-1} of the a accepted flips of a block
 // into fb.Tu[s] for every species s (collective; G is the G of the block
-// start).
+// start).  Per pivot the species' first warp finds it, exchanges the rows and
+// hands on the pivot row and reciprocal; then every warp takes its rows (lane:
+// column), two barriers in all.  (One warp doing it alone, a row at a time
+// through shared memory, took 35 kcycles for 21 Hubbard flips and 49 for the
+// 32 ends of a t-V block.)
 template <typename T, bool RES>
 __device__ __forceinline__ void block_inverse(Cta<T, RES>& x, int a, bool pivot) {
   FlipBuf<T>& fb = *x.fb;
   const int ld = x.c.ld, ns = x.nspec();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (int)blockDim.x >> 5;
+  // the warps of a species: every ns-th one
+  const int s = warp % ns, w = warp / ns, ws = nw / ns;
+  const unsigned full = 0xffffffffu;
   PQMC_FOR_2D(sl, 0, ns * a, m, 0, a) {
-    const int s = sl >= a ? 1 : 0, l = sl - s * a;
-    const T g = x.G(s)[(long)fb.gsite[l] * ld + fb.gsite[m]];
-    fb.Tu[s][l][m] = ((l == m) ? T(1) : T(0)) + ((l == m ? T(1) : T(0)) - g) * fb.cl[s][m];
+    const int sp = sl >= a ? 1 : 0, l = sl - sp * a;
+    const T g = x.G(sp)[(long)fb.gsite[l] * ld + fb.gsite[m]];
+    fb.Tu[sp][l][m] = ((l == m) ? T(1) : T(0)) + ((l == m ? T(1) : T(0)) - g) * fb.cl[sp][m];
   }
   __syncthreads();
-  if (warp < ns) {
-    const int s = warp;
-    T (*X)[kBlock + 1] = fb.Tu[s];
-    int* perm = x.sh.fperm;
-    for (int p = 0; p < a; ++p) {
+  T (*X)[kBlock + 1] = fb.Tu[s];
+  T* prow = fb.rs[s];                    // pivot row of the step
+  int* perm = x.sh.fperm;
+  for (int p = 0; p < a; ++p) {
+    if (w == 0) {
       if (pivot) {
         // largest |X_rp|, r >= p, ties to the lower row; swap rows r and p
         T best = T(-1);
@@ -546,8 +573,8 @@ __device__ __forceinline__ void block_inverse(Cta<T, RES>& x, int a, bool pivot)
         if (lane >= p && lane < a) { best = fabs(X[lane][p]); bi = lane; }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
-          const T ob = __shfl_xor_sync(0xffffffffu, best, o);
-          const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+          const T ob = __shfl_xor_sync(full, best, o);
+          const int oi = __shfl_xor_sync(full, bi, o);
           if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
         }
         if (lane == 0) perm[p] = bi;
@@ -558,34 +585,37 @@ __device__ __forceinline__ void block_inverse(Cta<T, RES>& x, int a, bool pivot)
         }
         __syncwarp();
       }
-      const T ip = T(1) / X[p][p];
-      const T xpl = lane < a ? X[p][lane] : T(0);
-      if (lane < a && lane != p)
-        for (int r = 0; r < a; ++r)
-          if (r != p) X[r][lane] = fma(-X[r][p] * ip, xpl, X[r][lane]);
-      __syncwarp();
-      if (lane < a) {
-        if (lane != p) X[p][lane] = xpl * ip;
-        X[lane][p] = lane == p ? ip : -X[lane][p] * ip;
-      }
-      __syncwarp();
+      if (lane < a) prow[lane] = X[p][lane];
     }
-    if (pivot) {
-      // the row interchanges of the factorisation become column
-      // interchanges of the inverse, undone last step first
-      for (int p = a - 1; p >= 0; --p) {
-        const int q = perm[p];
-        if (q != p && lane < a) {
-          const T t = X[lane][p];
-          X[lane][p] = X[lane][q];
-          X[lane][q] = t;
-        }
-        __syncwarp();
-      }
+    __syncthreads();
+    const T xpl = lane < a ? prow[lane] : T(0);
+    const T ip = T(1) / prow[p];
+    for (int r = w; r < a; r += ws) {
+      const T xrp = X[r][p], xrl = lane < a ? X[r][lane] : T(0);
+      __syncwarp();
+      T v;
+      if (r == p) v = lane == p ? ip : xpl * ip;
+      else v = lane == p ? -xrp * ip : fma(-xrp * ip, xpl, xrl);
+      if (lane < a) X[r][lane] = v;
     }
-    for (int l = 0; l < a; ++l)
-      if (lane < a) X[l][lane] *= fb.cl[s][l];
+    __syncthreads();
   }
+  if (w == 0 && pivot) {
+    // the row interchanges of the factorisation become column
+    // interchanges of the inverse, undone last step first
+    for (int p = a - 1; p >= 0; --p) {
+      const int q = perm[p];
+      if (q != p && lane < a) {
+        const T t = X[lane][p];
+        X[lane][p] = X[lane][q];
+        X[lane][q] = t;
+      }
+      __syncwarp();
+    }
+  }
+  __syncthreads();
+  for (int l = w; l < a; l += ws)
+    if (lane < a) X[l][lane] *= fb.cl[s][l];
   __syncthreads();
 }
 
@@ -593,7 +623,7 @@ template <typename T, bool RES>
 __device__ __forceinline__ void flush_block(Cta<T, RES>& x, int a, bool pivot) {
   const ChainDesc& c = x.c;
   FlipBuf<T>& fb = *x.fb;
-  const int N = c.N, ld = c.ld, ns = x.nspec();
+  const int N = c.N, ld = c.ld, ldu = x.ldu(), ns = x.nspec();
   T* Ubuf = x.Ub();                                    // kBlock x N  (U column-major, ld N)
   T* Wbuf = x.Wb();                                    // kBlock x ld (rows G_{S,:})
   block_inverse(x, a, pivot);
@@ -604,13 +634,13 @@ __device__ __forceinline__ void flush_block(Cta<T, RES>& x, int a, bool pivot) {
     T* Gs = x.G(s);
     PQMC_FOR_2D(m, 0, a, i, 0, N) {
       const int col = fb.gsite[m];
-      Ubuf[(long)m * N + i] = (i == col ? T(1) : T(0)) - Gs[(long)i * ld + col];
+      Ubuf[(long)m * ldu + i] = (i == col ? T(1) : T(0)) - Gs[(long)i * ld + col];
     }
     PQMC_FOR_2D(l, 0, a, q, 0, N) Wbuf[(long)l * ld + q] = Gs[(long)fb.gsite[l] * ld + q];
     __syncthreads();
     cta_gemm<T>(a, N, a, &fb.Tu[s][0][0], kBlock + 1, 1, Wbuf, ld, 1, MW, ld, 1, EpiStore());
     __syncthreads();
-    cta_gemm<T>(N, N, a, Ubuf, 1, N, MW, ld, 1, Gs, ld, 1, EpiSub());
+    cta_gemm<T>(N, N, a, Ubuf, 1, ldu, MW, ld, 1, Gs, ld, 1, EpiSub(), !std::is_same<T, double>::value);
     __syncthreads();
   }
   x.mark(kPhFlush);
@@ -652,34 +682,24 @@ __device__ __forceinline__ T& sm_u(T (*tab)[kBlock], int m, int p) { return tab[
 // row s_q, register p: column s_p; gives the U_m) or columns (transposed; the
 // V_m).  The two roles form the same elements and need no word of each other.
 template <typename T, bool RES>
-__device__ __forceinline__ void sm_core(Cta<T, RES>& x, int m0, int cnt) {
-  const ChainDesc& c = x.c;
+__device__ __forceinline__ void sm_core(Cta<T, RES>& x, int i0, int m0, int cnt) {
   FlipBuf<T>& fb = *x.fb;
-  const int N = c.N, ld = c.ld;
-  const int lane = threadIdx.x & 31;
-  for (int w = threadIdx.x >> 5; w < 4; w += blockDim.x >> 5) {
-    const int s = w >> 1;
+  const int lane = threadIdx.x & 31, nw = (int)blockDim.x >> 5;
+  for (int w = threadIdx.x >> 5; w < max(4, nw); w += nw) {
+    const int s = (w >> 1) & 1;
     const bool row = (w & 1) == 0;
-    const T* Gs = x.G(s);
-    const T* U = x.Uv(s);
-    const T* V = x.Vv(s);
     T (*tab)[kBlock] = fb.sv[s];
-    const int sq = fb.gsite[m0 + min(lane, cnt - 1)];
+    const int sq = min(fb.gsite[m0 + lane] - i0, kBlock - 1);
+    // element p of this line: block element (s_q, s_p) or (s_p, s_q), as staged
+    // for the decisions
     T a[kBlock];
 #pragma unroll
     for (int p = 0; p < kBlock; ++p) {
-      const int sp = fb.gsite[m0 + min(p, cnt - 1)];
-      a[p] = row ? Gs[(long)sq * ld + sp] : Gs[(long)sp * ld + sq];
+      const int sp = fb.gsite[m0 + p] - i0;
+      a[p] = row ? fb.Tu[s][sq][sp] : fb.Tu[s][sp][sq];
     }
-    for (int l = 0; l < m0; ++l) {
-      // flips of the delayed block's earlier sub-blocks
-      const T own = row ? U[(long)l * N + sq] : V[(long)l * ld + sq];
-#pragma unroll
-      for (int p = 0; p < kBlock; ++p) {
-        const int sp = fb.gsite[m0 + min(p, cnt - 1)];
-        a[p] = fma(-own, row ? V[(long)l * ld + sp] : U[(long)l * N + sp], a[p]);
-      }
-    }
+    __syncthreads();                     // the table takes the staged block's place
+    if (w >= 4) continue;
 #pragma unroll 1
     for (int m = 0; m < cnt; ++m) {
       const T f = fb.fr[s][m0 + m];
@@ -738,7 +758,8 @@ __device__ __forceinline__ void sm_four(T (&w)[kBlock], const T (*tab)[kBlock], 
   for (int p = 0; p + 4 < kW; ++p) w[p] = w[p + 4];
 }
 
-template <bool kRow, typename T, bool RES>
+// kLater: flips of the delayed block's earlier sub-blocks come first (m0 > 0)
+template <bool kRow, bool kLater, typename T, bool RES>
 __device__ __forceinline__ void sm_line(Cta<T, RES>& x, int s, int j, int m0, int cnt) {
   const ChainDesc& c = x.c;
   FlipBuf<T>& fb = *x.fb;
@@ -746,20 +767,18 @@ __device__ __forceinline__ void sm_line(Cta<T, RES>& x, int s, int j, int m0, in
   // element p of this line: G[j][s_p] (row) or G[s_p][j] (column)
   const T* g = kRow ? x.G(s) + (long)j * ld : x.G(s) + j;
   T* out = kRow ? x.Uv(s) + j : x.Vv(s) + j;
-  const long os = kRow ? c.N : ld;
+  const long os = ld;                    // (FP32: U and V share the row length)
   const int* site = fb.gsite + m0;
   T w[kBlock];
 #pragma unroll
-  for (int p = 0; p < kBlock; ++p) {
-    const int sp = site[min(p, cnt - 1)];
-    w[p] = g[kRow ? sp : sp * ld];
-  }
-  const T* other = kRow ? x.Vv(s) : x.Uv(s);
-  const long ot = kRow ? ld : c.N;
-  for (int l = 0; l < m0; ++l) {         // flips of the delayed block's earlier sub-blocks
-    const T a = out[l * os];
+  for (int p = 0; p < kBlock; ++p) w[p] = g[kRow ? site[p] : site[p] * ld];
+  if (kLater) {
+    const T* other = kRow ? x.Vv(s) : x.Uv(s);
+    for (int l = 0; l < m0; ++l) {
+      const T a = out[l * os];
 #pragma unroll
-    for (int p = 0; p < kBlock; ++p) w[p] = fma(-a, other[l * ot + site[min(p, cnt - 1)]], w[p]);
+      for (int p = 0; p < kBlock; ++p) w[p] = fma(-a, other[l * os + site[p]], w[p]);
+    }
   }
   out += m0 * os;
   int k = 0;
@@ -771,15 +790,15 @@ __device__ __forceinline__ void sm_line(Cta<T, RES>& x, int s, int j, int m0, in
 
 // every row of U and every column of V, both spins: a warp takes 32 rows or
 // 32 columns of one spin at a time
-template <typename T, bool RES>
+template <bool kLater, typename T, bool RES>
 __device__ __forceinline__ void sm_vectors(Cta<T, RES>& x, int m0, int cnt) {
   const int N = x.c.N, lane = threadIdx.x & 31;
   const int groups = (N + 31) >> 5;
   for (int t = threadIdx.x >> 5; t < 4 * groups; t += blockDim.x >> 5) {
     const int s = t & 1, j = 32 * (t >> 2) + lane;
     if (j >= N) continue;
-    if (t & 2) sm_line<true>(x, s, j, m0, cnt);
-    else sm_line<false>(x, s, j, m0, cnt);
+    if (t & 2) sm_line<true, kLater>(x, s, j, m0, cnt);
+    else sm_line<false, kLater>(x, s, j, m0, cnt);
   }
 }
 
@@ -791,7 +810,7 @@ template <typename T, bool RES>
 __device__ __forceinline__ void sm_vectors_by_flip(Cta<T, RES>& x, int m0, int m1) {
   const ChainDesc& c = x.c;
   FlipBuf<T>& fb = *x.fb;
-  const int N = c.N, ld = c.ld;
+  const int N = c.N, ld = c.ld, ldu = x.ldu();
   const int half = (int)blockDim.x >> 1;
   const int s = (int)threadIdx.x >= half ? 1 : 0;
   const int t = (int)threadIdx.x - s * half;
@@ -804,12 +823,12 @@ __device__ __forceinline__ void sm_vectors_by_flip(Cta<T, RES>& x, int m0, int m
     for (int o = t; o < 2 * N; o += half) {
       if (o < N) {
         T cv = Gs[(long)o * ld + sm];
-        for (int l = 0; l < m; ++l) cv = fma(-U[(long)l * N + o], V[(long)l * ld + sm], cv);
-        U[(long)m * N + o] = ((o == sm ? T(1) : T(0)) - cv) * f;
+        for (int l = 0; l < m; ++l) cv = fma(-U[(long)l * ldu + o], V[(long)l * ld + sm], cv);
+        U[(long)m * ldu + o] = ((o == sm ? T(1) : T(0)) - cv) * f;
       } else {
         const int j = o - N;
         T rv = Gs[(long)sm * ld + j];
-        for (int l = 0; l < m; ++l) rv = fma(-U[(long)l * N + sm], V[(long)l * ld + j], rv);
+        for (int l = 0; l < m; ++l) rv = fma(-U[(long)l * ldu + sm], V[(long)l * ld + j], rv);
         V[(long)m * ld + j] = rv;
       }
     }
@@ -826,29 +845,30 @@ __device__ __forceinline__ void apply_vectors(Cta<T, RES>& x, int a) {
   const int N = c.N, ld = c.ld;
   if constexpr (std::is_same<T, double>::value) {
     int* red = reinterpret_cast<int*>(x.sh.red);
+    const int ldu = x.ldu();
     for (int sp = 0; sp < 2; ++sp) {
       double* U = x.Uv(sp);
       double* V = x.Vv(sp);
       double* G = x.G(sp);
       int eu = kDigitNone, ev = kDigitNone;
       PQMC_FOR_2D(m, 0, a, i, 0, N) {
-        eu = max(eu, digit_exp(U[(long)m * N + i]));
+        eu = max(eu, digit_exp(U[(long)m * ldu + i]));
         ev = max(ev, digit_exp(V[(long)m * ld + i]));
       }
       const int EU = digit_cta_max(eu, red), EV = digit_cta_max(ev, red);
       unsigned long long* DU = reinterpret_cast<unsigned long long*>(U);
       unsigned long long* DV = reinterpret_cast<unsigned long long*>(V);
       PQMC_FOR_2D(m, 0, a, i, 0, N) {
-        DU[(long)m * N + i] = digit_pack(U[(long)m * N + i], EU);
+        DU[(long)m * ldu + i] = digit_pack(U[(long)m * ldu + i], EU);
         DV[(long)m * ld + i] = digit_pack(V[(long)m * ld + i], EV);
       }
       __syncthreads();
-      digit_gemm<false, false>(N, N, a, DU, 1, N, DV, 1, ld, [EU](int) { return EU; }, [EV](int) { return EV; }, false,
+      digit_gemm<false, false>(N, N, a, DU, 1, ldu, DV, 1, ld, [EU](int) { return EU; }, [EV](int) { return EV; }, false,
                                false, [G, ld](int i, int j, double v) { G[(long)i * ld + j] -= v; });
     }
   } else {
     for (int sp = 0; sp < 2; ++sp)
-      cta_gemm<T>(N, N, a, x.Uv(sp), 1, N, x.Vv(sp), ld, 1, x.G(sp), ld, 1, EpiSub());
+      cta_gemm<T>(N, N, a, x.Uv(sp), 1, x.ldu(), x.Vv(sp), ld, 1, x.G(sp), ld, 1, EpiSub(), true);
   }
   __syncthreads();
   x.mark(kPhFlush);
@@ -859,6 +879,25 @@ __device__ __forceinline__ void apply_vectors(Cta<T, RES>& x, int a) {
 // applied to G at once.  Within a delayed block a later sub-block reads its
 // diagonal block of G corrected by the update vectors of the flips already
 // accepted, G_SS - U_S V_S, so every decision sees the current G.
+// The diagonal block of G at sites i0 .. i0 + nbk - 1, both spins, into
+// fb.Tu (zero beyond nbk), brought up to date by the vectors of the a_done flips the
+// delayed block has accepted so far: G_SS - U_S V_S (collective).
+template <typename T, bool RES>
+__device__ __forceinline__ void stage_block(Cta<T, RES>& x, int i0, int nbk, int a_done) {
+  FlipBuf<T>& fb = *x.fb;
+  const int ld = x.c.ld;
+  for (int e = threadIdx.x; e < 2 * kBlock * kBlock; e += blockDim.x) {
+    const int s = e / (kBlock * kBlock), r = e / kBlock % kBlock, q = e % kBlock;
+    T v = T(0);
+    if (r < nbk && q < nbk) {
+      v = x.G(s)[(long)(i0 + r) * ld + i0 + q];
+      for (int l = 0; l < a_done; ++l) v = fma(-x.Uv(s)[(long)l * x.ldu() + i0 + r], x.Vv(s)[(long)l * ld + i0 + q], v);
+    }
+    fb.Tu[s][r][q] = v;
+  }
+  __syncthreads();
+}
+
 // The proposals of one decision sub-block, sites i0 .. i0 + nbk - 1 of slice
 // tau (nbk <= kBlock), after a_done flips of the delayed block were accepted
 // (their update vectors in the scratch correct the diagonal block read from
@@ -869,7 +908,6 @@ __device__ __forceinline__ void decide_sub_block(Cta<T, RES>& x, int tau, uint32
   const ChainDesc& c = x.c;
   Smem<T>& sh = x.sh;
   FlipBuf<T>& fb = *x.fb;
-  const int N = c.N, ld = c.ld;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int kap = x.gutz(tau) ? 1 : 0;
   int8_t* f = c.fields + (long)tau * c.nfld;
@@ -882,18 +920,7 @@ __device__ __forceinline__ void decide_sub_block(Cta<T, RES>& x, int tau, uint32
     T gs[kBlock];
     const bool colq = lane < nbk;
 #pragma unroll
-    for (int r = 0; r < kBlock; ++r) gs[r] = (colq && r < nbk) ? x.G(s)[(long)(i0 + r) * ld + i0 + lane] : T(0);
-    if (a_done > 0 && colq) {
-      // G_SS - U_S V_S over the vectors of the block's earlier flips
-      const T* U = reinterpret_cast<const T*>(x.scr + (s == 0 ? x.L.u : x.L.u2));
-      const T* V = reinterpret_cast<const T*>(x.scr + (s == 0 ? x.L.w : x.L.mw));
-      for (int l = 0; l < a_done; ++l) {
-        const T vq = V[(long)l * ld + i0 + lane];
-#pragma unroll
-        for (int r = 0; r < kBlock; ++r)
-          if (r < nbk) gs[r] = fma(-U[(long)l * N + i0 + r], vq, gs[r]);
-      }
-    }
+    for (int r = 0; r < kBlock; ++r) gs[r] = fb.Tu[s][r][lane];
     // lane j: uniform (in the decision precision) and field of site i0 + j
     T uj = T(2);
     int flj = 1;
@@ -912,6 +939,7 @@ __device__ __forceinline__ void decide_sub_block(Cta<T, RES>& x, int tau, uint32
         const T ds = dl[s][si];
         const T rs = T(1) + ds * (T(1) - __shfl_sync(0xffffffffu, gs[j], j));
         if (lane == 0) fb.rs[s][j] = rs;
+        __syncwarp();
         asm volatile("bar.sync 1, 64;" ::: "memory");
         const T R = fb.rs[0][j] * fb.rs[1][j];
         const bool acc = __shfl_sync(0xffffffffu, (int)(uj < (R < T(0) ? -R : R)), j) != 0;
@@ -958,7 +986,13 @@ __device__ __forceinline__ void decide_sub_block(Cta<T, RES>& x, int tau, uint32
 // by the operations of the two-warp form above, so the decisions and the
 // factors are the same bits.  What a decision leaves behind (fields, logs,
 // sites, Delta) is written after the loop, by all lanes at once.
-template <bool RES>
+// kRolled: the proposal loop stays rolled and the register window moves down
+// one row per proposal, so row j is always register 0.  In the one-CTA sweep,
+// whose phases evict one another from the instruction caches, the 40 KB of
+// the unrolled loop cost more to fetch than the moves (5.3 against 3.8 Mcycles
+// per sweep at 72 sites); in a kernel of its own (spread mode) the
+// unrolled loop is the faster one (13 against 20 kcycles per block).
+template <bool kRolled, bool RES>
 __device__ __forceinline__ void decide_sub_block_pair(Cta<float, RES>& x, int tau, uint32_t sweep, int i0, int nbk,
                                                              int a_done) {
   if (threadIdx.x >= 32) return;
@@ -966,35 +1000,15 @@ __device__ __forceinline__ void decide_sub_block_pair(Cta<float, RES>& x, int ta
   Smem<float>& sh = x.sh;
   FlipBuf<float>& fb = *x.fb;
   const unsigned full = 0xffffffffu;
-  const int N = c.N, ld = c.ld;
   const int lane = threadIdx.x, s = lane >> 4, q = lane & 15, half = lane & 16;
   const int kap = x.gutz(tau) ? 1 : 0;
   int8_t* f = c.fields + (long)tau * c.nfld;
   const float d0 = (float)c.delta[kap][s][0], d1 = (float)c.delta[kap][s][1];
-  const bool on0 = q < nbk, on1 = q + 16 < nbk;
   float ga[kBlock], gb[kBlock];
-  {
-    const float* G = x.G(s) + (long)i0 * ld + i0 + q;
 #pragma unroll
-    for (int r = 0; r < kBlock; ++r) {
-      ga[r] = (on0 && r < nbk) ? G[(long)r * ld] : 0.f;
-      gb[r] = (on1 && r < nbk) ? G[(long)r * ld + 16] : 0.f;
-    }
-  }
-  if (a_done > 0) {
-    // G_SS - U_S V_S over the vectors of the block's earlier flips
-    const float* U = reinterpret_cast<const float*>(x.scr + (s == 0 ? x.L.u : x.L.u2)) + i0;
-    const float* V = reinterpret_cast<const float*>(x.scr + (s == 0 ? x.L.w : x.L.mw)) + i0 + q;
-    for (int l = 0; l < a_done; ++l) {
-      const float va = on0 ? V[(long)l * ld] : 0.f, vb = on1 ? V[(long)l * ld + 16] : 0.f;
-#pragma unroll
-      for (int r = 0; r < kBlock; ++r)
-        if (r < nbk) {
-          const float u = U[(long)l * N + r];
-          if (on0) ga[r] = fma(-u, va, ga[r]);
-          if (on1) gb[r] = fma(-u, vb, gb[r]);
-        }
-    }
+  for (int r = 0; r < kBlock; ++r) {
+    ga[r] = fb.Tu[s][r][q];
+    gb[r] = fb.Tu[s][r][q + 16];
   }
   // lane j: uniform (in the decision precision) and field of site i0 + j
   float uj = 2.f;
@@ -1009,69 +1023,101 @@ __device__ __forceinline__ void decide_sub_block_pair(Cta<float, RES>& x, int ta
   unsigned accepted = 0;
   int a = a_done, bad = 0, nneg = 0;
   float* frs = &fb.fr[s][0];
-  // sites 0..15 (their columns in ga), then 16..31 (in gb).  The loops stay
-  // rolled: the register window moves down one row per proposal, so row j is
-  // always register 0 (see sm_core on code size).
-  const int n_lo = min(nbk, 16);
+  if constexpr (kRolled) {
+    // sites 0..15 (their columns in ga), then 16..31 (in gb)
+    const int n_lo = min(nbk, 16);
 #pragma unroll 1
-  for (int j = 0; j < n_lo; ++j) {
-    const float u = __shfl_sync(full, uj, j);
-    const float ds = ((up >> j) & 1u) ? d0 : d1;
-    const float rs = 1.f + ds * (1.f - __shfl_sync(full, ga[0], half | j));
-    const float R = rs * __shfl_xor_sync(full, rs, 16);
-    const float fac = ds / rs;
-    bad |= isfinite(R) ? 0 : 1;
-    const bool acc = u < fabsf(R);     // the same value in every lane
-    // G_rq += c G_rj G_jq for future rows r > j and columns q > j
-    const float ya = acc && q > j ? fac * ga[0] : 0.f, yb = acc ? fac * gb[0] : 0.f;
-    if (acc) {
-      accepted |= 1u << j;
-      nneg += R < 0.f ? 1 : 0;
-      if (q == 0) frs[a] = fac;
-      ++a;
+    for (int j = 0; j < n_lo; ++j) {
+      const float u = __shfl_sync(full, uj, j);
+      const float ds = ((up >> j) & 1u) ? d0 : d1;
+      const float rs = 1.f + ds * (1.f - __shfl_sync(full, ga[0], half | j));
+      const float R = rs * __shfl_xor_sync(full, rs, 16);
+      const float fac = ds / rs;
+      bad |= isfinite(R) ? 0 : 1;
+      const bool acc = u < fabsf(R);     // the same value in every lane
+      // G_rq += c G_rj G_jq for future rows r > j and columns q > j
+      const float ya = acc && q > j ? fac * ga[0] : 0.f, yb = acc ? fac * gb[0] : 0.f;
+      if (acc) {
+        accepted |= 1u << j;
+        nneg += R < 0.f ? 1 : 0;
+        if (q == 0) frs[a] = fac;
+        ++a;
 #pragma unroll
-      for (int r0 = 1; r0 < kBlock; r0 += 8)
-        if (r0 < nbk - j) {
+        for (int r0 = 1; r0 < kBlock; r0 += 8)
+          if (r0 < nbk - j) {
 #pragma unroll
-          for (int r = r0; r < (r0 + 8 < kBlock ? r0 + 8 : kBlock); ++r) {
-            const float xr = __shfl_sync(full, ga[r], half | j);
-            ga[r - 1] = fma(xr, ya, ga[r]);
-            gb[r - 1] = fma(xr, yb, gb[r]);
+            for (int r = r0; r < (r0 + 8 < kBlock ? r0 + 8 : kBlock); ++r) {
+              const float xr = __shfl_sync(full, ga[r], half | j);
+              ga[r - 1] = fma(xr, ya, ga[r]);
+              gb[r - 1] = fma(xr, yb, gb[r]);
+            }
           }
-        }
-    } else {
+      } else {
 #pragma unroll
-      for (int r = 1; r < kBlock; ++r) {
-        ga[r - 1] = ga[r];
-        gb[r - 1] = gb[r];
+        for (int r = 1; r < kBlock; ++r) {
+          ga[r - 1] = ga[r];
+          gb[r - 1] = gb[r];
+        }
       }
     }
-  }
 #pragma unroll 1
-  for (int j = 16; j < nbk; ++j) {
-    const float u = __shfl_sync(full, uj, j);
-    const float ds = ((up >> j) & 1u) ? d0 : d1;
-    const float rs = 1.f + ds * (1.f - __shfl_sync(full, gb[0], half | (j - 16)));
-    const float R = rs * __shfl_xor_sync(full, rs, 16);
-    const float fac = ds / rs;
-    bad |= isfinite(R) ? 0 : 1;
-    const bool acc = u < fabsf(R);
-    const float yb = acc && q + 16 > j ? fac * gb[0] : 0.f;
-    if (acc) {
-      accepted |= 1u << j;
-      nneg += R < 0.f ? 1 : 0;
-      if (q == 0) frs[a] = fac;
-      ++a;
+    for (int j = 16; j < nbk; ++j) {
+      const float u = __shfl_sync(full, uj, j);
+      const float ds = ((up >> j) & 1u) ? d0 : d1;
+      const float rs = 1.f + ds * (1.f - __shfl_sync(full, gb[0], half | (j - 16)));
+      const float R = rs * __shfl_xor_sync(full, rs, 16);
+      const float fac = ds / rs;
+      bad |= isfinite(R) ? 0 : 1;
+      const bool acc = u < fabsf(R);
+      const float yb = acc && q + 16 > j ? fac * gb[0] : 0.f;
+      if (acc) {
+        accepted |= 1u << j;
+        nneg += R < 0.f ? 1 : 0;
+        if (q == 0) frs[a] = fac;
+        ++a;
 #pragma unroll
-      for (int r0 = 1; r0 < 16; r0 += 8)
-        if (r0 < nbk - j) {
+        for (int r0 = 1; r0 < 16; r0 += 8)
+          if (r0 < nbk - j) {
 #pragma unroll
-          for (int r = r0; r < (r0 + 8 < 16 ? r0 + 8 : 16); ++r)
-            gb[r - 1] = fma(__shfl_sync(full, gb[r], half | (j - 16)), yb, gb[r]);
+            for (int r = r0; r < (r0 + 8 < 16 ? r0 + 8 : 16); ++r)
+              gb[r - 1] = fma(__shfl_sync(full, gb[r], half | (j - 16)), yb, gb[r]);
+          }
+      } else {
+#pragma unroll
+        for (int r = 1; r < 16; ++r) gb[r - 1] = gb[r];
+      }
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < kBlock; ++j) {
+      if (j < nbk) {
+        const float u = __shfl_sync(full, uj, j);
+        const float ds = ((up >> j) & 1u) ? d0 : d1;
+        const float rs = 1.f + ds * (1.f - __shfl_sync(full, j < 16 ? ga[j] : gb[j], half | (j & 15)));
+        const float R = rs * __shfl_xor_sync(full, rs, 16);
+        const float fac = ds / rs;
+        bad |= isfinite(R) ? 0 : 1;
+        if (u < fabsf(R)) {            // the same value in every lane
+          accepted |= 1u << j;
+          nneg += R < 0.f ? 1 : 0;
+          if (q == 0) frs[a] = fac;
+          ++a;
+          // G_rq += c G_rj G_jq for future rows r > j and columns q > j
+          if (j < 16) {
+            const float ya = q > j ? fac * ga[j] : 0.f, yb = fac * gb[j];
+#pragma unroll
+            for (int r = j + 1; r < kBlock; ++r) {
+              const float xr = __shfl_sync(full, ga[r], half | j);
+              ga[r] = fma(xr, ya, ga[r]);
+              gb[r] = fma(xr, yb, gb[r]);
+            }
+          } else {
+            const float yb = q + 16 > j ? fac * gb[j] : 0.f;
+#pragma unroll
+            for (int r = j + 1; r < kBlock; ++r) gb[r] = fma(__shfl_sync(full, gb[r], half | (j - 16)), yb, gb[r]);
+          }
         }
-    } else {
-#pragma unroll
-      for (int r = 1; r < 16; ++r) gb[r - 1] = gb[r];
+      }
     }
   }
   const bool mine = (accepted >> lane) & 1u;
@@ -1083,6 +1129,8 @@ __device__ __forceinline__ void decide_sub_block_pair(Cta<float, RES>& x, int ta
     fb.cl[1][at] = (float)c.delta[kap][1][si];
     f[i0 + lane] = (int8_t)-flj;
   }
+  // (the site list goes on with the last accepted site: sm_vectors reads whole blocks of it)
+  if (accepted && a + lane < a_done + kBlock) fb.gsite[a + lane] = i0 + 31 - __clz((int)accepted);
   const long long pos0 = sh.acc_pos;
   if (lane < nbk && pos0 + lane < c.acc_cap) c.acc_log[pos0 + lane] = mine ? 1 : 0;
   __syncwarp();
@@ -1097,28 +1145,29 @@ __device__ __forceinline__ void decide_sub_block_pair(Cta<float, RES>& x, int ta
 }
 
 // kPair: the one-warp form (FP32 kernels with room for its 64 block registers)
-template <bool kPair, typename T, bool RES>
+template <bool kPair, bool kRolled, typename T, bool RES>
 __device__ __forceinline__ void decide(Cta<T, RES>& x, int tau, uint32_t sweep, int i0, int nbk, int a_done) {
-  if constexpr (kPair && std::is_same<T, float>::value) decide_sub_block_pair(x, tau, sweep, i0, nbk, a_done);
+  stage_block(x, i0, nbk, a_done);
+  if constexpr (kPair && std::is_same<T, float>::value) decide_sub_block_pair<kRolled>(x, tau, sweep, i0, nbk, a_done);
   else decide_sub_block(x, tau, sweep, i0, nbk, a_done);
 }
 
 template <typename T, bool RES, bool kPair>
 __device__ __noinline__ void phase_decide(int tau, uint32_t sweep, int i0, int nbk, int a_done) {
   auto x = this_cta<T, RES>();
-  decide<kPair>(x, tau, sweep, i0, nbk, a_done);
+  decide<kPair, true>(x, tau, sweep, i0, nbk, a_done);
   __syncthreads();
   x.mark(kPhFlip);
 }
-template <typename T, bool RES>
-__device__ __noinline__ void phase_vectors(int m0, int m1) {
+template <typename T, bool RES, bool kLater>
+__device__ __noinline__ void phase_vectors(int i0, int m0, int m1) {
   auto x = this_cta<T, RES>();
   if constexpr (std::is_same<T, double>::value) {
     sm_vectors_by_flip(x, m0, m1);
   } else {
-    sm_core(x, m0, m1 - m0);
+    sm_core(x, i0, m0, m1 - m0);
     __syncthreads();
-    sm_vectors(x, m0, m1 - m0);
+    sm_vectors<kLater>(x, m0, m1 - m0);
   }
   __syncthreads();
   x.mark(kPhFlushVec);
@@ -1142,7 +1191,10 @@ __device__ __forceinline__ void update_slice(int tau, uint32_t sweep) {
     for (int i0 = d0; i0 < d1; i0 += sub) {
       phase_decide<T, RES, kPair>(tau, sweep, i0, min(sub, d1 - i0), a_done);
       const int a = x.sh.na;
-      if (a > a_done) phase_vectors<T, RES>(a_done, a);
+      if (a > a_done) {
+        if (a_done == 0 || std::is_same<T, double>::value) phase_vectors<T, RES, false>(i0, a_done, a);
+        else phase_vectors<T, RES, true>(i0, a_done, a);
+      }
       a_done = a;
     }
     if (a_done > 0) phase_apply<T, RES>(a_done);
@@ -1491,16 +1543,41 @@ __device__ __forceinline__ void qr_householder(Cta<T, RES>& x, int N, int ldm, i
   x.mark(kPhQRForm);
 }
 
-// 1 / x: the hardware's approximation (about 20 bits) and two Newton steps
-// y <- y + y (1 - x y), four dependent FMAs (65 cycles each) where the division
-// takes 646; outside the approximation's range the division.
+// 1 / x: the hardware's approximation (about 20 bits) and one step
+// y <- y + y (e + e^2), e = 1 - x y, of third order: three dependent FMAs (65
+// cycles each) where the division takes 646; outside the approximation's
+// range the division.
 static __device__ __forceinline__ double recip64(double x) {
-  const double ax = fabs(x);
-  if (!(ax > 1e-290 && ax < 1e290)) return 1.0 / x;
+  const int e = (__double2hiint(x) >> 20) & 0x7ff;
+  if (e < 60 || e > 1980) return 1.0 / x;
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  y = fma(y, fma(-x, y, 1.0), y);
-  return fma(y, fma(-x, y, 1.0), y);
+  const double r = fma(-x, y, 1.0);
+  return fma(y, fma(r, r, r), y);
+}
+
+// f(k, i, load(k, i)) for k < n, i < N over the CTA, flat (no idle lanes in a
+// row's tail), four loads in flight per thread
+template <typename L, typename F>
+__device__ __forceinline__ void for_flat4(int n, int N, L load, F f) {
+  const int step = (int)blockDim.x, sq = step / N, sr = step - sq * N;
+  int k = (int)threadIdx.x / N, i = (int)threadIdx.x - k * N;
+  while (k < n) {
+    int kk[4], ii[4];
+    decltype(load(0, 0)) v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      kk[u] = k;
+      ii[u] = i;
+      if (k < n) v[u] = load(k, i);
+      i += sr;
+      k += sq;
+      if (i >= N) { i -= N; ++k; }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (kk[u] < n) f(kk[u], ii[u], v[u]);
+  }
 }
 
 // Cholesky QR of a stack block M (N x n) of the reduced-precision paths:
@@ -1517,102 +1594,137 @@ static __device__ __forceinline__ double recip64(double x) {
 // 1e6); the caller then takes the Householder QR.  R has a positive diagonal,
 // so only log|det R| = (1/2) sum_k log(pivot_k) is returned.
 //
-// 72 sites, n = 36, one chain alone on its SM, per block and spin: the FP64
+// Both spins go through the elimination together, half of the CTA each.
+//
+// 72 sites, n = 36, one chain alone on its SM, both spins: the FP64
 // Gram matrix, factor (two barriers, a division and a row scaling per column)
-// and column-by-column Q took 122 + 57 kcycles.
+// and column-by-column Q took 358 kcycles.
+
+// digits of a block into D (ld digit_ld(N)); the exponent comes back
 template <typename T, bool RES, typename Elem>
-__device__ __forceinline__ bool qr_cholesky(Cta<T, RES>& x, int N, int n, double* Q, double& logabs, Elem M) {
-  Smem<T>& sh = x.sh;
+__device__ __forceinline__ int pack_block(Cta<T, RES>& x, int N, int n, Elem M) {
   unsigned long long* D = reinterpret_cast<unsigned long long*>(x.scr + x.L.m64);
-  unsigned long long* X = reinterpret_cast<unsigned long long*>(x.scr + x.L.mtq);   // the block's source is free by then
-  double* C = x.chol();                 // n x n row-major: see below
-  double* u[2] = {C + (long)n * n, C + (long)n * n + n};
-  double* dlim = u[1] + n;              // smallest pivot accepted
-  double* pv = dlim + n;                // pivots
-  double* isq = pv + n;                 // 1 / sqrt(pivot)
-  int* ex = reinterpret_cast<int*>(isq + n);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (int)blockDim.x >> 5;
-  const int ldd = digit_ld(N), ldx = digit_ld(n);
+  const int ldd = digit_ld(N);
   int E = kDigitNone;
-  PQMC_FOR_2D(i, 0, N, k, 0, n) E = max(E, digit_exp(M(i, k)));
-  E = digit_cta_max(E, reinterpret_cast<int*>(sh.red));
-  PQMC_FOR_2D(i, 0, N, k, 0, n) D[(long)k * ldd + i] = digit_pack(M(i, k), E);
-  if (threadIdx.x == 0) sh.chol_bad = 0;
+  for_flat4(N, n, M, [&](int, int, auto v) { E = max(E, digit_exp(v)); });
+  E = digit_cta_max(E, reinterpret_cast<int*>(x.sh.red));
+  for_flat4(N, n, M, [&](int i, int k, auto v) { D[(long)k * ldd + i] = digit_pack(v, E); });
   __syncthreads();
-  auto eM = [E](int) { return E; };
-  digit_gemm<true, true>(n, n, N, D, ldd, 1, D, ldd, 1, eM, eM, true, false,
-                   [C, n](int i, int j, double v) { C[(long)i * n + j] = v; });
+  return E;
+}
+
+// Elimination of [C | I] for both spins, the part of I that has filled in kept
+// below the diagonal: step k takes row k, u_j = row_kj / p_k, from the rows below,
+//     row_ij -= C_ki u_j   (C_ki = C_ik; column k, still zero: -C_ki / p_k).
+// Row k then holds the Schur complements C_kj right of the diagonal and row
+// k of L^{-1} (L unit lower, C = L diag(p) L^T) left of it.  One warp per spin
+// runs ahead: it takes row k + 1 first, its pivot, reciprocal and u, while the
+// others do the rest of step k: one barrier per column, the reciprocal's
+// latency beside the other rows' FMAs (a flat index with constant row
+// length: full FP64 warp instructions, no division).  The two warps that run
+// ahead sit on different sub-partitions.
+template <typename T, bool RES>
+__device__ __forceinline__ void chol_eliminate(Cta<T, RES>& x) {
+  Smem<T>& sh = x.sh;
+  const int H = x.nspec() == 2 ? (int)blockDim.x >> 1 : (int)blockDim.x;
+  const int s = (int)threadIdx.x / H, tid = (int)threadIdx.x - s * H, lane = threadIdx.x & 31;
+  const int nw = H >> 5, w = tid >> 5, ahead = s < nw ? s : 0;
+  const int n = x.nsig(s), ldc = digit_ld(x.nsig(s)), nmax = max(x.nsig(0), x.nsig(1));
+  double* C = x.chol(s);
+  double* u0 = C + (long)n * ldc;
+  double* dlim = u0 + 2 * n;            // smallest pivot accepted
+  double* pv = dlim + n;                // pivots
+  if (tid == 0) sh.chol_bad[s] = 0;
+  for (int k = tid; k < n; k += H) dlim[k] = 1e-12 * C[(long)k * ldc + k];
   __syncthreads();
-  for (int k = threadIdx.x; k < n; k += blockDim.x) dlim[k] = 1e-12 * C[(long)k * n + k];
-  __syncthreads();
-  x.mark(kPhOverlap);
-  // Elimination of [C | I], the part of I that has filled in kept below the
-  // diagonal: step k takes row k, u_j = row_kj / p_k, from the rows below,
-  //     row_ij -= C_ki u_j   (C_ki = C_ik; column k, still zero: -C_ki / p_k).
-  // Row k then holds the Schur complements C_kj right of the diagonal and row
-  // k of L^{-1} (L unit lower, C = L diag(p) L^T) left of it.  Warp 0 runs
-  // ahead: it takes row k + 1 first, its pivot, reciprocal and u, while the
-  // others do the rest of step k: one barrier per column, the reciprocal's
-  // latency beside the other rows' FMAs (a flat index with constant row
-  // length: full FP64 warp instructions, no division).
-  auto pivot_row = [&](int r, double* un) {
-    const double p = C[(long)r * n + r];
-    const bool ok = p > dlim[r];
+  auto pivot_row = [&](int r) {
+    double* un = u0 + (r & 1) * n;
+    const double p = C[(long)r * ldc + r];
+    // (positive doubles order like their bits)
+    const long long pb = __double_as_longlong(p);
+    const bool ok = pb > __double_as_longlong(dlim[r]) && pb < 0x7ff0000000000000ll;
     const double ip = ok ? recip64(p) : 0.0;
     if (lane == 0) {
       pv[r] = p;
-      if (!ok) sh.chol_bad = 1;
+      if (!ok) sh.chol_bad[s] = 1;
     }
-    for (int j = lane; j < n; j += 32) un[j] = j == r ? ip : C[(long)r * n + j] * ip;
+    for (int j = lane; j < n; j += 32) un[j] = j == r ? ip : C[(long)r * ldc + j] * ip;
   };
-  if (warp == 0) pivot_row(0, u[0]);
+  if (w == ahead && n > 0) pivot_row(0);
   __syncthreads();
-  {
-    const int rest = (int)blockDim.x - 32, tr = (int)threadIdx.x - 32;
-    const int sq = rest / n, sr = rest - sq * n;
-    const int i0 = tr / n, j0 = tr - i0 * n;
-    for (int k = 0; k + 1 < n && !sh.chol_bad; ++k) {
-      const double* uk = u[k & 1];
-      const double* Ck = C + (long)k * n;
-      if (warp == 0) {
+  const bool bulk = nw == 1 || w != ahead;
+  const int rest = nw == 1 ? H : H - 32, tr = nw == 1 ? tid : (w < ahead ? tid : tid - 32);
+  const int sq = n > 0 ? rest / n : 0, sr = n > 0 ? rest - sq * n : 0;
+  const int i0 = n > 0 && tr >= 0 ? tr / n : 0, j0 = tr - i0 * n;
+  for (int k = 0; k + 1 < nmax; ++k) {
+    if (k + 1 < n && !sh.chol_bad[s]) {
+      const double* uk = u0 + (k & 1) * n;
+      const double* Ck = C + (long)k * ldc;
+      if (w == ahead) {
         const int r = k + 1;
-        double* Cr = C + (long)r * n;
+        double* Cr = C + (long)r * ldc;
         const double m = Ck[r];
         for (int j = lane; j < n; j += 32) Cr[j] = fma(-m, uk[j], j == k ? 0.0 : Cr[j]);
         __syncwarp();
-        pivot_row(r, u[r & 1]);
-      } else {
+        pivot_row(r);
+      }
+      if (bulk) {
         int i = k + 2 + i0, j = j0;
         while (i < n) {
-          double* c = C + (long)i * n + j;
-          *c = fma(-Ck[i], uk[j], j == k ? 0.0 : *c);
+          // two elements in flight
+          const int i1 = i, j1 = j;
           j += sr;
           i += sq;
           if (j >= n) { j -= n; ++i; }
+          const bool two = i < n;
+          const int i2 = two ? i : i1, j2 = two ? j : j1;
+          double* p1 = C + i1 * ldc + j1;
+          double* p2 = C + i2 * ldc + j2;
+          const double f1 = Ck[i1], f2 = Ck[i2], u1 = uk[j1], u2 = uk[j2];
+          const double a1 = j1 == k ? 0.0 : *p1, a2 = j2 == k ? 0.0 : *p2;
+          const double v1 = fma(-f1, u1, a1), v2 = fma(-f2, u2, a2);
+          *p1 = v1;
+          if (two) {
+            *p2 = v2;
+            j += sr;
+            i += sq;
+            if (j >= n) { j -= n; ++i; }
+          }
         }
       }
-      __syncthreads();
     }
+    __syncthreads();
   }
+  double* isq = pv + n;                 // 1 / sqrt(pivot)
+  if (n > 0 && !sh.chol_bad[s])
+    for (int k = tid; k < n; k += H) isq[k] = rsqrt(pv[k]);
   __syncthreads();
-  if (sh.chol_bad) return false;
-  for (int k = threadIdx.x; k < n; k += blockDim.x) isq[k] = rsqrt(pv[k]);
-  __syncthreads();
-  x.mark(kPhQR);
-  // digits of R^{-1}: column j is row j of L^{-1} / sqrt(p_j), 1 / sqrt(p_j) on the diagonal
+}
+
+// Q = M R^{-1} of spin s to the stack block, from the block's digits (exponent
+// E) and the elimination; log|det R| comes back.  The factor's digits take its
+// place: column j of R^{-1} is row j of L^{-1} / sqrt(p_j), with 1 / sqrt(p_j)
+// on the diagonal.
+template <typename T, bool RES>
+__device__ __forceinline__ double chol_form_q(Cta<T, RES>& x, int s, int E, double* Q) {
+  Smem<T>& sh = x.sh;
+  const int N = x.c.N, n = x.nsig(s), ldd = digit_ld(N), ldc = digit_ld(n);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (int)blockDim.x >> 5;
+  const unsigned long long* D = reinterpret_cast<const unsigned long long*>(x.scr + x.L.m64);
+  double* C = x.chol(s);
+  const double* pv = C + (long)n * ldc + 3 * n;
+  const double* isq = pv + n;
+  int* ex = reinterpret_cast<int*>(C + (long)n * ldc);       // (u's place)
   for (int j = warp; j < n; j += nw) {
     const double f = isq[j];
+    double* row = C + (long)j * ldc;
+    unsigned long long* X = reinterpret_cast<unsigned long long*>(row);
     int e = lane == 0 ? digit_exp(f) : kDigitNone;
-    for (int c = lane; c < j; c += 32) e = max(e, digit_exp(C[(long)j * n + c] * f));
+    for (int c = lane; c < j; c += 32) e = max(e, digit_exp(row[c] * f));
     e = __reduce_max_sync(0xffffffffu, e);
-    for (int c = lane; c < ldx; c += 32)
-      X[(long)j * ldx + c] = c < j ? digit_pack(C[(long)j * n + c] * f, e) : c == j ? digit_pack(f, e) : kDigitZero;
+    for (int c = lane; c < ldc; c += 32) X[c] = c < j ? digit_pack(row[c] * f, e) : c == j ? digit_pack(f, e) : kDigitZero;
     if (lane == 0) ex[j] = e;
   }
-  __syncthreads();
-  digit_gemm<false, true>(N, n, n, D, 1, ldd, X, ldx, 1, eM, [ex](int j) { return ex[j]; }, false, true,
-                    [Q, N](int i, int j, double v) { Q[(long)j * N + i] = v; });
-  // log|det R|
   if (warp == 0) {
     double la = 0.0;
     for (int k = lane; k < n; k += 32) la += log(pv[k]);
@@ -1620,10 +1732,12 @@ __device__ __forceinline__ bool qr_cholesky(Cta<T, RES>& x, int N, int n, double
     if (lane == 0) sh.red[0] = 0.5 * la;
   }
   __syncthreads();
-  logabs = sh.red[0];
+  const double logabs = sh.red[0];
+  digit_gemm<false, true>(N, n, n, D, 1, ldd, reinterpret_cast<const unsigned long long*>(C), ldc, 1,
+                          [E](int) { return E; }, [ex](int j) { return ex[j]; }, false, true,
+                          [Q, N](int i, int j, double v) { Q[(long)j * N + i] = v; });
   __syncthreads();
-  x.mark(kPhQRForm);
-  return true;
+  return logabs;
 }
 
 // Invert O_s (n_s x n_s, row-major) in place for both spins at once by
@@ -1642,10 +1756,11 @@ __device__ __forceinline__ bool qr_cholesky(Cta<T, RES>& x, int N, int n, double
 template <typename T, bool RES>
 __device__ __forceinline__ void gj_invert2(Cta<T, RES>& x) {
   Smem<T>& sh = x.sh;
-  const int half = (int)blockDim.x >> 1;
-  const int s = (int)threadIdx.x >= half ? 1 : 0;
+  const int half = x.nspec() == 2 ? (int)blockDim.x >> 1 : (int)blockDim.x;   // threads per species
+  const int s = (int)threadIdx.x / half;
   const int tid = (int)threadIdx.x - s * half, lane = threadIdx.x & 31;
-  const bool first = tid < 32;
+  const int nw = half >> 5, w = tid >> 5, ahead = s < nw ? s : 0;   // (on different sub-partitions)
+  const bool first = w == ahead;
   const int n = x.nsig(s), nmax = max(x.nsig(0), x.nsig(1));
   double* A = x.Ob(s);
   double* f = x.gj_col(s);              // column j before step j, two steps in flight: f[(j & 1) n ..]
@@ -1681,7 +1796,7 @@ __device__ __forceinline__ void gj_invert2(Cta<T, RES>& x) {
     __syncwarp();
     pick(0);
   }
-  const int rest = half > 32 ? half - 32 : half, tr = half > 32 ? tid - 32 : tid;
+  const int rest = nw > 1 ? half - 32 : half, tr = nw == 1 || w < ahead ? tid : tid - 32;
   const int sq = n > 0 ? rest / n : 0, sr = n > 0 ? rest - sq * n : 0;
   const int i0 = n > 0 && tr >= 0 ? tr / n : 0, j0 = tr - i0 * n;
   __syncthreads();
@@ -1706,17 +1821,28 @@ __device__ __forceinline__ void gj_invert2(Cta<T, RES>& x) {
         __syncwarp();
         pick(j + 1);
       }
-      if (!first || half <= 32) {
+      if (!first || nw == 1) {
         int i = i0, c = j0;
         while (i < n) {
-          if (c != j + 1) {
-            double* a = A + (long)i * n + c;
-            const double v = fma(-fj[i], R[c], c == j ? 0.0 : *a);
-            *a = i == r ? R[c] : v;
-          }
+          // two elements in flight
+          const int i1 = i, c1 = c;
           c += sr;
           i += sq;
           if (c >= n) { c -= n; ++i; }
+          const bool two = i < n;
+          const int i2 = two ? i : i1, c2 = two ? c : c1;
+          double* p1 = A + i1 * n + c1;
+          double* p2 = A + i2 * n + c2;
+          const double f1 = fj[i1], f2 = fj[i2], r1 = R[c1], r2 = R[c2];
+          const double a1 = c1 == j ? 0.0 : *p1, a2 = c2 == j ? 0.0 : *p2;
+          const double v1 = i1 == r ? r1 : fma(-f1, r1, a1), v2 = i2 == r ? r2 : fma(-f2, r2, a2);
+          if (c1 != j + 1) *p1 = v1;
+          if (two && c2 != j + 1) *p2 = v2;
+          if (two) {
+            c += sr;
+            i += sq;
+            if (c >= n) { c -= n; ++i; }
+          }
         }
       }
     }
@@ -1809,14 +1935,14 @@ __device__ __forceinline__ double* stack_block(const Cta<T, RES>& x, double* bas
 // blocks at the ends of the projection.
 template <typename T, bool RES, typename F>
 __device__ __forceinline__ void with_block(Cta<T, RES>& x, int left, int s, F f) {
-  const int n = x.nsig(s), N = x.c.N;
+  const int ldn = x.ldn(s), N = x.c.N;
   if (x.sh.src == 2) {
     const double* P = x.c.P + (long)s * N * x.c.nmax;
     const int tau = left ? x.c.Ltau + 1 : 0;
     f([&x, P, tau, s, N](int i, int k) { return x.vexp(tau, s, i) * P[(long)k * N + i]; });
   } else {
-    const T* Mt = x.sh.src ? x.Mt2() : x.Mt();
-    f([Mt, n](int i, int k) { return Mt[(long)i * n + k]; });
+    const T* Mt = x.sh.src ? x.Mt2() : x.Mt(s);
+    f([Mt, ldn](int i, int k) { return Mt[(long)i * ldn + k]; });
   }
 }
 // M64 = that block, column-major
@@ -1840,8 +1966,8 @@ __device__ __noinline__ void phase_stack(int b, int left, int s) {
   auto x = this_cta<T, RES>();
   const ChainDesc& c = x.c;
   const int N = c.N, n_stab = c.n_stab;
-  const int n = x.nsig(s);
-  T* Mt = x.Mt();
+  const int n = x.nsig(s), ldn = x.ldn(s);
+  T* Mt = x.Mt(s);
   T* Mt2 = x.Mt2();
   constexpr bool f64 = std::is_same<T, double>::value;
   // Mt2 = e^{-dtau K} Mt: on the tensor cores in FP64 (digits of Mt in M64's place)
@@ -1851,16 +1977,16 @@ __device__ __noinline__ void phase_stack(int b, int left, int s) {
         const int ldd = digit_ld(N), ldk = N + (N & 1);
         unsigned long long* D = reinterpret_cast<unsigned long long*>(x.M64());
         int e = kDigitNone;
-        PQMC_FOR_2D(i, 0, N, k, 0, n) e = max(e, digit_exp(from[(long)i * n + k]));
+        PQMC_FOR_2D(i, 0, N, k, 0, n) e = max(e, digit_exp(from[(long)i * ldn + k]));
         const int E = digit_cta_max(e, reinterpret_cast<int*>(x.sh.red)), e1 = c.eEm;
-        PQMC_FOR_2D(i, 0, N, k, 0, n) D[(long)k * ldk + i] = digit_pack(from[(long)i * n + k], E);
+        PQMC_FOR_2D(i, 0, N, k, 0, n) D[(long)k * ldk + i] = digit_pack(from[(long)i * ldn + k], E);
         __syncthreads();
         digit_gemm<true, true>(N, n, N, c.dEm, ldd, 1, D, ldk, 1, [e1](int) { return e1; }, [E](int) { return E; }, false,
-                               false, [to, n](int i, int j, double v) { to[(long)i * n + j] = v; });
+                               false, [to, ldn](int i, int j, double v) { to[(long)i * ldn + j] = v; });
         return;
       }
     }
-    cta_gemm<T>(N, n, N, x.Em(), 1, c.ld, from, n, 1, to, n, 1, EpiStore());
+    cta_gemm<T>(N, n, N, x.Em(), 1, c.ld, from, ldn, 1, to, ldn, 1, EpiStore(), !f64);
   };
   int src = 0;
   if (left ? b == c.nb : b == 0) {
@@ -1869,11 +1995,11 @@ __device__ __noinline__ void phase_stack(int b, int left, int s) {
     src = 2;
   } else {
     const double* prev = left ? stack_block(x, c.Lst, b + 1, s) : stack_block(x, c.Rst, b - 1, s);
-    PQMC_FOR_2D(k, 0, n, i, 0, N) Mt[(long)i * n + k] = (T)prev[(long)k * N + i];
+    PQMC_FOR_2D(k, 0, n, i, 0, N) Mt[(long)i * ldn + k] = (T)prev[(long)k * N + i];
     if (!left) {
       for (int tau = (b - 1) * n_stab + 1; tau <= b * n_stab; ++tau) {
         x.stage(tau);
-        PQMC_FOR_2D(i, 0, N, k, 0, n) Mt[(long)i * n + k] *= x.vexpT(tau, s, i);
+        PQMC_FOR_2D(i, 0, N, k, 0, n) Mt[(long)i * ldn + k] *= x.vexpT(tau, s, i);
         __syncthreads();
         product(Mt, Mt2);
         __syncthreads();
@@ -1885,10 +2011,15 @@ __device__ __noinline__ void phase_stack(int b, int left, int s) {
       for (int tau = (b + 1) * n_stab; tau > b * n_stab; --tau) {
         product(Mt, Mt2);
         x.stage(tau);
-        PQMC_FOR_2D(i, 0, N, k, 0, n) Mt[(long)i * n + k] = x.vexpT(tau, s, i) * Mt2[(long)i * n + k];
+        PQMC_FOR_2D(i, 0, N, k, 0, n) Mt[(long)i * ldn + k] = x.vexpT(tau, s, i) * Mt2[(long)i * ldn + k];
         __syncthreads();
       }
     }
+  }
+  if (!f64 && src == 1) {
+    // (an odd number of products upwards: Mt is the work buffer now)
+    for (int e = threadIdx.x; e < N * ldn; e += blockDim.x) Mt2[e] = Mt[e];
+    src = 0;
   }
   if (threadIdx.x == 0) x.sh.src = src;
   __syncthreads();
@@ -1896,14 +2027,36 @@ __device__ __noinline__ void phase_stack(int b, int left, int s) {
   x.mark(kPhStack);
 }
 
+// digits of the block of spin s and, with gram, its Gram matrix (upper triangle)
 template <typename T, bool RES>
-__device__ __noinline__ bool phase_chol(int b, int left, int s, double* logabs) {
+__device__ __noinline__ int phase_digits(int left, int s, bool gram) {
   auto x = this_cta<T, RES>();
-  const int N = x.c.N, n = x.nsig(s);
-  double* Q = stack_block(x, left ? x.c.Lst : x.c.Rst, b, s);
-  bool ok = false;
-  with_block(x, left, s, [&](auto e) { ok = qr_cholesky(x, N, n, Q, *logabs, e); });
-  return ok;
+  const int N = x.c.N, n = x.nsig(s), ldd = digit_ld(N), ldc = digit_ld(n);
+  int E = 0;
+  with_block(x, left, s, [&](auto e) { E = pack_block(x, N, n, e); });
+  if (gram) {
+    const unsigned long long* D = reinterpret_cast<const unsigned long long*>(x.scr + x.L.m64);
+    double* C = x.chol(s);
+    auto eM = [E](int) { return E; };
+    digit_gemm<true, true>(n, n, N, D, ldd, 1, D, ldd, 1, eM, eM, true, false,
+                           [C, ldc](int i, int j, double v) { C[(long)i * ldc + j] = v; });
+    __syncthreads();
+  }
+  x.mark(kPhOverlap);
+  return E;
+}
+template <typename T, bool RES>
+__device__ __noinline__ void phase_factor() {
+  auto x = this_cta<T, RES>();
+  chol_eliminate(x);
+  x.mark(kPhQR);
+}
+template <typename T, bool RES>
+__device__ __noinline__ double phase_form_q(int b, int left, int s, int E) {
+  auto x = this_cta<T, RES>();
+  const double la = chol_form_q(x, s, E, stack_block(x, left ? x.c.Lst : x.c.Rst, b, s));
+  x.mark(kPhQRForm);
+  return la;
 }
 template <typename T, bool RES>
 __device__ __noinline__ void phase_householder(int b, int left, int s, double* logabs, double* sgn) {
@@ -1920,12 +2073,7 @@ template <typename T, bool RES>
 __device__ __forceinline__ void push_block(int b, int left) {
   auto x = this_cta<T, RES>();
   const ChainDesc& c = x.c;
-  for (int s = 0; s < x.nspec(); ++s) {
-    phase_stack<T, RES>(b, left, s);
-    double la, sg = 1.0;
-    bool done = false;
-    if constexpr (!std::is_same<T, double>::value) done = phase_chol<T, RES>(b, left, s, &la);
-    if (!done) phase_householder<T, RES>(b, left, s, &la, &sg);
+  auto weight = [&](int s, double la, double sg) {
     if (threadIdx.x == 0) {
       double* lg = left ? c.Llog : c.Rlog;
       const bool first = left ? b == c.nb : b == 0;
@@ -1934,6 +2082,31 @@ __device__ __forceinline__ void push_block(int b, int left) {
       lg[(b * 2 + s) * 2 + 1] = (first ? 1.0 : lg[(bp * 2 + s) * 2 + 1]) * sg;
     }
     __syncthreads();
+  };
+  double la, sg;
+  if constexpr (std::is_same<T, double>::value) {
+    for (int s = 0; s < x.nspec(); ++s) {
+      phase_stack<T, RES>(b, left, s);
+      phase_householder<T, RES>(b, left, s, &la, &sg);
+      weight(s, la, sg);
+    }
+  } else {
+    for (int s = 0; s < x.nspec(); ++s) phase_stack<T, RES>(b, left, s);
+    int E = 0;
+    for (int s = 0; s < x.nspec(); ++s) E = phase_digits<T, RES>(left, s, true);
+    phase_factor<T, RES>();
+    // the digits at hand are the last species'
+    const bool bad[2] = {x.sh.chol_bad[0] != 0, x.sh.chol_bad[1] != 0};
+    for (int s = x.nspec() - 1; s >= 0; --s) {
+      if (bad[s]) continue;
+      if (s < x.nspec() - 1) E = phase_digits<T, RES>(left, s, false);
+      weight(s, phase_form_q<T, RES>(b, left, s, E), 1.0);
+    }
+    for (int s = 0; s < x.nspec(); ++s)
+      if (bad[s]) {
+        phase_householder<T, RES>(b, left, s, &la, &sg);
+        weight(s, la, sg);
+      }
   }
 }
 
@@ -2003,10 +2176,10 @@ __device__ __forceinline__ void assemble_spin(Cta<T, RES>& x, int s, const doubl
     }
     T* qrt = x.QRt();
     T* qlt = x.QLt();
-    PQMC_FOR_2D(k, 0, ns, i, 0, N) {
-      qrt[(long)k * N + i] = (T)QR[(long)k * N + i];
-      qlt[(long)k * N + i] = (T)QL[(long)k * N + i];
-    }
+    for_flat4(ns, N, [QR, N](int k, int i) { return QR[(long)k * N + i]; },
+              [qrt, ld](int k, int i, double v) { qrt[(long)k * ld + i] = (T)v; });
+    for_flat4(ns, N, [QL, N](int k, int i) { return QL[(long)k * N + i]; },
+              [qlt, ld](int k, int i, double v) { qlt[(long)k * ld + i] = (T)v; });
     qr = qrt;
     ql = qlt;
     __syncthreads();
@@ -2017,18 +2190,20 @@ __device__ __forceinline__ void assemble_spin(Cta<T, RES>& x, int s, const doubl
     // O^{-1} to the path precision once (in the order of its rows and columns),
     // then a path-precision product
     T* ot = x.Ot();
+    const int ldo = pad4(ns);
     if (c.dg64) {
-      for (int e = threadIdx.x; e < ns * ns; e += blockDim.x) ot[e] = (T)Xinv[e];
+      PQMC_FOR_2D(j, 0, ns, k, 0, ns) ot[(long)j * ldo + k] = (T)Xinv[(long)j * ns + k];
     } else {
       const int* rows = x.gj_rows(s);
-      PQMC_FOR_2D(j, 0, ns, k, 0, ns) ot[(long)j * ns + rows[k]] = (T)Xinv[(long)rows[j] * ns + k];
+      PQMC_FOR_2D(j, 0, ns, k, 0, ns) ot[(long)j * ldo + rows[k]] = (T)Xinv[(long)rows[j] * ns + k];
     }
     __syncthreads();
-    cta_gemm<T>(ns, N, ns, ot, ns, 1, ql, N, 1, Y, ld, 1, EpiStore());
+    cta_gemm<T>(ns, N, ns, ot, ldo, 1, ql, ld, 1, Y, ld, 1, EpiStore(), true);
   }
   __syncthreads();
   EpiFresh<T> epi{x.G(s), ld, &dmax};
-  cta_gemm<T>(N, N, ns, qr, 1, N, Y, ld, 1, (T*)nullptr, 0, 0, epi);
+  cta_gemm<T>(N, N, ns, qr, 1, std::is_same<T, double>::value ? N : ld, Y, ld, 1, (T*)nullptr, 0, 0, epi,
+              !std::is_same<T, double>::value);
   if constexpr (!std::is_same<T, double>::value) {
     if (c.dg64 == 2 && record) {
       // the refreshed G itself against G_FP64 (the path-precision copies of
@@ -2068,12 +2243,14 @@ __device__ __noinline__ void phase_overlap(int b) {
     int E = 1;
     for (int pass = 0; pass < 2; ++pass) {
       int e = kDigitNone;
-      PQMC_FOR_2D(k, 0, n, i, 0, N) {
-        const double l = QL[(long)k * N + i], r = QR[(long)k * N + i];
-        e = max(e, max(digit_exp(l), digit_exp(r)));
-        DL[(long)k * ldd + i] = digit_pack(l, E);
-        DR[(long)k * ldd + i] = digit_pack(r, E);
-      }
+      auto pack = [&](const double* Q, unsigned long long* D) {
+        for_flat4(n, N, [Q, N](int k, int i) { return Q[(long)k * N + i]; }, [&](int k, int i, double v) {
+          e = max(e, digit_exp(v));
+          D[(long)k * ldd + i] = digit_pack(v, E);
+        });
+      };
+      pack(QL, DL);
+      pack(QR, DR);
       const bool again = __syncthreads_or(e > E) != 0;
       if (!again) break;
       E = digit_cta_max(e, reinterpret_cast<int*>(x.sh.red));
