@@ -179,6 +179,11 @@ struct SpBuf {
   __device__ __host__ SpBuf(unsigned char* base, int N, int ld, int nmax, int tsize = (int)sizeof(T))
       : b(base), L(spread_layout(N, ld, nmax, tsize)) {}
   __device__ __host__ T* mt(int s, int k) const { return reinterpret_cast<T*>(b + L.mt[s][k]); }
+  __device__ __host__ unsigned long long* dq(int s, int k) const {
+    return reinterpret_cast<unsigned long long*>(b + L.dq[s][k]);
+  }
+  __device__ __host__ int* em() const { return reinterpret_cast<int*>(b + L.misc + 40); }
+  __device__ __host__ int* eq() const { return reinterpret_cast<int*>(b + L.misc + 48); }
   __device__ __host__ double* m64(int s) const { return reinterpret_cast<double*>(b + L.m64[s]); }
   __device__ __host__ double* c64(int s) const { return reinterpret_cast<double*>(b + L.c64[s]); }
   __device__ __host__ double* rinv(int s) const { return reinterpret_cast<double*>(b + L.rinv[s]); }
@@ -202,6 +207,12 @@ struct SpBuf {
   }
   __device__ __host__ double* lchol() const { return reinterpret_cast<double*>(b + L.misc + 24); }
 };
+
+// largest digit exponent over a grid, in global memory (every thread of a warp calls)
+__device__ __forceinline__ void sp_exp_max(int* to, int e) {
+  e = __reduce_max_sync(0xffffffffu, e);
+  if ((threadIdx.x & 31) == 0) atomicMax(to, e);
+}
 
 // e^{V_sigma(s_tau)} at site i in FP64, as the single-CTA path tabulates it
 __device__ __forceinline__ double sp_vexp(const ChainDesc& c, int tau, int s, int i) {
@@ -384,13 +395,17 @@ __global__ void sp_stack_first_kernel(const ChainDesc* chains, int tau0, int lef
   const int N = c.N, s = blockIdx.y, n = s == 0 ? c.nup : c.ndn, ldn = c.nmax;
   SpBuf<T> sp(c.spread, N, c.ld, c.nmax);
   const long stride = (long)gridDim.x * blockDim.x;
+  int ex = kDigitNone;
   if (tau0 >= 0) {
     const double* P = c.P + (long)s * N * c.nmax;
     double* M = sp.m64(s);
     for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < (long)N * n; e += stride) {
       const int q = (int)(e / N), i = (int)(e % N);
-      M[(long)q * N + i] = sp_vexp(c, tau0, s, i) * P[(long)q * N + i];
+      const double v = sp_vexp(c, tau0, s, i) * P[(long)q * N + i];
+      M[(long)q * N + i] = v;
+      ex = max(ex, digit_exp(v));
     }
+    sp_exp_max(sp.em() + s, ex);
   } else {
     const double* prev = (left ? c.Lst : c.Rst) + ((long)b_prev * 2 + s) * N * c.nmax;
     T* Mt = sp.mt(s, 0);
@@ -410,10 +425,14 @@ __global__ void sp_to64_kernel(const ChainDesc* chains, int k) {
   SpBuf<T> sp(c.spread, N, c.ld, c.nmax);
   const T* Mt = sp.mt(s, k);
   double* M = sp.m64(s);
+  int ex = kDigitNone;
   for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < (long)N * n; e += (long)gridDim.x * blockDim.x) {
     const int q = (int)(e / N), i = (int)(e % N);
-    M[(long)q * N + i] = (double)Mt[(long)i * ldn + q];
+    const double v = (double)Mt[(long)i * ldn + q];
+    M[(long)q * N + i] = v;
+    ex = max(ex, digit_exp(v));
   }
+  sp_exp_max(sp.em() + s, ex);
 }
 
 // path-precision copies of O^{-1}, Q_R and Q_L for the assembly
@@ -461,6 +480,39 @@ static __global__ void sp_stack_log_kernel(const ChainDesc* chains, int b, int l
   }
 }
 
+// The sums over all pairs of sites of a measurement (kinetic energy, staggered
+// exchange, see measure), one row of G per warp at a time; each CTA leaves its
+// pair of partial sums in M64's place, free until the next stack block.  (One
+// CTA did them in 3.6 ms at 648 sites.)
+constexpr int kSpMeasCtas = 76;
+template <typename T>
+__global__ void __launch_bounds__(256) sp_measure_kernel(const ChainDesc* chains) {
+  __shared__ double red[32];
+  const ChainDesc& c = chains[blockIdx.z];
+  if (c.st->err) return;
+  const int N = c.N, ld = c.ld, lane = threadIdx.x & 31;
+  const T* G0 = static_cast<const T*>(c.G);
+  double ek = 0.0, ex = 0.0;
+  for (int i = blockIdx.x * 8 + (int)(threadIdx.x >> 5); i < N; i += 8 * kSpMeasCtas)
+    for (int j = lane; j < N; j += 32) {
+      const double k = c.K64[(long)i * N + j], ee = c.eps[i] * c.eps[j];
+#pragma unroll
+      for (int s = 0; s < 2; ++s) {
+        const T* G = G0 + (long)s * N * ld;
+        const double gji = (i == j ? 1.0 : 0.0) - (double)G[(long)j * ld + i];
+        if (k != 0.0) ek += k * gji;
+        ex += ee * gji * (double)G[(long)i * ld + j];
+      }
+    }
+  ek = cta_sum(ek, red);
+  ex = cta_sum(ex, red);
+  if (threadIdx.x == 0) {
+    double* out = SpBuf<T>(c.spread, N, ld, c.nmax).m64(0) + 2 * blockIdx.x;
+    out[0] = ek;
+    out[1] = ex;
+  }
+}
+
 // End of a stabilisation, one CTA per chain: the weight of G from the stack
 // blocks' weights and O's pivots,
 // the recorded max |G - G_fresh| (flags & kSpRecord), the measurement
@@ -500,6 +552,7 @@ __global__ void __launch_bounds__(256) sp_tail_kernel(const ChainDesc* chains, u
   if (threadIdx.x == 0) {
     const double dmax = __longlong_as_double((long long)*sp.dmax());
     *sp.dmax() = 0ull;
+    sp.eq()[0] = sp.eq()[1] = 0;
     if (flags & kSpRecord) {
       if (!isfinite(dmax)) sh.err |= kErrNaN;
       sh.dGmax = fmax(sh.dGmax, dmax);
@@ -510,7 +563,7 @@ __global__ void __launch_bounds__(256) sp_tail_kernel(const ChainDesc* chains, u
     c.st->sign_stack = sign_total;
   }
   __syncthreads();
-  if (flags & kSpMeasure) measure(x);
+  if (flags & kSpMeasure) measure(x, sp.m64(0), kSpMeasCtas);
   store_state(x, err);
 }
 
@@ -520,6 +573,9 @@ __global__ void __launch_bounds__(256) sp_tail_kernel(const ChainDesc* chains, u
 
 // FP64 tile product over the jobs of g
 cudaError_t sp_dgemm(SpGemm& g, int mode, int max_m, int max_n, cudaStream_t st);
+// Gram matrix of M64 (upper triangle), or with b >= 0 the overlap Q_L^T Q_R of
+// stack blocks b, on the tensor cores
+cudaError_t sp_digit_products(const ChainDesc* d, int nc, int N, int nmax, int b, int tsize, cudaStream_t st);
 // Cholesky factor C = R^T R, panel p: the diagonal block R_PP and its inverse
 // (the block row R_{P,rest} = R_PP^{-T} C_{P,rest} and the trailing update
 // are sp_dgemm products)
@@ -658,16 +714,7 @@ cudaError_t spread_sweep_t(const SpreadPlan& P, int mode, int measure, cudaStrea
       ok(cudaSuccess);
     }
     // Cholesky QR: Gram matrix, blocked factor, Q = M R^{-1}
-    {
-      SpGemm g{};
-      g.njobs = 2 * nc;
-      g.sai = N; g.sak = 1; g.sbk = 1; g.sbj = N; g.sci = ldn; g.scj = 1;
-      g.upper = 1;   // the factorisation reads the upper triangle only
-      for (int c = 0; c < nc; ++c)
-        for (int s = 0; s < 2; ++s)
-          g.job[2 * c + s] = SpJob{buf(c).m64(s), buf(c).m64(s), buf(c).c64(s), nullptr, nullptr, nsig[s], nsig[s], N, 0};
-      ok(sp_dgemm(g, kSpStore, ldn, ldn, st));
-    }
+    ok(sp_digit_products(D, nc, N, ldn, -1, ts, st));
     for (int p0 = 0; p0 < ldn && e == cudaSuccess; p0 += kSpPanel) {
       const int p = p0 / kSpPanel;
       ok(sp_chol_panel(D, nc, ldn, p, ts, st));
@@ -711,16 +758,7 @@ cudaError_t spread_sweep_t(const SpreadPlan& P, int mode, int measure, cudaStrea
   };
   // G = 1 - Q_R (Q_L^T Q_R)^{-1} Q_L^T at stabilisation point b
   auto refresh = [&](int b, bool left, int flags) {
-    {
-      SpGemm g{};
-      g.njobs = 2 * nc;
-      g.sai = N; g.sak = 1; g.sbk = 1; g.sbj = N; g.sci = ldn; g.scj = 1;
-      for (int c = 0; c < nc; ++c)
-        for (int s = 0; s < 2; ++s)
-          g.job[2 * c + s] =
-              SpJob{stack_block(c, true, b, s), stack_block(c, false, b, s), buf(c).o64(s), nullptr, nullptr, nsig[s], nsig[s], N, 0};
-      ok(sp_dgemm(g, kSpStore, ldn, ldn, st));
-    }
+    ok(sp_digit_products(D, nc, N, ldn, b, ts, st));
     for (int p0 = 0; p0 < ldn && e == cudaSuccess; p0 += kSpGJ) {
       ok(sp_gj_panel(D, nc, ldn, p0 / kSpGJ, ts, st));
       SpGemm g{};
@@ -758,6 +796,10 @@ cudaError_t spread_sweep_t(const SpreadPlan& P, int mode, int measure, cudaStrea
     ok(sp_gemm_t<T>(gy, kSpStore, ldn, N, st));
     ok(sp_gemm_t<T>(gg, kSpFresh, N, N, st));
     cur = 0;
+    if (flags & kSpMeasure) {
+      sp_measure_kernel<T><<<dim3(kSpMeasCtas, 1, nc), 256, 0, st>>>(D);
+      ok(cudaSuccess);
+    }
     sp_tail_kernel<T><<<nc, 256, smem_cta, st>>>(D, P.seed, b, left ? 1 : 0, flags, P.d_err);
     ok(cudaSuccess);
   };

@@ -2,6 +2,8 @@
 // stabilisation steps that both paths call.
 #include "spread.cuh"
 
+#include <cooperative_groups.h>
+
 namespace pqmc {
 
 namespace {
@@ -11,18 +13,75 @@ __device__ __forceinline__ SpBuf<double> fp64_bufs(const ChainDesc& c, int tsize
 }
 __device__ __forceinline__ int nsig_of(const ChainDesc& c, int s) { return s == 0 ? c.nup : c.ndn; }
 
-// Cholesky factor, diagonal block of panel p (one CTA per spin, chain), on a
-// shared-memory copy: step k takes the pivot C_kk, writes row k of R
-// (R_kj = C_kj / sqrt(C_kk)) and then updates the rows below by
-// C_ij -= R_ki R_kj (one FP64 instruction per element); then R_PP^{-1} by
-// back substitution on the identity, one barrier per row.  Panel 0 first records the Gram diagonal and clears the chain's
-// breakdown flag and log det R.
+// Digits of M64 (b < 0) or of stack blocks b, Q_L and Q_R (grid: .., spin, chain).
+// M64 is packed against the exponent its writer left in em; the columns of
+// Q are orthonormal, |q| < 2, and an element beyond that (or a NaN) marks eq, which
+// makes the product NaN.
+__global__ void __launch_bounds__(256) sp_digits_kernel(const ChainDesc* chains, int b, int tsize) {
+  const ChainDesc& c = chains[blockIdx.z];
+  if (c.st->err) return;
+  const int s = blockIdx.y, n = nsig_of(c, s), N = c.N, ldd = digit_ld(N);
+  SpBuf<double> sp = fp64_bufs(c, tsize);
+  const long stride = (long)gridDim.x * blockDim.x, e0 = blockIdx.x * (long)blockDim.x + threadIdx.x;
+  if (b < 0) {
+    const double* M = sp.m64(s);
+    unsigned long long* D = sp.dq(s, 0);
+    const int E = sp.em()[s];
+    for (long e = e0; e < (long)N * n; e += stride) {
+      const int k = (int)(e / N), i = (int)(e % N);
+      D[(long)k * ldd + i] = digit_pack(M[e], E);
+    }
+  } else {
+    const long off = ((long)b * 2 + s) * N * c.nmax;
+    bool bad = false;
+    for (int q = 0; q < 2; ++q) {
+      const double* Q = (q == 0 ? c.Lst : c.Rst) + off;
+      unsigned long long* D = sp.dq(s, q);
+      for (long e = e0; e < (long)N * n; e += stride) {
+        const int k = (int)(e / N), i = (int)(e % N);
+        const double v = Q[e];
+        bad |= digit_exp(v) > 1;
+        D[(long)k * ldd + i] = digit_pack(v, 1);
+      }
+    }
+    if (bad) atomicMax(sp.eq() + s, kDigitBad);
+  }
+}
+
+// One 32 x 32 block of the Gram matrix (b < 0, upper triangle) or of O per CTA
+// (digit_gemm.cuh; 648 x 324: 36 MMAs per 16-deep step on 8 warps, against the FP64
+// pipe's 74% in a tiled FMA product).
+__global__ void __launch_bounds__(256) sp_digit_gemm_kernel(const ChainDesc* chains, int b, int tsize) {
+  const ChainDesc& c = chains[blockIdx.z];
+  if (c.st->err) return;
+  const int s = blockIdx.y, n = nsig_of(c, s), N = c.N, ldd = digit_ld(N), ldn = c.nmax;
+  const int tn = (c.nmax + 31) >> 5;
+  const int i0 = 32 * (int)(blockIdx.x / tn), j0 = 32 * (int)(blockIdx.x % tn);
+  if (i0 >= n || j0 >= n || (b < 0 && i0 > j0)) return;
+  SpBuf<double> sp = fp64_bufs(c, tsize);
+  const unsigned long long* A = sp.dq(s, 0) + (long)i0 * ldd;
+  const unsigned long long* B = sp.dq(s, b < 0 ? 0 : 1) + (long)j0 * ldd;
+  double* C = (b < 0 ? sp.c64(s) : sp.o64(s)) + (long)i0 * ldn + j0;
+  const int bad = b < 0 ? 0 : sp.eq()[s];
+  const int E = b < 0 ? sp.em()[s] : bad > 0 ? bad : 1;
+  auto ex = [E](int) { return E; };
+  digit_gemm<true, true>(min(32, n - i0), min(32, n - j0), N, A, ldd, 1, B, ldd, 1, ex, ex, false, false,
+                         [C, ldn](int i, int j, double v) { C[(long)i * ldn + j] = v; });
+}
+
+// Cholesky factor, diagonal block of panel p (one CTA per spin, chain), and its
+// inverse, by the elimination of [C | I] in shared memory (chol_eliminate):
+// step k takes row k, u_j = row_kj / p_k, from the rows below; right of the
+// diagonal stay the Schur complements (R_kj = C_kj / sqrt(p_k)), left of it the
+// rows of L^{-1} (R_PP^{-1} = L^{-T} diag(p)^{-1/2}).  Warp 0 runs one step ahead (row
+// k + 1, its pivot and reciprocal), so a column costs one barrier and the
+// reciprocal's latency passes beside the other rows' FMAs; factor and
+// back substitution as two chains of 32 steps took 42.6 us.  Panel 0 first
+// records the Gram diagonal and clears the chain's breakdown flag and log det R.
 __global__ void __launch_bounds__(256) chol_panel_kernel(const ChainDesc* chains, int p, int tsize) {
-  __shared__ double A[kSpPanel][kSpPanel + 1];    // Schur complements
-  __shared__ double R[kSpPanel][kSpPanel + 1];    // the factor's rows
-  __shared__ double X[1][kSpPanel][kSpPanel + 1]; // inverse, rows in progress
-  __shared__ double Xf[kSpPanel][kSpPanel + 1];   // its final rows
-  __shared__ double ikk[kSpPanel];
+  __shared__ double A[kSpPanel][kSpPanel + 1];
+  __shared__ double u[2][kSpPanel];
+  __shared__ double pv[kSpPanel], isq[kSpPanel], dlim[kSpPanel];
   __shared__ int bad;
   const ChainDesc& c = chains[blockIdx.y];
   if (c.st->err) return;
@@ -38,36 +97,41 @@ __global__ void __launch_bounds__(256) chol_panel_kernel(const ChainDesc* chains
     if (threadIdx.x == 0) {
       sp.bad()[s] = 0;
       sp.lchol()[s] = 0.0;
+      sp.em()[s] = kDigitNone;          // (the block's digits have been used: ready for the next block)
     }
   }
-  __shared__ double dlim[kSpPanel];
   __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int e = threadIdx.x; e < kSpPanel * kSpPanel; e += blockDim.x) {
     const int i = e / kSpPanel, j = e % kSpPanel;
-    A[i][j] = (i < bw && j < bw) ? C[(long)(p0 + i) * ldn + p0 + j] : 0.0;
-    R[i][j] = 0.0;
+    A[i][j] = (i < bw && j < bw && j >= i) ? C[(long)(p0 + i) * ldn + p0 + j] : 0.0;
   }
   if ((int)threadIdx.x < bw) dlim[threadIdx.x] = 1e-12 * d0[p0 + threadIdx.x];
   if (threadIdx.x == 0) bad = 0;
   __syncthreads();
-  // upper-triangle pairs (i, j), i <= j, of the trailing block, enumerated so
-  // that every FP64 instruction carries a full warp (the FP64 unit takes as
-  // long for a partial warp)
-  for (int k = 0; k < bw; ++k) {
-    const double piv = A[k][k];
-    if (!(piv > dlim[k])) {   // the same value in every thread: uniform exit
-      if (threadIdx.x == 0) bad = 1;
-      break;
+  auto pivot_row = [&](int r) {
+    const double piv = A[r][r];
+    // (positive doubles order like their bits)
+    const long long pb = __double_as_longlong(piv);
+    const bool ok = pb > __double_as_longlong(dlim[r]) && pb < 0x7ff0000000000000ll;
+    const double ip = ok ? recip64(piv) : 0.0;
+    if (lane == 0) {
+      pv[r] = piv;
+      if (!ok) bad = 1;
     }
-    const double ir = rsqrt(piv);
-    if ((int)threadIdx.x >= k && (int)threadIdx.x < bw) R[k][threadIdx.x] = threadIdx.x == k ? piv * ir : A[k][threadIdx.x] * ir;
-    __syncthreads();
-    const int m = bw - k - 1;
-    for (int e = threadIdx.x; e < m * (m + 1) / 2; e += blockDim.x) {
-      int i = 0, r = e;
-      while (r >= m - i) { r -= m - i; ++i; }
-      const int ii = k + 1 + i, jj = ii + r;
-      A[ii][jj] = fma(-R[k][ii], R[k][jj], A[ii][jj]);
+    u[r & 1][lane] = lane == r ? ip : A[r][lane] * ip;
+  };
+  if (warp == 0) pivot_row(0);
+  __syncthreads();
+  for (int k = 0; k + 1 < bw && !bad; ++k) {
+    const double uk = u[k & 1][lane];
+    if (warp == 0) {
+      const int r = k + 1;
+      A[r][lane] = fma(-A[k][r], uk, lane == k ? 0.0 : A[r][lane]);
+      __syncwarp();
+      pivot_row(r);
+    } else {
+      for (int i = k + 1 + warp; i < bw; i += 7) A[i][lane] = fma(-A[k][i], uk, lane == k ? 0.0 : A[i][lane]);
     }
     __syncthreads();
   }
@@ -76,39 +140,20 @@ __global__ void __launch_bounds__(256) chol_panel_kernel(const ChainDesc* chains
     if (threadIdx.x == 0) sp.bad()[s] = 1;
     return;
   }
-  for (int e = threadIdx.x; e < bw * bw; e += blockDim.x) {
-    const int i = e / bw, j = e % bw;
-    if (i <= j) C[(long)(p0 + i) * ldn + p0 + j] = R[i][j];
-  }
+  if ((int)threadIdx.x < bw) isq[threadIdx.x] = rsqrt(pv[threadIdx.x]);
   if (threadIdx.x < 32) {
     // log det R_PP: one logarithm per lane, summed over the warp
-    double la = (int)threadIdx.x < bw ? log(R[threadIdx.x][threadIdx.x]) : 0.0;
+    double la = (int)threadIdx.x < bw ? log(pv[threadIdx.x]) : 0.0;
     la = warp_sum(la);
-    if (threadIdx.x == 0) sp.lchol()[s] += la;
+    if (threadIdx.x == 0) sp.lchol()[s] += 0.5 * la;
   }
-  // X = R_PP^{-1} by back substitution on the identity: for k = bw-1 .. 0,
-  // row k of X is final once scaled by 1 / R_kk (kept in Xf), then the rows
-  // i < k take away R_ik times it (one FP64 instruction per element)
-  for (int e = threadIdx.x; e < kSpPanel * kSpPanel; e += blockDim.x) {
-    const int i = e / kSpPanel, j = e % kSpPanel;
-    X[0][i][j] = (i == j && i < bw) ? 1.0 : 0.0;
-    Xf[i][j] = 0.0;
-  }
-  if ((int)threadIdx.x < bw) ikk[threadIdx.x] = 1.0 / R[threadIdx.x][threadIdx.x];
   __syncthreads();
-  for (int k = bw - 1; k >= 0; --k) {
-    if ((int)threadIdx.x < bw) Xf[k][threadIdx.x] = X[0][k][threadIdx.x] * ikk[k];
-    __syncthreads();
-    for (int e = threadIdx.x; e < k * bw; e += blockDim.x) {
-      const int i = e / bw, j = e % bw;
-      X[0][i][j] = fma(-R[i][k], Xf[k][j], X[0][i][j]);
-    }
-    __syncthreads();
-  }
   double* Ri = sp.rinv(s) + (long)p * kSpPanel * kSpPanel;
   for (int e = threadIdx.x; e < kSpPanel * kSpPanel; e += blockDim.x) {
     const int i = e / kSpPanel, j = e % kSpPanel;
-    Ri[e] = (i < bw && j < bw) ? Xf[i][j] : 0.0;
+    const bool in = i < bw && j < bw;
+    if (in && i <= j) C[(long)(p0 + i) * ldn + p0 + j] = i == j ? pv[i] * isq[i] : A[i][j] * isq[i];
+    Ri[e] = !in || i > j ? 0.0 : i == j ? isq[i] : A[j][i] * isq[j];
   }
 }
 
@@ -161,161 +206,165 @@ __global__ void __launch_bounds__(256) qform_kernel(const ChainDesc* chains, int
   }
 }
 
-// Gauss-Jordan panel p (columns P = [p0, p1)) of O, one CTA per spin, chain:
-// for each column j of P the largest |O_ij|, i >= j (ties to the lower row),
-// the interchange of rows j and i, then the elimination of column j
+// Gauss-Jordan panel p (columns P = [p0, p1)) of O, one cluster of kGJRanks CTAs
+// per spin and chain: for each column j of P the largest |O_ij| over the rows
+// not used yet (ties to the lower row), then the elimination of column j
 // restricted to the panel's columns (the rest of the row operations is the
-// block update that follows, from the block row saved at the end).  The
-// panel stays in shared memory for all its steps, each thread owning one
-// panel column on every 16th row (one FP64 FMA per eliminated element); the
-// pass that eliminates column j also hands on column j + 1 and its pivot
-// candidates, so a step takes two CTA barriers.  The interchanges reach the
-// other columns once, in order, at the end.
-constexpr int kGJLd = kSpGJ + 1;
-constexpr int kGJThreads = 512;
-constexpr int kGJRowStep = kGJThreads / kSpGJ;
-static_assert(kGJThreads % kSpGJ == 0 && kSpGJ <= 32, "each thread owns one panel column");
-size_t gj_panel_smem(int nmax) { return (size_t)nmax * kGJLd * 8; }
+// block update that follows, from the block row saved at the end).  The rows
+// are dealt out to the cluster's CTAs and stay in their shared memory; a step
+// costs one cluster barrier: every CTA hands its best candidate, the whole
+// panel row, to all eight (distributed shared memory), and each takes the
+// best of the eight and eliminates its own rows.  (One CTA per spin had n x 16
+// FP64 FMAs per column on one SM and two barriers with a division between
+// them: 71.7 us per panel at n = 324.)  Rows are interchanged once, at the end: the
+// panel's interchanges composed into one permutation of at most 2 bw rows
+// (place rows[e] takes row src[e]), applied to the panel as it is written back
+// and to the other columns, which the CTAs share.
+constexpr int kGJRanks = 8;
+constexpr int kGJRows = kMaxSigma / kGJRanks;     // rows per CTA
+static_assert(kMaxSigma % kGJRanks == 0 && kGJRows == 4 * 16 && kSpGJ == 16, "four rows per thread and column");
+struct GJCand {
+  unsigned long long best;
+  int row, pad;
+  double v[kSpGJ];
+};
 
-__global__ void __launch_bounds__(kGJThreads) gj_panel_kernel(const ChainDesc* chains, int p, int tsize) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  double (*Ap)[kGJLd] = reinterpret_cast<double (*)[kGJLd]>(smem_raw);   // n x bw panel
-  __shared__ double fbuf[2][kMaxSigma];   // column j of the panel before step j (two steps in flight)
-  __shared__ double prow[kSpGJ];          // pivot row of the step, after the interchange
-  __shared__ double ips;
-  __shared__ unsigned long long wbest[kGJThreads / 32];
-  __shared__ int wbi[kGJThreads / 32];
-  __shared__ int piv[kSpGJ];
+__global__ void __cluster_dims__(kGJRanks, 1, 1) __launch_bounds__(256)
+    gj_panel_kernel(const ChainDesc* chains, int p, int tsize) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  __shared__ double Ap[kGJRows][kSpGJ + 1];
+  __shared__ GJCand cand[2][kGJRanks];              // two steps in flight
+  __shared__ int used[kGJRows], place[kGJRows], pivrow[kSpGJ];
+  __shared__ int rows[2 * kSpGJ], src[2 * kSpGJ], nrows;
   const ChainDesc& c = chains[blockIdx.y];
-  if (c.st->err) return;
-  const int s = blockIdx.x, n = nsig_of(c, s), ldn = c.nmax;
+  if (c.st->err) return;                            // (the whole cluster)
+  const int s = blockIdx.x / kGJRanks, rank = blockIdx.x % kGJRanks, n = nsig_of(c, s), ldn = c.nmax;
   const int p0 = p * kSpGJ;
   if (p0 >= n) return;
   const int p1 = min(p0 + kSpGJ, n), bw = p1 - p0;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int col = threadIdx.x % kSpGJ, row0 = threadIdx.x / kSpGJ;
+  const int col = threadIdx.x % kSpGJ, r0 = threadIdx.x / kSpGJ;
+  const int nl = rank < n ? (n - rank + kGJRanks - 1) / kGJRanks : 0;   // local row l: rank + 8 l
   SpBuf<double> sp = fp64_bufs(c, tsize);
   double* A = sp.o64(s);
-  // load; the owners of column 0 hand it on with its pivot candidates
-  unsigned long long best = 0;
-  int bi = p0;
-  for (int i = row0; i < n; i += kGJRowStep) {
-    if (col < bw) {
-      const double v = A[(long)i * ldn + p0 + col];
-      Ap[i][col] = v;
-      if (col == 0) {
-        fbuf[0][i] = v;
-        const unsigned long long av = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
-        if (i >= p0 && av > best) { best = av; bi = i; }
-      }
-    }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int l = r0 + 16 * q;
+    if (l < nl) Ap[l][col] = col < bw ? A[(long)(rank + kGJRanks * l) * ldn + p0 + col] : 0.0;
   }
+  for (int l = threadIdx.x; l < kGJRows; l += blockDim.x) {
+    used[l] = rank + kGJRanks * l < p0 ? 1 : 0;     // rows before the panel are pivot rows already
+    place[l] = rank + kGJRanks * l;
+  }
+  cl.sync();                                        // every CTA of the cluster runs before its memory is written
   for (int jj = 0; jj < bw; ++jj) {
     const int j = p0 + jj;
-    double* f = fbuf[jj & 1];
-    double* fnext = fbuf[(jj + 1) & 1];
-    // candidates of column j: per warp, then warp 0 over the warps
+    GJCand* cd = cand[jj & 1];
+    if (warp == 0) {
+      // this CTA's candidate, handed to every CTA
+      unsigned long long best = 0;
+      int bl = -1;
+      for (int l = lane; l < nl; l += 32) {
+        const unsigned long long v = (unsigned long long)__double_as_longlong(Ap[l][jj]) & 0x7fffffffffffffffull;
+        if (!used[l] && (bl < 0 || v > best)) { best = v; bl = l; }
+      }
+      const unsigned hi = __reduce_max_sync(0xffffffffu, bl < 0 ? 0u : (unsigned)(best >> 32));
+      const unsigned lo = __reduce_max_sync(0xffffffffu, bl >= 0 && (unsigned)(best >> 32) == hi ? (unsigned)best : 0u);
+      const bool mine = bl >= 0 && (unsigned)(best >> 32) == hi && (unsigned)best == lo;
+      const unsigned l = __reduce_min_sync(0xffffffffu, mine ? (unsigned)bl : 0xffffffffu);   // ties to the lower row
+      const bool any = l != 0xffffffffu;
+      for (int t = 0; t < kGJRanks; ++t) {
+        GJCand* to = cl.map_shared_rank(&cd[rank], t);
+        if (lane < kSpGJ) to->v[lane] = any ? Ap[l][lane] : 0.0;
+        if (lane == 16) to->best = any ? ((unsigned long long)hi << 32) | lo : 0ull;
+        if (lane == 17) to->row = any ? rank + kGJRanks * (int)l : 0x7fffffff;
+      }
+    }
+    cl.sync();
+    // the best of the eight, ties to the lower row
+    int b = 0;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const unsigned long long ob = __shfl_xor_sync(0xffffffffu, best, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-    }
-    if (lane == 0) { wbest[warp] = best; wbi[warp] = bi; }
-    __syncthreads();
-    if (threadIdx.x < 32) {
-      unsigned long long bb = 0;
-      int ii = j;
-      if (lane < kGJThreads / 32) { bb = wbest[lane]; ii = wbi[lane]; }
+    for (int t = 1; t < kGJRanks; ++t)
+      if (cd[t].row != 0x7fffffff &&
+          (cd[b].row == 0x7fffffff || cd[t].best > cd[b].best || (cd[t].best == cd[b].best && cd[t].row < cd[b].row)))
+        b = t;
+    const int r = cd[b].row;
+    const double pvt = cd[b].v[jj];
+    const double ip = pvt != 0.0 ? recip64(pvt) : 0.0;
+    const double x = col == jj ? ip : cd[b].v[col] * ip;
+    // eliminate column j: v = add - f_i x, one FP64 instruction per element
+    double f[4], v[4];
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long ob = __shfl_xor_sync(0xffffffffu, bb, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, ii, o);
-        if (ob > bb || (ob == bb && oi < ii)) { bb = ob; ii = oi; }
-      }
-      if (ii != j) {
-        if (lane < bw) {
-          const double t = Ap[j][lane];
-          Ap[j][lane] = Ap[ii][lane];
-          Ap[ii][lane] = t;
-        }
-        if (lane == 0) {
-          const double t = f[j];
-          f[j] = f[ii];
-          f[ii] = t;
-        }
-      }
-      __syncwarp();
-      if (lane < bw) prow[lane] = Ap[j][lane];
-      if (lane == 0) {
-        const double pv = Ap[j][jj];
-        ips = pv != 0.0 ? 1.0 / pv : 0.0;
-        piv[jj] = ii;
-        sp.perm(s)[j] = ii;
-        sp.pval(s)[j] = pv;
-        if (pv == 0.0) sp.bad()[s] = 1;
+    for (int q = 0; q < 4; ++q) {
+      const int l = r0 + 16 * q;
+      if (l < nl) {
+        f[q] = Ap[l][jj];
+        v[q] = col == jj ? 0.0 : Ap[l][col];
       }
     }
     __syncthreads();
-    // eliminate column j from the panel; the owners of column j + 1 hand it on
-    const double ip = ips;
-    best = 0;
-    bi = j + 1;
-    if (col < bw) {
-      // one FP64 instruction per element: v = add - f_i x with (x, add) =
-      // (1 / pivot, 0) on the pivot column, (pivot row / pivot, O_ic) elsewhere
-      const bool pc = col == jj;
-      const double x = pc ? ip : prow[col] * ip;
-      for (int i = row0; i < n; i += kGJRowStep) {
-        const double add = pc ? 0.0 : Ap[i][col];
-        const double v = i == j ? x : fma(-f[i], x, add);
-        Ap[i][col] = v;
-        if (col == jj + 1) {
-          fnext[i] = v;
-          const unsigned long long av = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
-          if (i > j && av > best) { best = av; bi = i; }
-        }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int l = r0 + 16 * q;
+      if (l < nl) Ap[l][col] = rank + kGJRanks * l == r ? x : fma(-f[q], x, v[q]);
+    }
+    if (threadIdx.x == 0) {
+      pivrow[jj] = r;
+      if (r % kGJRanks == rank) used[r / kGJRanks] = 1;
+      if (rank == 0) {
+        sp.pval(s)[j] = pvt;
+        if (pvt == 0.0) sp.bad()[s] = 1;
       }
     }
+    __syncthreads();
   }
-  __syncthreads();
-  for (int e = threadIdx.x; e < n * bw; e += blockDim.x) A[(long)(e / bw) * ldn + p0 + e % bw] = Ap[e / bw][e % bw];
-  // the panel back; the other columns take the panel's interchanges composed
-  // into one permutation of at most 2 bw rows (new row rows[e] = old row
-  // src[e]), read once and written once, and the block row of the update
-  __shared__ int rows[2 * kSpGJ], src[2 * kSpGJ], nrows;
-  if (threadIdx.x == 0) {
-    int m = 0;
-    for (int jj = 0; jj < bw; ++jj) { rows[m] = p0 + jj; src[m] = p0 + jj; ++m; }
+  // the interchanges: entry e (lane e) is place rows[e] and the row it takes
+  if (warp == 0) {
+    int pl = lane < bw ? p0 + lane : -1, id = pl, m = bw;
     for (int jj = 0; jj < bw; ++jj) {
-      const int j = p0 + jj, r = piv[jj];
-      if (r == j) continue;
-      int ej = -1, er = -1;
-      for (int e = 0; e < m; ++e) {
-        if (rows[e] == j) ej = e;
-        if (rows[e] == r) er = e;
+      const int r = pivrow[jj];
+      const unsigned at = __ballot_sync(0xffffffffu, lane < m && id == r);
+      const int other = __shfl_sync(0xffffffffu, id, jj);          // the row now at place p0 + jj
+      int e = __ffs((int)at) - 1;
+      if (at == 0) {                                               // row r is still at place r
+        e = m++;
+        if (lane == e) { pl = r; id = r; }
       }
-      if (er < 0) { rows[m] = r; src[m] = r; er = m++; }
-      const int t = src[ej];
-      src[ej] = src[er];
-      src[er] = t;
+      const int pr = __shfl_sync(0xffffffffu, pl, e);
+      if (e != jj) {
+        if (lane == e) id = other;
+        if (lane == jj) id = r;
+      }
+      if (rank == 0 && lane == 0) sp.perm(s)[p0 + jj] = pr;
     }
-    nrows = m;
+    if (lane < m) {
+      rows[lane] = pl;
+      src[lane] = id;
+      if (id % kGJRanks == rank) place[id / kGJRanks] = pl;
+    }
+    if (lane == 0) nrows = m;
   }
   __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int l = r0 + 16 * q;
+    if (l < nl && col < bw) A[(long)place[l] * ldn + p0 + col] = Ap[l][col];
+  }
+  // the other columns, and the block row of the update (rows[e] = p0 + e for e < bw)
   const int m = nrows;
   double* Tb = sp.tgj(s);
-  for (int col = threadIdx.x; col < n; col += blockDim.x) {
-    if (col >= p0 && col < p1) continue;
+  for (int cc = rank * 64 + (int)threadIdx.x; cc < n && threadIdx.x < 64; cc += 64 * kGJRanks) {
+    if (cc >= p0 && cc < p1) continue;
     double v[2 * kSpGJ];
 #pragma unroll
     for (int e = 0; e < 2 * kSpGJ; ++e)
-      if (e < m) v[e] = A[(long)src[e] * ldn + col];
+      if (e < m) v[e] = A[(long)src[e] * ldn + cc];
 #pragma unroll
     for (int e = 0; e < 2 * kSpGJ; ++e)
       if (e < m) {
-        A[(long)rows[e] * ldn + col] = v[e];
-        if (e < bw) Tb[(long)e * ldn + col] = v[e];   // rows[e] = p0 + e for e < bw
+        A[(long)rows[e] * ldn + cc] = v[e];
+        if (e < bw) Tb[(long)e * ldn + cc] = v[e];
       }
   }
 }
@@ -346,6 +395,15 @@ cudaError_t sp_dgemm(SpGemm& g, int mode, int max_m, int max_n, cudaStream_t st)
   return sp_gemm_t<double>(g, mode, max_m, max_n, st);
 }
 
+cudaError_t sp_digit_products(const ChainDesc* d, int nc, int N, int nmax, int b, int tsize, cudaStream_t st) {
+  const int t = (nmax + 31) / 32;
+  sp_digits_kernel<<<dim3((unsigned)std::min(512, (N * nmax + 255) / 256), 2, nc), 256, 0, st>>>(d, b, tsize);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  sp_digit_gemm_kernel<<<dim3(t * t, 2, nc), 256, 0, st>>>(d, b, tsize);
+  return cudaGetLastError();
+}
+
 cudaError_t sp_chol_panel(const ChainDesc* d, int nc, int nmax, int p, int tsize, cudaStream_t st) {
   (void)nmax;
   chol_panel_kernel<<<dim3(2, nc), 256, 0, st>>>(d, p, tsize);
@@ -359,14 +417,12 @@ cudaError_t sp_qform(const ChainDesc* d, int nc, int N, int nmax, int left, int 
 }
 
 cudaError_t sp_gj_panel(const ChainDesc* d, int nc, int nmax, int p, int tsize, cudaStream_t st) {
-  gj_panel_kernel<<<dim3(2, nc), kGJThreads, gj_panel_smem(nmax), st>>>(d, p, tsize);
+  (void)nmax;
+  gj_panel_kernel<<<dim3(2 * kGJRanks, nc), 256, 0, st>>>(d, p, tsize);
   return cudaGetLastError();
 }
 
-cudaError_t spread_prepare() {
-  return cudaFuncSetAttribute(gj_panel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)gj_panel_smem(kMaxSigma));
-}
+cudaError_t spread_prepare() { return cudaSuccess; }
 
 cudaError_t sp_gj_unswap(const ChainDesc* d, int nc, int nmax, int tsize, cudaStream_t st) {
   gj_unswap_kernel<<<dim3((nmax + 127) / 128, 2, nc), 128, 0, st>>>(d, tsize);

@@ -94,11 +94,7 @@ static __device__ double cta_max(double v, double* red) {
 // on load; the epilogue receives (i, j, value).  Every thread owns 4x4
 // outputs.  When A is contiguous in i and B in j (sai = sbj = 1, strides and
 // pointers 16-byte aligned, same type as T) the operands are read with
-// 16-byte vector loads.  pad: the caller's rows of A and B can be read up to
-// the next multiple of four elements, whatever they hold there, so that sizes
-// that are no multiple of four take the vector loads too (162 sites: rank-21
-// update, stack products and assembly 29 + 22 + 24 Mcycles per 42 slices with
-// scalar loads and a bounds check per element).
+// 16-byte vector loads.
 
 struct EpiStore {
   static constexpr bool kRow4 = true;   // supports 4 contiguous outputs of a row at once
@@ -143,18 +139,18 @@ __device__ __forceinline__ bool vec_ok(const T* p, long stride) {
 
 template <typename T, typename TA, typename TB, typename TC, typename Epi>
 __device__ void cta_gemm(int M, int Nn, int K, const TA* A, int sai, int sak, const TB* B, int sbk, int sbj,
-                         TC* C, int sci, int scj, Epi epi, bool pad = false) {
+                         TC* C, int sci, int scj, Epi epi) {
   const int tm = (M + 3) >> 2, tn = (Nn + 3) >> 2;
   bool vec = false, vec_row = false, st_row = false;
   if constexpr (std::is_same<T, TA>::value && std::is_same<T, TB>::value) {
     vec = sai == 1 && sbj == 1 && vec_ok<T>((const T*)A, sak) && vec_ok<T>((const T*)B, sbk) &&
-          (pad || ((M % 4 == 0) && (Nn % 4 == 0)));
+          (M % 4 == 0) && (Nn % 4 == 0);
     // A contiguous along k (row-major): 4 x 4 blocks of A per four k-steps
     vec_row = !vec && sak == 1 && sbj == 1 && vec_ok<T>((const T*)A, sai) && vec_ok<T>((const T*)B, sbk) &&
-              (pad || (Nn % 4 == 0));
+              (M % 4 == 0) && (Nn % 4 == 0) && (K % 4 == 0);
   }
   if constexpr (std::is_same<T, TC>::value && HasRow4<Epi>::value) {
-    st_row = scj == 1 && vec_ok<T>((const T*)C, sci);
+    st_row = scj == 1 && vec_ok<T>((const T*)C, sci) && (Nn % 4 == 0);
   }
   for (int t = threadIdx.x; t < tm * tn; t += blockDim.x) {
     const int i0 = (t / tn) << 2, j0 = (t % tn) << 2;
@@ -181,15 +177,12 @@ __device__ void cta_gemm(int M, int Nn, int K, const TA* A, int sai, int sak, co
     }
     if constexpr (std::is_same<T, TA>::value && std::is_same<T, TB>::value) {
       if (vec_row) {
-        const T* pa[4];
-#pragma unroll
-        for (int r = 0; r < 4; ++r) pa[r] = (const T*)A + (long)min(i0 + r, M - 1) * sai;
+        const T* pa = (const T*)A + (long)i0 * sai;
         const T* pb = (const T*)B + j0;
-        int k = 0;
-        for (; k + 4 <= K; k += 4) {
+        for (int k = 0; k < K; k += 4) {
           T a[4][4], b[4][4];
 #pragma unroll
-          for (int r = 0; r < 4; ++r) Vec4<T>::load(pa[r] + k, a[r]);
+          for (int r = 0; r < 4; ++r) Vec4<T>::load(pa + (long)r * sai + k, a[r]);
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk) Vec4<T>::load(pb + (long)(k + kk) * sbk, b[kk]);
 #pragma unroll
@@ -198,16 +191,6 @@ __device__ void cta_gemm(int M, int Nn, int K, const TA* A, int sai, int sak, co
             for (int r = 0; r < 4; ++r)
 #pragma unroll
               for (int q = 0; q < 4; ++q) acc[r][q] = fma(a[r][kk], b[kk][q], acc[r][q]);
-        }
-        for (; k < K; ++k) {
-          T b[4];
-          Vec4<T>::load(pb + (long)k * sbk, b);
-#pragma unroll
-          for (int r = 0; r < 4; ++r) {
-            const T ar = pa[r][k];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) acc[r][q] = fma(ar, b[q], acc[r][q]);
-          }
         }
       }
     }
@@ -225,7 +208,7 @@ __device__ void cta_gemm(int M, int Nn, int K, const TA* A, int sai, int sak, co
       }
     }
     if constexpr (std::is_same<T, TC>::value && HasRow4<Epi>::value) {
-      if (st_row && j0 + 4 <= Nn) {
+      if (st_row) {
 #pragma unroll
         for (int r = 0; r < 4; ++r)
           if (i0 + r < M) epi.row4((T*)C + (long)(i0 + r) * sci + j0, acc[r]);
@@ -237,6 +220,90 @@ __device__ void cta_gemm(int M, int Nn, int K, const TA* A, int sai, int sak, co
 #pragma unroll
       for (int q = 0; q < 4; ++q)
         if (i0 + r < M && j0 + q < Nn) epi(C, sci, scj, i0 + r, j0 + q, acc[r][q]);
+  }
+}
+
+// The same in FP32 for operands laid out in whole vectors, which is how the
+// reduced paths keep theirs: A(i,k) = A[i + k lda], or with kRowA A[i lda + k];
+// B(k,j) = B[k ldb + j], C row-major; lda, ldb, ldc multiples of four, bases
+// 16-byte aligned, and rows of A and B readable up to the next multiple of
+// four elements (whatever they hold there).  One layout per instantiation:
+// no fallback to scalar loads inside, so the loop keeps its registers and the
+// phase its code small.  (162 sites: rank-21 update, stack products and
+// assembly took 29 + 22 + 24 Mcycles per 42 slices with scalar loads and a
+// bounds check per element; 288 sites: a single function choosing at run
+// time took 74 for the wrap, this one %s.)
+template <bool kRowA, typename Epi>
+__device__ __forceinline__ void cta_gemm_f32(int M, int Nn, int K, const float* A, int lda, const float* B, int ldb,
+                                             float* C, int ldc, Epi epi) {
+  const int tm = (M + 3) >> 2, tn = (Nn + 3) >> 2;
+  for (int t = threadIdx.x; t < tm * tn; t += blockDim.x) {
+    const int i0 = (t / tn) << 2, j0 = (t % tn) << 2;
+    float acc[4][4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[r][q] = 0.f;
+    const float* pb = B + j0;
+    if constexpr (!kRowA) {
+      const float* pa = A + i0;
+#pragma unroll 4
+      for (int k = 0; k < K; ++k) {
+        float a[4], b[4];
+        Vec4<float>::load(pa + (long)k * lda, a);
+        Vec4<float>::load(pb + (long)k * ldb, b);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) acc[r][q] = fma(a[r], b[q], acc[r][q]);
+      }
+    } else {
+      // 4 x 4 blocks of A per four k-steps (the last rows of a ragged M are read again)
+      const int l1 = min(1, M - 1 - i0) * lda, l2 = min(2, M - 1 - i0) * lda, l3 = min(3, M - 1 - i0) * lda;
+      const float* pa = A + (long)i0 * lda;
+      int k = 0;
+      for (; k + 4 <= K; k += 4) {
+        float a[4][4], b[4][4];
+        Vec4<float>::load(pa + k, a[0]);
+        Vec4<float>::load(pa + l1 + k, a[1]);
+        Vec4<float>::load(pa + l2 + k, a[2]);
+        Vec4<float>::load(pa + l3 + k, a[3]);
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) Vec4<float>::load(pb + (long)(k + kk) * ldb, b[kk]);
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk)
+#pragma unroll
+          for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[r][q] = fma(a[r][kk], b[kk][q], acc[r][q]);
+      }
+#pragma unroll 1
+      for (; k < K; ++k) {
+        float a[4], b[4];
+        a[0] = pa[k];
+        a[1] = pa[l1 + k];
+        a[2] = pa[l2 + k];
+        a[3] = pa[l3 + k];
+        Vec4<float>::load(pb + (long)k * ldb, b);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) acc[r][q] = fma(a[r], b[q], acc[r][q]);
+      }
+    }
+    if constexpr (HasRow4<Epi>::value) {
+      if (j0 + 4 <= Nn) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+          if (i0 + r < M) epi.row4(C + (long)(i0 + r) * ldc + j0, acc[r]);
+        continue;
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (i0 + r < M && j0 + q < Nn) epi(C, ldc, 1, i0 + r, j0 + q, acc[r][q]);
   }
 }
 
@@ -492,10 +559,12 @@ __device__ __forceinline__ Cta<T, RES> this_cta() {
 // writing G: it runs in FP32 on the CUDA cores on the BF16X3 path too
 // (measured faster than either tensor-core form at 162-648 sites, and exact
 // to FP32).  FP32 and FP64 paths: CUDA-core FMA.
-template <bool kTc, typename T, bool RES, typename Epi>
-__device__ __forceinline__ void wrap_gemm(Cta<T, RES>& x, int n, const T* A, int sai, int sak, const T* B, T* C, int ld,
-                                          Epi epi) {
-  if constexpr (std::is_same<T, float>::value) {
+// kRowA: A is row-major (ld ld), else A(i, k) = A[i + k ld].
+template <bool kTc, bool kRowA, typename T, bool RES, typename Epi>
+__device__ __forceinline__ void wrap_gemm(Cta<T, RES>& x, int n, const T* A, const T* B, T* C, int ld, Epi epi) {
+  constexpr bool f32 = std::is_same<T, float>::value;
+  const int sai = kRowA ? ld : 1, sak = kRowA ? 1 : ld;
+  if constexpr (f32) {
     if (x.c.tc) {
       if constexpr (kTc && !RES) {
         if (x.sh.tcs_off) {
@@ -507,8 +576,10 @@ __device__ __forceinline__ void wrap_gemm(Cta<T, RES>& x, int n, const T* A, int
       cta_gemm_bf16x3(n, n, n, A, sai, sak, B, ld, 1, C, ld, 1, epi);
       return;
     }
+    cta_gemm_f32<kRowA>(n, n, n, A, ld, B, ld, C, ld, epi);
+  } else {
+    cta_gemm<T>(n, n, n, A, sai, sak, B, ld, 1, C, ld, 1, epi);
   }
-  cta_gemm<T>(n, n, n, A, sai, sak, B, ld, 1, C, ld, 1, epi, !std::is_same<T, double>::value);
 }
 
 // --------------------------------------------------------------------------
@@ -640,7 +711,8 @@ __device__ __forceinline__ void flush_block(Cta<T, RES>& x, int a, bool pivot) {
     __syncthreads();
     cta_gemm<T>(a, N, a, &fb.Tu[s][0][0], kBlock + 1, 1, Wbuf, ld, 1, MW, ld, 1, EpiStore());
     __syncthreads();
-    cta_gemm<T>(N, N, a, Ubuf, 1, ldu, MW, ld, 1, Gs, ld, 1, EpiSub(), !std::is_same<T, double>::value);
+    if constexpr (std::is_same<T, double>::value) cta_gemm<T>(N, N, a, Ubuf, 1, ldu, MW, ld, 1, Gs, ld, 1, EpiSub());
+    else cta_gemm_f32<false>(N, N, a, Ubuf, ldu, MW, ld, Gs, ld, EpiSub());
     __syncthreads();
   }
   x.mark(kPhFlush);
@@ -867,8 +939,7 @@ __device__ __forceinline__ void apply_vectors(Cta<T, RES>& x, int a) {
                                false, [G, ld](int i, int j, double v) { G[(long)i * ld + j] -= v; });
     }
   } else {
-    for (int sp = 0; sp < 2; ++sp)
-      cta_gemm<T>(N, N, a, x.Uv(sp), 1, x.ldu(), x.Vv(sp), ld, 1, x.G(sp), ld, 1, EpiSub(), true);
+    for (int sp = 0; sp < 2; ++sp) cta_gemm_f32<false>(N, N, a, x.Uv(sp), ld, x.Vv(sp), ld, x.G(sp), ld, EpiSub());
   }
   __syncthreads();
   x.mark(kPhFlush);
@@ -1403,17 +1474,17 @@ __device__ __forceinline__ void wrap(Cta<T, RES>& x, int tau, int dir) {
     if (gz) return;
     // Gt = e^{-dtau K} G, G = Gt e^{+dtau K}
     for (int s = 0; s < x.nspec(); ++s) {
-      wrap_gemm<kTc>(x, N, Em, 1, ld, x.G(s), Gt, ld, EpiStore());
+      wrap_gemm<kTc, false>(x, N, Em, x.G(s), Gt, ld, EpiStore());
       __syncthreads();
-      wrap_gemm<kTc>(x, N, Gt, ld, 1, Ep, x.G(s), ld, EpiStore());
+      wrap_gemm<kTc, true>(x, N, Gt, Ep, x.G(s), ld, EpiStore());
       __syncthreads();
     }
   } else {
     if (!gz) {
       for (int s = 0; s < x.nspec(); ++s) {
-        wrap_gemm<kTc>(x, N, Ep, 1, ld, x.G(s), Gt, ld, EpiStore());
+        wrap_gemm<kTc, false>(x, N, Ep, x.G(s), Gt, ld, EpiStore());
         __syncthreads();
-        wrap_gemm<kTc>(x, N, Gt, ld, 1, Em, x.G(s), ld, EpiStore());
+        wrap_gemm<kTc, true>(x, N, Gt, Em, x.G(s), ld, EpiStore());
         __syncthreads();
       }
     }
@@ -1986,7 +2057,8 @@ __device__ __noinline__ void phase_stack(int b, int left, int s) {
         return;
       }
     }
-    cta_gemm<T>(N, n, N, x.Em(), 1, c.ld, from, ldn, 1, to, ldn, 1, EpiStore(), !f64);
+    if constexpr (f64) cta_gemm<T>(N, n, N, x.Em(), 1, c.ld, from, ldn, 1, to, ldn, 1, EpiStore());
+    else cta_gemm_f32<false>(N, n, N, x.Em(), c.ld, from, ldn, to, ldn, EpiStore());
   };
   int src = 0;
   if (left ? b == c.nb : b == 0) {
@@ -2198,12 +2270,12 @@ __device__ __forceinline__ void assemble_spin(Cta<T, RES>& x, int s, const doubl
       PQMC_FOR_2D(j, 0, ns, k, 0, ns) ot[(long)j * ldo + rows[k]] = (T)Xinv[(long)rows[j] * ns + k];
     }
     __syncthreads();
-    cta_gemm<T>(ns, N, ns, ot, ldo, 1, ql, ld, 1, Y, ld, 1, EpiStore(), true);
+    cta_gemm_f32<true>(ns, N, ns, ot, ldo, ql, ld, Y, ld, EpiStore());
   }
   __syncthreads();
   EpiFresh<T> epi{x.G(s), ld, &dmax};
-  cta_gemm<T>(N, N, ns, qr, 1, std::is_same<T, double>::value ? N : ld, Y, ld, 1, (T*)nullptr, 0, 0, epi,
-              !std::is_same<T, double>::value);
+  if constexpr (std::is_same<T, double>::value) cta_gemm<T>(N, N, ns, qr, 1, N, Y, ld, 1, (T*)nullptr, 0, 0, epi);
+  else cta_gemm_f32<false>(N, N, ns, qr, ld, Y, ld, nullptr, 0, epi);
   if constexpr (!std::is_same<T, double>::value) {
     if (c.dg64 == 2 && record) {
       // the refreshed G itself against G_FP64 (the path-precision copies of
@@ -2361,8 +2433,10 @@ __device__ __forceinline__ void measure_tv(Cta<T, RES>& x) {
   __syncthreads();
 }
 
+// grid_sums: the sums over i, j (ek, ex) formed elsewhere, n_sums pairs to add
+// up (a chain swept by the whole GPU), or null.
 template <typename T, bool RES>
-__device__ __forceinline__ void measure(Cta<T, RES>& x) {
+__device__ __forceinline__ void measure(Cta<T, RES>& x, const double* grid_sums = nullptr, int n_sums = 0) {
   const ChainDesc& c = x.c;
   if (c.tv) {
     measure_tv(x);
@@ -2371,13 +2445,20 @@ __device__ __forceinline__ void measure(Cta<T, RES>& x) {
   Smem<T>& sh = x.sh;
   const int N = c.N, ld = c.ld;
   double ek = 0.0, dc = 0.0, st = 0.0, ex = 0.0;
-  PQMC_FOR_2D(i, 0, N, j, 0, N) {
-    const double k = c.K64[(long)i * N + j];
-    const double ee = c.eps[i] * c.eps[j];
-    for (int s = 0; s < 2; ++s) {
-      const double gji = (i == j ? 1.0 : 0.0) - (double)x.G(s)[(long)j * ld + i];
-      ek += k * gji;
-      ex += ee * gji * (double)x.G(s)[(long)i * ld + j];
+  if (grid_sums) {
+    for (int q = threadIdx.x; q < n_sums; q += blockDim.x) {
+      ek += grid_sums[2 * q];
+      ex += grid_sums[2 * q + 1];
+    }
+  } else {
+    PQMC_FOR_2D(i, 0, N, j, 0, N) {
+      const double k = c.K64[(long)i * N + j];
+      const double ee = c.eps[i] * c.eps[j];
+      for (int s = 0; s < 2; ++s) {
+        const double gji = (i == j ? 1.0 : 0.0) - (double)x.G(s)[(long)j * ld + i];
+        ek += k * gji;
+        ex += ee * gji * (double)x.G(s)[(long)i * ld + j];
+      }
     }
   }
   for (int i = threadIdx.x; i < N; i += blockDim.x) {
