@@ -419,6 +419,19 @@ pqmc_status pqmc_probe_pipes(double* out);
 pqmc_status pqmc_test_tc_gemm(int M, int N, int K, const float* d_A, int trans_a, const float* d_B, float* d_C,
                               void* stream);
 
+/* Test hook of the FP64 product on the tensor cores that the stabilisation and
+ * the FP64 path use (no counterpart in the paper): one CTA rounds A and B to
+ * 63-bit fixed point against the largest element of each, takes them apart
+ * into eight 8-bit digits and adds up the digit products with i + j <= 7 in
+ * exact integer sums, rounded once to FP64.  Device pointers, FP64, row-major:
+ * A is M x K, B is K x N, C is M x N (written).  strided != 0 runs the form that
+ * reads the packed operands across their rows.  An operand that holds a NaN or
+ * an infinity makes every element of C NaN.  1 <= M, N, K <= 1024.  Runs on
+ * `stream` (NULL: the legacy default stream), allocates a work buffer on it and
+ * synchronises it. */
+pqmc_status pqmc_test_digit_gemm(int M, int N, int K, const double* d_A, const double* d_B, double* d_C, int strided,
+                                 void* stream);
+
 /* Error bar of the sign-reweighted estimator <s O>/<s> of the Method
  * section, as pqmc_measure computes it: the records are split into n_groups
  * groups (bins of consecutive sweeps of one chain, or whole chains when

@@ -97,6 +97,29 @@ __global__ void __launch_bounds__(512, 1) tc_gemm_test_kernel(int M, int N, int 
 }
 
 // --------------------------------------------------------------------------
+// Test kernel of the FP64 digit product (pqmc_test_digit_gemm).
+
+__global__ void __launch_bounds__(256, 1) digit_gemm_test_kernel(int M, int N, int K, const double* A, const double* B,
+                                                                double* C, unsigned long long* D, int strided) {
+  __shared__ int red[8];
+  const int ld = digit_ld(K);
+  unsigned long long* DA = D;
+  unsigned long long* DB = D + (size_t)M * ld;
+  int ea = kDigitNone, eb = kDigitNone;
+  PQMC_FOR_2D(i, 0, M, k, 0, K) ea = max(ea, digit_exp(A[(size_t)i * K + k]));
+  PQMC_FOR_2D(k, 0, K, j, 0, N) eb = max(eb, digit_exp(B[(size_t)k * N + j]));
+  const int EA = digit_cta_max(ea, red), EB = digit_cta_max(eb, red);
+  PQMC_FOR_2D(i, 0, M, k, 0, K) DA[strided ? (size_t)k * M + i : (size_t)i * ld + k] = digit_pack(A[(size_t)i * K + k], EA);
+  PQMC_FOR_2D(k, 0, K, j, 0, N) DB[strided ? (size_t)k * N + j : (size_t)j * ld + k] = digit_pack(B[(size_t)k * N + j], EB);
+  __syncthreads();
+  auto fa = [EA](int) { return EA; };
+  auto fb = [EB](int) { return EB; };
+  auto epi = [C, N](int i, int j, double v) { C[(size_t)i * N + j] = v; };
+  if (strided) digit_gemm<false, false>(M, N, K, DA, 1, M, DB, 1, N, fa, fb, false, false, epi);
+  else digit_gemm<true, true>(M, N, K, DA, ld, 1, DB, ld, 1, fa, fb, false, false, epi);
+}
+
+// --------------------------------------------------------------------------
 // Allocation-free initialisation of one chain (pqmc_green_noalloc).
 //
 // Runs init_kernel for a single FP64 chain with every buffer the kernel needs
@@ -324,6 +347,29 @@ extern "C" pqmc_status pqmc_test_tc_gemm(int M, int N, int K, const float* d_A, 
   if (herr & kErrTimeout) {
     set_init_error("pqmc_test_tc_gemm: tensor-core completion wait gave up");
     return PQMC_ETIMEOUT;
+  }
+  return PQMC_OK;
+}
+
+extern "C" pqmc_status pqmc_test_digit_gemm(int M, int N, int K, const double* d_A, const double* d_B, double* d_C,
+                                            int strided, void* stream) {
+  using namespace pqmc;
+  if (M < 1 || N < 1 || K < 1 || M > 1024 || N > 1024 || K > 1024 || !d_A || !d_B || !d_C) {
+    set_init_error("pqmc_test_digit_gemm: bad sizes or NULL pointer");
+    return PQMC_EINVAL;
+  }
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  unsigned long long* d_work = nullptr;
+  cudaError_t e = cudaMallocAsync(&d_work, (size_t)(M + N) * digit_ld(K) * 8, st);
+  if (e == cudaSuccess) {
+    digit_gemm_test_kernel<<<1, 256, 0, st>>>(M, N, K, d_A, d_B, d_C, d_work, strided ? 1 : 0);
+    e = cudaGetLastError();
+  }
+  if (d_work) cudaFreeAsync(d_work, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) {
+    set_init_error(std::string("pqmc_test_digit_gemm: ") + cudaGetErrorString(e));
+    return PQMC_ECUDA;
   }
   return PQMC_OK;
 }

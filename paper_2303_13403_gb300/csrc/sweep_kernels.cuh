@@ -1001,7 +1001,7 @@ __device__ __forceinline__ void decide_sub_block(Cta<T, RES>& x, int tau, uint32
       uj = uniform_of<T>(((uint64_t)w.x0 << 21) | (uint64_t)(w.x1 >> 11));
       flj = (int)f[i0 + lane];
     }
-    int a = a_done, bad = 0, nneg = 0;
+    int a = a_done, bad = 0, nneg = 0, last = i0;
     const long long pos0 = sh.acc_pos;
 #pragma unroll
     for (int j = 0; j < kBlock; ++j) {
@@ -1034,10 +1034,13 @@ __device__ __forceinline__ void decide_sub_block(Cta<T, RES>& x, int tau, uint32
             fb.cl[1][a] = dl[1][si];
             nneg += R < T(0) ? 1 : 0;
           }
+          last = i0 + j;
           ++a;
         }
       }
     }
+    // (the site list goes on with the last accepted site: sm_vectors reads whole blocks of it)
+    if (s == 0 && a > a_done && a + lane < a_done + kBlock) fb.gsite[a + lane] = last;
     if (s == 0 && lane == 0) {
       sh.na = a;
       sh.acc_pos = pos0 + nbk;
@@ -2532,7 +2535,8 @@ __device__ __forceinline__ void sweep_once(uint32_t sweep, bool do_measure) {
   }
 }
 
-template <typename T, bool RES>
+// kTables: the slice exponentials too (the wrap and the stack products read them)
+template <bool kTables = true, typename T, bool RES>
 __device__ __forceinline__ void load_state(Cta<T, RES>& x) {
   if (threadIdx.x == 0) {
     const ChainState& st = *x.c.st;
@@ -2548,7 +2552,7 @@ __device__ __forceinline__ void load_state(Cta<T, RES>& x) {
     x.sh.logw_spin[0] = st.logw[0][0];
     x.sh.logw_spin[1] = st.logw[1][0];
   }
-  if (threadIdx.x < 28) {
+  if (kTables && threadIdx.x < 28) {
     const int k = threadIdx.x / 14, sp = (threadIdx.x / 7) % 2, m = threadIdx.x % 7 - 3;
     double v = 1.0;
     if (x.c.tv) {

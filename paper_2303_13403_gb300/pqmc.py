@@ -111,6 +111,8 @@ SIGNATURES = [
     ("pqmc_probe_pipes", C.c_int, [C.POINTER(C.c_double)]),
     ("pqmc_test_tc_gemm", C.c_int, [C.c_int, C.c_int, C.c_int, C.c_void_p, C.c_int, C.c_void_p, C.c_void_p,
                                     C.c_void_p]),
+    ("pqmc_test_digit_gemm", C.c_int, [C.c_int, C.c_int, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p, C.c_int,
+                                       C.c_void_p]),
 ]
 
 
@@ -362,6 +364,12 @@ def test_tc_gemm(M, N, K, d_A, trans_a, d_B, d_C, stream=None):
     """pqmc_test_tc_gemm: device pointers (ints); C = A B by the tensor-core split-BF16 product."""
     _check(load().pqmc_test_tc_gemm(M, N, K, C.c_void_p(d_A), 1 if trans_a else 0, C.c_void_p(d_B),
                                     C.c_void_p(d_C), C.c_void_p(stream) if stream else None))
+
+
+def test_digit_gemm(M, N, K, d_A, d_B, d_C, strided=False, stream=None):
+    """pqmc_test_digit_gemm: device pointers (ints); C = A B in FP64 by the tensor-core digit product."""
+    _check(load().pqmc_test_digit_gemm(M, N, K, C.c_void_p(d_A), C.c_void_p(d_B), C.c_void_p(d_C),
+                                       1 if strided else 0, C.c_void_p(stream) if stream else None))
 
 
 def host_jackknife(sO, s):
