@@ -171,33 +171,34 @@ __global__ void __launch_bounds__(256) sp_gemm_kernel(SpGemm g) {
 // Per-chain pointers of the spread buffers.
 
 // (tsize: the path precision's element size, which places the FP64 buffers
-// too)
+// too; the spin is a choice between two offsets, not an index, so that a kernel
+// computes the offsets it needs in registers instead of a table in local memory)
 template <typename T>
 struct SpBuf {
   unsigned char* b;
   SpreadLayout L;
   __device__ __host__ SpBuf(unsigned char* base, int N, int ld, int nmax, int tsize = (int)sizeof(T))
       : b(base), L(spread_layout(N, ld, nmax, tsize)) {}
-  __device__ __host__ T* mt(int s, int k) const { return reinterpret_cast<T*>(b + L.mt[s][k]); }
+  __device__ __host__ T* mt(int s, int k) const { return reinterpret_cast<T*>(b + (s ? (k ? L.mt[1][1] : L.mt[1][0]) : (k ? L.mt[0][1] : L.mt[0][0]))); }
   __device__ __host__ unsigned long long* dq(int s, int k) const {
-    return reinterpret_cast<unsigned long long*>(b + L.dq[s][k]);
+    return reinterpret_cast<unsigned long long*>(b + (s ? (k ? L.dq[1][1] : L.dq[1][0]) : (k ? L.dq[0][1] : L.dq[0][0])));
   }
   __device__ __host__ int* em() const { return reinterpret_cast<int*>(b + L.misc + 40); }
   __device__ __host__ int* eq() const { return reinterpret_cast<int*>(b + L.misc + 48); }
-  __device__ __host__ double* m64(int s) const { return reinterpret_cast<double*>(b + L.m64[s]); }
-  __device__ __host__ double* c64(int s) const { return reinterpret_cast<double*>(b + L.c64[s]); }
-  __device__ __host__ double* rinv(int s) const { return reinterpret_cast<double*>(b + L.rinv[s]); }
-  __device__ __host__ double* o64(int s) const { return reinterpret_cast<double*>(b + L.o64[s]); }
-  __device__ __host__ double* tgj(int s) const { return reinterpret_cast<double*>(b + L.tgj[s]); }
-  __device__ __host__ double* pval(int s) const { return reinterpret_cast<double*>(b + L.pval[s]); }
-  __device__ __host__ int* perm(int s) const { return reinterpret_cast<int*>(b + L.perm[s]); }
-  __device__ __host__ double* d0(int s) const { return reinterpret_cast<double*>(b + L.d0[s]); }
-  __device__ __host__ T* xt(int s) const { return reinterpret_cast<T*>(b + L.xt[s]); }
-  __device__ __host__ T* qrt(int s) const { return reinterpret_cast<T*>(b + L.qrt[s]); }
-  __device__ __host__ T* qlt(int s) const { return reinterpret_cast<T*>(b + L.qlt[s]); }
-  __device__ __host__ T* y(int s) const { return reinterpret_cast<T*>(b + L.y[s]); }
-  __device__ __host__ T* gt(int s) const { return reinterpret_cast<T*>(b + L.gt[s]); }
-  __device__ __host__ T* mb(int s) const { return reinterpret_cast<T*>(b + L.mb[s]); }
+  __device__ __host__ double* m64(int s) const { return reinterpret_cast<double*>(b + (s ? L.m64[1] : L.m64[0])); }
+  __device__ __host__ double* c64(int s) const { return reinterpret_cast<double*>(b + (s ? L.c64[1] : L.c64[0])); }
+  __device__ __host__ double* rinv(int s) const { return reinterpret_cast<double*>(b + (s ? L.rinv[1] : L.rinv[0])); }
+  __device__ __host__ double* o64(int s) const { return reinterpret_cast<double*>(b + (s ? L.o64[1] : L.o64[0])); }
+  __device__ __host__ double* tgj(int s) const { return reinterpret_cast<double*>(b + (s ? L.tgj[1] : L.tgj[0])); }
+  __device__ __host__ double* pval(int s) const { return reinterpret_cast<double*>(b + (s ? L.pval[1] : L.pval[0])); }
+  __device__ __host__ int* perm(int s) const { return reinterpret_cast<int*>(b + (s ? L.perm[1] : L.perm[0])); }
+  __device__ __host__ double* d0(int s) const { return reinterpret_cast<double*>(b + (s ? L.d0[1] : L.d0[0])); }
+  __device__ __host__ T* xt(int s) const { return reinterpret_cast<T*>(b + (s ? L.xt[1] : L.xt[0])); }
+  __device__ __host__ T* qrt(int s) const { return reinterpret_cast<T*>(b + (s ? L.qrt[1] : L.qrt[0])); }
+  __device__ __host__ T* qlt(int s) const { return reinterpret_cast<T*>(b + (s ? L.qlt[1] : L.qlt[0])); }
+  __device__ __host__ T* y(int s) const { return reinterpret_cast<T*>(b + (s ? L.y[1] : L.y[0])); }
+  __device__ __host__ T* gt(int s) const { return reinterpret_cast<T*>(b + (s ? L.gt[1] : L.gt[0])); }
+  __device__ __host__ T* mb(int s) const { return reinterpret_cast<T*>(b + (s ? L.mb[1] : L.mb[0])); }
   __device__ __host__ T* g2() const { return reinterpret_cast<T*>(b + L.g2); }
   __device__ __host__ int* sites() const { return reinterpret_cast<int*>(b + L.misc + 64); }
   __device__ __host__ int* na() const { return reinterpret_cast<int*>(b + L.misc); }
@@ -237,7 +238,7 @@ __global__ void __launch_bounds__(256) sp_decide_kernel(const ChainDesc* chains,
   if (chains[blockIdx.x].st->err) return;
   setup_cta<T>(chains[blockIdx.x], 0, seed);
   auto x = this_cta<T, false>();
-  load_state(x);
+  load_state<false>(x);
   const ChainDesc& c = x.c;
   x.Gp = sp_gcur<T>(c, alt);
   decide<true, false>(x, tau, *sweep_ctr, i0, min(kBlock, c.N - i0), 0);
@@ -261,83 +262,105 @@ __global__ void __launch_bounds__(256) sp_decide_kernel(const ChainDesc* chains,
 
 // Block update on one 64 x 64 tile of G per CTA (grid: tiles, spin, chain):
 // G_new = G_old - (E_S - G_old[:, S]) M G_old[S, :], G_old the current buffer
-// (alt), G_new the other one; a copy when no flip was accepted.
+// (alt), G_new the other one; a copy when no flip was accepted.  The tile moves
+// little data and few FMAs; what it waits for is the chain of dependent loads
+// (descriptor, number of flips, sites, rows and columns of G), so every stage
+// issues all its loads before it uses one, and the tile itself is read first
+// (one load per loop turn in each stage took 17 us per block at 648 sites).
 template <typename T>
-__global__ void __launch_bounds__(256) sp_flush_kernel(const ChainDesc* chains, int i0, int alt) {
-  constexpr int TT = 64;
+__global__ void __launch_bounds__(256) sp_flush_kernel(const ChainDesc* chains, int alt) {
+  constexpr int TT = 64, kQ = kBlock / 4;
   __shared__ T Ms[kBlock][kBlock + 1];
   __shared__ T MW[kBlock][TT];
   __shared__ T Ws[kBlock][TT];
   __shared__ T Us[TT][kBlock + 1];
   __shared__ int st[kBlock];
   const ChainDesc& c = chains[blockIdx.z];
-  if (c.st->err) return;
   const int N = c.N, ld = c.ld, s = blockIdx.y;
+  const ChainState* state = c.st;
   SpBuf<T> sp(c.spread, N, ld, c.nmax);
-  const T* Gin = sp_gcur<T>(c, alt) + (long)s * N * ld;
-  T* Gout = sp_gcur<T>(c, alt ^ 1) + (long)s * N * ld;
-  const int a = *sp.na();
+  const T* own = static_cast<const T*>(c.G);
+  const T* Gin = (alt ? sp.g2() : own) + (long)s * N * ld;
+  T* Gout = const_cast<T*>(alt ? own : sp.g2()) + (long)s * N * ld;
   const int tn = (N + TT - 1) / TT;
   const int r0 = (blockIdx.x / tn) * TT, c0 = (blockIdx.x % tn) * TT;
   if (r0 >= N) return;
   const int nr = min(TT, N - r0), nc = min(TT, N - c0);
-  if (a == 0) {
-    for (int e = threadIdx.x; e < nr * nc; e += blockDim.x) {
-      const long o = (long)(r0 + e / nc) * ld + c0 + e % nc;
-      Gout[o] = Gin[o];
-    }
-    return;
-  }
-  const T* Mb = sp.mb(s);
-  if ((int)threadIdx.x < a) st[threadIdx.x] = sp.sites()[threadIdx.x];
-  for (int e = threadIdx.x; e < a * a; e += blockDim.x) Ms[e / a][e % a] = Mb[(e / a) * kBlock + e % a];
-  __syncthreads();
-  // W = G_old[S, tile columns]; U = E_S - G_old[tile rows, S]
-  for (int e = threadIdx.x; e < a * nc; e += blockDim.x) {
-    const int l = e / nc, j = e % nc;
-    Ws[l][j] = Gin[(long)st[l] * ld + c0 + j];
-  }
-  for (int e = threadIdx.x; e < a * nr; e += blockDim.x) {
-    const int i = e / a, m = e % a;
-    Us[i][m] = (r0 + i == st[m] ? T(1) : T(0)) - Gin[(long)(r0 + i) * ld + st[m]];
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < a * nc; e += blockDim.x) {
-    const int l = e / nc, j = e % nc;
-    T v = T(0);
-    for (int m = 0; m < a; ++m) v = fma(Ms[l][m], Ws[m][j], v);
-    MW[l][j] = v;
-  }
-  __syncthreads();
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, x64 = tid & 63, y4 = tid >> 6;
+  const int a = *sp.na(), stopped = state->err;
+  if (tid < kBlock) st[tid] = sp.sites()[tid];
   // 4 x 4 outputs per thread, rows and columns interleaved by 16
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  T g[4][4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = ty + 16 * r, j = tx + 16 * q;
+      g[r][q] = i < nr && j < nc ? Gin[(long)(r0 + i) * ld + c0 + j] : T(0);
+    }
+  if (stopped) return;
   T acc[4][4];
 #pragma unroll
   for (int r = 0; r < 4; ++r)
 #pragma unroll
     for (int q = 0; q < 4; ++q) acc[r][q] = T(0);
-  for (int m = 0; m < a; ++m) {
-    T u[4], w[4];
+  if (a > 0) {
+    const T* Mb = sp.mb(s);
+    T m[4];
 #pragma unroll
-    for (int r = 0; r < 4; ++r) u[r] = Us[ty + 16 * r][m];
+    for (int q = 0; q < 4; ++q) {
+      const int l = (tid >> 5) + 8 * q, k = tid & 31;
+      m[q] = l < a && k < a ? Mb[l * kBlock + k] : T(0);
+    }
+    __syncthreads();
+    // W = G_old[S, tile columns]; U = E_S - G_old[tile rows, S]
+    T w[kQ], u[kQ];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) w[q] = MW[m][tx + 16 * q];
+    for (int q = 0; q < kQ; ++q) {
+      const int l = y4 + 4 * q;
+      w[q] = l < a && x64 < nc ? Gin[(long)st[l] * ld + c0 + x64] : T(0);
+      u[q] = l < a && x64 < nr ? Gin[(long)(r0 + x64) * ld + st[l]] : T(0);
+    }
 #pragma unroll
-    for (int r = 0; r < 4; ++r)
+    for (int q = 0; q < 4; ++q) Ms[(tid >> 5) + 8 * q][tid & 31] = m[q];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) acc[r][q] = fma(u[r], w[q], acc[r][q]);
+    for (int q = 0; q < kQ; ++q) {
+      const int l = y4 + 4 * q;
+      Ws[l][x64] = w[q];
+      if (l < a) Us[x64][l] = (r0 + x64 == st[l] ? T(1) : T(0)) - u[q];
+    }
+    __syncthreads();
+    // M W: column x64 and every fourth row from y4 per thread
+    T v[kQ];
+#pragma unroll
+    for (int q = 0; q < kQ; ++q) v[q] = T(0);
+    for (int k = 0; k < a; ++k) {
+      const T wk = Ws[k][x64];
+#pragma unroll
+      for (int q = 0; q < kQ; ++q) v[q] = fma(Ms[y4 + 4 * q][k], wk, v[q]);
+    }
+#pragma unroll
+    for (int q = 0; q < kQ; ++q) MW[y4 + 4 * q][x64] = v[q];
+    __syncthreads();
+    for (int k = 0; k < a; ++k) {
+      T uu[4], ww[4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) uu[r] = Us[ty + 16 * r][k];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) ww[q] = MW[k][tx + 16 * q];
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[r][q] = fma(uu[r], ww[q], acc[r][q]);
+    }
   }
 #pragma unroll
   for (int r = 0; r < 4; ++r)
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int i = ty + 16 * r, j = tx + 16 * q;
-      if (i < nr && j < nc) {
-        const long o = (long)(r0 + i) * ld + c0 + j;
-        Gout[o] = Gin[o] - acc[r][q];
-      }
+      if (i < nr && j < nc) Gout[(long)(r0 + i) * ld + c0 + j] = g[r][q] - acc[r][q];
     }
-  (void)i0;
 }
 
 // G (both spins) from the second copy back into the chain's own buffer
@@ -525,7 +548,7 @@ __global__ void __launch_bounds__(256) sp_tail_kernel(const ChainDesc* chains, u
   if (chains[blockIdx.x].st->err) return;
   setup_cta<T>(chains[blockIdx.x], 0, seed);
   auto x = this_cta<T, false>();
-  load_state(x);
+  load_state<false>(x);
   const ChainDesc& c = x.c;
   Smem<T>& sh = x.sh;
   SpBuf<T> sp(c.spread, c.N, c.ld, c.nmax);
@@ -640,7 +663,7 @@ cudaError_t spread_sweep_t(const SpreadPlan& P, int mode, int measure, cudaStrea
     for (int i0 = 0; i0 < N && e == cudaSuccess; i0 += kBlock) {
       sp_decide_kernel<T><<<nc, 256, smem_cta, st>>>(D, P.seed, P.d_sweep, tau, i0, cur, P.d_err);
       ok(cudaSuccess);
-      sp_flush_kernel<T><<<dim3(tn * tn, 2, nc), 256, 0, st>>>(D, i0, cur);
+      sp_flush_kernel<T><<<dim3(tn * tn, 2, nc), 256, 0, st>>>(D, cur);
       ok(cudaSuccess);
       cur ^= 1;
     }
