@@ -145,7 +145,8 @@ typedef struct {
                                (reduced paths only, one chain per SM); 0 picks for FP64 256,
                                128 or 64 (up to one, up to two, more chains per SM of the
                                device), and for the reduced paths 256, or 512 when a chain has 128
-                               sites or more. Smaller CTAs put more chains on one SM
+                               sites or more or when the batch has at most one chain per
+                               SM and a chain of 64 sites or more. Smaller CTAs put more chains on one SM
                                (FP64: 256/cta_threads per SM, others twice that) */
     int dense_chains;       /* reduced paths only: kernels built for twice as many chains per SM
                                (fewer registers per thread); needs cta_threads 64 or 128 */

@@ -439,7 +439,16 @@ pqmc_status build_ctx(int n, const pqmc_chain_spec* specs, const pqmc_opts* opts
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int fp64_tpb = n <= sms ? 256 : n <= 2 * sms ? 128 : 64;
-  const int reduced_tpb = (nmax_sites >= 128 && !o.dense_chains) ? 512 : 256;
+  // (a reduced-path batch of at most one chain per SM takes 512 threads from
+  // 64 sites on: 72 sites 16.6 -> 14.4 ms per sweep, 98 sites 12.0 -> 7.2, while
+  // 18 and 32 sites do not gain; BF16X3 only where every chain stays in
+  // shared memory, because a 512-thread CTA wraps the others by another
+  // tensor-core product, whose rounding differs)
+  bool roomy = n <= sms && nmax_sites >= 64;
+  if (ctx->prec == PQMC_BF16X3)
+    for (const HostChain& h : ctx->chains)
+      roomy = roomy && resident_bytes(h.N, h.ld, h.nmax, (int)ctx->tsize, o.delay_k) <= smem_resident_cap(ctx->prec, 512, 0);
+  const int reduced_tpb = ((nmax_sites >= 128 || roomy) && !o.dense_chains) ? 512 : 256;
   ctx->tpb = o.cta_threads != 0 ? o.cta_threads : (ctx->prec == PQMC_FP64 ? (o.spread ? 256 : fp64_tpb) : reduced_tpb);
   {
     ctx->boost = (ctx->prec != PQMC_FP64 && o.dense_chains) ? 1 : 0;
