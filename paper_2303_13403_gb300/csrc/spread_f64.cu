@@ -223,18 +223,16 @@ __global__ void __launch_bounds__(256) qform_kernel(const ChainDesc* chains, int
 constexpr int kGJRanks = 8;
 constexpr int kGJRows = kMaxSigma / kGJRanks;     // rows per CTA
 static_assert(kMaxSigma % kGJRanks == 0 && kGJRows == 4 * 16 && kSpGJ == 16, "four rows per thread and column");
-struct GJCand {
-  unsigned long long best;
-  int row, pad;
-  double v[kSpGJ];
-};
+// a CTA's candidate: the scaled pivot row it would give (16), the pivot, its
+// absolute value's bits and its row
+constexpr int kGJWords = kSpGJ + 3;
 
 __global__ void __cluster_dims__(kGJRanks, 1, 1) __launch_bounds__(256)
     gj_panel_kernel(const ChainDesc* chains, int p, int tsize) {
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
   __shared__ double Ap[kGJRows][kSpGJ + 1];
-  __shared__ GJCand cand[2][kGJRanks];              // two steps in flight
+  __shared__ unsigned long long cand[2][kGJRanks][kGJWords];   // two steps in flight
   __shared__ int used[kGJRows], place[kGJRows], pivrow[kSpGJ];
   __shared__ int rows[2 * kSpGJ], src[2 * kSpGJ], nrows;
   const ChainDesc& c = chains[blockIdx.y];
@@ -260,9 +258,10 @@ __global__ void __cluster_dims__(kGJRanks, 1, 1) __launch_bounds__(256)
   cl.sync();                                        // every CTA of the cluster runs before its memory is written
   for (int jj = 0; jj < bw; ++jj) {
     const int j = p0 + jj;
-    GJCand* cd = cand[jj & 1];
+    auto cd = cand[jj & 1];
     if (warp == 0) {
-      // this CTA's candidate, handed to every CTA
+      // this CTA's candidate, handed to every CTA; its owner takes the
+      // reciprocal and scales the row, so that the choice below is integer work
       unsigned long long best = 0;
       int bl = -1;
       for (int l = lane; l < nl; l += 32) {
@@ -274,25 +273,32 @@ __global__ void __cluster_dims__(kGJRanks, 1, 1) __launch_bounds__(256)
       const bool mine = bl >= 0 && (unsigned)(best >> 32) == hi && (unsigned)best == lo;
       const unsigned l = __reduce_min_sync(0xffffffffu, mine ? (unsigned)bl : 0xffffffffu);   // ties to the lower row
       const bool any = l != 0xffffffffu;
-      for (int t = 0; t < kGJRanks; ++t) {
-        GJCand* to = cl.map_shared_rank(&cd[rank], t);
-        if (lane < kSpGJ) to->v[lane] = any ? Ap[l][lane] : 0.0;
-        if (lane == 16) to->best = any ? ((unsigned long long)hi << 32) | lo : 0ull;
-        if (lane == 17) to->row = any ? rank + kGJRanks * (int)l : 0x7fffffff;
+      const double pvt = any ? Ap[l][jj] : 0.0;
+      const double ip = pvt != 0.0 ? recip64(pvt) : 0.0;
+      const double x = lane == jj ? ip : any && lane < kSpGJ ? Ap[l][lane] * ip : 0.0;
+      unsigned long long w = (unsigned long long)__double_as_longlong(lane == kSpGJ ? pvt : x);
+      if (lane == kSpGJ + 1) w = ((unsigned long long)hi << 32) | lo;
+      if (lane == kSpGJ + 2) w = any ? (unsigned long long)(rank + kGJRanks * (int)l) : 0x7fffffffull;
+      if (lane < kGJWords) {
+#pragma unroll
+        for (int t = 0; t < kGJRanks; ++t) *cl.map_shared_rank(&cd[rank][lane], t) = w;
       }
     }
     cl.sync();
     // the best of the eight, ties to the lower row
-    int b = 0;
-#pragma unroll
-    for (int t = 1; t < kGJRanks; ++t)
-      if (cd[t].row != 0x7fffffff &&
-          (cd[b].row == 0x7fffffff || cd[t].best > cd[b].best || (cd[t].best == cd[b].best && cd[t].row < cd[b].row)))
-        b = t;
-    const int r = cd[b].row;
-    const double pvt = cd[b].v[jj];
-    const double ip = pvt != 0.0 ? recip64(pvt) : 0.0;
-    const double x = col == jj ? ip : cd[b].v[col] * ip;
+    int b;
+    {
+      const int row = lane < kGJRanks ? (int)cd[lane][kSpGJ + 2] : 0x7fffffff;
+      const unsigned long long best = lane < kGJRanks && row != 0x7fffffff ? cd[lane][kSpGJ + 1] : 0ull;
+      const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(best >> 32));
+      const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(best >> 32) == hi ? (unsigned)best : 0u);
+      const bool top = (unsigned)(best >> 32) == hi && (unsigned)best == lo;
+      const unsigned low = __reduce_min_sync(0xffffffffu, top ? (unsigned)row : 0xffffffffu);
+      b = __ffs((int)__ballot_sync(0xffffffffu, top && (unsigned)row == low)) - 1;
+    }
+    const int r = (int)cd[b][kSpGJ + 2];
+    const double pvt = __longlong_as_double((long long)cd[b][kSpGJ]);
+    const double x = __longlong_as_double((long long)cd[b][col]);
     // eliminate column j: v = add - f_i x, one FP64 instruction per element
     double f[4], v[4];
 #pragma unroll
@@ -354,19 +360,20 @@ __global__ void __cluster_dims__(kGJRanks, 1, 1) __launch_bounds__(256)
   // the other columns, and the block row of the update (rows[e] = p0 + e for e < bw)
   const int m = nrows;
   double* Tb = sp.tgj(s);
-  for (int cc = rank * 64 + (int)threadIdx.x; cc < n && threadIdx.x < 64; cc += 64 * kGJRanks) {
-    if (cc >= p0 && cc < p1) continue;
-    double v[2 * kSpGJ];
+  static_assert(kMaxSigma <= 64 * kGJRanks, "one column per 64 threads and rank");
+  const int cc = rank * 64 + (int)(threadIdx.x & 63), eg = (int)(threadIdx.x >> 6) * 8;   // eight entries per thread
+  const bool mover = cc < n && (cc < p0 || cc >= p1);
+  double mv[8];
 #pragma unroll
-    for (int e = 0; e < 2 * kSpGJ; ++e)
-      if (e < m) v[e] = A[(long)src[e] * ldn + cc];
+  for (int e = 0; e < 8; ++e)
+    if (mover && eg + e < m) mv[e] = A[(long)src[eg + e] * ldn + cc];
+  __syncthreads();                                  // a column's rows are all read before one is written
 #pragma unroll
-    for (int e = 0; e < 2 * kSpGJ; ++e)
-      if (e < m) {
-        A[(long)rows[e] * ldn + cc] = v[e];
-        if (e < bw) Tb[(long)e * ldn + cc] = v[e];
-      }
-  }
+  for (int e = 0; e < 8; ++e)
+    if (mover && eg + e < m) {
+      A[(long)rows[eg + e] * ldn + cc] = mv[e];
+      if (eg + e < bw) Tb[(long)(eg + e) * ldn + cc] = mv[e];
+    }
 }
 
 // row i: the interchanges of the elimination applied to the columns, last first

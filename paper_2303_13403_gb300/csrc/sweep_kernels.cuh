@@ -661,14 +661,35 @@ __device__ __forceinline__ void block_inverse(Cta<T, RES>& x, int a, bool pivot)
     __syncthreads();
     const T xpl = lane < a ? prow[lane] : T(0);
     const T ip = T(1) / prow[p];
-    for (int r = w; r < a; r += ws) {
-      const T xrp = X[r][p], xrl = lane < a ? X[r][lane] : T(0);
-      __syncwarp();
-      T v;
-      if (r == p) v = lane == p ? ip : xpl * ip;
-      else v = lane == p ? -xrp * ip : fma(-xrp * ip, xpl, xrl);
-      if (lane < a) X[r][lane] = v;
-    }
+    // several rows of a warp in flight: eight without a branch where a warp has
+    // up to eight rows (two FP32 species), four with the absent ones left out where
+    // that would be idle work (one species) or FP64 instructions
+    auto eliminate = [&](auto in_flight, auto skip) {
+      constexpr int kU = decltype(in_flight)::value;
+      for (int r0 = w; r0 < a; r0 += kU * ws) {
+        T xrp[kU], xrl[kU];
+#pragma unroll
+        for (int q = 0; q < kU; ++q) {
+          const int r = min(r0 + q * ws, a - 1);
+          xrp[q] = X[r][p];
+          xrl[q] = X[r][lane];
+        }
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < kU; ++q) {
+          const int r = r0 + q * ws;     // (the same in the whole warp)
+          if (decltype(skip)::value && r >= a) continue;
+          const T m = xrp[q] * ip;
+          T v = fma(-m, xpl, xrl[q]);
+          if (lane == p) v = -m;
+          if (r == p) v = lane == p ? ip : xpl * ip;
+          if (r < a && lane < a) X[r][lane] = v;
+        }
+        __syncwarp();
+      }
+    };
+    if (std::is_same<T, double>::value || ns == 1) eliminate(std::integral_constant<int, 4>(), std::true_type());
+    else eliminate(std::integral_constant<int, 8>(), std::false_type());
     __syncthreads();
   }
   if (w == 0 && pivot) {
