@@ -427,8 +427,8 @@ pqmc_status build_ctx(int n, const pqmc_chain_spec* specs, const pqmc_opts* opts
   ctx->off_last = take((size_t)n * kRecord * 8);
   // default CTA size (measured on GB300): the FP64 path packs 4 chains of 64
   // threads per SM, or 2 of 128 or 1 of 256 when the batch leaves the SMs room
-  // (304 chains of 72 sites, 2Theta = 4: 90.4 ms per sweep with 64 threads,
-  // 74.6 with 128; one chain of 72 sites finishes in half the time with 256);
+  // (304 chains of 72 sites, 2Theta = 4: 70.6 ms per sweep with 64 threads,
+  // 43.9 with 128, 44.8 with 256);
   // the reduced paths 2 chains of 256 threads, whose G and
   // scratch then fit in shared memory at 72 sites, and one chain of 512
   // threads per SM once a chain has 128 sites or more (its G lives in global

@@ -266,7 +266,8 @@ __global__ void __launch_bounds__(256) sp_decide_kernel(const ChainDesc* chains,
 // little data and few FMAs; what it waits for is the chain of dependent loads
 // (descriptor, number of flips, sites, rows and columns of G), so every stage
 // issues all its loads before it uses one, and the tile itself is read first
-// (one load per loop turn in each stage took 17 us per block at 648 sites).
+// (one load per loop turn in each stage took 17.3 us per block at 648 sites,
+// this form 8.6).
 template <typename T>
 __global__ void __launch_bounds__(256) sp_flush_kernel(const ChainDesc* chains, int alt) {
   constexpr int TT = 64, kQ = kBlock / 4;

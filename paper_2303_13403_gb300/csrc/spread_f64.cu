@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(256) sp_digit_gemm_kernel(const ChainDesc* cha
 // rows of L^{-1} (R_PP^{-1} = L^{-T} diag(p)^{-1/2}).  Warp 0 runs one step ahead (row
 // k + 1, its pivot and reciprocal), so a column costs one barrier and the
 // reciprocal's latency passes beside the other rows' FMAs; factor and
-// back substitution as two chains of 32 steps took 42.6 us.  Panel 0 first
+// back substitution as two chains of 32 steps took 42.6 us, this form 17.0.  Panel 0 first
 // records the Gram diagonal and clears the chain's breakdown flag and log det R.
 __global__ void __launch_bounds__(256) chol_panel_kernel(const ChainDesc* chains, int p, int tsize) {
   __shared__ double A[kSpPanel][kSpPanel + 1];
@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(256) qform_kernel(const ChainDesc* chains, int
 // panel row, to all eight (distributed shared memory), and each takes the
 // best of the eight and eliminates its own rows.  (One CTA per spin had n x 16
 // FP64 FMAs per column on one SM and two barriers with a division between
-// them: 71.7 us per panel at n = 324.)  Rows are interchanged once, at the end: the
+// them: 71.7 us per panel at n = 324, this form 27.9.)  Rows are interchanged once, at the end: the
 // panel's interchanges composed into one permutation of at most 2 bw rows
 // (place rows[e] takes row src[e]), applied to the panel as it is written back
 // and to the other columns, which the CTAs share.

@@ -231,8 +231,7 @@ __device__ void cta_gemm(int M, int Nn, int K, const TA* A, int sai, int sak, co
 // no fallback to scalar loads inside, so the loop keeps its registers and the
 // phase its code small.  (162 sites: rank-21 update, stack products and
 // assembly took 29 + 22 + 24 Mcycles per 42 slices with scalar loads and a
-// bounds check per element; 288 sites: a single function choosing at run
-// time took 74 for the wrap, this one %s.)
+// bounds check per element)
 template <bool kRowA, typename Epi>
 __device__ __forceinline__ void cta_gemm_f32(int M, int Nn, int K, const float* A, int lda, const float* B, int ldb,
                                              float* C, int ldc, Epi epi) {
