@@ -123,7 +123,10 @@ __global__ void __launch_bounds__(256) chol_panel_kernel(const ChainDesc* chains
   };
   if (warp == 0) pivot_row(0);
   __syncthreads();
-  for (int k = 0; k + 1 < bw && !bad; ++k) {
+  // (every step runs to its barrier whatever the pivots are: warp 0 sets bad
+  // one step ahead, so it is read only after the last barrier; past a bad
+  // pivot the rows take u = 0)
+  for (int k = 0; k + 1 < bw; ++k) {
     const double uk = u[k & 1][lane];
     if (warp == 0) {
       const int r = k + 1;
@@ -135,7 +138,6 @@ __global__ void __launch_bounds__(256) chol_panel_kernel(const ChainDesc* chains
     }
     __syncthreads();
   }
-  __syncthreads();
   if (bad) {
     if (threadIdx.x == 0) sp.bad()[s] = 1;
     return;

@@ -1,0 +1,65 @@
+"""Stack blocks that the Cholesky QR cannot factorise.
+
+With 2 Theta = 0 the stack blocks are e^{V(s)} P alone, formed in FP64, and a
+large g makes them as ill-conditioned as wanted: the Gutzwiller factor scales
+the sites of field +1 up (spin down: those of field -1) and the others down,
+so a spin with fewer scaled-up sites than particles has a block with
+cond ~ e^{2 kappa}, kappa = arccosh(e^{g/2}) (g = 18: 2.6e8), beyond the
+1e6 that the factorisation takes.  The host decides which blocks break from
+the fields; a block in between is left to neither side."""
+import numpy as np
+import pytest
+
+from oracle import philox, pqmc as opq
+from paper_2303_13403_gb300 import pqmc, workloads
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def cuda():
+    import torch
+    torch.cuda.set_device(0)
+    pqmc.load()
+
+
+def vmc(L, g, **kw):
+    return workloads.honeycomb(L, U=4.0, dtau=0.1, two_theta=0.0, g=g, M_N=0.21, **kw)
+
+
+def model_of(spec):
+    return opq.Model(opq.Params(kind=spec.kind, Lx=spec.Lx, Ly=spec.Ly, U=spec.U, dtau=spec.dtau, two_theta=spec.two_theta,
+                                g=spec.g, M_N=spec.M_N, n_up=spec.n_up, n_dn=spec.n_dn, n_stab=1))
+
+
+def smallest_pivot(m, fields, sg):
+    """Smallest pivot of the blocks' Gram matrices relative to its diagonal (both end slices)."""
+    out = 1.0
+    for f in fields:
+        M = np.exp(sg * np.arccosh(np.exp(m.p.g / 2)) * f)[:, None] * m.P[sg]
+        r = np.abs(np.diag(np.linalg.qr(M)[1]))
+        out = min(out, float((r ** 2 / (M ** 2).sum(0)).min()))
+    return out
+
+
+@pytest.mark.parametrize("prec", [pqmc.FP64, pqmc.FP32])
+@pytest.mark.parametrize("L,g", [(3, 18.0), (6, 18.0), (6, 0.6)])
+def test_spread_reports_a_breakdown(L, g, prec):
+    """The whole-GPU sweep has no other factorisation: it stops with ESTAB, at
+    whichever column the pivot fails, and the next context runs."""
+    spec = vmc(L, g)
+    m = model_of(spec)
+    seen = set()
+    for seed in range(1, 9):
+        f = philox.initial_fields(seed, 0, 2, spec.n_sites)
+        pivot = min(smallest_pivot(m, f, sg) for sg in (1, -1))
+        if 2e-13 < pivot < 5e-12:
+            continue
+        try:
+            pqmc.Context([spec], prec=prec, seed=seed, n_stab=1, spread=1).close()
+            status = 0
+        except pqmc.PQMCError as e:
+            status = e.status
+        assert status == (pqmc.ESTAB if pivot < 1e-12 else 0), (seed, pivot)
+        seen.add(status)
+    assert seen == {pqmc.ESTAB} if g > 1 else seen == {0}
