@@ -823,6 +823,29 @@ __device__ __forceinline__ void sm_core(Cta<T, RES>& x, int i0, int m0, int cnt)
   }
 }
 
+// Where sm_four reads a spin's table (flat, four elements from there): for flip
+// k + i the elements of the flips k + q .. k + q + 3, in the place of sm_v (rows)
+// or sm_u (columns, the four in reverse).  A window that reaches past the last
+// flip of the block reads the last four once more instead (its elements there
+// stand for no flip), so that no read leaves the flip's row.
+__host__ __device__ constexpr int sm_at(bool row, int k, int i, int q) {
+  const int qc = q < kBlock - 4 - k ? q : kBlock - 4 - k;
+  return row ? (k + i) * kBlock + k + qc : (kBlock - 1 - k - i) * kBlock + kBlock - 4 - k - qc;
+}
+constexpr bool sm_reads_in_row() {
+  for (int k = 0; k < kBlock; k += 4)
+    for (int i = 0; i < 4; ++i)
+      for (int q = 0; q < kBlock; q += 4) {
+        const int v = sm_at(true, k, i, q), u = sm_at(false, k, i, q);
+        if (v / kBlock != k + i || (v + 3) / kBlock != k + i || u < 0 || u / kBlock != kBlock - 1 - k - i ||
+            (u + 3) / kBlock != kBlock - 1 - k - i)
+          return false;
+        if (k + q < kBlock && (v % kBlock != k + q || u % kBlock != kBlock - 4 - k - q)) return false;
+      }
+  return true;
+}
+static_assert(kBlock % 4 == 0 && sm_reads_in_row(), "the update vectors' table reads");
+
 // Four flips k .. k + 3 on a thread's window w of kW elements (register i:
 // flip k + i): the flips' vector elements go out, the later elements take
 // their updates.  No branch inside: the table rows are read ahead of the
@@ -830,7 +853,7 @@ __device__ __forceinline__ void sm_core(Cta<T, RES>& x, int i0, int m0, int cnt)
 template <bool kRow, int kW, typename T>
 __device__ __forceinline__ void sm_four(T (&w)[kBlock], const T (*tab)[kBlock], int k, int cnt, int j, const int* site,
                                         const T* fr, T* out, long os) {
-  const T* tr = kRow ? &tab[k][k] : &tab[kBlock - 1 - k][kBlock - 4 - k];
+  const T* t0 = &tab[0][0];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     T cv = w[i];
@@ -840,7 +863,7 @@ __device__ __forceinline__ void sm_four(T (&w)[kBlock], const T (*tab)[kBlock], 
     for (int q = 0; q < kW; q += 4)
       if (q + 3 > i) {
         T t[4];
-        Vec4<T>::load(kRow ? tr + i * kBlock + q : tr - i * kBlock - q, t);
+        Vec4<T>::load(t0 + sm_at(kRow, k, i, q), t);
 #pragma unroll
         for (int h = 0; h < 4; ++h)
           if (q + h > i) w[q + h] = fma(-cv, kRow ? t[h] : t[3 - h], w[q + h]);
