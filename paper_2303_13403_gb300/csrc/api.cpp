@@ -210,10 +210,11 @@ void put(Staged& a, size_t off, const std::vector<double>& src, int rows, int co
     for (int j = 0; j < cols; ++j) p[(size_t)i * ld + j] = (T)src[(size_t)i * cols + j];
 }
 
-// smallest E with |x| < 2^E for every x of v
+// smallest E with |x| < 2^E for every x of v; kDigitBad when one is not finite
 int max_exponent(const std::vector<double>& v) {
-  int e = -1000;
+  int e = kDigitNone;
   for (double x : v) {
+    if (!std::isfinite(x)) return kDigitBad;
     int k = 0;
     std::frexp(x, &k);
     if (x != 0.0) e = std::max(e, k);
@@ -222,12 +223,14 @@ int max_exponent(const std::vector<double>& v) {
 }
 
 // Digits of an N x N matrix for digit_gemm.cuh: element (b, a) at
-// a digit_ld(N) + b, x = X 2^{E - 62} packed as X + 0x80...80.
+// a digit_ld(N) + b, x = X 2^{E - 62} packed as X + 0x80...80 (a matrix that
+// is not finite has no digits: its exponent makes every product NaN).
 void pack_digits(uint64_t* dig, const std::vector<double>& m, int N, int E) {
   const int ldd = digit_ld(N);
   for (int a = 0; a < N; ++a)
     for (int b = 0; b < N; ++b)
-      dig[(size_t)a * ldd + b] = (uint64_t)std::llround(std::ldexp(m[(size_t)b * N + a], 62 - E)) + 0x8080808080808080ull;
+      dig[(size_t)a * ldd + b] =
+          (E == kDigitBad ? 0 : (uint64_t)std::llround(std::ldexp(m[(size_t)b * N + a], 62 - E))) + kDigitZero;
 }
 
 void put_raw(Staged& a, size_t off, const void* src, size_t n) { memcpy(a.at(off, n), src, n); }

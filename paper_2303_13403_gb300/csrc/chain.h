@@ -148,6 +148,11 @@ PQMC_HDI constexpr int m64_ld(int N) { return N | 1; }
 // n rounded up to whole 16-byte vectors of FP32
 PQMC_HDI constexpr int pad4(int n) { return (n + 3) & ~3; }
 PQMC_HDI constexpr int digit_ld(int K) { return ((K + 5) & ~7) + 2; }
+// packed digits (digit_gemm.cuh): exponents of an operand with a NaN or an
+// infinity and of one that is all zero; a packed zero
+constexpr int kDigitBad = 1 << 20;
+constexpr int kDigitNone = -(1 << 19);
+constexpr unsigned long long kDigitZero = 0x8080808080808080ull;
 
 PQMC_HDI ScratchLayout scratch_layout(int N, int ld, int n, int tsize, int kd) {
   ScratchLayout L;

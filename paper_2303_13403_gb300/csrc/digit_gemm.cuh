@@ -33,10 +33,6 @@
 
 namespace pqmc {
 
-constexpr int kDigitBad = 1 << 20;                       // exponent of an operand with a NaN or an infinity
-constexpr int kDigitNone = -(1 << 19);                   // exponent of an operand that is all zero
-constexpr unsigned long long kDigitZero = 0x8080808080808080ull;   // packed zero
-
 // smallest E with |x| < 2^E
 static __device__ __forceinline__ int digit_exp(double x) {
   const int e = (__double2hiint(x) >> 20) & 0x7ff;

@@ -63,3 +63,17 @@ def test_spread_reports_a_breakdown(L, g, prec):
         assert status == (pqmc.ESTAB if pivot < 1e-12 else 0), (seed, pivot)
         seen.add(status)
     assert seen == {pqmc.ESTAB} if g > 1 else seen == {0}
+
+
+def test_overflowing_exponential_is_reported():
+    """e^{+dtau K} beyond the FP64 range (4 x 4, t' = -0.5: e^{720}, where
+    e^{-dtau K} reaches e^{240}): the propagated G is NaN, which the first
+    decisions taken on it report."""
+    spec = workloads.ChainSpec(kind=workloads.SQUARE, Lx=4, Ly=4, tp=-0.5, U=0.0, dtau=120.0, two_theta=240.0, g=0.0,
+                               n_up=7, n_dn=7)
+    ctx = pqmc.Context([spec], prec=pqmc.FP64, seed=3, n_stab=1)
+    with pytest.raises(pqmc.PQMCError) as e:
+        ctx.sweep(2)
+        ctx.synchronize()
+    assert e.value.status == pqmc.ENAN
+    ctx.close()
