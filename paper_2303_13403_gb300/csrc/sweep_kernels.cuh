@@ -2087,19 +2087,31 @@ __device__ __noinline__ void phase_stack(int b, int left, int s) {
   T* Mt = x.Mt(s);
   T* Mt2 = x.Mt2();
   constexpr bool f64 = std::is_same<T, double>::value;
-  // Mt2 = e^{-dtau K} Mt: on the tensor cores in FP64 (digits of Mt in M64's place)
+  // Mt2 = e^{-dtau K} Mt: on the tensor cores in FP64 (digits of Mt in M64's
+  // place).  The columns of a block grow apart by up to e^{6 dtau} per slice
+  // and the product mixes rows only, so each column has its own exponent: a
+  // shared one cost the small columns their digits (free fermions, 72 sites, 10
+  // slices of dtau = 0.8: log det off by 2.7e-9, now by less than 1e-12).
+  // It enters as a factor 2^e of the result: as a second exponent in the
+  // digits' assembly it took 1.6% of a one-chain sweep of 18 sites.
   auto product = [&](const T* from, T* to) {
     if constexpr (f64) {
       if (c.dEm) {
-        const int ldd = digit_ld(N), ldk = N + (N & 1);
+        const int ldd = digit_ld(N), ldk = N + (N & 1), e1 = c.eEm;
         unsigned long long* D = reinterpret_cast<unsigned long long*>(x.M64());
-        int e = kDigitNone;
-        PQMC_FOR_2D(i, 0, N, k, 0, n) e = max(e, digit_exp(from[(long)i * ldn + k]));
-        const int E = digit_cta_max(e, reinterpret_cast<int*>(x.sh.red)), e1 = c.eEm;
-        PQMC_FOR_2D(i, 0, N, k, 0, n) D[(long)k * ldk + i] = digit_pack(from[(long)i * ldn + k], E);
+        double* sc = x.qbeta();                        // (the QR's vectors come later)
+        for (int k = threadIdx.x >> 5; k < n; k += blockDim.x >> 5) {
+          int e = kDigitNone;
+          for (int i = threadIdx.x & 31; i < N; i += 32) e = max(e, digit_exp(from[(long)i * ldn + k]));
+          e = __reduce_max_sync(0xffffffffu, e);
+          for (int i = threadIdx.x & 31; i < N; i += 32) D[(long)k * ldk + i] = digit_pack(from[(long)i * ldn + k], e);
+          // (2^{e - 1}: every exponent's is a normal number)
+          if ((threadIdx.x & 31) == 0)
+            sc[k] = __longlong_as_double(e == kDigitBad ? 0x7ff8000000000000ll : e == kDigitNone ? 0ll : (long long)(e + 1022) << 52);
+        }
         __syncthreads();
-        digit_gemm<true, true>(N, n, N, c.dEm, ldd, 1, D, ldk, 1, [e1](int) { return e1; }, [E](int) { return E; }, false,
-                               false, [to, ldn](int i, int j, double v) { to[(long)i * ldn + j] = v; });
+        digit_gemm<true, true>(N, n, N, c.dEm, ldd, 1, D, ldk, 1, [e1](int) { return e1; }, [](int) { return 1; }, false,
+                               false, [to, ldn, sc](int i, int j, double v) { to[(long)i * ldn + j] = v * sc[j]; });
         return;
       }
     }
