@@ -231,14 +231,14 @@ PQMC_HDI ScratchLayout scratch_layout(int N, int ld, int n, int tsize, int kd) {
 //                 alternate between G and g2 (read one, write the other)
 //   mb[s]       : M (kBlock x kBlock, T) of the flips accepted in one block
 //   dq[s][0..1] : packed digits (digit_gemm.cuh, ld digit_ld(N)) of a block to factor or of Q_L and Q_R
+//   dx[s][0..1] : their columns' exponents (n, int)
 //   misc        : int na (accepted flips of the block), int bad[2] (Cholesky
 //                 breakdown), then 8-aligned: uint64 dmax (bits of max |G - G_fresh|),
-//                 double lchol[2] (log det R); at 40: int em[2] (exponent of M64's digits), eq[2] (of
-//                 Q_L and Q_R's); at 64: int sites[kBlock] (accepted sites)
+//                 double lchol[2] (log det R); at 64: int sites[kBlock] (accepted sites)
 constexpr int kSpPanel = 32;   // Cholesky panel width
 constexpr int kSpGJ = 16;      // Gauss-Jordan panel width
 struct SpreadLayout {
-  size_t mt[2][2], dq[2][2], m64[2], c64[2], rinv[2], o64[2], tgj[2], pval[2], perm[2], d0[2], xt[2], qrt[2], qlt[2], y[2],
+  size_t mt[2][2], dq[2][2], dx[2][2], m64[2], c64[2], rinv[2], o64[2], tgj[2], pval[2], perm[2], d0[2], xt[2], qrt[2], qlt[2], y[2],
       gt[2], mb[2], g2, misc, total;
 };
 
@@ -256,6 +256,8 @@ PQMC_HDI SpreadLayout spread_layout(int N, int ld, int n, int tsize) {
     L.mt[s][1] = take(Nn * tsize);
     L.dq[s][0] = take((size_t)digit_ld(N) * n * 8);
     L.dq[s][1] = take((size_t)digit_ld(N) * n * 8);
+    L.dx[s][0] = take((size_t)n * 4);
+    L.dx[s][1] = take((size_t)n * 4);
     L.m64[s] = take(Nn * 8 > 2048 ? Nn * 8 : 2048);   // (also the partial sums of a measurement)
     L.c64[s] = take(nn * 8);
     L.rinv[s] = take(np * kSpPanel * kSpPanel * 8);

@@ -183,8 +183,7 @@ struct SpBuf {
   __device__ __host__ unsigned long long* dq(int s, int k) const {
     return reinterpret_cast<unsigned long long*>(b + (s ? (k ? L.dq[1][1] : L.dq[1][0]) : (k ? L.dq[0][1] : L.dq[0][0])));
   }
-  __device__ __host__ int* em() const { return reinterpret_cast<int*>(b + L.misc + 40); }
-  __device__ __host__ int* eq() const { return reinterpret_cast<int*>(b + L.misc + 48); }
+  __device__ __host__ int* dexp(int s, int k) const { return reinterpret_cast<int*>(b + (s ? (k ? L.dx[1][1] : L.dx[1][0]) : (k ? L.dx[0][1] : L.dx[0][0]))); }
   __device__ __host__ double* m64(int s) const { return reinterpret_cast<double*>(b + (s ? L.m64[1] : L.m64[0])); }
   __device__ __host__ double* c64(int s) const { return reinterpret_cast<double*>(b + (s ? L.c64[1] : L.c64[0])); }
   __device__ __host__ double* rinv(int s) const { return reinterpret_cast<double*>(b + (s ? L.rinv[1] : L.rinv[0])); }
@@ -208,12 +207,6 @@ struct SpBuf {
   }
   __device__ __host__ double* lchol() const { return reinterpret_cast<double*>(b + L.misc + 24); }
 };
-
-// largest digit exponent over a grid, in global memory (every thread of a warp calls)
-__device__ __forceinline__ void sp_exp_max(int* to, int e) {
-  e = __reduce_max_sync(0xffffffffu, e);
-  if ((threadIdx.x & 31) == 0) atomicMax(to, e);
-}
 
 // e^{V_sigma(s_tau)} at site i in FP64, as the single-CTA path tabulates it
 __device__ __forceinline__ double sp_vexp(const ChainDesc& c, int tau, int s, int i) {
@@ -419,17 +412,13 @@ __global__ void sp_stack_first_kernel(const ChainDesc* chains, int tau0, int lef
   const int N = c.N, s = blockIdx.y, n = s == 0 ? c.nup : c.ndn, ldn = c.nmax;
   SpBuf<T> sp(c.spread, N, c.ld, c.nmax);
   const long stride = (long)gridDim.x * blockDim.x;
-  int ex = kDigitNone;
   if (tau0 >= 0) {
     const double* P = c.P + (long)s * N * c.nmax;
     double* M = sp.m64(s);
     for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < (long)N * n; e += stride) {
       const int q = (int)(e / N), i = (int)(e % N);
-      const double v = sp_vexp(c, tau0, s, i) * P[(long)q * N + i];
-      M[(long)q * N + i] = v;
-      ex = max(ex, digit_exp(v));
+      M[(long)q * N + i] = sp_vexp(c, tau0, s, i) * P[(long)q * N + i];
     }
-    sp_exp_max(sp.em() + s, ex);
   } else {
     const double* prev = (left ? c.Lst : c.Rst) + ((long)b_prev * 2 + s) * N * c.nmax;
     T* Mt = sp.mt(s, 0);
@@ -449,14 +438,10 @@ __global__ void sp_to64_kernel(const ChainDesc* chains, int k) {
   SpBuf<T> sp(c.spread, N, c.ld, c.nmax);
   const T* Mt = sp.mt(s, k);
   double* M = sp.m64(s);
-  int ex = kDigitNone;
   for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < (long)N * n; e += (long)gridDim.x * blockDim.x) {
     const int q = (int)(e / N), i = (int)(e % N);
-    const double v = (double)Mt[(long)i * ldn + q];
-    M[(long)q * N + i] = v;
-    ex = max(ex, digit_exp(v));
+    M[(long)q * N + i] = (double)Mt[(long)i * ldn + q];
   }
-  sp_exp_max(sp.em() + s, ex);
 }
 
 // path-precision copies of O^{-1}, Q_R and Q_L for the assembly
@@ -576,7 +561,6 @@ __global__ void __launch_bounds__(256) sp_tail_kernel(const ChainDesc* chains, u
   if (threadIdx.x == 0) {
     const double dmax = __longlong_as_double((long long)*sp.dmax());
     *sp.dmax() = 0ull;
-    sp.eq()[0] = sp.eq()[1] = 0;
     if (flags & kSpRecord) {
       if (!isfinite(dmax)) sh.err |= kErrNaN;
       sh.dGmax = fmax(sh.dGmax, dmax);

@@ -13,39 +13,40 @@ __device__ __forceinline__ SpBuf<double> fp64_bufs(const ChainDesc& c, int tsize
 }
 __device__ __forceinline__ int nsig_of(const ChainDesc& c, int s) { return s == 0 ? c.nup : c.ndn; }
 
-// Digits of M64 (b < 0) or of stack blocks b, Q_L and Q_R (grid: .., spin, chain).
-// M64 is packed against the exponent its writer left in em; the columns of
-// Q are orthonormal, |q| < 2, and an element beyond that (or a NaN) marks eq, which
-// makes the product NaN.
+// Digits of M64 (b < 0, q = 0) or of stack blocks b, Q_L (q = 0) and Q_R (q = 1),
+// one column per CTA with the column's own exponent (grid: column of q = 0, then
+// of q = 1; spin; chain): the columns of M64 grow apart by up to e^{6 dtau} per
+// slice, and the Gram matrix has to keep the small ones' diagonal (against the
+// block's largest element a pivot of free fermions, 72 sites, 10 slices of
+// dtau = 0.8, failed).  A thread holds its rows in registers between the search
+// and the packing.
 __global__ void __launch_bounds__(256) sp_digits_kernel(const ChainDesc* chains, int b, int tsize) {
+  __shared__ int red[8];
+  constexpr int kRows = kMaxN / 256;
+  static_assert(kMaxN % 256 == 0, "rows per thread");
   const ChainDesc& c = chains[blockIdx.z];
   if (c.st->err) return;
-  const int s = blockIdx.y, n = nsig_of(c, s), N = c.N, ldd = digit_ld(N);
+  const int s = blockIdx.y, n = nsig_of(c, s), N = c.N;
+  const int q = blockIdx.x >= c.nmax ? 1 : 0, k = blockIdx.x - q * c.nmax;
+  if (k >= n) return;
   SpBuf<double> sp = fp64_bufs(c, tsize);
-  const long stride = (long)gridDim.x * blockDim.x, e0 = blockIdx.x * (long)blockDim.x + threadIdx.x;
-  if (b < 0) {
-    const double* M = sp.m64(s);
-    unsigned long long* D = sp.dq(s, 0);
-    const int E = sp.em()[s];
-    for (long e = e0; e < (long)N * n; e += stride) {
-      const int k = (int)(e / N), i = (int)(e % N);
-      D[(long)k * ldd + i] = digit_pack(M[e], E);
-    }
-  } else {
-    const long off = ((long)b * 2 + s) * N * c.nmax;
-    bool bad = false;
-    for (int q = 0; q < 2; ++q) {
-      const double* Q = (q == 0 ? c.Lst : c.Rst) + off;
-      unsigned long long* D = sp.dq(s, q);
-      for (long e = e0; e < (long)N * n; e += stride) {
-        const int k = (int)(e / N), i = (int)(e % N);
-        const double v = Q[e];
-        bad |= digit_exp(v) > 1;
-        D[(long)k * ldd + i] = digit_pack(v, 1);
-      }
-    }
-    if (bad) atomicMax(sp.eq() + s, kDigitBad);
+  const double* col = (b < 0 ? sp.m64(s) : (q == 0 ? c.Lst : c.Rst) + ((long)b * 2 + s) * N * c.nmax) + (long)k * N;
+  double v[kRows];
+  int e = kDigitNone;
+#pragma unroll
+  for (int r = 0; r < kRows; ++r) {
+    const int i = threadIdx.x + 256 * r;
+    v[r] = i < N ? col[i] : 0.0;
+    e = max(e, digit_exp(v[r]));
   }
+  e = digit_cta_max(e, red);
+  unsigned long long* D = sp.dq(s, q) + (long)k * digit_ld(N);
+#pragma unroll
+  for (int r = 0; r < kRows; ++r) {
+    const int i = threadIdx.x + 256 * r;
+    if (i < N) D[i] = digit_pack(v[r], e);
+  }
+  if (threadIdx.x == 0) sp.dexp(s, q)[k] = e;
 }
 
 // One 32 x 32 block of the Gram matrix (b < 0, upper triangle) or of O per CTA
@@ -59,13 +60,14 @@ __global__ void __launch_bounds__(256) sp_digit_gemm_kernel(const ChainDesc* cha
   const int i0 = 32 * (int)(blockIdx.x / tn), j0 = 32 * (int)(blockIdx.x % tn);
   if (i0 >= n || j0 >= n || (b < 0 && i0 > j0)) return;
   SpBuf<double> sp = fp64_bufs(c, tsize);
+  const int qb = b < 0 ? 0 : 1;
   const unsigned long long* A = sp.dq(s, 0) + (long)i0 * ldd;
-  const unsigned long long* B = sp.dq(s, b < 0 ? 0 : 1) + (long)j0 * ldd;
+  const unsigned long long* B = sp.dq(s, qb) + (long)j0 * ldd;
+  const int* ea = sp.dexp(s, 0) + i0;
+  const int* eb = sp.dexp(s, qb) + j0;
   double* C = (b < 0 ? sp.c64(s) : sp.o64(s)) + (long)i0 * ldn + j0;
-  const int bad = b < 0 ? 0 : sp.eq()[s];
-  const int E = b < 0 ? sp.em()[s] : bad > 0 ? bad : 1;
-  auto ex = [E](int) { return E; };
-  digit_gemm<true, true>(min(32, n - i0), min(32, n - j0), N, A, ldd, 1, B, ldd, 1, ex, ex, false, false,
+  digit_gemm<true, true>(min(32, n - i0), min(32, n - j0), N, A, ldd, 1, B, ldd, 1, [ea](int i) { return ea[i]; },
+                         [eb](int j) { return eb[j]; }, false, false,
                          [C, ldn](int i, int j, double v) { C[(long)i * ldn + j] = v; });
 }
 
@@ -97,7 +99,6 @@ __global__ void __launch_bounds__(256) chol_panel_kernel(const ChainDesc* chains
     if (threadIdx.x == 0) {
       sp.bad()[s] = 0;
       sp.lchol()[s] = 0.0;
-      sp.em()[s] = kDigitNone;          // (the block's digits have been used: ready for the next block)
     }
   }
   __syncthreads();
@@ -406,7 +407,8 @@ cudaError_t sp_dgemm(SpGemm& g, int mode, int max_m, int max_n, cudaStream_t st)
 
 cudaError_t sp_digit_products(const ChainDesc* d, int nc, int N, int nmax, int b, int tsize, cudaStream_t st) {
   const int t = (nmax + 31) / 32;
-  sp_digits_kernel<<<dim3((unsigned)std::min(512, (N * nmax + 255) / 256), 2, nc), 256, 0, st>>>(d, b, tsize);
+  (void)N;
+  sp_digits_kernel<<<dim3((b < 0 ? 1 : 2) * nmax, 2, nc), 256, 0, st>>>(d, b, tsize);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   sp_digit_gemm_kernel<<<dim3(t * t, 2, nc), 256, 0, st>>>(d, b, tsize);

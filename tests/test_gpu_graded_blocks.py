@@ -44,3 +44,13 @@ def test_weight_of_graded_blocks_fp64(L, dtau):
         w = ctx.weight()
         assert abs(w[0] - exact[0]) < 1e-13 * abs(exact[0]) + 1e-13 and abs(w[2] - exact[1]) < 1e-13 * abs(exact[1]) + 1e-13, (w, exact)
         ctx.close()
+
+
+@pytest.mark.parametrize("L,dtau", [(3, 0.5), (6, 0.1), (6, 0.8), (9, 0.5)])
+def test_weight_of_graded_blocks_spread(L, dtau):
+    """The same by the whole-GPU sweep, whose factor comes from the Gram matrix."""
+    spec, exact = free(L, dtau)
+    ctx = pqmc.Context([spec], prec=pqmc.FP64, seed=1, n_stab=10, spread=1)
+    w = ctx.weight()
+    assert abs(w[0] - exact[0]) < 1e-13 * abs(exact[0]) + 1e-13 and abs(w[2] - exact[1]) < 1e-13 * abs(exact[1]) + 1e-13, (w, exact)
+    ctx.close()
