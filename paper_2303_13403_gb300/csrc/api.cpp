@@ -210,29 +210,6 @@ void put(Staged& a, size_t off, const std::vector<double>& src, int rows, int co
     for (int j = 0; j < cols; ++j) p[(size_t)i * ld + j] = (T)src[(size_t)i * cols + j];
 }
 
-// smallest E with |x| < 2^E for every x of v; kDigitBad when one is not finite
-int max_exponent(const std::vector<double>& v) {
-  int e = kDigitNone;
-  for (double x : v) {
-    if (!std::isfinite(x)) return kDigitBad;
-    int k = 0;
-    std::frexp(x, &k);
-    if (x != 0.0) e = std::max(e, k);
-  }
-  return e;
-}
-
-// Digits of an N x N matrix for digit_gemm.cuh: element (b, a) at
-// a digit_ld(N) + b, x = X 2^{E - 62} packed as X + 0x80...80 (a matrix that
-// is not finite has no digits: its exponent makes every product NaN).
-void pack_digits(uint64_t* dig, const std::vector<double>& m, int N, int E) {
-  const int ldd = digit_ld(N);
-  for (int a = 0; a < N; ++a)
-    for (int b = 0; b < N; ++b)
-      dig[(size_t)a * ldd + b] =
-          (E == kDigitBad ? 0 : (uint64_t)std::llround(std::ldexp(m[(size_t)b * N + a], 62 - E))) + kDigitZero;
-}
-
 void put_raw(Staged& a, size_t off, const void* src, size_t n) { memcpy(a.at(off, n), src, n); }
 
 pqmc_status sync_check(pqmc_ctx* ctx) {
@@ -370,8 +347,8 @@ pqmc_status build_ctx(int n, const pqmc_chain_spec* specs, const pqmc_opts* opts
       if (!sym_eig(h.N, mt.K, mt.w, mt.V)) { delete ctx; return fail(nullptr, PQMC_EINVAL, "eigensolver failed on K"); }
       expm_from_eig(h.N, mt.w, mt.V, -s.dtau, mt.expKm);
       expm_from_eig(h.N, mt.w, mt.V, +s.dtau, mt.expKp);
-      mt.eEm = max_exponent(mt.expKm);
-      mt.eEp = max_exponent(mt.expKp);
+      mt.eEm = digit_exponent(mt.expKm);
+      mt.eEp = digit_exponent(mt.expKp);
       models[key] = std::move(mt);
       const size_t Tm = (size_t)h.N * h.ld * ctx->tsize;
       const size_t o1 = take(Tm);
@@ -477,9 +454,9 @@ pqmc_status build_ctx(int n, const pqmc_chain_spec* specs, const pqmc_opts* opts
         put<double>(A, h.off_expKm, mt.expKm, h.N, h.N, h.ld);
         put<double>(A, h.off_expKp, mt.expKp, h.N, h.N, h.ld);
         const size_t tab = (size_t)h.N * digit_ld(h.N);
-        uint64_t* dig = reinterpret_cast<uint64_t*>(A.at(h.off_digits, 2 * tab * 8));
-        pack_digits(dig, mt.expKm, h.N, mt.eEm);
-        pack_digits(dig + tab, mt.expKp, h.N, mt.eEp);
+        unsigned long long* dig = reinterpret_cast<unsigned long long*>(A.at(h.off_digits, 2 * tab * 8));
+        digit_table(dig, mt.expKm, h.N, mt.eEm);
+        digit_table(dig + tab, mt.expKp, h.N, mt.eEp);
       } else {
         put<float>(A, h.off_expKm, mt.expKm, h.N, h.N, h.ld);
         put<float>(A, h.off_expKp, mt.expKp, h.N, h.N, h.ld);

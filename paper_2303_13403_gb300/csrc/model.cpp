@@ -1,6 +1,8 @@
 // Host-side FP64 model set-up (see model.h).
 #include "model.h"
 
+#include "chain.h"
+
 #include <algorithm>
 #include <limits>
 #include <cmath>
@@ -203,6 +205,25 @@ bool trial_orbitals(const Lattice& lat, const std::vector<double>& K, const std:
     for (int k = 0; k < n_sigma; ++k) P[(size_t)i * n_sigma + k] = V[(size_t)i * N + k];
   gap = n_sigma < N ? w[n_sigma] - w[n_sigma - 1] : INFINITY;
   return true;
+}
+
+int digit_exponent(const std::vector<double>& m) {
+  int e = kDigitNone;
+  for (double x : m) {
+    if (!std::isfinite(x)) return kDigitBad;
+    int k = 0;
+    std::frexp(x, &k);
+    if (x != 0.0) e = std::max(e, k);
+  }
+  return e;
+}
+
+void digit_table(unsigned long long* dig, const std::vector<double>& m, int N, int E) {
+  const int ldd = digit_ld(N);
+  for (int a = 0; a < N; ++a)
+    for (int b = 0; b < N; ++b)
+      dig[(size_t)a * ldd + b] =
+          (E == kDigitBad ? 0 : (unsigned long long)std::llround(std::ldexp(m[(size_t)b * N + a], 62 - E))) + kDigitZero;
 }
 
 double hs_coupling(double x) { return std::acosh(std::exp(0.5 * x)); }

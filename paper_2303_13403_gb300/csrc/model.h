@@ -36,6 +36,13 @@ bool trial_orbitals(const Lattice& lat, const std::vector<double>& K, const std:
                     double M_N, double tiebreak, int sigma, int n_sigma, std::vector<double>& P,
                     double& gap);
 
+// Digits of an N x N matrix (row-major) for digit_gemm.cuh: element (b, a) at
+// a digit_ld(N) + b, x = X 2^{E - 62} packed as X + 0x80...80, E =
+// digit_exponent(m) the smallest with |x| < 2^E for every element.  A matrix that is
+// not finite has no digits: its exponent, kDigitBad, makes every product NaN.
+int digit_exponent(const std::vector<double>& m);
+void digit_table(unsigned long long* dig, const std::vector<double>& m, int N, int E);
+
 // cosh(kappa) = exp(x / 2): the Ising coupling of Eq. (1) in the spin-channel
 // reading (x = g) and of the Trotterised U term (x = dtau U).
 double hs_coupling(double x);

@@ -180,10 +180,7 @@ extern "C" pqmc_status pqmc_green_noalloc(const pqmc_chain_spec* spec, int n_sta
   const size_t o_desc = take256(off, sizeof(ChainDesc));
   const size_t o_state = take256(off, sizeof(ChainState));
   const size_t o_err = take256(off, sizeof(int));
-  const size_t o_em = take256(off, (size_t)N * ld * 8);
-  const size_t o_ep = take256(off, (size_t)N * ld * 8);
-  const size_t o_em64 = take256(off, (size_t)N * N * 8);
-  const size_t o_k64 = take256(off, (size_t)N * N * 8);
+  const size_t o_em = take256(off, (size_t)N * digit_ld(N) * 8);
   const size_t o_P = take256(off, 2 * blk);
   const size_t upload = off;                   // everything above is uploaded each call
   const size_t o_rst = take256(off, (size_t)(nb + 1) * 2 * blk);
@@ -222,14 +219,13 @@ extern "C" pqmc_status pqmc_green_noalloc(const pqmc_chain_spec* spec, int n_sta
 
   // host model set-up (FP64), same as context creation
   Lattice lat{lt.kind, lt.Lx, lt.Ly, lt.t, lt.tp};
-  std::vector<double> K, eps, w, V, em, ep, P[2];
+  std::vector<double> K, eps, w, V, em, P[2];
   build_hopping(lat, K, eps);
   if (!sym_eig(N, K, w, V)) {
     set_init_error("pqmc_green_noalloc: eigensolver failed on K");
     return PQMC_EINVAL;
   }
   expm_from_eig(N, w, V, -spec->dtau, em);
-  expm_from_eig(N, w, V, +spec->dtau, ep);
   for (int sp = 0; sp < 2; ++sp) {
     double gap = 0;
     if (!trial_orbitals(lat, K, eps, spec->trial.M_N, spec->trial.tiebreak, sp == 0 ? 1 : -1, sp == 0 ? nup : ndn,
@@ -257,10 +253,9 @@ extern "C" pqmc_status pqmc_green_noalloc(const pqmc_chain_spec* spec, int n_sta
       }
   d.fields = const_cast<int8_t*>(d_fields);
   d.G = base + o_G;
-  d.expKm = base + o_em;
-  d.expKp = base + o_ep;
-  d.expKm64 = reinterpret_cast<const double*>(base + o_em64);
-  d.K64 = reinterpret_cast<const double*>(base + o_k64);
+  // (the only slice wrapped is a Gutzwiller slice: the stack products' table is enough)
+  d.dEm = reinterpret_cast<const unsigned long long*>(base + o_em);
+  d.eEm = digit_exponent(em);
   d.P = reinterpret_cast<const double*>(base + o_P);
   d.Rst = reinterpret_cast<double*>(base + o_rst);
   d.Lst = reinterpret_cast<double*>(base + o_lst);
@@ -273,15 +268,7 @@ extern "C" pqmc_status pqmc_green_noalloc(const pqmc_chain_spec* spec, int n_sta
   st.sign_running = 1.0;
   st.logw[0][1] = st.logw[1][1] = 1.0;
   memcpy(h.data() + o_state, &st, sizeof st);
-  double* hem = reinterpret_cast<double*>(h.data() + o_em);
-  double* hep = reinterpret_cast<double*>(h.data() + o_ep);
-  for (int i = 0; i < N; ++i)
-    for (int j = 0; j < N; ++j) {
-      hem[(size_t)i * ld + j] = em[(size_t)i * N + j];
-      hep[(size_t)i * ld + j] = ep[(size_t)i * N + j];
-    }
-  memcpy(h.data() + o_em64, em.data(), (size_t)N * N * 8);
-  memcpy(h.data() + o_k64, K.data(), (size_t)N * N * 8);
+  digit_table(reinterpret_cast<unsigned long long*>(h.data() + o_em), em, N, d.eEm);
   double* hP = reinterpret_cast<double*>(h.data() + o_P);
   for (int sp = 0; sp < 2; ++sp) {
     const int ns = sp == 0 ? nup : ndn;

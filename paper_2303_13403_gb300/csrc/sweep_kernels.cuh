@@ -2096,27 +2096,24 @@ __device__ __noinline__ void phase_stack(int b, int left, int s) {
   // digits' assembly it took 1.6% of a one-chain sweep of 18 sites.
   auto product = [&](const T* from, T* to) {
     if constexpr (f64) {
-      if (c.dEm) {
-        const int ldd = digit_ld(N), ldk = N + (N & 1), e1 = c.eEm;
-        unsigned long long* D = reinterpret_cast<unsigned long long*>(x.M64());
-        double* sc = x.qbeta();                        // (the QR's vectors come later)
-        for (int k = threadIdx.x >> 5; k < n; k += blockDim.x >> 5) {
-          int e = kDigitNone;
-          for (int i = threadIdx.x & 31; i < N; i += 32) e = max(e, digit_exp(from[(long)i * ldn + k]));
-          e = __reduce_max_sync(0xffffffffu, e);
-          for (int i = threadIdx.x & 31; i < N; i += 32) D[(long)k * ldk + i] = digit_pack(from[(long)i * ldn + k], e);
-          // (2^{e - 1}: every exponent's is a normal number)
-          if ((threadIdx.x & 31) == 0)
-            sc[k] = __longlong_as_double(e == kDigitBad ? 0x7ff8000000000000ll : e == kDigitNone ? 0ll : (long long)(e + 1022) << 52);
-        }
-        __syncthreads();
-        digit_gemm<true, true>(N, n, N, c.dEm, ldd, 1, D, ldk, 1, [e1](int) { return e1; }, [](int) { return 1; }, false,
-                               false, [to, ldn, sc](int i, int j, double v) { to[(long)i * ldn + j] = v * sc[j]; });
-        return;
+      const int ldd = digit_ld(N), ldk = N + (N & 1), e1 = c.eEm;
+      unsigned long long* D = reinterpret_cast<unsigned long long*>(x.M64());
+      double* sc = x.qbeta();                        // (the QR's vectors come later)
+      for (int k = threadIdx.x >> 5; k < n; k += blockDim.x >> 5) {
+        int e = kDigitNone;
+        for (int i = threadIdx.x & 31; i < N; i += 32) e = max(e, digit_exp(from[(long)i * ldn + k]));
+        e = __reduce_max_sync(0xffffffffu, e);
+        for (int i = threadIdx.x & 31; i < N; i += 32) D[(long)k * ldk + i] = digit_pack(from[(long)i * ldn + k], e);
+        // (2^{e - 1}: every exponent's is a normal number)
+        if ((threadIdx.x & 31) == 0)
+          sc[k] = __longlong_as_double(e == kDigitBad ? 0x7ff8000000000000ll : e == kDigitNone ? 0ll : (long long)(e + 1022) << 52);
       }
+      __syncthreads();
+      digit_gemm<true, true>(N, n, N, c.dEm, ldd, 1, D, ldk, 1, [e1](int) { return e1; }, [](int) { return 1; }, false,
+                             false, [to, ldn, sc](int i, int j, double v) { to[(long)i * ldn + j] = v * sc[j]; });
+    } else {
+      cta_gemm_f32<false>(N, n, N, x.Em(), c.ld, from, ldn, to, ldn, EpiStore());
     }
-    if constexpr (f64) cta_gemm<T>(N, n, N, x.Em(), 1, c.ld, from, ldn, 1, to, ldn, 1, EpiStore());
-    else cta_gemm_f32<false>(N, n, N, x.Em(), c.ld, from, ldn, to, ldn, EpiStore());
   };
   int src = 0;
   if (left ? b == c.nb : b == 0) {
