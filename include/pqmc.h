@@ -147,7 +147,9 @@ typedef struct {
                                device), and for the reduced paths 256, or 512 when a chain has 128
                                sites or more or when the batch has at most one chain per
                                SM and a chain of 64 sites or more. Smaller CTAs put more chains on one SM
-                               (FP64: 256/cta_threads per SM, others twice that) */
+                               (FP64: 256/cta_threads per SM, others twice that). A chain's fields, G,
+                               weight and records are the same bits with every size
+                               (BF16X3: with those of one wrap product, 512 or up to 256) */
     int dense_chains;       /* reduced paths only: kernels built for twice as many chains per SM
                                (fewer registers per thread); needs cta_threads 64 or 128 */
     int dg_fp64;            /* reduced paths only, diagnostic: nonzero makes the error recorded at

@@ -2443,11 +2443,34 @@ __device__ __forceinline__ void refresh(int b, bool record) {
   phase_assemble<T, RES>(b, record);
 }
 
-// Wick estimates on the fresh G at the middle slice: E/site for Eq. (2),
-// docc/site, kinetic/site, with the weight sign and the running sign, and the
-// staggered S^z structure factor S = (1/N^2) sum_ij eps_i eps_j <S^z_i S^z_j>
-// = [(sum_i eps_i m_i)^2 + sum_s sum_ij eps_i eps_j (delta_ij - G_s,ji) G_s,ij]
-// / (4 N^2), m_i = n_i,up - n_i,dn (the spins are independent at fixed fields).
+// Two sums over i, j < N of the terms that term(i, j, a, b) adds (collective): one
+// row at a time per warp, the rows' sums through the scratch (no phase's buffers
+// are in use), so that the order of the additions, and with it the last bit
+// of a record, does not depend on the number of threads, which the default takes
+// from the batch.  Lanes of warp 0 leave with parts to add up over the warp, in a and b.
+template <typename T, bool RES, typename F>
+__device__ __forceinline__ void row_sums(Cta<T, RES>& x, F term, double& a, double& b) {
+  const int N = x.c.N, lane = threadIdx.x & 31;
+  double* rows = reinterpret_cast<double*>(x.scr);     // 2 N of them: less than any phase holds
+  __syncthreads();
+  for (int i = threadIdx.x >> 5; i < N; i += blockDim.x >> 5) {
+    double p = 0.0, q = 0.0;
+    for (int j = lane; j < N; j += 32) term(i, j, p, q);
+    p = warp_sum(p);
+    q = warp_sum(q);
+    if (lane == 0) {
+      rows[2 * i] = p;
+      rows[2 * i + 1] = q;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < 32)
+    for (int i = lane; i < N; i += 32) {
+      a += rows[2 * i];
+      b += rows[2 * i + 1];
+    }
+}
+
 // Wick estimates of the spinless t-V model on the fresh G at the middle
 // slice: E/site of Eq. (4), interaction energy/site
 // V sum_<ij> [(n_i - 1/2)(n_j - 1/2) - G_ji G_ij] / N, kinetic/site, the weight
@@ -2460,21 +2483,23 @@ __device__ __forceinline__ void measure_tv(Cta<T, RES>& x) {
   const int N = c.N, ld = c.ld;
   const T* G = x.G(0);
   double ek = 0.0, eb = 0.0, st = 0.0, ex = 0.0;
-  PQMC_FOR_2D(i, 0, N, j, 0, N) {
+  row_sums(x, [&](int i, int j, double& k, double& e) {
     const double gji = (i == j ? 1.0 : 0.0) - (double)G[(long)j * ld + i];
-    ek += c.K64[(long)i * N + j] * gji;
-    ex += c.eps[i] * c.eps[j] * gji * (double)G[(long)i * ld + j];
+    k += c.K64[(long)i * N + j] * gji;
+    e += c.eps[i] * c.eps[j] * gji * (double)G[(long)i * ld + j];
+  }, ek, ex);
+  if (threadIdx.x < 32) {
+    for (int i = threadIdx.x; i < N; i += 32) st += c.eps[i] * (0.5 - (double)G[(long)i * ld + i]);
+    for (int b = threadIdx.x; b < c.nfld; b += 32) {
+      const int i = c.bond_ends[2 * b], j = c.bond_ends[2 * b + 1];
+      const double di = 0.5 - (double)G[(long)i * ld + i], dj = 0.5 - (double)G[(long)j * ld + j];
+      eb += di * dj - (double)G[(long)j * ld + i] * (double)G[(long)i * ld + j];
+    }
+    ek = warp_sum(ek);
+    eb = warp_sum(eb) * c.U;
+    st = warp_sum(st);
+    ex = warp_sum(ex);
   }
-  for (int i = threadIdx.x; i < N; i += blockDim.x) st += c.eps[i] * (0.5 - (double)G[(long)i * ld + i]);
-  for (int b = threadIdx.x; b < c.nfld; b += blockDim.x) {
-    const int i = c.bond_ends[2 * b], j = c.bond_ends[2 * b + 1];
-    const double di = 0.5 - (double)G[(long)i * ld + i], dj = 0.5 - (double)G[(long)j * ld + j];
-    eb += di * dj - (double)G[(long)j * ld + i] * (double)G[(long)i * ld + j];
-  }
-  ek = cta_sum(ek, sh.red);
-  eb = cta_sum(eb, sh.red) * c.U;
-  st = cta_sum(st, sh.red);
-  ex = cta_sum(ex, sh.red);
   if (threadIdx.x == 0) {
     const int m = c.st->n_meas;
     const double rec[kRecord] = {sh.sign_spin[0] * sh.sign_spin[1], (ek + eb) / N, eb / N, ek / N,
@@ -2488,6 +2513,11 @@ __device__ __forceinline__ void measure_tv(Cta<T, RES>& x) {
   __syncthreads();
 }
 
+// Wick estimates on the fresh G at the middle slice: E/site for Eq. (2),
+// docc/site, kinetic/site, with the weight sign and the running sign, and the
+// staggered S^z structure factor S = (1/N^2) sum_ij eps_i eps_j <S^z_i S^z_j>
+// = [(sum_i eps_i m_i)^2 + sum_s sum_ij eps_i eps_j (delta_ij - G_s,ji) G_s,ij]
+// / (4 N^2), m_i = n_i,up - n_i,dn (the spins are independent at fixed fields).
 // grid_sums: the sums over i, j (ek, ex) formed elsewhere, n_sums pairs to add
 // up (a chain swept by the whole GPU), or null.
 template <typename T, bool RES>
@@ -2501,30 +2531,32 @@ __device__ __forceinline__ void measure(Cta<T, RES>& x, const double* grid_sums 
   const int N = c.N, ld = c.ld;
   double ek = 0.0, dc = 0.0, st = 0.0, ex = 0.0;
   if (grid_sums) {
-    for (int q = threadIdx.x; q < n_sums; q += blockDim.x) {
+    for (int q = threadIdx.x < 32 ? (int)threadIdx.x : n_sums; q < n_sums; q += 32) {
       ek += grid_sums[2 * q];
       ex += grid_sums[2 * q + 1];
     }
   } else {
-    PQMC_FOR_2D(i, 0, N, j, 0, N) {
+    row_sums(x, [&](int i, int j, double& kin, double& stag) {
       const double k = c.K64[(long)i * N + j];
       const double ee = c.eps[i] * c.eps[j];
       for (int s = 0; s < 2; ++s) {
         const double gji = (i == j ? 1.0 : 0.0) - (double)x.G(s)[(long)j * ld + i];
-        ek += k * gji;
-        ex += ee * gji * (double)x.G(s)[(long)i * ld + j];
+        kin += k * gji;
+        stag += ee * gji * (double)x.G(s)[(long)i * ld + j];
       }
+    }, ek, ex);
+  }
+  if (threadIdx.x < 32) {
+    for (int i = threadIdx.x; i < N; i += 32) {
+      const double g0 = (double)x.G(0)[(long)i * ld + i], g1 = (double)x.G(1)[(long)i * ld + i];
+      dc += (1.0 - g0) * (1.0 - g1);
+      st += c.eps[i] * (g1 - g0);
     }
+    ek = warp_sum(ek);
+    dc = warp_sum(dc);
+    st = warp_sum(st);
+    ex = warp_sum(ex);
   }
-  for (int i = threadIdx.x; i < N; i += blockDim.x) {
-    const double g0 = (double)x.G(0)[(long)i * ld + i], g1 = (double)x.G(1)[(long)i * ld + i];
-    dc += (1.0 - g0) * (1.0 - g1);
-    st += c.eps[i] * (g1 - g0);
-  }
-  ek = cta_sum(ek, sh.red);
-  dc = cta_sum(dc, sh.red);
-  st = cta_sum(st, sh.red);
-  ex = cta_sum(ex, sh.red);
   if (threadIdx.x == 0) {
     const int m = c.st->n_meas;
     const double rec[kRecord] = {sh.sign_spin[0] * sh.sign_spin[1], (ek + c.U * dc) / N, dc / N, ek / N,
