@@ -435,6 +435,11 @@ pqmc_status pqmc_test_tc_gemm(int M, int N, int K, const float* d_A, int trans_a
 pqmc_status pqmc_test_digit_gemm(int M, int N, int K, const double* d_A, const double* d_B, double* d_C, int strided,
                                  void* stream);
 
+/* Test hook of the reciprocal that the stabilisation takes of its pivots (no
+ * counterpart in the paper): y_i = 1 / x_i for n FP64 values (device pointers)
+ * on `stream` (NULL: the legacy default stream), which it synchronises. */
+pqmc_status pqmc_test_recip(int n, const double* d_x, double* d_y, void* stream);
+
 /* Error bar of the sign-reweighted estimator <s O>/<s> of the Method
  * section, as pqmc_measure computes it: the records are split into n_groups
  * groups (bins of consecutive sweeps of one chain, or whole chains when

@@ -120,6 +120,13 @@ __global__ void __launch_bounds__(256, 1) digit_gemm_test_kernel(int M, int N, i
 }
 
 // --------------------------------------------------------------------------
+// Test kernel of the pivots' reciprocal (pqmc_test_recip).
+
+__global__ void recip_test_kernel(int n, const double* x, double* y) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) y[i] = recip64(x[i]);
+}
+
+// --------------------------------------------------------------------------
 // Allocation-free initialisation of one chain (pqmc_green_noalloc).
 //
 // Runs init_kernel for a single FP64 chain with every buffer the kernel needs
@@ -356,6 +363,23 @@ extern "C" pqmc_status pqmc_test_digit_gemm(int M, int N, int K, const double* d
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) {
     set_init_error(std::string("pqmc_test_digit_gemm: ") + cudaGetErrorString(e));
+    return PQMC_ECUDA;
+  }
+  return PQMC_OK;
+}
+
+extern "C" pqmc_status pqmc_test_recip(int n, const double* d_x, double* d_y, void* stream) {
+  using namespace pqmc;
+  if (n < 1 || !d_x || !d_y) {
+    set_init_error("pqmc_test_recip: bad size or NULL pointer");
+    return PQMC_EINVAL;
+  }
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  recip_test_kernel<<<64, 256, 0, st>>>(n, d_x, d_y);
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) {
+    set_init_error(std::string("pqmc_test_recip: ") + cudaGetErrorString(e));
     return PQMC_ECUDA;
   }
   return PQMC_OK;

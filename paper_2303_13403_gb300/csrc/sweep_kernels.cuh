@@ -1660,10 +1660,13 @@ __device__ __forceinline__ void qr_householder(Cta<T, RES>& x, int N, int ldm, i
   x.mark(kPhQRForm);
 }
 
-// 1 / x: the hardware's approximation (about 20 bits) and one step
-// y <- y + y (e + e^2), e = 1 - x y, of third order: three dependent FMAs (65
-// cycles each) where the division takes 646; outside the approximation's
-// range the division.
+// 1 / x by the geometric series: with y an approximation and e = 1 - x y,
+// 1 / x = y / (1 - e) = y (1 + e + e^2 + ...); cut after e^2, which is Chebyshev's
+// third-order iteration for the root of 1 / y - x (Householder, The Numerical
+// Treatment of a Single Nonlinear Equation, 1970).  y is PTX's
+// rcp.approx.ftz.f64, good to some 20 bits, so the terms left out are below 2^-60 and the result
+// is within 0.5 + 2^-6 ulp.  Three dependent FMAs (65 cycles each) where the division takes
+// 646 cycles on the pivots' serial chain; outside the approximation's range the division.
 static __device__ __forceinline__ double recip64(double x) {
   const int e = (__double2hiint(x) >> 20) & 0x7ff;
   if (e < 60 || e > 1980) return 1.0 / x;

@@ -113,6 +113,7 @@ SIGNATURES = [
                                     C.c_void_p]),
     ("pqmc_test_digit_gemm", C.c_int, [C.c_int, C.c_int, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p, C.c_int,
                                        C.c_void_p]),
+    ("pqmc_test_recip", C.c_int, [C.c_int, C.c_void_p, C.c_void_p, C.c_void_p]),
 ]
 
 
@@ -370,6 +371,11 @@ def test_digit_gemm(M, N, K, d_A, d_B, d_C, strided=False, stream=None):
     """pqmc_test_digit_gemm: device pointers (ints); C = A B in FP64 by the tensor-core digit product."""
     _check(load().pqmc_test_digit_gemm(M, N, K, C.c_void_p(d_A), C.c_void_p(d_B), C.c_void_p(d_C),
                                        1 if strided else 0, C.c_void_p(stream) if stream else None))
+
+
+def test_recip(n, d_x, d_y, stream=None):
+    """pqmc_test_recip: device pointers (ints); y = 1 / x as the stabilisation takes it."""
+    _check(load().pqmc_test_recip(n, C.c_void_p(d_x), C.c_void_p(d_y), C.c_void_p(stream) if stream else None))
 
 
 def host_jackknife(sO, s):
