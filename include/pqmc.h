@@ -383,7 +383,9 @@ typedef struct {
  * key made of the precision, n_stab, the fixed options and the multiset of
  * chain shapes (N, N_up, N_dn, Ltau, model); with the environment variable
  * PQMC_AUTOTUNE_CACHE naming a file, the cache is also read from and written
- * to that file as JSON.  pqmc_init / pqmc_init_batch call this when
+ * to that file as JSON.  A file's pick carries the build of the library that
+ * timed it and is timed again by another build; a pick without a build is
+ * taken as it stands.  pqmc_init / pqmc_init_batch call this when
  * opts->delay_k is 0.  Allocates a temporary context (device memory).
  * PQMC_EINVAL for bad specs or options, PQMC_ECUDA when no candidate ran. */
 pqmc_status pqmc_autotune(int n, const pqmc_chain_spec* specs, const pqmc_opts* opts, pqmc_tune* out);

@@ -1,4 +1,5 @@
 """Build libpqmc.so in-tree for sm_103a (nvcc + g++, translation units compiled in parallel)."""
+import hashlib
 import os
 import subprocess
 import sys
@@ -16,6 +17,15 @@ CU_SOURCES = ["sweep.cu", "sweep_f64.cu", "sweep_f32.cu", "sweep_f32_256.cu", "s
 CPP_SOURCES = ["api.cpp", "model.cpp"]
 
 
+def build_id():
+    """Hash of the sources: the autotuner's cache holds timings of one build."""
+    h = hashlib.sha1()
+    for f in sorted(os.listdir(CSRC)):
+        with open(os.path.join(CSRC, f), "rb") as fh:
+            h.update(f.encode() + fh.read())
+    return h.hexdigest()[:12]
+
+
 def _cmds():
     os.makedirs(OUT_DIR, exist_ok=True)
     inc = ["-I" + CSRC, "-I" + os.path.join(os.path.dirname(HERE), "include"), "-I" + os.path.join(CUDA, "include")]
@@ -27,7 +37,7 @@ def _cmds():
         objs.append(o)
     for s in CPP_SOURCES:
         o = os.path.join(OUT_DIR, s + ".o")
-        cmds.append(["g++", "-O2", "-std=c++17", "-fPIC", "-Wall", *inc, "-c", os.path.join(CSRC, s), "-o", o])
+        cmds.append(["g++", "-O2", "-std=c++17", "-fPIC", "-Wall", '-DPQMC_BUILD_ID="%s"' % build_id(), *inc, "-c", os.path.join(CSRC, s), "-o", o])
         objs.append(o)
     link = [NVCC, *ARCH, "-shared", "-cudart", "shared", "-o", LIB, *objs,
             "-Xlinker", "-rpath," + os.path.join(CUDA, "lib64")]

@@ -688,13 +688,18 @@ std::string tune_key(int n, const pqmc_chain_spec* specs, const pqmc_opts& o) {
   return k.str();
 }
 
-struct TuneEntry { int delay_k, cta_threads; double ms; };
+// (build: the build that timed the pick; empty for one that a file gives without)
+#ifndef PQMC_BUILD_ID
+#define PQMC_BUILD_ID "0"
+#endif
+struct TuneEntry { int delay_k, cta_threads; double ms; std::string build; };
 std::mutex g_tune_mu;
 std::map<std::string, TuneEntry> g_tune;
 bool g_tune_file_read = false;
 
-// the JSON cache: an object of {"key": {"delay_k": k, "cta_threads": t, "ms_per_sweep": m}}
-// entries (whitespace anywhere; keys hold no quotes)
+// the JSON cache: an object of {"key": {"delay_k": k, "cta_threads": t, "ms_per_sweep": m, "build": "b"}}
+// entries (whitespace anywhere; keys hold no quotes).  A pick that another build
+// has timed is left aside: its kernels were others.  One without a build stands.
 void tune_file_read(const char* path) {
   std::ifstream f(path);
   std::stringstream ss;
@@ -724,9 +729,16 @@ void tune_file_read(const char* path) {
     if (e == std::string::npos) break;
     const std::string key = txt.substr(q0 + 1, q1 - q0 - 1), obj = txt.substr(b, e - b + 1);
     double k = 0, t = 0, m = NAN;
-    if (field(obj, "delay_k", k) && field(obj, "cta_threads", t)) {
+    std::string build;
+    const size_t bp = obj.find("\"build\"");
+    if (bp != std::string::npos) {
+      const size_t c = obj.find(':', bp);
+      const size_t b0 = c == std::string::npos ? c : obj.find('"', c), b1 = b0 == std::string::npos ? b0 : obj.find('"', b0 + 1);
+      if (b1 != std::string::npos) build = obj.substr(b0 + 1, b1 - b0 - 1);
+    }
+    if (field(obj, "delay_k", k) && field(obj, "cta_threads", t) && (bp == std::string::npos || build == PQMC_BUILD_ID)) {
       field(obj, "ms_per_sweep", m);
-      const TuneEntry te{(int)k, (int)t, m >= 0 ? m : NAN};
+      const TuneEntry te{(int)k, (int)t, m >= 0 ? m : NAN, build};
       if (valid_delay(te.delay_k) && te.cta_threads > 0 && !g_tune.count(key)) g_tune[key] = te;
     }
     pos = e + 1;
@@ -739,9 +751,11 @@ void tune_file_write(const char* path) {
   size_t i = 0;
   for (auto& kv : g_tune) {
     char buf[160];
-    snprintf(buf, sizeof buf, "{\"delay_k\": %d, \"cta_threads\": %d, \"ms_per_sweep\": %.6g}", kv.second.delay_k,
+    snprintf(buf, sizeof buf, "{\"delay_k\": %d, \"cta_threads\": %d, \"ms_per_sweep\": %.6g", kv.second.delay_k,
              kv.second.cta_threads, std::isfinite(kv.second.ms) ? kv.second.ms : -1.0);
-    f << "  \"" << kv.first << "\": " << buf << (++i < g_tune.size() ? ",\n" : "\n");
+    f << "  \"" << kv.first << "\": " << buf;
+    if (!kv.second.build.empty()) f << ", \"build\": \"" << kv.second.build << "\"";
+    f << "}" << (++i < g_tune.size() ? ",\n" : "\n");
   }
   f << "}\n";
 }
@@ -820,7 +834,7 @@ pqmc_status autotune_cached(int n, const pqmc_chain_spec* specs, const pqmc_opts
   const pqmc_status st = autotune_run(n, specs, o, out);
   if (st != PQMC_OK) return st;
   std::lock_guard<std::mutex> lk(g_tune_mu);
-  g_tune[key] = TuneEntry{out->delay_k, out->cta_threads, out->ms_per_sweep};
+  g_tune[key] = TuneEntry{out->delay_k, out->cta_threads, out->ms_per_sweep, PQMC_BUILD_ID};
   if (path && *path) tune_file_write(path);
   return PQMC_OK;
 }
