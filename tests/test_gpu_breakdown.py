@@ -77,3 +77,40 @@ def test_overflowing_exponential_is_reported():
         ctx.synchronize()
     assert e.value.status == pqmc.ENAN
     ctx.close()
+
+
+# (L, N_up, N_dn, sites of field +1): spin up breaks when these are fewer than N_up, spin down when the others
+# are fewer than N_dn
+BROKEN = [(3, 9, 9, 6), (3, 9, 9, 12), (3, 11, 11, 9), (6, 36, 36, 30), (6, 36, 36, 42), (6, 38, 38, 36), (6, 38, 34, 36),
+          (6, 34, 38, 36), (9, 81, 81, 75), (9, 81, 81, 87)]
+
+
+@pytest.mark.parametrize("prec", [pqmc.FP32, pqmc.BF16X3])
+@pytest.mark.parametrize("tpb", [64, 256, 512])
+@pytest.mark.parametrize("L,n_up,n_dn,plus", BROKEN)
+def test_reduced_paths_fall_back_to_householder(L, n_up, n_dn, plus, tpb, prec):
+    """One spin's block or both spins' beyond the Cholesky QR, in shared memory
+    and (162 sites) global memory: G at tau = 0 and the weights of the FP64 path.
+    Both end slices hold the same fields, so Q_L and Q_R span one space and G is
+    1 minus a projector with elements of at most 1: three FP32 roundings and two
+    sums of n terms, 2 (n + 3) 2^-24 = 1e-5 at n = 81."""
+    spec = vmc(L, 18.0, n_up=n_up, n_dn=n_dn)
+    rng = np.random.default_rng(plus)
+    f = np.full(spec.n_sites, -1, np.int8)
+    f[rng.permutation(spec.n_sites)[:plus]] = 1
+    fields = np.stack([f, f])
+    m = model_of(spec)
+    for sg, broken in ((1, plus < n_up), (-1, spec.n_sites - plus < n_dn)):
+        pivot = smallest_pivot(m, fields, sg)
+        assert pivot < 1e-13 if broken else pivot > 1e-10
+    out = []
+    for p, threads in ((pqmc.FP64, 0), (prec, tpb)):
+        ctx = pqmc.Context([spec], prec=p, seed=1, n_stab=1, cta_threads=threads)
+        ctx.set_fields(fields)
+        out.append(([ctx.green_at(0, 0, s) for s in (0, 1)], ctx.weight()))
+        ctx.close()
+    (G64, w64), (G, w) = out
+    for s in (0, 1):
+        assert np.abs(G64[s]).max() < 1 + 1e-6
+        assert np.abs(G[s] - G64[s]).max() < 1e-5
+    assert np.allclose(w, w64, rtol=0, atol=1e-6)
