@@ -56,7 +56,7 @@ struct HostChain {
   pqmc_chain_spec spec;
   int N, ld, nup, ndn, nmax, Ltau, nb, nfld;
   size_t off_fields, off_G, off_Rst, off_Lst, off_Rlog, off_Llog, off_meas, off_dG,
-      off_acc, off_state, off_P, off_scratch, off_expKm, off_expKp, off_digits, off_expKm64, off_K64, off_eps, off_bonds,
+      off_acc, off_state, off_P, off_scratch, off_expKm, off_expKp, off_digits, off_K64, off_eps, off_bonds,
       off_sbonds, off_spread;
 };
 
@@ -355,7 +355,6 @@ pqmc_status build_ctx(int n, const pqmc_chain_spec* specs, const pqmc_opts* opts
       take(Tm);
       if (ctx->prec == PQMC_FP64) take(2 * (size_t)h.N * digit_ld(h.N) * 8);   // digits of e^{-+dtau K}
       take((size_t)h.N * h.N * 8);
-      take((size_t)h.N * h.N * 8);
       take((size_t)h.N * 8);
       take((size_t)h.N * 3 * 4);             // bond ends (3N/2 x 2 int)
       take((size_t)h.N * 3 * 4);             // site bonds (N x 3 int)
@@ -383,8 +382,7 @@ pqmc_status build_ctx(int n, const pqmc_chain_spec* specs, const pqmc_opts* opts
     h.off_expKm = model_off[key];
     h.off_expKp = h.off_expKm + align_up((size_t)h.N * h.ld * ctx->tsize, 256);
     h.off_digits = h.off_expKp + align_up((size_t)h.N * h.ld * ctx->tsize, 256);
-    h.off_expKm64 = h.off_digits + (ctx->prec == PQMC_FP64 ? align_up(2 * (size_t)h.N * digit_ld(h.N) * 8, 256) : 0);
-    h.off_K64 = h.off_expKm64 + align_up((size_t)h.N * h.N * 8, 256);
+    h.off_K64 = h.off_digits + (ctx->prec == PQMC_FP64 ? align_up(2 * (size_t)h.N * digit_ld(h.N) * 8, 256) : 0);
     h.off_eps = h.off_K64 + align_up((size_t)h.N * h.N * 8, 256);
     h.off_bonds = h.off_eps + align_up((size_t)h.N * 8, 256);
     h.off_sbonds = h.off_bonds + align_up((size_t)h.N * 3 * 4, 256);
@@ -461,7 +459,6 @@ pqmc_status build_ctx(int n, const pqmc_chain_spec* specs, const pqmc_opts* opts
         put<float>(A, h.off_expKm, mt.expKm, h.N, h.N, h.ld);
         put<float>(A, h.off_expKp, mt.expKp, h.N, h.N, h.ld);
       }
-      put<double>(A, h.off_expKm64, mt.expKm, h.N, h.N, h.N);
       put<double>(A, h.off_K64, mt.K, h.N, h.N, h.N);
       put_raw(A, h.off_eps, mt.eps.data(), (size_t)h.N * 8);
       if (is_tv(s)) {
@@ -542,7 +539,6 @@ pqmc_status build_ctx(int n, const pqmc_chain_spec* specs, const pqmc_opts* opts
       d.eEm = mt.eEm;
       d.eEp = mt.eEp;
     }
-    d.expKm64 = reinterpret_cast<const double*>(b + h.off_expKm64);
     d.K64 = reinterpret_cast<const double*>(b + h.off_K64);
     d.eps = reinterpret_cast<const double*>(b + h.off_eps);
     d.bond_ends = reinterpret_cast<const int*>(b + h.off_bonds);
@@ -592,7 +588,6 @@ pqmc_status build_ctx(int n, const pqmc_chain_spec* specs, const pqmc_opts* opts
   if (e == cudaSuccess) e = upload_run_order(ctx);
   if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_err, 0, 2 * sizeof(int), ctx->stream);
   if (e == cudaSuccess) e = prepare_sweep(ctx->prec, ctx->tpb, ctx->boost, ctx->res_bytes);
-  if (e == cudaSuccess && ctx->spread) e = spread_prepare();
   if (e != cudaSuccess) { pqmc_free(ctx); return cuda_fail(nullptr, e, "upload"); }
   if (ctx->spread) {
     e = spread_init(ctx->plan, ctx->stream);

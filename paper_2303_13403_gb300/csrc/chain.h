@@ -63,7 +63,6 @@ struct ChainDesc {
   void* G;                 // 2 x N x ld (T)
   const void* expKm;       // N x ld (T): e^{-dtau K}
   const void* expKp;       // N x ld (T): e^{+dtau K}
-  const double* expKm64;   // N x N FP64
   const unsigned long long* dEm;  // FP64 path: packed digits of e^{-dtau K}, element (b, a) at a digit_ld(N) + b, or null
   const unsigned long long* dEp;  // the same of e^{+dtau K}
   int eEm, eEp;            // their exponents
@@ -133,7 +132,7 @@ PQMC_HDI constexpr size_t al16(size_t v) { return (v + 15) & ~(size_t)15; }
 // sweep_kernels.cuh.
 PQMC_HDI constexpr size_t flipbuf_bytes(int tsize) {
   return al16(2 * (size_t)kBlock * (kBlock + 1) * tsize + 2 * (size_t)kBlock * tsize +
-              4 * (size_t)kMaxDelay * tsize + 2 * (size_t)kMaxDelay * 4);
+              4 * (size_t)kMaxDelay * tsize + (size_t)kMaxDelay * 4);
 }
 
 // kd: the delayed-update block of the chain (its update vectors are sized

@@ -39,7 +39,4 @@ cudaError_t spread_sweep(const SpreadPlan& p, int parity, int measure, cudaStrea
 // right block 0, G at tau = -1, running sign) with the same kernels.
 cudaError_t spread_init(const SpreadPlan& p, cudaStream_t stream);
 
-// Kernel attributes of the spread sequence (once per process, before capture).
-cudaError_t spread_prepare();
-
 }  // namespace pqmc

@@ -433,8 +433,6 @@ cudaError_t sp_gj_panel(const ChainDesc* d, int nc, int nmax, int p, int tsize, 
   return cudaGetLastError();
 }
 
-cudaError_t spread_prepare() { return cudaSuccess; }
-
 cudaError_t sp_gj_unswap(const ChainDesc* d, int nc, int nmax, int tsize, cudaStream_t st) {
   gj_unswap_kernel<<<dim3((nmax + 127) / 128, 2, nc), 128, 0, st>>>(d, tsize);
   return cudaGetLastError();

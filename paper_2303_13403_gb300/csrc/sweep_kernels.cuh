@@ -404,7 +404,6 @@ struct FlipBuf {
   T rs[2][kBlock];                  // ratio R_sigma of each proposal of the decision sub-block
   T cl[2][kMaxDelay];               // Delta of each accepted flip of the delayed block (diagonal of Gamma)
   T fr[2][kMaxDelay];               // Delta / R_sigma of each accepted flip
-  int sites[kMaxDelay];             // (unused slot kept for the layout)
   int gsite[kMaxDelay];             // site of each accepted flip
 };
 static_assert(sizeof(FlipBuf<double>) <= flipbuf_bytes(8) && sizeof(FlipBuf<float>) <= flipbuf_bytes(4),
@@ -424,7 +423,6 @@ struct Smem {
   long long t_mark;
   signed char fr[kMaxN];            // fields of the staged slice
   int na;                           // accepted flips in the block
-  int piv;
   int nswap[2];
   int chol_bad[2];                  // the spin's Cholesky factor broke down
   int fperm[kBlock];                // row interchanges of the flush inverse (t-V)
@@ -549,7 +547,7 @@ __device__ __forceinline__ Cta<T, RES> this_cta() {
   }
 }
 
-// Product of the wrap in the path's arithmetic.  On the BF16X3 path it runs
+// Product of the reduced paths' wrap.  On the BF16X3 path it runs
 // as split-precision tensor-core products: tcgen05 MMAs into tensor memory
 // when the CTA holds a staging area for them (kTc: 512-thread CTAs, a chain
 // kept in global memory; a kernel that holds tcgen05 code runs one CTA per
@@ -557,28 +555,23 @@ __device__ __forceinline__ Cta<T, RES> this_cta() {
 // delayed update is a rank-a correction (a <= 64) whose cost is reading and
 // writing G: it runs in FP32 on the CUDA cores on the BF16X3 path too
 // (measured faster than either tensor-core form at 162-648 sites, and exact
-// to FP32).  FP32 and FP64 paths: CUDA-core FMA.
+// to FP32).  FP32 path: CUDA-core FMA.
 // kRowA: A is row-major (ld ld), else A(i, k) = A[i + k ld].
-template <bool kTc, bool kRowA, typename T, bool RES, typename Epi>
-__device__ __forceinline__ void wrap_gemm(Cta<T, RES>& x, int n, const T* A, const T* B, T* C, int ld, Epi epi) {
-  constexpr bool f32 = std::is_same<T, float>::value;
+template <bool kTc, bool kRowA, bool RES, typename Epi>
+__device__ __forceinline__ void wrap_gemm(Cta<float, RES>& x, int n, const float* A, const float* B, float* C, int ld, Epi epi) {
   const int sai = kRowA ? ld : 1, sak = kRowA ? 1 : ld;
-  if constexpr (f32) {
-    if (x.c.tc) {
-      if constexpr (kTc && !RES) {
-        if (x.sh.tcs_off) {
-          cta_gemm_tc(n, n, n, A, sai, sak, B, ld, 1, C, ld, 1, epi, x.tcs(), x.sh.tmem, &x.sh.err, kErrTimeout);
-          __syncthreads();
-          return;
-        }
+  if (x.c.tc) {
+    if constexpr (kTc && !RES) {
+      if (x.sh.tcs_off) {
+        cta_gemm_tc(n, n, n, A, sai, sak, B, ld, 1, C, ld, 1, epi, x.tcs(), x.sh.tmem, &x.sh.err, kErrTimeout);
+        __syncthreads();
+        return;
       }
-      cta_gemm_bf16x3(n, n, n, A, sai, sak, B, ld, 1, C, ld, 1, epi);
-      return;
     }
-    cta_gemm_f32<kRowA>(n, n, n, A, ld, B, ld, C, ld, epi);
-  } else {
-    cta_gemm<T>(n, n, n, A, sai, sak, B, ld, 1, C, ld, 1, epi);
+    cta_gemm_bf16x3(n, n, n, A, sai, sak, B, ld, 1, C, ld, 1, epi);
+    return;
   }
+  cta_gemm_f32<kRowA>(n, n, n, A, ld, B, ld, C, ld, epi);
 }
 
 // --------------------------------------------------------------------------
@@ -711,13 +704,13 @@ __device__ __forceinline__ void block_inverse(Cta<T, RES>& x, int a, bool pivot)
 }
 
 template <typename T, bool RES>
-__device__ __forceinline__ void flush_block(Cta<T, RES>& x, int a, bool pivot) {
+__device__ __forceinline__ void flush_block(Cta<T, RES>& x, int a) {
   const ChainDesc& c = x.c;
   FlipBuf<T>& fb = *x.fb;
   const int N = c.N, ld = c.ld, ldu = x.ldu(), ns = x.nspec();
   T* Ubuf = x.Ub();                                    // kBlock x N  (U column-major, ld N)
   T* Wbuf = x.Wb();                                    // kBlock x ld (rows G_{S,:})
-  block_inverse(x, a, pivot);
+  block_inverse(x, a, true);
   // per species: A_S = E_S - G_{:,S} (N x a, column-major) and W = G_{S,:}
   // (a x N) gathered before G changes, then MW = M W and G -= A_S MW
   T* MW = reinterpret_cast<T*>(x.scr + x.L.mw);
@@ -1428,7 +1421,7 @@ __device__ __forceinline__ void update_slice_tv(Cta<T, RES>& x, int tau, uint32_
       x.mark(kPhFlip);
       const int a = sh.na;
       if (a == 0) continue;
-      flush_block(x, a, true);
+      flush_block(x, a);
     }
   }
 }
@@ -1468,36 +1461,48 @@ __device__ __forceinline__ void wrap_digits(Cta<T, RES>& x, int s, const unsigne
   __syncthreads();
 }
 
-template <bool kTc, typename T, bool RES>
-__device__ __forceinline__ void wrap(Cta<T, RES>& x, int tau, int dir) {
+// e^{V} G_s e^{-V} (dir > 0) or e^{-V} G_s e^{V}, slice tau staged
+template <typename T, bool RES>
+__device__ __forceinline__ void scale_slice(Cta<T, RES>& x, int tau, int dir, int s) {
+  const int N = x.c.N, ld = x.c.ld;
+  T* G = x.G(s);
+  if (dir > 0) {
+    PQMC_FOR_2D(i, 0, N, j, 0, N) G[(long)i * ld + j] *= x.vexpT(tau, s, i) * x.vinvT(tau, s, j);
+  } else {
+    PQMC_FOR_2D(i, 0, N, j, 0, N) G[(long)i * ld + j] *= x.vexpT(tau, s, j) * x.vinvT(tau, s, i);
+  }
+}
+
+template <bool kTc, bool RES>
+__device__ __forceinline__ void wrap(Cta<double, RES>& x, int tau, int dir) {
+  const ChainDesc& c = x.c;
+  const bool gz = x.gutz(tau);
+  x.stage(tau);
+  for (int s = 0; s < x.nspec(); ++s) {
+    if (!gz && dir > 0) {
+      wrap_digits(x, s, c.dEm, c.eEm, c.dEp, c.eEp,
+                  [&](int i, int j) { return x.vexpT(tau, s, i) * x.vinvT(tau, s, j); });
+    } else {
+      if (!gz) wrap_digits(x, s, c.dEp, c.eEp, c.dEm, c.eEm, [](int, int) { return 1.0; });
+      scale_slice(x, tau, dir, s);
+    }
+  }
+  __syncthreads();
+}
+
+template <bool kTc, bool RES>
+__device__ __forceinline__ void wrap(Cta<float, RES>& x, int tau, int dir) {
   const ChainDesc& c = x.c;
   const int N = c.N, ld = c.ld;
   const bool gz = x.gutz(tau);
-  T* Gt = x.Gt();
-  if constexpr (std::is_same<T, double>::value) {
-    if (!gz && c.dEm) {
-      x.stage(tau);
-      for (int s = 0; s < x.nspec(); ++s) {
-        if (dir > 0) {
-          wrap_digits(x, s, c.dEm, c.eEm, c.dEp, c.eEp,
-                      [&](int i, int j) { return x.vexpT(tau, s, i) * x.vinvT(tau, s, j); });
-        } else {
-          wrap_digits(x, s, c.dEp, c.eEp, c.dEm, c.eEm, [](int, int) { return 1.0; });
-          T* Gs = x.G(s);
-          PQMC_FOR_2D(i, 0, N, j, 0, N) Gs[(long)i * ld + j] *= x.vexpT(tau, s, j) * x.vinvT(tau, s, i);
-        }
-      }
-      __syncthreads();
-      return;
-    }
-  }
-  const T* Em = x.Em();
-  const T* Ep = x.Ep();
+  float* Gt = x.Gt();
+  const float* Em = x.Em();
+  const float* Ep = x.Ep();
   if (!gz && RES && x.L.em) {
     // a chain resident in shared memory reads e^{-+dtau K} there: the two
     // tables are copied in from the L2-resident copy shared by all chains
     // (the wrap phase leaves room for them in the scratch)
-    const int chunks = N * ld * (int)sizeof(T) / 16;
+    const int chunks = N * ld * (int)sizeof(float) / 16;
     int4* dm = reinterpret_cast<int4*>(x.scr + x.L.em);
     int4* dp = reinterpret_cast<int4*>(x.scr + x.L.ep);
     const int4* sm = reinterpret_cast<const int4*>(Em);
@@ -1506,16 +1511,13 @@ __device__ __forceinline__ void wrap(Cta<T, RES>& x, int tau, int dir) {
       dm[e] = sm[e];
       dp[e] = sp[e];
     }
-    Em = reinterpret_cast<const T*>(dm);
-    Ep = reinterpret_cast<const T*>(dp);
+    Em = reinterpret_cast<const float*>(dm);
+    Ep = reinterpret_cast<const float*>(dp);
     __syncthreads();
   }
   x.stage(tau);
   if (dir > 0) {
-    for (int s = 0; s < x.nspec(); ++s) {
-      T* Gs = x.G(s);
-      PQMC_FOR_2D(i, 0, N, j, 0, N) Gs[(long)i * ld + j] *= x.vexpT(tau, s, i) * x.vinvT(tau, s, j);
-    }
+    for (int s = 0; s < x.nspec(); ++s) scale_slice(x, tau, +1, s);
     __syncthreads();
     if (gz) return;
     // Gt = e^{-dtau K} G, G = Gt e^{+dtau K}
@@ -1534,10 +1536,7 @@ __device__ __forceinline__ void wrap(Cta<T, RES>& x, int tau, int dir) {
         __syncthreads();
       }
     }
-    for (int s = 0; s < x.nspec(); ++s) {
-      T* Gs = x.G(s);
-      PQMC_FOR_2D(i, 0, N, j, 0, N) Gs[(long)i * ld + j] *= x.vexpT(tau, s, j) * x.vinvT(tau, s, i);
-    }
+    for (int s = 0; s < x.nspec(); ++s) scale_slice(x, tau, -1, s);
     __syncthreads();
   }
 }
@@ -2754,7 +2753,7 @@ __global__ void __launch_bounds__(TPB, MINB) init_kernel(const ChainDesc* chains
 }
 
 template <typename T, bool RES, bool kPair, bool kTc>
-__device__ __forceinline__ void run_sweeps(uint32_t sweep0, int n_sweeps, int do_measure, int* err) {
+__device__ __forceinline__ void run_sweeps(uint32_t sweep0, int n_sweeps, int do_measure) {
   auto x = this_cta<T, RES>();
   Smem<T>& sh = x.sh;
   const long long t_start = clock64();
@@ -2764,7 +2763,6 @@ __device__ __forceinline__ void run_sweeps(uint32_t sweep0, int n_sweeps, int do
     if (sh.err) break;
   }
   if (threadIdx.x == 0) sh.cyc[kPhTotal] += clock64() - t_start;
-  (void)err;
 }
 
 template <typename T, int TPB, int MINB>
@@ -2778,7 +2776,7 @@ __global__ void __launch_bounds__(TPB, MINB) sweep_kernel(const ChainDesc* chain
   if (sh.res) {
     auto x = this_cta<T, true>();
     load_state(x);
-    run_sweeps<T, true, kPair, (TPB == 512)>(sweep0, n_sweeps, do_measure, err);
+    run_sweeps<T, true, kPair, (TPB == 512)>(sweep0, n_sweeps, do_measure);
     write_back<T, true>();
     store_state(x, err);
   } else {
@@ -2802,7 +2800,7 @@ __global__ void __launch_bounds__(TPB, MINB) sweep_kernel(const ChainDesc* chain
         __syncthreads();
       }
     }
-    run_sweeps<T, false, kPair, (TPB == 512)>(sweep0, n_sweeps, do_measure, err);
+    run_sweeps<T, false, kPair, (TPB == 512)>(sweep0, n_sweeps, do_measure);
     if constexpr (std::is_same<T, float>::value && TPB == 512) {
       if (sh.tcs_off) tc_free(sh.tmem);
     }
