@@ -2066,7 +2066,7 @@ __device__ __forceinline__ void with_block(Cta<T, RES>& x, int left, int s, F f)
 }
 // M64 = that block, column-major
 template <typename T, bool RES>
-__device__ __forceinline__ void block_to_m64(Cta<T, RES>& x, int b, int left, int s) {
+__device__ __forceinline__ void block_to_m64(Cta<T, RES>& x, int left, int s) {
   const int ldm = m64_ld(x.c.N);
   double* M = x.M64();
   with_block(x, left, s, [&](auto e) {
@@ -2152,7 +2152,7 @@ __device__ __noinline__ void phase_stack(int b, int left, int s) {
   }
   if (threadIdx.x == 0) x.sh.src = src;
   __syncthreads();
-  if (f64) block_to_m64(x, b, left, s);
+  if (f64) block_to_m64(x, left, s);
   x.mark(kPhStack);
 }
 
@@ -2174,6 +2174,76 @@ __device__ __noinline__ int phase_digits(int left, int s, bool gram) {
   x.mark(kPhOverlap);
   return E;
 }
+
+// Up to 16 orbitals the reduced paths' three FP64 products of a stabilisation
+// (Gram matrix, Q, overlap) are FMA loops, one element per thread: the fixed work
+// of a digit tile (packing, fragments, assembly) is more than these few FMAs.
+// ms per sweep by digits and by FMAs, 20 slices: 8 sites x 608 chains 1.65, 1.29; 18
+// sites x 304 1.21, 1.01; 32 sites (n = 16) x 304 1.89, 1.66, packed densely (x 1216, 64
+// threads) 13.5, 10.3; 72 sites with n = 19 4.67, 4.74; 50 sites (n = 25) x 608 6.41, 6.53; 64
+// sites with n = 28 x 256 (120 slices) 21.5, 28.0.  One function for all of it, its loops
+// rolled (dense packing, 32 sites: 11.5 unrolled); what it adds to the code costs
+// the larger chains 0.2 to 0.6%.
+constexpr int kSmallOrbitals = 16;
+template <typename T, bool RES>
+__device__ __forceinline__ bool small_products(const Cta<T, RES>& x) {
+  return x.c.nmax <= kSmallOrbitals;
+}
+
+// C(i, j) = sum_k A[i lda + k] B[j ldb + k] (with upper, only j >= i)
+static __device__ __forceinline__ void small_product(int M, int Nn, int K, const double* A, int lda, const double* B, int ldb,
+                                                     bool upper, double* C, int ldc) {
+#pragma unroll 1
+  for (int e = threadIdx.x; e < M * Nn; e += blockDim.x) {
+    const int i = e / Nn, j = e - i * Nn;
+    if (upper && j < i) continue;
+    const double* a = A + i * lda;
+    const double* b = B + j * ldb;
+    double v0 = 0.0, v1 = 0.0;
+    int k = 0;
+#pragma unroll 1
+    for (; k + 1 < K; k += 2) {
+      v0 = fma(a[k], b[k], v0);
+      v1 = fma(a[k + 1], b[k + 1], v1);
+    }
+    if (k < K) v0 = fma(a[k], b[k], v0);
+    C[i * ldc + j] = v0 + v1;
+  }
+}
+
+// the block of spin s in M64 and, with gram, its Gram matrix
+template <typename T, bool RES>
+__device__ __forceinline__ void small_gram(Cta<T, RES>& x, int left, int s, bool gram) {
+  const int N = x.c.N, n = x.nsig(s);
+  block_to_m64(x, left, s);
+  if (gram) {
+    small_product(n, n, N, x.M64(), m64_ld(N), x.M64(), m64_ld(N), true, x.chol(s), digit_ld(n));
+    __syncthreads();
+  }
+}
+// Q = M R^{-1} from M64: q_ij = (m_ij + sum_{k < j} m_ik (L^{-1})_jk) / sqrt(p_j); log|det R| comes back
+template <typename T, bool RES>
+__device__ __forceinline__ double small_form_q(Cta<T, RES>& x, int s, double* Q) {
+  const int N = x.c.N, n = x.nsig(s), ldc = digit_ld(n), ldm = m64_ld(N);
+  const double* M = x.M64();
+  const double* C = x.chol(s);
+  const double* pv = C + (long)n * ldc + 3 * n;
+  const double* isq = pv + n;
+  if (threadIdx.x < 32) {
+    const double la = warp_sum((int)threadIdx.x < n ? log(pv[threadIdx.x]) : 0.0);
+    if (threadIdx.x == 0) x.sh.red[0] = 0.5 * la;
+  }
+#pragma unroll 1
+  for (int e = threadIdx.x; e < N * n; e += blockDim.x) {
+    const int j = e / N, i = e - j * N;
+    double v = M[j * ldm + i];
+#pragma unroll 1
+    for (int k = 0; k < j; ++k) v = fma(M[k * ldm + i], C[j * ldc + k], v);
+    Q[e] = v * isq[j];
+  }
+  __syncthreads();
+  return x.sh.red[0];
+}
 template <typename T, bool RES>
 __device__ __noinline__ void phase_factor() {
   auto x = this_cta<T, RES>();
@@ -2191,36 +2261,85 @@ template <typename T, bool RES>
 __device__ __noinline__ void phase_householder(int b, int left, int s, double* logabs, double* sgn) {
   auto x = this_cta<T, RES>();
   const int N = x.c.N, n = x.nsig(s);
-  if (!std::is_same<T, double>::value) block_to_m64(x, b, left, s);
+  if (!std::is_same<T, double>::value) block_to_m64(x, left, s);
   qr_householder(x, N, m64_ld(N), n, x.M64(), x.Q64(), *logabs, *sgn);
   copy_block(x.Q64(), stack_block(x, left ? x.c.Lst : x.c.Rst, b, s), N * n);
   x.mark(kPhQR);
+}
+
+// the weight of stack block b of spin s, log|det R| and sign of R given
+template <typename T, bool RES>
+__device__ __forceinline__ void stack_weight(Cta<T, RES>& x, int b, int left, int s, double la, double sg) {
+  const ChainDesc& c = x.c;
+  if (threadIdx.x == 0) {
+    double* lg = left ? c.Llog : c.Rlog;
+    const bool first = left ? b == c.nb : b == 0;
+    const int bp = left ? b + 1 : b - 1;
+    lg[(b * 2 + s) * 2 + 0] = (first ? 0.0 : lg[(bp * 2 + s) * 2 + 0]) + la;
+    lg[(b * 2 + s) * 2 + 1] = (first ? 1.0 : lg[(bp * 2 + s) * 2 + 1]) * sg;
+  }
+  __syncthreads();
+}
+
+// spins whose Cholesky factor broke down
+template <typename T, bool RES>
+__device__ __forceinline__ void householder_fallback(Cta<T, RES>& x, int b, int left, const bool bad[2]) {
+  double la, sg;
+  for (int s = 0; s < x.nspec(); ++s)
+    if (bad[s]) {
+      phase_householder<T, RES>(b, left, s, &la, &sg);
+      stack_weight(x, b, left, s, la, sg);
+    }
+}
+
+template <typename T, bool RES>
+__device__ __forceinline__ void small_overlap(Cta<T, RES>& x, int b) {
+  const int N = x.c.N;
+  for (int s = 0; s < x.nspec(); ++s)
+    small_product(x.nsig(s), x.nsig(s), N, stack_block(x, x.c.Lst, b, s), N, stack_block(x, x.c.Rst, b, s), N, false, x.Ob(s),
+                  x.nsig(s));
+  __syncthreads();
+  x.mark(kPhOverlap);
+}
+
+// Cholesky QR of both species' blocks by the small products, or (left < 0) the overlap
+template <typename T, bool RES>
+__device__ __noinline__ void phase_small(int b, int left) {
+  auto x = this_cta<T, RES>();
+  if (left < 0) {
+    small_overlap(x, b);
+    return;
+  }
+  for (int s = 0; s < x.nspec(); ++s) small_gram(x, left, s, true);
+  x.mark(kPhOverlap);
+  phase_factor<T, RES>();
+  const bool bad[2] = {x.sh.chol_bad[0] != 0, x.sh.chol_bad[1] != 0};
+  for (int s = x.nspec() - 1; s >= 0; --s) {
+    if (bad[s]) continue;
+    if (s < x.nspec() - 1) small_gram(x, left, s, false);   // (M64 holds the last species' block)
+    stack_weight(x, b, left, s, small_form_q(x, s, stack_block(x, left ? x.c.Lst : x.c.Rst, b, s)), 1.0);
+  }
+  x.mark(kPhQRForm);
+  householder_fallback(x, b, left, bad);
 }
 
 // the new stack block b of both species
 template <typename T, bool RES>
 __device__ __forceinline__ void push_block(int b, int left) {
   auto x = this_cta<T, RES>();
-  const ChainDesc& c = x.c;
-  auto weight = [&](int s, double la, double sg) {
-    if (threadIdx.x == 0) {
-      double* lg = left ? c.Llog : c.Rlog;
-      const bool first = left ? b == c.nb : b == 0;
-      const int bp = left ? b + 1 : b - 1;
-      lg[(b * 2 + s) * 2 + 0] = (first ? 0.0 : lg[(bp * 2 + s) * 2 + 0]) + la;
-      lg[(b * 2 + s) * 2 + 1] = (first ? 1.0 : lg[(bp * 2 + s) * 2 + 1]) * sg;
-    }
-    __syncthreads();
-  };
-  double la, sg;
   if constexpr (std::is_same<T, double>::value) {
+    double la, sg;
     for (int s = 0; s < x.nspec(); ++s) {
       phase_stack<T, RES>(b, left, s);
       phase_householder<T, RES>(b, left, s, &la, &sg);
-      weight(s, la, sg);
+      stack_weight(x, b, left, s, la, sg);
     }
   } else {
     for (int s = 0; s < x.nspec(); ++s) phase_stack<T, RES>(b, left, s);
+    if (small_products(x)) {
+      phase_small<T, RES>(b, left);
+      return;
+    }
     int E = 0;
     for (int s = 0; s < x.nspec(); ++s) E = phase_digits<T, RES>(left, s, true);
     phase_factor<T, RES>();
@@ -2229,13 +2348,9 @@ __device__ __forceinline__ void push_block(int b, int left) {
     for (int s = x.nspec() - 1; s >= 0; --s) {
       if (bad[s]) continue;
       if (s < x.nspec() - 1) E = phase_digits<T, RES>(left, s, false);
-      weight(s, phase_form_q<T, RES>(b, left, s, E), 1.0);
+      stack_weight(x, b, left, s, phase_form_q<T, RES>(b, left, s, E), 1.0);
     }
-    for (int s = 0; s < x.nspec(); ++s)
-      if (bad[s]) {
-        phase_householder<T, RES>(b, left, s, &la, &sg);
-        weight(s, la, sg);
-      }
+    householder_fallback(x, b, left, bad);
   }
 }
 
@@ -2440,7 +2555,12 @@ __device__ __noinline__ void phase_assemble(int b, bool record) {
 
 template <typename T, bool RES>
 __device__ __forceinline__ void refresh(int b, bool record) {
-  phase_overlap<T, RES>(b);
+  bool small = false;
+  if constexpr (!std::is_same<T, double>::value) {
+    small = small_products(this_cta<T, RES>());
+    if (small) phase_small<T, RES>(b, -1);
+  }
+  if (!small) phase_overlap<T, RES>(b);
   phase_inverse<T, RES>();
   phase_assemble<T, RES>(b, record);
 }
