@@ -405,8 +405,10 @@ pqmc_status build_ctx(int n, const pqmc_chain_spec* specs, const pqmc_opts* opts
   ctx->off_last = take((size_t)n * kRecord * 8);
   // default CTA size (measured on GB300): the FP64 path packs 4 chains of 64
   // threads per SM, or 2 of 128 or 1 of 256 when the batch leaves the SMs room
-  // (304 chains of 72 sites, 2Theta = 4: 70.6 ms per sweep with 64 threads,
-  // 43.9 with 128, 44.8 with 256);
+  // (ms per sweep with 64 / 128 / 256 threads, 2Theta = 2: 72 sites x 304 chains
+  // 37.4 / 23.1 / 23.5, x 456 42.8 / 44.8 / 35.2, x 608 47.9 / 46.5 / 47.0; 18
+  // sites x 608 at 2Theta = 4 10.0 / 10.2 / 14.9: above two chains per SM none is
+  // ahead throughout, and delay_k = 0 lets the autotuner choose);
   // the reduced paths 2 chains of 256 threads, whose G and
   // scratch then fit in shared memory at 72 sites, and one chain of 512
   // threads per SM once a chain has 128 sites or more (its G lives in global

@@ -135,17 +135,14 @@ PQMC_HDI constexpr size_t flipbuf_bytes(int tsize) {
               4 * (size_t)kMaxDelay * tsize + (size_t)kMaxDelay * 4);
 }
 
-// kd: the delayed-update block of the chain (its update vectors are sized
-// for max(kd, kBlock) flips)
 // leading dimension of the stack phase's FP64 block M in the scratch: odd, so
-// that the Gram matrix's threads, each on its own columns, read different
-// shared-memory banks
+// that threads on different columns read different shared-memory banks
 PQMC_HDI constexpr int m64_ld(int N) { return N | 1; }
+// n rounded up to whole 16-byte vectors of FP32
+PQMC_HDI constexpr int pad4(int n) { return (n + 3) & ~3; }
 // leading dimension of packed digits (digit_gemm.cuh) for K contiguous elements:
 // = 2 mod 8, so that the fragments' 16-byte loads along K and 8-byte loads
 // across it meet few bank conflicts (and K pairs stay 16-byte aligned)
-// n rounded up to whole 16-byte vectors of FP32
-PQMC_HDI constexpr int pad4(int n) { return (n + 3) & ~3; }
 PQMC_HDI constexpr int digit_ld(int K) { return ((K + 5) & ~7) + 2; }
 // packed digits (digit_gemm.cuh): exponents of an operand with a NaN or an
 // infinity and of one that is all zero; a packed zero
@@ -153,6 +150,8 @@ constexpr int kDigitBad = 1 << 20;
 constexpr int kDigitNone = -(1 << 19);
 constexpr unsigned long long kDigitZero = 0x8080808080808080ull;
 
+// kd: the delayed-update block of the chain (its update vectors are sized
+// for max(kd, kBlock) flips)
 PQMC_HDI ScratchLayout scratch_layout(int N, int ld, int n, int tsize, int kd) {
   ScratchLayout L;
   const size_t Nn = (size_t)N * n;

@@ -24,9 +24,11 @@
 //
 // Precision: T (double or float) is the path precision of G, the ratios,
 // the wrap, the delayed updates, the products that advance the stack blocks
-// and the assembly of G from them.  The Householder QR of the stack blocks,
-// the product Q_L^T Q_R, its inverse and the log-determinant / sign are FP64
-// in every path.
+// and the assembly of G from them.  The QR of the stack blocks (Householder on
+// the FP64 path; Cholesky on the reduced paths, Householder where that breaks
+// down), the product Q_L^T Q_R, its inverse and the log-determinant / sign are
+// FP64 in every path.  FP64 products run as exact digit products on the tensor
+// cores where that is faster (digit_gemm.cuh).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -446,10 +448,12 @@ struct Smem {
 
 // One chain CTA: its descriptor, shared memory, and where G and the phase
 // scratch live (RES: shared memory, when they fit; else the chain's global
-// buffers).  Each phase of the sweep is a function of its own (not inlined:
-// ptxas gives every phase the whole register budget, where one inlined kernel
-// spilled) that builds its Cta from the shared-memory base, so that with RES
-// every access is a shared-memory instruction on a 32-bit address.
+// buffers).  Each phase of the sweep is a function of its own (not inlined), so
+// that ptxas gives it the whole register budget, and builds its Cta from the
+// shared-memory base, so that with RES every access is a shared-memory
+// instruction on a 32-bit address.  At 128 registers the FP32 kernels still spill
+// 156 bytes around the calls and up to 104 in a phase (the digit products and
+// the assembly); the FP64 kernels (206 registers) and spread mode's do not.
 template <typename T, bool RES>
 struct Cta {
   static constexpr bool resident = RES;
@@ -599,10 +603,13 @@ __device__ __forceinline__ T uniform_of(uint64_t m53) {
 // Applies the a accepted flips of a block, recorded in fb (global sites
 // gsite, Delta per species cl), to the whole G of every species:
 //     G <- G - (E_S - G_{:,S}) Gamma (1 + (1 - G_SS) Gamma)^{-1} G_{S,:}
-// with G the G of the block start.  X = 1 + (1 - G_SS) Gamma is inverted in
-// place; Hubbard blocks need no pivoting (its pivots
-// are the accepted ratios), the bond blocks of the t-V model pivot on rows
-// (a single end of an accepted bond may have a vanishing ratio).
+// with G the G of the block start (flush_block, t-V blocks; a Hubbard chain
+// swept by the whole GPU takes the middle factor from block_inverse).
+// X = 1 + (1 - G_SS) Gamma is inverted in place; Hubbard blocks need no
+// pivoting (its pivots are the accepted ratios), the bond blocks of the t-V
+// model pivot on rows (a single end of an accepted bond may have a vanishing
+// ratio).
+
 // M = Gamma (1 + (1 - G_SS) Gamma)^{-1} of the a accepted flips of a block
 // into fb.Tu[s] for every species s (collective; G is the G of the block
 // start).  Per pivot the species' first warp finds it, exchanges the rows and
@@ -981,11 +988,6 @@ __device__ __forceinline__ void apply_vectors(Cta<T, RES>& x, int a) {
   x.mark(kPhFlush);
 }
 
-// Hubbard slice: delayed blocks of c.kb sites (8, 16, 32 or 64), each
-// decided in sub-blocks of up to kBlock sites (one warp per spin) and then
-// applied to G at once.  Within a delayed block a later sub-block reads its
-// diagonal block of G corrected by the update vectors of the flips already
-// accepted, G_SS - U_S V_S, so every decision sees the current G.
 // The diagonal block of G at sites i0 .. i0 + nbk - 1, both spins, into
 // fb.Tu (zero beyond nbk), brought up to date by the vectors of the a_done flips the
 // delayed block has accepted so far: G_SS - U_S V_S (collective).
@@ -1288,6 +1290,11 @@ __device__ __noinline__ void phase_apply(int a) {
   apply_vectors(x, a);
 }
 
+// Hubbard slice: delayed blocks of c.kb sites (8, 16, 32 or 64), each
+// decided in sub-blocks of up to kBlock sites (FP32: by one warp, else one warp
+// per spin) and then applied to G at once.  Within a delayed block a later
+// sub-block reads its diagonal block of G corrected by the update vectors of the
+// flips already accepted, G_SS - U_S V_S, so every decision sees the current G.
 template <typename T, bool RES, bool kPair>
 __device__ __forceinline__ void update_slice(int tau, uint32_t sweep) {
   auto x = this_cta<T, RES>();
@@ -1705,19 +1712,23 @@ __device__ __forceinline__ void for_flat4(int n, int N, L load, F f) {
 // orthogonality grows like eps cond(M)^2, Yamamoto et al., ETNA 44 (2015)).
 // With two slices per stabilisation cond(M) stays near 1e2.  The two products,
 // M^T M and M R^{-1}, run on the tensor cores from the digits of M
-// (digit_gemm.cuh); the factor and its inverse come from one elimination of
-// [C | I] on the FP64 pipe.  M(i, k): element of the block.
-// Q goes column-major (ld N) to the stack block.  Returns false, with nothing
-// written, when a
-// pivot falls below 1e-12 of its original diagonal entry (cond(M) above about
-// 1e6); the caller then takes the Householder QR.  R has a positive diagonal,
-// so only log|det R| = (1/2) sum_k log(pivot_k) is returned.
+// (digit_gemm.cuh), or as FMA loops for few orbitals; the factor and its inverse
+// come from one elimination of [C | I] on the FP64 pipe, both spins together, half
+// of the CTA each.  Q goes column-major (ld N) to the stack block.  A block with a
+// pivot below 1e-12 of its original diagonal entry (cond(M) above about 1e6)
+// takes the Householder QR instead.  R has a positive diagonal, so only
+// log|det R| = (1/2) sum_k log(pivot_k) is kept.
 //
-// Both spins go through the elimination together, half of the CTA each.
+// The block's digits share one exponent, so the Gram matrix is off by about
+// N 2^-58 of the largest element squared, and a column smaller by a factor r sees
+// N r^2 2^-58 of its own diagonal.  That is below (r 2^-24)^2, what the FP32
+// products leave of the large columns in the small one, for every N; a pivot
+// that it spoils falls under the limit and takes the Householder QR.
 //
-// 72 sites, n = 36, one chain alone on its SM, both spins: the FP64
-// Gram matrix, factor (two barriers, a division and a row scaling per column)
-// and column-by-column Q took 358 kcycles.
+// 72 sites, n = 36, one chain alone on its SM, both spins, per stabilisation: the
+// Gram matrix, factor (two barriers, a division and a row scaling per column) and
+// column-by-column Q on the FP64 pipe took 358 kcycles; this form takes 187,
+// the overlap included.
 
 // digits of a block into D (ld digit_ld(N)); the exponent comes back
 template <typename T, bool RES, typename Elem>
@@ -2464,12 +2475,6 @@ __device__ __forceinline__ void assemble_spin(Cta<T, RES>& x, int s, const doubl
   __syncthreads();
 }
 
-// G <- 1 - Q_R (Q_L^T Q_R)^{-1} Q_L^T at stabilisation point b; records
-// max |G - G_fresh| when record != 0, and the weight's log|det| and sign.
-// With c.dg64 (reduced paths) the recorded error is max |G - G_FP64|, the
-// propagated G against the same formula assembled in FP64 from the FP64
-// factors; the G that replaces the propagated one is still the
-// path-precision assembly, so the chain itself is unchanged.
 // O_s = Q_L^T Q_R of both spins, from the digits of the two blocks (columns of
 // orthonormal matrices: exponent 1; should an element reach 2, the blocks are
 // packed again against the largest).
@@ -2553,6 +2558,12 @@ __device__ __noinline__ void phase_assemble(int b, bool record) {
   __syncthreads();
 }
 
+// G <- 1 - Q_R (Q_L^T Q_R)^{-1} Q_L^T at stabilisation point b; records
+// max |G - G_fresh| when record != 0, and the weight's log|det| and sign.
+// With c.dg64 (reduced paths) the recorded error is max |G - G_FP64|, the
+// propagated G against the same formula assembled in FP64 from the FP64
+// factors; the G that replaces the propagated one is still the
+// path-precision assembly, so the chain itself is unchanged.
 template <typename T, bool RES>
 __device__ __forceinline__ void refresh(int b, bool record) {
   bool small = false;
