@@ -177,30 +177,34 @@ def fp32_peak_tflops(sm_mhz):
 
 # ---------------------------------------------------------------- our arm
 def sweep_flops(N, n, Ltau, n_stab, acc, prec):
-    """Algorithmic flops per sweep per chain, both spins: (path-precision, FP64).
+    """Flops per sweep per chain, both spins, by the pipe that runs them: (FP32 or BF16X3, FP64, digits).
 
-    Path precision, per interaction slice per spin: wrap 4 N^3, delayed-update
-    flush 2 acc N^3, stack slice products 2 N^2 n.  FP64, per stabilisation per
-    spin, Ltau / n_stab stabilisations per sweep: the QR of the N x n stack
-    block 2 n^2 (N - n/3), the overlap Q_L^T Q_R 2 n^2 N and its inverse 2 n^3
-    (the method's arithmetic, whatever QR variant the kernel runs; the
-    kernel's Cholesky QR on the reduced paths does more, N n (n + 1) + n^3/3
-    + N n^2, and is not counted)."""
-    path = 2 * Ltau * (4 * N ** 3 + 2 * acc * N ** 3 + 2 * N * N * n)
-    stab = (Ltau // n_stab) * 2 * (2 * n * n * (N - n / 3) + 2 * n * n * N + 2 * n ** 3)
-    return path, stab
+    Per interaction slice and spin: wrap 4 N^3, delayed-update product 2 acc N^3,
+    stack slice products 2 N^2 n.  Per stabilisation and spin, Ltau / n_stab of
+    them: overlap Q_L^T Q_R 2 n^2 N, its inverse 2 n^3, and the QR of the N x n
+    stack block: on the FP64 path Householder, 2 n^2 (N - n / 3); on the reduced
+    paths Cholesky, Gram matrix n^2 N, elimination of [C | I] n^3, Q n^2 N.
+    Digits: FP64 products on the tensor cores, counted as the FP64 flops they stand
+    for (36 FP16 multiply-adds each): all but the QR's and the inverse's."""
+    slices = 2 * Ltau * (4 * N ** 3 + 2 * acc * N ** 3 + 2 * N * N * n)
+    stabs = 2 * (Ltau // n_stab)
+    if prec == "fp64":
+        return 0.0, stabs * (2 * n * n * (N - n / 3) + 2 * n ** 3), slices + stabs * 2 * n * n * N
+    return slices, stabs * 3 * n ** 3, stabs * 4 * n * n * N
 
 
 # FP64 peak from the unit counts and the clock: 152 SMs x 2 FP64 FMA lanes per
 # clock x 2 flop x 2070 MHz = 1.26 TFLOP/s, the part's nominal 1.25 TFLOP/s
-# (an FMA-throughput probe on this pool measured 1.2 TFLOP/s).
+# (the library's FMA-throughput probe measures 1.06).  FP16 mma.sync: 1024 multiply-adds
+# per cycle and SM (measured 1023).
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2070e6 / 1e12
+MMA_PEAK_TFLOPS = 152 * 1024 * 2 * 2070e6 / 1e12
 
 # DRAM bytes (read + write) per chain and sweep of the sweep kernel, by
 # (precision, N, Ltau, delayed block, CTA threads), from one ncu capture of
-# that launch shape (profiles/sweep_kernel_gutz72_ncu.md: 304 chains, one
-# sweep, 550.7 + 499.6 MB).
-DRAM_BYTES_PER_CHAIN_SWEEP = {("fp32", 72, 80, 32, 256): (550.736384e6 + 499.562496e6) / 304}
+# that launch shape (profiles/sweep_kernel_gutz72_phases_ncu.md: 304 chains, one
+# sweep, 559.0 + 554.4 MB).
+DRAM_BYTES_PER_CHAIN_SWEEP = {("fp32", 72, 80, 32, 256): (559.01184e6 + 554.353408e6) / 304}
 
 
 def run_ours(a):
@@ -489,18 +493,16 @@ def run_ours(a):
     e2e_value = updates / float(t.item())
     ctx.close()
 
-    # roofline of the sweep kernel (one launch per step): the binding pipe is
-    # FP64 for every path (the stabilisation in the reduced paths, everything
-    # in the FP64 path)
-    path_f, stab_f = sweep_flops(N, N // 2, Ltau, n_stab, res["accept"], head)
+    # roofline of the sweep kernel (one launch per step): the FP64 pipe, which
+    # holds the serial part of the stabilisation, and beside it the FP32 and the tensor pipe
+    fp32_f, fp64_f, digit_f = sweep_flops(N, N // 2, Ltau, n_stab, res["accept"], head)
     launch_s = ms / 1e3 / a.steps
-    fp64_f = stab_f + (path_f if head == "fp64" else 0.0)
     fp64_achieved = fp64_f * a.chains / launch_s / 1e12
-    fp32_achieved = (path_f * a.chains / launch_s / 1e12) if head != "fp64" else 0.0
+    fp32_achieved = fp32_f * a.chains / launch_s / 1e12
+    mma_achieved = 36 * digit_f * a.chains / launch_s / 1e12
     fp32_peak = fp32_peak_tflops(2070.0)
-    # time the two pipes need at their peaks, as a fraction of the launch
-    bound_s = fp64_f * a.chains / (FP64_PEAK_TFLOPS * 1e12) + (
-        path_f * a.chains / (fp32_peak * 1e12) if head != "fp64" else 0.0)
+    # time the FP64 and FP32 pipes need at their peaks, as a fraction of the launch
+    bound_s = fp64_f * a.chains / (FP64_PEAK_TFLOPS * 1e12) + fp32_f * a.chains / (fp32_peak * 1e12)
     shape_key = (head, N, Ltau, r["launch"]["delay_k"], r["launch"]["cta_threads"])
     traffic = (DRAM_BYTES_PER_CHAIN_SWEEP[shape_key] * a.chains if shape_key in DRAM_BYTES_PER_CHAIN_SWEEP
                else None)
@@ -540,7 +542,11 @@ def run_ours(a):
                      "two_pipe_bound_frac": bound_s / launch_s,
                      "fp32_pipe": {"achieved": fp32_achieved, "peak": fp32_peak,
                                    "frac": fp32_achieved / fp32_peak,
-                                   "peak_source": "152 SMs x 128 FP32 lanes x 2 flop x 2070 MHz"}},
+                                   "peak_source": "152 SMs x 128 FP32 lanes x 2 flop x 2070 MHz"},
+                     "tensor_pipe": {"achieved": mma_achieved, "peak": MMA_PEAK_TFLOPS,
+                                     "frac": mma_achieved / MMA_PEAK_TFLOPS,
+                                     "note": "FP64 products as FP16 digit products, 36 FP16 flops per FP64 flop",
+                                     "peak_source": "152 SMs x 1024 FP16 multiply-adds x 2 flop x 2070 MHz (mma.sync)"}},
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d // max(a.steps, 1),
                 "d2h_bytes_per_step": d2h // max(a.steps, 1),
                 "note": "timed: context creation (host FP64 model build, device allocation and clearing, upload "
