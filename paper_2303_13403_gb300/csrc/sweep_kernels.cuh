@@ -2191,10 +2191,10 @@ __device__ __noinline__ int phase_digits(int left, int s, bool gram) {
 // of a digit tile (packing, fragments, assembly) is more than these few FMAs.
 // ms per sweep by digits and by FMAs, 20 slices: 8 sites x 608 chains 1.65, 1.29; 18
 // sites x 304 1.21, 1.01; 32 sites (n = 16) x 304 1.89, 1.66, packed densely (x 1216, 64
-// threads) 13.5, 10.3; 72 sites with n = 19 4.67, 4.74; 50 sites (n = 25) x 608 6.41, 6.53; 64
-// sites with n = 28 x 256 (120 slices) 21.5, 28.0.  One function for all of it, its loops
-// rolled (dense packing, 32 sites: 11.5 unrolled); what it adds to the code costs
-// the larger chains 0.2 to 0.6%.
+// threads) 13.5, 10.1; 72 sites with n = 19 4.67, 4.74; 50 sites (n = 25) x 608 6.41, 6.53; 64
+// sites with n = 28 x 256 (120 slices) 21.5, 28.0.  One function for all of it and one
+// for the product, loops rolled (unrolled and inlined: 11.5 for the dense case),
+// because what they add to the code costs the larger chains 0.1 to 0.2% (inlined 0.2 to 0.6).
 constexpr int kSmallOrbitals = 16;
 template <typename T, bool RES>
 __device__ __forceinline__ bool small_products(const Cta<T, RES>& x) {
@@ -2202,7 +2202,7 @@ __device__ __forceinline__ bool small_products(const Cta<T, RES>& x) {
 }
 
 // C(i, j) = sum_k A[i lda + k] B[j ldb + k] (with upper, only j >= i)
-static __device__ __forceinline__ void small_product(int M, int Nn, int K, const double* A, int lda, const double* B, int ldb,
+static __device__ __noinline__ void small_product(int M, int Nn, int K, const double* A, int lda, const double* B, int ldb,
                                                      bool upper, double* C, int ldc) {
 #pragma unroll 1
   for (int e = threadIdx.x; e < M * Nn; e += blockDim.x) {
