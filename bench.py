@@ -203,8 +203,8 @@ MMA_PEAK_TFLOPS = 152 * 1024 * 2 * 2070e6 / 1e12
 # DRAM bytes (read + write) per chain and sweep of the sweep kernel, by
 # (precision, N, Ltau, delayed block, CTA threads), from one ncu capture of
 # that launch shape (profiles/sweep_kernel_gutz72_phases_ncu.md: 304 chains, one
-# sweep, 559.0 + 554.4 MB).
-DRAM_BYTES_PER_CHAIN_SWEEP = {("fp32", 72, 80, 32, 256): (559.01184e6 + 554.353408e6) / 304}
+# sweep, 560.8 + 554.0 MB).
+DRAM_BYTES_PER_CHAIN_SWEEP = {("fp32", 72, 80, 32, 256): (560.804352e6 + 553.951232e6) / 304}
 
 
 def run_ours(a):
