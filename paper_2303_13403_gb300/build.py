@@ -20,7 +20,7 @@ CPP_SOURCES = ["api.cpp", "model.cpp"]
 def build_id():
     """Hash of the sources: the autotuner's cache holds timings of one build."""
     h = hashlib.sha1()
-    for f in sorted(os.listdir(CSRC)):
+    for f in sorted(f for f in os.listdir(CSRC) if f.endswith((".cu", ".cuh", ".cpp", ".h"))):
         with open(os.path.join(CSRC, f), "rb") as fh:
             h.update(f.encode() + fh.read())
     return h.hexdigest()[:12]
